@@ -73,8 +73,17 @@ enum { DD_F_KL = 1, DD_F_TV = 2, DD_F_KLT = 4 };
  *                 (exponent plus hardware mantissa log) and is within ln2 *
  *                 DD_FAST_LOG_SPREAD + 2^-24 (2 ln k + 2 KL + 2) of the exact
  *                 form; every (row, target) pair whose KL there is below
- *                 DD_TILE_EXACT_BELOW is recomputed in the exact form.  In
- *                 both cases the rows near the target (x = t among them) come
+ *                 DD_TILE_EXACT_BELOW is recomputed in the exact form.  For
+ *                 more than two targets on a map with n_v k_pad >= 2^20 (and
+ *                 without dd_log_poisson_kernel) KL is formed on the tensor
+ *                 cores from BF16 slices of P and log2 P that sum exactly, as
+ *                 e_x - sum_b P[x,b] log P[t,b]; it is as accurate (against
+ *                 64 bits two to three times more, above 0.25), and the
+ *                 pairs below 0.07 are recomputed in the exact form.  The
+ *                 slices (8 bytes an entry of P) are built on the first such
+ *                 call, which synchronizes, and kept with the map; a P with
+ *                 entries outside [0, 2] or row sums above 1.01, or no room
+ *                 for them, keeps the FP32 sums.  In all cases the rows near the target (x = t among them) come
  *                 from the exact form and every value keeps 1e-5 relative
  *                 accuracy.
  *  DD_PREC_BF16X3 KL cross term sum_b P[x,b] log P[t,b] as a tensor-core GEMM
@@ -289,8 +298,8 @@ dd_status dd_sparsify(dd_ctx *ctx, int32_t mesh, double theta, int64_t *kept, in
  * exact KL is +inf and the result is finite and at least 87; KLT is +inf on
  * every boundary row and the result there is at least 50.
  * Memory: the first DD_PREC_FP32 call with T > 2 on a mesh stores a tiled
- * copy of P and of its log2 beside P (2 x 4 n_v k_pad bytes, rounded up to
- * whole tiles; kept until P is recomputed, refined or replaced or the mesh
+ * copy of P beside P (4 n_v k_pad bytes, rounded up to whole tiles; as much
+ * again for its log2 where KL takes the tile pass; kept until P is recomputed, refined or replaced or the mesh
  * unloaded), and every such call stages its targets in the same layout
  * (context scratch, 8 T k_pad bytes rounded up): the pipelined tile pass
  * reads them.  When either does not fit, the call runs the staged tile
@@ -386,11 +395,12 @@ dd_status dd_query(dd_ctx *ctx, int32_t mesh, const int32_t *targets, int32_t T,
  * fields of all items are computed by one persistent launch, then the paths
  * of all items by one tracer launch.  The launch is staged (each item in the
  * tile shape the autotuner picks for it) or pipelined (every item in 128 x 64
- * tiles on the meshes' tiled copies of P, as dd_distance builds them: 2 x 4
- * n_v k_pad bytes per mesh, kept with the mesh; without room for them the
+ * tiles on the meshes' tiled copies of P, as dd_distance builds them: 4 or 8
+ * bytes times n_v k_pad per mesh, kept with the mesh; without room for them the
  * launch stays staged), whichever the autotuner measured faster for the
  * class of the batch (dd_tuning_table).  Same arithmetic as dd_query with
- * FP32: both launches give the same fields, bit for bit.
+ * FP32 (KL on the tensor cores when every map qualifies): both launches give
+ * the same fields, bit for bit.
  *   n_items   number of items (>= 1)
  *   mesh_ids  host [n_items] loaded meshes with a Poisson kernel
  *   T_per     host [n_items] targets per item (>= 1)

@@ -168,11 +168,19 @@ void drop_sparse(DevMesh &m) {
     m.sp_theta = 0.f;
 }
 
+// the operands of the tensor-core KL
+void drop_kl_mma(DevMesh &m) {
+    release(m, m.kl_a, (int64_t)kl_mma_row_bytes(m));
+    release(m, m.kl_ex, (int64_t)kl_mma_ex_bytes(m));
+    m.kl_state = 0;
+}
+
 // what was derived from the stored P (the BF16 split, the row entropies, the
 // sparse rows) goes when P is recomputed or replaced
 void drop_derived(DevMesh &m) {
     release(m, m.LP, m.n_v * m.k_pad * (int64_t)sizeof(float));
     drop_tiled(m);
+    drop_kl_mma(m);
     release(m, m.p_hi, m.n_v * m.kb * 2);
     release(m, m.p_lo, m.n_v * m.kb * 2);
     release(m, m.ex, m.n_v * (int64_t)sizeof(float));
@@ -258,11 +266,30 @@ dd_status fields_into(dd_ctx *ctx, DevMesh &m, const int32_t *d_targets, int32_t
         // targets staged in the same layout make the pipelined tile available
         TiledArgs ta{};
         const TiledArgs *tiled = nullptr;
+        KlMmaArgs ka{};
+        const KlMmaArgs *kl_mma = nullptr;
         // (without room for them the staged tile shapes, which need none, run instead)
         if (T > 2) {
             std::string err;
-            if (prepare_tiled(m, ctx->stream, err) == DD_OK &&
-                ensure_scratch(ctx, S_TSTAGE, tiled_target_bytes(m.k_pad, T)) == DD_OK) {
+            bool mma_ok = false;
+            if (kl && kl_mma_wanted(m)) {
+                if ((st = prepare_kl_mma(m, ctx->stream, &mma_ok, err)) != DD_OK) return set_err(ctx, st, err);
+                if (mma_ok &&
+                    ensure_scratch(ctx, S_KLMMA, kl_mma_target_bytes(m.k_pad, T, kl_mma_tile(T))) != DD_OK) {
+                    cudaGetLastError();
+                    ctx->err.clear();
+                    mma_ok = false;
+                }
+            }
+            if (mma_ok) {
+                ka = KlMmaArgs{m.kl_a, m.kl_ex, reinterpret_cast<uint8_t *>(ctx->scratch[S_KLMMA])};
+                kl_mma = &ka;
+            }
+            const bool tile_logs = kl && !kl_mma;
+            if (!tile_logs && !tv) {
+                // KL from the tensor cores alone: no tile pass
+            } else if (prepare_tiled(m, tile_logs, ctx->stream, err) == DD_OK &&
+                       ensure_scratch(ctx, S_TSTAGE, tiled_target_bytes(m.k_pad, T)) == DD_OK) {
                 float *ts = reinterpret_cast<float *>(ctx->scratch[S_TSTAGE]);
                 ta = TiledArgs{m.pt_p, m.pt_l, ts, ts + tiled_target_bytes(m.k_pad, T) / (2 * sizeof(float)),
                                m.pt_kt};
@@ -273,7 +300,7 @@ dd_status fields_into(dd_ctx *ctx, DevMesh &m, const int32_t *d_targets, int32_t
             }
         }
         launch_fields_fp32(m.P, m.n_v, m.k_pad, stage, T, kl, tv, ctx->d_err, ctx->stream, -1, m.LP != nullptr,
-                           tiled, tile_done);
+                           tiled, tile_done, kl_mma);
     } else if (tile_done) {
         CK(cudaEventRecord(tile_done, ctx->stream), "fields event");
     }
@@ -638,6 +665,7 @@ dd_status dd_log_poisson_kernel(dd_ctx *ctx, int32_t mesh, double tol, int32_t m
         release(*m, m->p_lo, m->n_v * m->kb * 2);
         release(*m, m->ex, m->n_v * (int64_t)sizeof(float));
         drop_tiled(*m);
+        drop_kl_mma(*m);
         m->kb = 0;
         drop_sparse(*m);
         std::string err;
@@ -1157,6 +1185,34 @@ dd_status dd_query_batch(dd_ctx *ctx, int32_t n_items, const int32_t *mesh_ids, 
             q.out_kl = (f_mask & DD_F_KL) ? base : nullptr;
             q.out_tv = (f_mask & DD_F_TV) ? base + ((f_mask & DD_F_KL) ? (int64_t)T_per[i] * m.n_v : 0) : nullptr;
         }
+        // KL from the tensor cores when every map qualifies (and there is room), as in dd_distance
+        bool mma = (f_mask & DD_F_KL) != 0;
+        int32_t max_T = 0;
+        size_t kb_bytes = 0;
+        for (int i = 0; i < n_items && mma; ++i) {
+            std::string err;
+            mma = kl_mma_wanted(*ms[i]);
+            if (mma && (st = prepare_kl_mma(*ms[i], ctx->stream, &mma, err)) != DD_OK) return set_err(ctx, st, err);
+            kb_bytes += kl_mma_target_bytes(ms[i]->k_pad, T_per[i], 64);
+            max_T = std::max(max_T, T_per[i]);
+        }
+        if (mma && ensure_scratch(ctx, S_KLMMA, kb_bytes) != DD_OK) {
+            cudaGetLastError();
+            ctx->err.clear();
+            mma = false;
+        }
+        if (mma) {
+            uint8_t *kb = reinterpret_cast<uint8_t *>(ctx->scratch[S_KLMMA]);
+            for (int i = 0; i < n_items; ++i) {
+                BatchProblem &q = probs[i];
+                q.KA = ms[i]->kl_a;
+                q.kex = ms[i]->kl_ex;
+                q.KB = kb;
+                q.knch = kl_mma_chunks(ms[i]->k_pad);
+                kb += kl_mma_target_bytes(ms[i]->k_pad, T_per[i], 64);
+            }
+        }
+        const bool tile_kl = (f_mask & DD_F_KL) && !mma;      // KL in the tile pass
         const size_t o_tprob = 0, o_tloc = align256(nT * sizeof(int32_t));
         const size_t o_probs = o_tloc + align256(nT * sizeof(int32_t));
         const size_t o_doms = o_probs + align256(n_items * sizeof(BatchProblem));
@@ -1175,9 +1231,11 @@ dd_status dd_query_batch(dd_ctx *ctx, int32_t n_items, const int32_t *mesh_ids, 
                            reinterpret_cast<const int32_t *>(dmeta + o_tloc),
                            reinterpret_cast<const int32_t *>(ctx->scratch[S_TARGETS]), nT, max_k, ctx->stream);
         CK(cudaGetLastError(), "batch staging launch");
-        for (int i = 0; i < n_items; ++i)
-            probs[i].variant = tile_variant_for(probs[i].P, probs[i].n_v, probs[i].k_pad, probs[i].sP, probs[i].sL,
-                                                probs[i].sE, probs[i].T, probs[i].out_kl, probs[i].out_tv, ctx->stream);
+        if (tile_kl || (f_mask & DD_F_TV))
+            for (int i = 0; i < n_items; ++i)
+                probs[i].variant = tile_variant_for(probs[i].P, probs[i].n_v, probs[i].k_pad, probs[i].sP, probs[i].sL,
+                                                probs[i].sE, probs[i].T, tile_kl ? probs[i].out_kl : nullptr,
+                                                probs[i].out_tv, ctx->stream);
         // items: every output tile, larger row extents first for balance
         std::vector<std::pair<int64_t, BatchItem>> order;
         for (int i = 0; i < n_items; ++i) {
@@ -1197,7 +1255,7 @@ dd_status dd_query_batch(dd_ctx *ctx, int32_t n_items, const int32_t *mesh_ids, 
         int64_t tstage_bytes = 0, max_tiles = 0;
         for (int i = 0; i < n_items && pipe_ok; ++i) {
             std::string err;
-            if (prepare_tiled(*ms[i], ctx->stream, err) != DD_OK) pipe_ok = false;
+            if (prepare_tiled(*ms[i], tile_kl, ctx->stream, err) != DD_OK) pipe_ok = false;
             tstage_bytes += (int64_t)tiled_target_bytes(ms[i]->k_pad, T_per[i]);
             max_tiles = std::max<int64_t>(max_tiles, (T_per[i] + 63) / 64 * (tiled_k32(ms[i]->k_pad) / 32));
         }
@@ -1205,22 +1263,25 @@ dd_status dd_query_batch(dd_ctx *ctx, int32_t n_items, const int32_t *mesh_ids, 
             cudaGetLastError();
             pipe_ok = false;
         }
+        // (the tensor-core KL takes the same 128 x 64 items, with or without the tiled copies)
         std::vector<std::pair<int64_t, BatchItem>> order_pipe;
-        if (pipe_ok) {
-            float *ts = reinterpret_cast<float *>(ctx->scratch[S_TSTAGE]);
+        if (pipe_ok || mma) {
+            float *ts = pipe_ok ? reinterpret_cast<float *>(ctx->scratch[S_TSTAGE]) : nullptr;
             for (int i = 0; i < n_items; ++i) {
                 BatchProblem &q = probs[i];
                 const DevMesh &m = *ms[i];
-                const int64_t half = (int64_t)tiled_target_bytes(m.k_pad, T_per[i]) / (2 * sizeof(float));
-                q.PT = m.pt_p;
-                q.LT = m.pt_l;
-                q.kt = m.pt_kt;
-                q.TQ = ts;
-                q.TL = ts + half;
-                ts += 2 * half;
+                if (pipe_ok) {
+                    const int64_t half = (int64_t)tiled_target_bytes(m.k_pad, T_per[i]) / (2 * sizeof(float));
+                    q.PT = m.pt_p;
+                    q.LT = m.pt_l;
+                    q.kt = m.pt_kt;
+                    q.TQ = ts;
+                    q.TL = ts + half;
+                    ts += 2 * half;
+                }
                 for (int64_t xt = 0; xt * 128 < m.n_v; ++xt)
                     for (int at = 0; at * 64 < T_per[i]; ++at)
-                        order_pipe.push_back({m.pt_kt, BatchItem{i, (int32_t)xt, at, 0}});
+                        order_pipe.push_back({tiled_k32(m.k_pad), BatchItem{i, (int32_t)xt, at, 0}});
             }
             std::stable_sort(order_pipe.begin(), order_pipe.end(),
                              [](const std::pair<int64_t, BatchItem> &x, const std::pair<int64_t, BatchItem> &y) {
@@ -1253,16 +1314,19 @@ dd_status dd_query_batch(dd_ctx *ctx, int32_t n_items, const int32_t *mesh_ids, 
         }
         const BatchProblem *dprobs = reinterpret_cast<const BatchProblem *>(dmeta + o_probs);
         int32_t *dcounter = reinterpret_cast<int32_t *>(dmeta + o_counter);
+        const BatchItem *ditems_pipe = reinterpret_cast<const BatchItem *>(dmeta + o_items_pipe);
+        const BatchKlMma kl{ditems_pipe, (int32_t)order_pipe.size(), max_T, ctx->d_err, (f_mask & DD_F_TV) != 0};
+        const BatchKlMma *klp = mma ? &kl : nullptr;
         auto staged = [&]() {
             launch_batch_fields(dprobs, (int32_t)n_items, reinterpret_cast<const BatchItem *>(dmeta + o_items),
-                                (int32_t)order.size(), dcounter, ctx->stream, fix_blocks);
+                                (int32_t)order.size(), dcounter, ctx->stream, fix_blocks, klp);
         };
         auto pipelined = [&]() {
-            launch_batch_fields_pipe(dprobs, (int32_t)n_items, reinterpret_cast<const BatchItem *>(dmeta + o_items_pipe),
-                                     (int32_t)order_pipe.size(), dcounter, ctx->d_err, ctx->stream, fix_blocks,
-                                     max_tiles, (f_mask & DD_F_KL) != 0, (f_mask & DD_F_TV) != 0);
+            launch_batch_fields_pipe(dprobs, (int32_t)n_items, ditems_pipe, (int32_t)order_pipe.size(), dcounter,
+                                     ctx->d_err, ctx->stream, fix_blocks, max_tiles, (f_mask & DD_F_KL) != 0,
+                                     (f_mask & DD_F_TV) != 0, klp);
         };
-        if (pipe_ok && batch_launch_choice(n_items, work, f_mask, staged, pipelined, ctx->stream) == 1)
+        if (pipe_ok && batch_launch_choice(n_items, work, f_mask | (mma ? kBatchTensorKl : 0), staged, pipelined, ctx->stream) == 1)
             pipelined();
         else
             staged();

@@ -637,7 +637,7 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
 }
 
 // P and fast_l2(P) of one row tile x 32 columns into the tiled layout (zero
-// past n_v and k_pad; fast_l2(0) = -127 is finite)
+// past n_v and k_pad; fast_l2(0) = -127 is finite); a null output is left out
 __global__ void tiled_layout_kernel(const float *__restrict__ P, int64_t n_v, int64_t k_pad, int64_t k32,
                                     float *__restrict__ PT, float *__restrict__ LT) {
     __shared__ float t[kTiledRows][33];
@@ -660,8 +660,8 @@ __global__ void tiled_layout_kernel(const float *__restrict__ P, int64_t n_v, in
         const int c = idx / kTiledRows, r = idx % kTiledRows;
         const float v = t[r][c];
         const int64_t o = (xt * k32 + b0 + c) * kTiledRows + r;
-        PT[o] = v;
-        LT[o] = fast_l2(v);
+        if (PT) PT[o] = v;
+        if (LT) LT[o] = fast_l2(v);
     }
 }
 
@@ -1057,7 +1057,7 @@ struct FixSmem {
 template <bool PF>
 __device__ __forceinline__ void fix_rows(const float *__restrict__ P, int64_t n_v, int64_t k_pad, int32_t T,
                                          const float *__restrict__ sL, const float *__restrict__ sE,
-                                         float *__restrict__ out_kl, int64_t x0, FixSmem &sh) {
+                                         float *__restrict__ out_kl, int64_t x0, float below, FixSmem &sh) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int w0 = 0; w0 < T; w0 += kFixTW) {
         const int tw = min(kFixTW, T - w0);
@@ -1072,7 +1072,7 @@ __device__ __forceinline__ void fix_rows(const float *__restrict__ P, int64_t n_
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     const int a = a0 + i;
-                    low[i] = a < tw && x < n_v && out_kl[(int64_t)(w0 + a) * n_v + x] < kTileExactBelow;
+                    low[i] = a < tw && x < n_v && out_kl[(int64_t)(w0 + a) * n_v + x] < below;
                 }
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
@@ -1173,10 +1173,10 @@ __global__ void __launch_bounds__(256, PF ? 3 : 4) fix_kl_rows_kernel(const floa
                                                                      int64_t k_pad, int32_t T,
                                                                      const float *__restrict__ sL,
                                                                      const float *__restrict__ sE,
-                                                                     float *__restrict__ out_kl) {
+                                                                     float *__restrict__ out_kl, float below) {
     __shared__ FixSmem sh;
     build_log_table(sh.tab);
-    fix_rows<PF>(P, n_v, k_pad, T, sL, sE, out_kl, (int64_t)blockIdx.x * kFixRB, sh);
+    fix_rows<PF>(P, n_v, k_pad, T, sL, sE, out_kl, (int64_t)blockIdx.x * kFixRB, below, sh);
 }
 
 // Many problems: CTA g takes row block g of the problems' row blocks in
@@ -1184,7 +1184,7 @@ __global__ void __launch_bounds__(256, PF ? 3 : 4) fix_kl_rows_kernel(const floa
 // a block-wide prefix sum over the problems' row-block counts.
 template <bool PF>
 __global__ void __launch_bounds__(256, PF ? 3 : 4) fix_kl_rows_batch_kernel(const BatchProblem *__restrict__ probs,
-                                                                           int32_t n_probs) {
+                                                                           int32_t n_probs, float below) {
     __shared__ FixSmem sh;
     __shared__ int64_t wsum[8];
     __shared__ int found_prob;
@@ -1218,7 +1218,7 @@ __global__ void __launch_bounds__(256, PF ? 3 : 4) fix_kl_rows_batch_kernel(cons
     }
     if (found_prob < 0) return;
     const BatchProblem &q = probs[found_prob];
-    fix_rows<PF>(q.P, q.n_v, q.k_pad, q.T, q.sL, q.sE, q.out_kl, found_x0, sh);
+    fix_rows<PF>(q.P, q.n_v, q.k_pad, q.T, q.sL, q.sE, q.out_kl, found_x0, below, sh);
 }
 
 // the three shapes the autotuner chooses from
@@ -1276,6 +1276,8 @@ bool fix_prefetch(int64_t blocks) { return blocks <= 3 * (int64_t)num_sms(); }
 // ------------------------------------------------------------------ multi-problem persistent launch
 // Work items are output tiles of several problems (domains); CTAs pull items
 // from an atomic counter, largest rows first, and run the item's tile shape.
+// (KL false: TV alone, for batches whose KL the tensor cores form)
+template <bool KL>
 __global__ void __launch_bounds__(256, 2) batch_tile_kernel(const BatchProblem *__restrict__ probs,
                                                          const BatchItem *__restrict__ items, int32_t n_items,
                                                          int32_t *__restrict__ counter) {
@@ -1294,15 +1296,15 @@ __global__ void __launch_bounds__(256, 2) batch_tile_kernel(const BatchProblem *
         const BatchProblem q = probs[w.prob];
         switch (q.variant) {
             case 0:
-                tile_body<64, 64, 4, 4>(q.P, q.n_v, q.k_pad, q.sP, q.sL, q.sE, nullptr, q.T, q.out_kl, q.out_tv,
+                tile_body<64, 64, 4, 4, KL>(q.P, q.n_v, q.k_pad, q.sP, q.sL, q.sE, nullptr, q.T, q.out_kl, q.out_tv,
                                         (int64_t)w.x_tile * 64, w.a_tile * 64, tsm, tab);
                 break;
             case 1:
-                tile_body<128, 32, 4, 4>(q.P, q.n_v, q.k_pad, q.sP, q.sL, q.sE, nullptr, q.T, q.out_kl, q.out_tv,
+                tile_body<128, 32, 4, 4, KL>(q.P, q.n_v, q.k_pad, q.sP, q.sL, q.sE, nullptr, q.T, q.out_kl, q.out_tv,
                                          (int64_t)w.x_tile * 128, w.a_tile * 32, tsm, tab);
                 break;
             default:
-                tile_body<256, 16, 8, 2>(q.P, q.n_v, q.k_pad, q.sP, q.sL, q.sE, nullptr, q.T, q.out_kl, q.out_tv,
+                tile_body<256, 16, 8, 2, KL>(q.P, q.n_v, q.k_pad, q.sP, q.sL, q.sE, nullptr, q.T, q.out_kl, q.out_tv,
                                          (int64_t)w.x_tile * 256, w.a_tile * 16, tsm, tab);
                 break;
         }
@@ -1381,7 +1383,7 @@ void launch_variant(int v, const float *P, int64_t n_v, int64_t k_pad, const flo
 // The first time a (rows, columns, targets) class is seen, every tile shape
 // runs on the actual problem (three timed launches each, after a warm-up) and
 // the fastest is kept for the class.  Classes: rows and k_pad in powers of
-// two, targets in powers of two up to 256.
+// two, targets in powers of two up to 256, TV alone apart from the rest.
 std::mutex g_tune_mutex;
 std::map<std::tuple<int, int, int>, int> g_tune;
 
@@ -1407,6 +1409,7 @@ int tune_variant(const float *P, int64_t n_v, int64_t k_pad, const float *sP, co
     // the classes of launches with and without the tiled layout are kept apart
     auto key = tune_key(n_v, k_pad, T);
     if (pipe) std::get<2>(key) += 100;
+    if (!out_kl) std::get<2>(key) += 1000;      // TV alone
     {
         std::lock_guard<std::mutex> lock(g_tune_mutex);
         auto it = g_tune.find(key);
@@ -1460,13 +1463,15 @@ size_t tiled_target_bytes(int64_t k_pad, int32_t T) {
     return 2 * (size_t)((T + kTiledRows - 1) / kTiledRows) * (size_t)tiled_k32(k_pad) * kTiledRows * sizeof(float);
 }
 
-dd_status prepare_tiled(DevMesh &m, cudaStream_t s, std::string &err) {
-    if (m.pt_p) return DD_OK;
+dd_status prepare_tiled(DevMesh &m, bool logs, cudaStream_t s, std::string &err) {
+    const bool need_p = !m.pt_p, need_l = logs && !m.pt_l;
+    if (!need_p && !need_l) return DD_OK;
     // row tiles in pairs (a CTA of the wide shape takes two), columns to a multiple of 64
     const int64_t k32 = tiled_k32(m.k_pad), nt = (m.n_v + 2 * kTiledRows - 1) / (2 * kTiledRows) * 2;
     const size_t ne = (size_t)nt * k32 * kTiledRows;
     void *pp = nullptr, *pl = nullptr;
-    if (cudaMalloc(&pp, ne * sizeof(float)) != cudaSuccess || cudaMalloc(&pl, ne * sizeof(float)) != cudaSuccess) {
+    if ((need_p && cudaMalloc(&pp, ne * sizeof(float)) != cudaSuccess) ||
+        (need_l && cudaMalloc(&pl, ne * sizeof(float)) != cudaSuccess)) {
         cudaGetLastError();
         if (pp) cudaFree(pp);
         if (pl) cudaFree(pl);
@@ -1480,23 +1485,28 @@ dd_status prepare_tiled(DevMesh &m, cudaStream_t s, std::string &err) {
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
-        cudaFree(pp);
-        cudaFree(pl);
+        if (pp) cudaFree(pp);
+        if (pl) cudaFree(pl);
         err = std::string("tiled layout launch failed: ") + cudaGetErrorString(e);
         return DD_ECUDA;
     }
-    m.pt_p = (float *)pp;
-    m.pt_l = (float *)pl;
     m.pt_kt = k32;
-    m.owned.push_back(pp);
-    m.owned.push_back(pl);
-    m.bytes += (int64_t)(2 * ne * sizeof(float));
+    if (pp) {
+        m.pt_p = (float *)pp;
+        m.owned.push_back(pp);
+        m.bytes += (int64_t)(ne * sizeof(float));
+    }
+    if (pl) {
+        m.pt_l = (float *)pl;
+        m.owned.push_back(pl);
+        m.bytes += (int64_t)(ne * sizeof(float));
+    }
     return DD_OK;
 }
 
 void launch_fields_fp32(const float *P, int64_t n_v, int64_t k_pad, const float4 *stage, int32_t T, float *out_kl,
                         float *out_tv, int *err_flag, cudaStream_t s, int variant, bool staged_logs,
-                        const TiledArgs *tiled, cudaEvent_t tile_done) {
+                        const TiledArgs *tiled, cudaEvent_t tile_done, const KlMmaArgs *kl_mma) {
     const float *sP = reinterpret_cast<const float *>(stage);
     const float *sL = sP + (int64_t)T * k_pad;
     const float *sE = sL + (int64_t)T * k_pad;
@@ -1524,24 +1534,30 @@ void launch_fields_fp32(const float *P, int64_t n_v, int64_t k_pad, const float4
         if (tile_done) cudaEventRecord(tile_done, s);
         return;
     }
-    if (tiled) {
-        // the staged targets in the tiled layout (P and the target-side log2)
-        KMark km_("tiled_targets_kernel", s);
-        tiled_targets_kernel<<<dim3((unsigned)((T + kTiledRows - 1) / kTiledRows), (unsigned)(tiled->kt / 32)), 256,
-                               0, s>>>(sP, sE, tF, T, k_pad, tiled->kt, tiled->TQ, tiled->TL);
+    // the tile pass: every field asked for, or TV alone when the tensor cores form KL
+    float *tile_kl = kl_mma ? nullptr : out_kl;
+    if (tile_kl || out_tv) {
+        if (tiled) {
+            // the staged targets in the tiled layout (P and the target-side log2)
+            KMark km_("tiled_targets_kernel", s);
+            tiled_targets_kernel<<<dim3((unsigned)((T + kTiledRows - 1) / kTiledRows), (unsigned)(tiled->kt / 32)),
+                                   256, 0, s>>>(sP, sE, tF, T, k_pad, tiled->kt, tiled->TQ, tiled->TL);
+        }
+        const int v = (variant >= 0 && variant < kNumShapes)
+                          ? variant
+                          : tune_variant(P, n_v, k_pad, sP, sL, sE, tF, T, tile_kl, out_tv, s, tiled, err_flag);
+        launch_variant(v, P, n_v, k_pad, sP, sL, sE, tF, T, tile_kl, out_tv, s, tiled, err_flag);
     }
-    const int v = (variant >= 0 && variant < kNumShapes)
-                      ? variant
-                      : tune_variant(P, n_v, k_pad, sP, sL, sE, tF, T, out_kl, out_tv, s, tiled, err_flag);
-    launch_variant(v, P, n_v, k_pad, sP, sL, sE, tF, T, out_kl, out_tv, s, tiled, err_flag);
     if (tile_done) cudaEventRecord(tile_done, s);
     if (out_kl) {
+        if (kl_mma) launch_kl_mma(*kl_mma, sP, n_v, k_pad, T, out_kl, err_flag, s);
+        const float below = kl_mma ? kMmaExactBelow : kTileExactBelow;
         KMark km_("fix_kl_kernel", s);        // the timing hook's name of the exact recompute
         const int64_t blocks = (n_v + kFixRB - 1) / kFixRB;
         if (fix_prefetch(blocks))
-            fix_kl_rows_kernel<true><<<(unsigned)blocks, 256, 0, s>>>(P, n_v, k_pad, T, sL, sE, out_kl);
+            fix_kl_rows_kernel<true><<<(unsigned)blocks, 256, 0, s>>>(P, n_v, k_pad, T, sL, sE, out_kl, below);
         else
-            fix_kl_rows_kernel<false><<<(unsigned)blocks, 256, 0, s>>>(P, n_v, k_pad, T, sL, sE, out_kl);
+            fix_kl_rows_kernel<false><<<(unsigned)blocks, 256, 0, s>>>(P, n_v, k_pad, T, sL, sE, out_kl, below);
     }
 }
 
@@ -1564,59 +1580,68 @@ void launch_batch_stage(const BatchProblem *d_probs, const int32_t *d_tprob, con
     }
 }
 
+namespace {
+// the exact recompute of a batch
+void launch_batch_fix(const BatchProblem *d_probs, int32_t n_probs, int64_t fix_blocks, float below, cudaStream_t s) {
+    if (fix_blocks <= 0) return;
+    KMark km_("fix_kl_batch_kernel", s);      // the timing hook's name of the exact recompute
+    if (fix_prefetch(fix_blocks))
+        fix_kl_rows_batch_kernel<true><<<(unsigned)fix_blocks, 256, 0, s>>>(d_probs, n_probs, below);
+    else
+        fix_kl_rows_batch_kernel<false><<<(unsigned)fix_blocks, 256, 0, s>>>(d_probs, n_probs, below);
+}
+}  // namespace
+
 void launch_batch_fields(const BatchProblem *d_probs, int32_t n_probs, const BatchItem *d_items, int32_t n_items,
-                         int32_t *d_counter, cudaStream_t s, int64_t fix_blocks) {
+                         int32_t *d_counter, cudaStream_t s, int64_t fix_blocks, const BatchKlMma *kl_mma) {
     if (n_items <= 0) return;
     const size_t smem = (size_t)(2 * kTileB + kTileB + 4) * (256 + 16) * sizeof(float);
-    cudaFuncSetAttribute(batch_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_tile_kernel, 256, smem);
-    if (per_sm < 1) per_sm = 1;
-    int64_t grid = (int64_t)num_sms() * per_sm;
-    if (grid > n_items) grid = n_items;
-    cudaMemsetAsync(d_counter, 0, sizeof(int32_t), s);
-    {
+    auto tile = [&](auto kern) {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        int per_sm = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem);
+        if (per_sm < 1) per_sm = 1;
+        int64_t grid = (int64_t)num_sms() * per_sm;
+        if (grid > n_items) grid = n_items;
+        cudaMemsetAsync(d_counter, 0, sizeof(int32_t), s);
         KMark km_("batch_tile_kernel", s);
-        batch_tile_kernel<<<(unsigned)grid, 256, smem, s>>>(d_probs, d_items, n_items, d_counter);
-    }
-    if (fix_blocks > 0) {
-        KMark km_("fix_kl_batch_kernel", s);      // the timing hook's name of the exact recompute
-        if (fix_prefetch(fix_blocks))
-            fix_kl_rows_batch_kernel<true><<<(unsigned)fix_blocks, 256, 0, s>>>(d_probs, n_probs);
-        else
-            fix_kl_rows_batch_kernel<false><<<(unsigned)fix_blocks, 256, 0, s>>>(d_probs, n_probs);
-    }
+        kern<<<(unsigned)grid, 256, smem, s>>>(d_probs, d_items, n_items, d_counter);
+    };
+    if (!kl_mma)
+        tile(batch_tile_kernel<true>);
+    else if (kl_mma->tv)
+        tile(batch_tile_kernel<false>);
+    if (kl_mma) launch_batch_kl_mma(d_probs, n_probs, kl_mma->items, kl_mma->n_items, kl_mma->max_T, kl_mma->err, s);
+    launch_batch_fix(d_probs, n_probs, fix_blocks, kl_mma ? kMmaExactBelow : kTileExactBelow, s);
 }
 
 void launch_batch_fields_pipe(const BatchProblem *d_probs, int32_t n_probs, const BatchItem *d_items,
                               int32_t n_items, int32_t *d_counter, int *err, cudaStream_t s, int64_t fix_blocks,
-                              int64_t max_tiles, bool f_kl, bool f_tv) {
+                              int64_t max_tiles, bool f_kl, bool f_tv, const BatchKlMma *kl_mma) {
     if (n_items <= 0) return;
-    {
-        KMark km_("tiled_targets_kernel", s);
-        batch_tiled_targets_kernel<<<dim3((unsigned)max_tiles, (unsigned)n_probs), 256, 0, s>>>(d_probs);
-    }
-    constexpr size_t smem = (size_t)2 * 6 * 64 * kTiledRows * sizeof(float);
-    cudaMemsetAsync(d_counter, 0, sizeof(int32_t), s);
-    const unsigned grid = (unsigned)std::min<int64_t>(num_sms(), n_items);
-    auto go = [&](auto kern) {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        KMark km_("batch_tile_kernel", s);
-        kern<<<grid, 512, smem, s>>>(d_probs, d_items, n_items, d_counter, err);
-    };
-    if (f_kl && f_tv)
-        go(batch_pipe_kernel<true, true>);
-    else if (f_kl)
-        go(batch_pipe_kernel<true, false>);
-    else
-        go(batch_pipe_kernel<false, true>);
-    if (fix_blocks > 0) {
-        KMark km_("fix_kl_batch_kernel", s);
-        if (fix_prefetch(fix_blocks))
-            fix_kl_rows_batch_kernel<true><<<(unsigned)fix_blocks, 256, 0, s>>>(d_probs, n_probs);
+    if (kl_mma) f_kl = false;        // in the tile pass
+    if (f_kl || f_tv) {
+        {
+            KMark km_("tiled_targets_kernel", s);
+            batch_tiled_targets_kernel<<<dim3((unsigned)max_tiles, (unsigned)n_probs), 256, 0, s>>>(d_probs);
+        }
+        constexpr size_t smem = (size_t)2 * 6 * 64 * kTiledRows * sizeof(float);
+        cudaMemsetAsync(d_counter, 0, sizeof(int32_t), s);
+        const unsigned grid = (unsigned)std::min<int64_t>(num_sms(), n_items);
+        auto go = [&](auto kern) {
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            KMark km_("batch_tile_kernel", s);
+            kern<<<grid, 512, smem, s>>>(d_probs, d_items, n_items, d_counter, err);
+        };
+        if (f_kl && f_tv)
+            go(batch_pipe_kernel<true, true>);
+        else if (f_kl)
+            go(batch_pipe_kernel<true, false>);
         else
-            fix_kl_rows_batch_kernel<false><<<(unsigned)fix_blocks, 256, 0, s>>>(d_probs, n_probs);
+            go(batch_pipe_kernel<false, true>);
     }
+    if (kl_mma) launch_batch_kl_mma(d_probs, n_probs, kl_mma->items, kl_mma->n_items, kl_mma->max_T, kl_mma->err, s);
+    launch_batch_fix(d_probs, n_probs, fix_blocks, kl_mma ? kMmaExactBelow : kTileExactBelow, s);
 }
 
 int64_t fix_row_blocks(int64_t n_v) { return (n_v + kFixRB - 1) / kFixRB; }
@@ -1671,15 +1696,18 @@ std::string tuning_table() {
     for (auto &kv : g_tune) {
         char buf[160];
         const int tk = std::get<2>(kv.first);
-        std::snprintf(buf, sizeof buf, "rows<=2^%d k_pad<=2^%d T<=2^%d%s: %s\n", std::get<0>(kv.first),
-                      std::get<1>(kv.first), tk % 100, tk >= 100 ? " (tiled copy of P)" : "", names[kv.second]);
+        std::snprintf(buf, sizeof buf, "rows<=2^%d k_pad<=2^%d T<=2^%d%s%s: %s\n", std::get<0>(kv.first),
+                      std::get<1>(kv.first), tk % 100, tk % 1000 >= 100 ? " (tiled copy of P)" : "",
+                      tk >= 1000 ? " (TV)" : "", names[kv.second]);
         out += buf;
     }
     for (auto &kv : g_batch_tune) {
         char buf[160];
         const int fm = std::get<0>(kv.first);
         std::snprintf(buf, sizeof buf, "batch of problems<=2^%d n*k*T<=2^%d (%s): %s\n", std::get<1>(kv.first),
-                      std::get<2>(kv.first), fm == 3 ? "KL+TV" : (fm == 1 ? "KL" : "TV"),
+                      std::get<2>(kv.first),
+                      (fm & 3) == 2 ? "TV" : (std::string((fm & 3) == 3 ? "KL+TV" : "KL") +
+                                      ((fm & kBatchTensorKl) ? ", KL on the tensor cores" : "")).c_str(),
                       kv.second ? "pipelined persistent launch" : "staged persistent launch");
         out += buf;
     }

@@ -73,6 +73,12 @@ struct DevMesh {
     // log2 of every entry
     float *pt_p = nullptr, *pt_l = nullptr;
     int64_t pt_kt = 0;
+    // BF16 slices of P in chunk images and e_x in two parts, for the
+    // tensor-core KL of many targets (dd_klmma.cu; built on the first such
+    // request): 0 not built, 1 ready, -1 P does not qualify
+    uint8_t *kl_a = nullptr;
+    float2 *kl_ex = nullptr;
+    int kl_state = 0;
     // sparse fields (dd_sparsify): the threshold relative to the row maximum,
     // the sparsified P as CSR (each row's kept entries in column order), and
     // the exact total of every stored row (for the merged-bin extension)
@@ -123,15 +129,17 @@ struct TiledArgs {
     float *TQ, *TL;              // [ceil(T / 64)][kt][64], filled by launch_fields_fp32
     int64_t kt;
 };
+struct KlMmaArgs;
 int64_t tiled_k32(int64_t k_pad);
 size_t tiled_target_bytes(int64_t k_pad, int32_t T);
-dd_status prepare_tiled(DevMesh &m, cudaStream_t s, std::string &err);
+// logs: the log2 copy too (the KL of the pipelined tile; TV reads P alone)
+dd_status prepare_tiled(DevMesh &m, bool logs, cudaStream_t s, std::string &err);
 // tile_done: null, or an event recorded on s when the many-target tile pass
 // has ended (TV final; KL still to be recomputed near the targets).
 void launch_fields_fp32(const float *P, int64_t n_v, int64_t k_pad, const float4 *stage, int32_t T,
                         float *out_kl, float *out_tv, int *err_flag, cudaStream_t s, int variant = -1,
                         bool staged_logs = false, const TiledArgs *tiled = nullptr,
-                        cudaEvent_t tile_done = nullptr);
+                        cudaEvent_t tile_done = nullptr, const KlMmaArgs *kl_mma = nullptr);
 // One problem of a multi-domain field launch, and one output tile of it.
 struct BatchProblem {
     const float *P;
@@ -144,6 +152,12 @@ struct BatchProblem {
     const float *PT, *LT;
     float *TQ, *TL;
     int64_t kt;
+    // the tensor-core KL: the mesh's row slices and e_x, this problem's target
+    // slices (tiles of 64), chunks of 64 columns (null: KL in the tile pass)
+    const uint8_t *KA;
+    uint8_t *KB;
+    const float2 *kex;
+    int32_t knch;
 };
 struct BatchItem {
     int32_t prob, x_tile, a_tile, pad;
@@ -157,8 +171,15 @@ void launch_batch_stage(const BatchProblem *d_probs, const int32_t *d_tprob, con
                         const int32_t *d_targets, int32_t n_targets, int64_t k_max, cudaStream_t s);
 // tile pass over every item, then the exact recompute by row blocks of every
 // problem with KL output (fix_blocks: the sum of their fix_row_blocks(n_v))
+// (kl_mma: KL comes from launch_batch_kl_mma before the recompute; the tile pass sums TV alone)
+struct BatchKlMma {
+    const BatchItem *items;      // 128 rows x 64 targets
+    int32_t n_items, max_T;
+    int *err;
+    bool tv;                     // TV is asked for
+};
 void launch_batch_fields(const BatchProblem *d_probs, int32_t n_probs, const BatchItem *d_items, int32_t n_items,
-                         int32_t *d_counter, cudaStream_t s, int64_t fix_blocks);
+                         int32_t *d_counter, cudaStream_t s, int64_t fix_blocks, const BatchKlMma *kl_mma = nullptr);
 // The pipelined multi-domain launch: every problem carries its tiled arrays
 // (PT, LT, TQ, TL, kt) and the items are 128-row x 64-target tiles (BatchItem
 // x_tile counts pairs of 64-row tiles); the targets are first put into the
@@ -167,13 +188,40 @@ void launch_batch_fields(const BatchProblem *d_probs, int32_t n_probs, const Bat
 // all problems ask for), then the exact recompute.
 void launch_batch_fields_pipe(const BatchProblem *d_probs, int32_t n_probs, const BatchItem *d_items,
                               int32_t n_items, int32_t *d_counter, int *err, cudaStream_t s, int64_t fix_blocks,
-                              int64_t max_tiles, bool f_kl, bool f_tv);
+                              int64_t max_tiles, bool f_kl, bool f_tv, const BatchKlMma *kl_mma = nullptr);
 int64_t fix_row_blocks(int64_t n_v);
+
+// The KL fields of more than two targets on the tensor cores, as accurate as
+// FP32 sums (dd_klmma.cu).  prepare_kl_mma builds the mesh's operands once;
+// *usable is false where there is no room for them or P does not qualify.
+// launch_kl_mma: the targets' slices into args.B (kl_mma_target_bytes with
+// kl_mma_tile's N), then out_kl [T][n_v]; the values below kMmaExactBelow are
+// then for the exact recompute.
+constexpr float kMmaExactBelow = 0.07f;
+struct KlMmaArgs {
+    const uint8_t *A;
+    const float2 *ex;
+    uint8_t *B;
+};
+bool kl_mma_wanted(const DevMesh &m);
+int32_t kl_mma_chunks(int64_t k_pad);
+int kl_mma_tile(int32_t T);
+size_t kl_mma_target_bytes(int64_t k_pad, int32_t T, int N);
+size_t kl_mma_row_bytes(const DevMesh &m);
+size_t kl_mma_ex_bytes(const DevMesh &m);
+dd_status prepare_kl_mma(DevMesh &m, cudaStream_t s, bool *usable, std::string &err);
+void launch_kl_mma(const KlMmaArgs &args, const float *sP, int64_t n_v, int64_t k_pad, int32_t T, float *out_kl,
+                   int *err, cudaStream_t s);
+// every problem's KL (KA, KB, kex, knch set; items of 128 rows x 64 targets)
+void launch_batch_kl_mma(const BatchProblem *d_probs, int32_t n_probs, const BatchItem *d_items, int32_t n_items,
+                         int32_t max_T, int *err, cudaStream_t s);
 // The autotuner's choice between the staged (0) and the pipelined (1)
 // multi-domain launch: the first time a class of batches is seen (the fields
 // asked for, problems and n k T work in powers of two) both run (a warm-up
 // and two timed launches each, on the caller's stream) and the faster is kept
-// for the class.  DD_BATCH_PIPE=0 or 1 pins the choice.
+// for the class.  DD_BATCH_PIPE=0 or 1 pins the choice.  kBatchTensorKl in
+// f_mask: KL comes from the tensor cores (a class of its own).
+constexpr uint32_t kBatchTensorKl = 8;
 int batch_launch_choice(int32_t n_probs, int64_t work, uint32_t f_mask, const std::function<void()> &staged,
                         const std::function<void()> &pipelined, cudaStream_t s);
 std::string tuning_table();
@@ -247,7 +295,7 @@ void launch_batch_trace(const void *d_doms, const int32_t *d_tdom, const int32_t
 
 // ---------------------------------------------------------------- context
 enum ScratchId { S_TARGETS, S_SOURCES, S_STAGE, S_FIELDS, S_XY, S_LEN, S_STATUS, S_GRAD, S_GEMM, S_META,
-                 S_TSTAGE, S_COUNT };
+                 S_TSTAGE, S_KLMMA, S_COUNT };
 
 struct MeshSlot {
     bool live = false;
