@@ -22,7 +22,7 @@
 // 2^-33 of the chunk's largest entry times the largest log.  After every chunk
 // A is split at multiples of 2^-15: the upper part goes into a total of
 // such multiples (exact below 2^9), the rest and B into a second total.
-// e_x is formed once per mesh in FP64 and kept in the same two parts.
+// e_x is summed once per mesh in pairs of floats and kept in the same two parts.
 //
 // Against 64 bits (KL above 0.07, three obstacle grids of 60 to 140 cells a
 // side) the relative error is 3e-8 .. 7e-8 in the root mean square and at most
@@ -297,33 +297,43 @@ __global__ void __launch_bounds__(320, 1) kl_mma_kernel(const KlOne one, const B
 }
 
 // ---------------------------------------------------------------- operands
-// log2 of a positive normal FP32 number in FP64: Tang's table method (128
-// midpoints; r_j = 1 / c_j rounded to FP32, so m r_j - 1 is exact in FP64) with
-// the Taylor series of log(1 + u) to u^6 (|u| <= 2^-8: below 2^-58 beyond it)
+// log2 of a positive normal FP32 number as hi + lo, hi a multiple of 2^-12 (an
+// FP32 number exactly), |lo| < 2^-7: Tang's table method (128 midpoints c_j,
+// r_j = 1 / c_j rounded) with the Taylor series of log(1 + u), u = m r_j - 1
+// rounded once (|u| <= 2^-8, so to 2^-33).  The pair errs by less than 2^-31.
+// In FP64, of which this part does one operation for 60 in FP32, the logs of a
+// map's slices were most of its first call (201 x 201 cells: 1.0 ms).
 constexpr int kTab = 128;
 struct Log2Tab {
-    float r[kTab];
-    double l[kTab];
+    float r[kTab], h[kTab], l[kTab];
 };
 __device__ __forceinline__ void build_log2_table(Log2Tab &t) {
     for (int j = threadIdx.x; j < kTab; j += blockDim.x) {
         const float r = (float)(1.0 / (1.0 + (j + 0.5) / kTab));
+        const double l = -log2((double)r), h = rint(l * 4096.0) / 4096.0;
         t.r[j] = r;
-        t.l[j] = -log2((double)r);
+        t.h[j] = (float)h;
+        t.l[j] = (float)(l - h);
     }
 }
-__device__ __forceinline__ double log2_exact(float p, const Log2Tab &t) {
+__device__ __forceinline__ float2 log2_pair(float p, const Log2Tab &t) {
     const int i = __float_as_int(p);
     const int j = (i >> 16) & (kTab - 1);
-    const double m = (double)__int_as_float((i & 0x007FFFFF) | 0x3F800000);
-    const double u = fma(m, (double)t.r[j], -1.0);
-    double s = -1.0 / 6.0;
-    s = fma(s, u, 1.0 / 5.0);
-    s = fma(s, u, -1.0 / 4.0);
-    s = fma(s, u, 1.0 / 3.0);
-    s = fma(s, u, -0.5);
-    s = fma(s * u, u, u);
-    return fma(s, 1.4426950408889634074, t.l[j]) + (double)((i >> 23) - 127);
+    const float u = __fmaf_rn(__int_as_float((i & 0x007FFFFF) | 0x3F800000), t.r[j], -1.0f);
+    float s = __fmaf_rn(0.2f, u, -0.25f);
+    s = __fmaf_rn(s, u, 1.0f / 3.0f);
+    s = __fmaf_rn(s, u, -0.5f);
+    const float v = __fmaf_rn(__fmul_rn(s, u), u, u);                       // log(1 + u)
+    // times log2 e as the sum of its rounding and the rest
+    constexpr float c = 1.44269504f, cl = (float)(1.4426950408889634074 - (double)1.44269504f);
+    const float w = __fmaf_rn(v, c, __fmaf_rn(v, cl, t.l[j]));
+    return make_float2((float)((i >> 23) - 127) + t.h[j], w);
+}
+// (s, c) += a: two-sum
+__device__ __forceinline__ void pair_add(float &s, float &c, float a) {
+    const float t = __fadd_rn(s, a), b = __fsub_rn(t, s);
+    c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(a, b)));
+    s = t;
 }
 
 // The slices of P's rows and e_x, one warp per row (rows past n_v: zeros), two
@@ -338,7 +348,7 @@ __global__ void __launch_bounds__(256) kl_rows_kernel(const float *__restrict__ 
     const int lane = threadIdx.x & 31;
     const int64_t nw = (int64_t)gridDim.x * 8;
     for (int64_t x = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); x < n_pad; x += nw) {
-        double e = 0.0;
+        float es = 0.0f, ec = 0.0f;      // this lane's part of e_x, a pair
         float sum = 0.0f;
         bool wrong = false;
         uint8_t *img = A + (x / BM) * nch * A_BYTES + image_at((int)(x % BM), 2 * lane);
@@ -348,8 +358,16 @@ __global__ void __launch_bounds__(256) kl_rows_kernel(const float *__restrict__ 
             if (x < n_v && b < k_pad) p = *reinterpret_cast<const float2 *>(P + x * k_pad + b);   // k_pad is a multiple of 4
             wrong |= !(p.x >= 0.f && p.y >= 0.f && p.x <= 2.f && p.y <= 2.f);
             sum += p.x + p.y;
-            if (p.x >= FLT_MIN) e = fma((double)p.x, log2_exact(p.x, tab), e);
-            if (p.y >= FLT_MIN) e = fma((double)p.y, log2_exact(p.y, tab), e);
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const float pv = i ? p.y : p.x;
+                if (pv >= FLT_MIN) {
+                    const float2 l = log2_pair(pv, tab);
+                    const float a = __fmul_rn(pv, l.x);
+                    ec = __fadd_rn(ec, __fmaf_rn(pv, l.y, __fmaf_rn(pv, l.x, -a)));
+                    pair_add(es, ec, a);
+                }
+            }
             // entries are not negative: their bit patterns order as the numbers do
             unsigned mx = __reduce_max_sync(0xffffffffu, max(__float_as_uint(p.x), __float_as_uint(p.y)));
             // grid 2^-7 of the largest entry's power of two (chunks below 2^-87: of that)
@@ -366,6 +384,7 @@ __global__ void __launch_bounds__(256) kl_rows_kernel(const float *__restrict__ 
                 iq *= 0x1p9f;
             }
         }
+        double e = (double)es + (double)ec;
         for (int o = 16; o > 0; o >>= 1) {
             e += __shfl_xor_sync(0xffffffffu, e, o);
             sum += __shfl_xor_sync(0xffffffffu, sum, o);
@@ -385,17 +404,17 @@ __device__ __forceinline__ void kl_targets_chunk(const float *__restrict__ sP, i
                                                  int c, int32_t nch, uint8_t *__restrict__ B, const Log2Tab &tab) {
     const int lane = threadIdx.x & 31;
     const int64_t b = (int64_t)c * BK + 2 * lane;
-    // log2 as an unevaluated sum of two floats: the slices reach 2^-19 of the
-    // chunk's grid, far above the pair's 2^-48
+    // log2 as a normalised sum of two floats: the slices reach 2^-19 of the
+    // chunk's grid (2^-23 and up), above the pair's error
     float l[2] = {0.f, 0.f}, t[2] = {0.f, 0.f};
     if (a < T && b < k_pad) {
         const float2 p = *reinterpret_cast<const float2 *>(sP + (int64_t)a * k_pad + b);
         const float pv[2] = {p.x, p.y};
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-            const double d = log2_exact(fmaxf(pv[i], FLT_MIN), tab);
-            l[i] = (float)d;
-            t[i] = (float)(d - (double)l[i]);
+            const float2 d = log2_pair(fmaxf(pv[i], FLT_MIN), tab);
+            l[i] = __fadd_rn(d.x, d.y);
+            t[i] = __fsub_rn(d.y, __fsub_rn(l[i], d.x));
         }
     }
     // the chunk's grid, 2^-7 of the largest magnitude's power of two among those up to 32
@@ -475,18 +494,16 @@ dd_status prepare_kl_mma(DevMesh &m, cudaStream_t s, bool *usable, std::string &
     const int64_t nt = (m.n_v + BM - 1) / BM;
     const size_t abytes = (size_t)nt * nch * A_BYTES, ebytes = (size_t)nt * BM * sizeof(float2);
     uint8_t *a = nullptr, *e = nullptr;
-    int *bad = nullptr;
     auto drop = [&]() {
         if (a) cudaFree(a);
         if (e) cudaFree(e);
-        if (bad) cudaFree(bad);
     };
-    if (cudaMalloc((void **)&a, abytes) != cudaSuccess || cudaMalloc((void **)&e, ebytes) != cudaSuccess ||
-        cudaMalloc((void **)&bad, sizeof(int)) != cudaSuccess) {
+    if (cudaMalloc((void **)&a, abytes) != cudaSuccess || cudaMalloc((void **)&e, ebytes + sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
         drop();
         return DD_OK;      // no room: the FP32 tile kernels, which need none, run instead
     }
+    int *bad = reinterpret_cast<int *>(e + ebytes);
     int flag = 0;
     cudaError_t ce = cudaMemsetAsync(bad, 0, sizeof(int), s);
     if (ce == cudaSuccess) {
@@ -502,8 +519,6 @@ dd_status prepare_kl_mma(DevMesh &m, cudaStream_t s, bool *usable, std::string &
         err = std::string("slicing P for the tensor-core KL failed: ") + cudaGetErrorString(ce);
         return DD_ECUDA;
     }
-    cudaFree(bad);
-    bad = nullptr;
     if (flag) {
         drop();
         m.kl_state = -1;
