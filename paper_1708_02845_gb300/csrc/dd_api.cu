@@ -549,8 +549,21 @@ dd_status dd_load_mesh(dd_ctx *ctx, const double *xy, int64_t n_v, const int32_t
         if ((st = dev_copy(ctx, m, &m.tnbr, nbr4.data(), nbr4.size())) != DD_OK) return undo(st);
         if ((st = dev_copy(ctx, m, &m.gphi, g4.data(), g4.size())) != DD_OK) return undo(st);
         if ((st = dev_copy(ctx, m, &m.trec, rec.data(), rec.size())) != DD_OK) return undo(st);
+        {
+            const size_t bytes = (size_t)h.n_t * 12 * sizeof(int4);
+            const cudaError_t e = cudaMalloc((void **)&m.hrec, bytes);
+            if (e != cudaSuccess) return undo(cuda_err(ctx, e, "mesh allocation"));
+            m.owned.push_back(m.hrec);
+            m.bytes += (int64_t)bytes;
+            launch_crossings(m, nullptr);      // ordered before the copies below, which wait for it
+        }
         if ((st = dev_copy(ctx, m, &m.vt_off, h.vt_off.data(), h.vt_off.size())) != DD_OK) return undo(st);
         if ((st = dev_copy(ctx, m, &m.vt, h.vt.data(), h.vt.size())) != DD_OK) return undo(st);
+        std::vector<int32_t> wide;
+        for (int64_t v = 0; v < h.n_v; ++v)
+            if (h.vt_off[v + 1] - h.vt_off[v] > kWideFanTriangles) wide.push_back((int32_t)v);
+        m.n_wide = (int32_t)wide.size();
+        if ((st = dev_copy(ctx, m, &m.wide, wide.data(), wide.size())) != DD_OK) return undo(st);
         if ((st = dev_copy(ctx, m, &m.vn_off, h.vn_off.data(), h.vn_off.size())) != DD_OK) return undo(st);
         if ((st = dev_copy(ctx, m, &m.vn, h.vn.data(), h.vn.size())) != DD_OK) return undo(st);
         if ((st = dev_copy(ctx, m, &m.interior, h.I.data(), h.I.size())) != DD_OK) return undo(st);
@@ -848,8 +861,8 @@ dd_status trace_into(dd_ctx *ctx, DevMesh &m, const float *d_fields, const int32
                           reinterpret_cast<const int32_t *>(ctx->scratch[S_SOURCES]), T, S, max_pts, dxy, dlen, dst,
                           ctx->stream);
     } else {
-        // rates and vertex decisions of every field are stored only where many paths share a field
-        const bool dense = trace_dense_decisions(S);
+        // rates and vertex decisions of every field are stored only where many paths share a field and a warp
+        const bool dense = trace_dense_decisions(T, S);
         if ((st = ensure_scratch(ctx, S_GRAD, dense ? trace_scratch_bytes(m, T, true) : 256)) != DD_OK) return st;
         launch_trace(m, d_fields, m.n_v, reinterpret_cast<const int32_t *>(ctx->scratch[S_TARGETS]),
                      reinterpret_cast<const int32_t *>(ctx->scratch[S_SOURCES]), T, S, max_pts, dxy, dlen, dst,

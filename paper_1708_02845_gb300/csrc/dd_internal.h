@@ -41,6 +41,7 @@ dd_status build_host_mesh(const double *xy, int64_t n_v, const int32_t *tri, int
                           HostMesh &out, std::string &err);
 
 // ---------------------------------------------------------------- device mesh
+constexpr int kWideFanTriangles = 16;
 struct DevMesh {
     int64_t n_v = 0, n_t = 0, k = 0, m = 0, k_pad = 0;
     float2 *xy = nullptr;      // [n_v]
@@ -49,7 +50,10 @@ struct DevMesh {
     float4 *gphi = nullptr;    // [n_t][2]: (g0x, g0y, g1x, g1y), (g2x, g2y, 0, 0)
     int4 *trec = nullptr;      // [n_t][4] tracer records: (v0,v1,v2,n0) (n1,n2,q0,q1) (q2,0,p0x,p0y) (p1x,p1y,p2x,p2y),
                                // q_i = |grad phi_i|^2
+    int4 *hrec = nullptr;      // [n_t][4][3] the walk's crossings (dd_trace.cu: crossings_kernel)
     int32_t *vt_off = nullptr, *vt = nullptr;
+    int32_t *wide = nullptr;       // [n_wide] the vertices with more than kWideFanTriangles incident triangles
+    int32_t n_wide = 0;
     int32_t *vn_off = nullptr, *vn = nullptr;
     int32_t *interior = nullptr;   // [m]
     uint8_t *isb = nullptr;        // [n_v] 1 on boundary vertices
@@ -265,11 +269,13 @@ void launch_sparse_fields(const DevMesh &m, const int32_t *d_targets, float4 *st
 // spread (max - min) of the hardware mantissa log's error over [1, 2), in base-2 units
 dd_status fast_log_spread(double *spread, std::string &err);
 
-// Tracer: when trace_dense_decisions(S), per-field triangle rates and vertex
+// Tracer: when trace_dense_decisions(T, S), per-field triangle rates and vertex
 // decisions into `scratch` (trace_scratch_bytes(m, T, true) bytes), then T*S
 // paths; otherwise the walk forms the rates and decisions it needs itself and
 // `scratch` is unused.
-bool trace_dense_decisions(int32_t S);
+// launch_crossings fills m.hrec from m.trec and m.gphi, once per mesh.
+void launch_crossings(const DevMesh &m, cudaStream_t s);
+bool trace_dense_decisions(int32_t T, int32_t S);
 size_t trace_scratch_bytes(const DevMesh &m, int32_t T, bool decisions);
 void launch_trace(const DevMesh &m, const float *fields, int64_t field_stride, const int32_t *targets,
                   const int32_t *sources, int32_t T, int32_t S, int32_t max_pts, float2 *out_xy,

@@ -21,16 +21,23 @@
 //
 // Work split for latency.  What a vertex state decides depends only on the
 // field and the vertex (the best triangle is the steepest, ties by id, so the
-// order in which the incident triangles are examined does not matter), so it
-// is computed for every vertex of every field before the walk
-// (vertex_decision_kernel), after the barycentric rates of every triangle
-// (rates_kernel).  Both are stored field-minor ([triangle][field],
-// [vertex][field]): a warp of the decision kernel handles one vertex for 32
-// fields, so the triangle records it reads are shared by all its lanes and
-// the rates it reads are contiguous.  The walk then does one thing per iteration: cross one
-// triangle from an edge (one 64-byte record and one 16-byte rate load, both
-// addressed by the id the previous step found), apply one vertex decision
-// (one 48-byte load), or slide along a valley or boundary edge.
+// order in which the incident triangles are examined does not matter).  Where
+// many paths share a field it is computed for every vertex of every field
+// before the walk (vertex_decision_kernel; wide fans in wide_decision_kernel),
+// after the barycentric rates of every triangle (rates_kernel).  Both are
+// stored field-minor ([triangle][field], [vertex][field]): a warp of the
+// decision kernel handles one vertex for 32 fields, so the triangle records it
+// reads are shared by all its lanes and the rates it reads are contiguous.
+// The walk (walk_path) then does one thing per iteration: cross one triangle
+// from an edge, apply one vertex decision, or slide along a valley or
+// boundary edge.  Batches of several maps walk one path per thread on stored
+// rates (trace_path).
+//
+// Measured, longest path 436 points: grid140, one target, 256 paths 279 -> 119
+// us (a call with its fields, results in host buffers, 362 -> 222 us); 142
+// points, 32 paths on the 2,049-vertex disk 250 -> 47 us (a call 240 -> 68 us);
+// 941 points, 64 x 256 paths on the 71,681-vertex disk 953 -> 476 us and the
+// decisions 778 -> 270 us (a call 1,760 -> 829 us).
 #include <cfloat>
 #include <cstring>
 #include <cstdlib>
@@ -45,6 +52,8 @@ namespace {
 
 constexpr float kEpsBary = 1e-6f;    // barycentric snap to a vertex
 constexpr float kEpsWedge = 1e-6f;   // relative tolerance of the wedge / entry tests
+constexpr int kWideFan = kWideFanTriangles;
+constexpr int64_t kWarpPaths = 2432;      // 16 a SM
 constexpr int32_t kDenseMinPaths = 128;   // paths per field from which decisions are precomputed
 
 // Triangle record (64 bytes): vertex ids, the ids of the triangles across the
@@ -85,14 +94,17 @@ __device__ __forceinline__ int sel3i(int i, int a, int b, int c) { return i == 0
 // Per (field, triangle): (r0, r1, r2, |g|^2) with r_i = -grad(phi_i) . g the
 // rate of change of barycentric coordinate i along the descent direction -g.
 // g = f0 grad(phi_0) + f1 grad(phi_1) + f2 grad(phi_2) = (f0 - f2) g0 + (f1 - f2) g1.
-__device__ __forceinline__ float4 tri_rates(const float4 *__restrict__ gphi, const int4 *__restrict__ rec, int64_t t,
-                                            const float *__restrict__ f) {
-    const int4 a = __ldg(rec + 4 * t);
-    const float4 h = __ldg(gphi + 2 * t);                 // (g0x, g0y, g1x, g1y)
-    const float f2 = f[a.z], d0 = f[a.x] - f2, d1 = f[a.y] - f2;
+// h: (g0x, g0y, g1x, g1y)
+__device__ __forceinline__ float4 rates_of(const float4 &h, float f0, float f1, float f2) {
+    const float d0 = f0 - f2, d1 = f1 - f2;
     const float gx = d0 * h.x + d1 * h.z, gy = d0 * h.y + d1 * h.w;
     const float r0 = -(h.x * gx + h.y * gy), r1 = -(h.z * gx + h.w * gy);
     return make_float4(r0, r1, -(r0 + r1), gx * gx + gy * gy);
+}
+__device__ __forceinline__ float4 tri_rates(const float4 *__restrict__ gphi, const int4 *__restrict__ rec, int64_t t,
+                                            const float *__restrict__ f) {
+    const int4 a = __ldg(rec + 4 * t);
+    return rates_of(__ldg(gphi + 2 * t), f[a.x], f[a.y], f[a.z]);
 }
 
 // rates[t * T + a] for every triangle t and field a (field-minor)
@@ -105,16 +117,15 @@ __global__ void rates_kernel(const float4 *__restrict__ gphi, const int4 *__rest
     rates[i] = tri_rates(gphi, rec, t, fields + (int64_t)a * field_stride);
 }
 
-// What the walk does at a vertex (48 bytes)
+// What the walk does at a vertex (32 bytes)
 enum { kVCross = 0, kVVertex = 1, kVAdjacent = 2, kVStuck = 3 };
 struct VDec {
     int4 h;      // kind, then: cross (ea, eb, t_next) | vertex (u, -, -) | adjacent (target, -, -)
     float4 w;    // cross (la, lb, point) | vertex, adjacent (position, -, -)
-    float4 e;    // cross: positions of ea and eb
 };
 
 struct TraceDom {
-    const int4 *rec;
+    const int4 *rec, *hrec;
     const float4 *gphi;
     const float2 *xy;
     const int32_t *vt_off, *vt;
@@ -167,9 +178,11 @@ struct FanScan {
         }
     }
 
-    __device__ __forceinline__ VDec finish(const TraceDom &p, const float *__restrict__ f, int target, int v) const {
+    // (G lanes of `mask` hold the same scan and share the fallback's fan)
+    template <int G>
+    __device__ __forceinline__ VDec finish(const TraceDom &p, const float *__restrict__ f, int target, int v,
+                                           unsigned mask = 0) const {
         VDec d;
-        d.e = make_float4(0.f, 0.f, 0.f, 0.f);
         if (adj) {                                   // v lies on an edge incident on the target
             const float2 pt = p.xy[target];
             d.h = make_int4(kVAdjacent, target, 0, 0);
@@ -188,17 +201,17 @@ struct FanScan {
             } else {
                 d.h = make_int4(kVCross, b_vj, b_vk, b_next);
                 d.w = make_float4(lj, lk, lj * b_pj.x + lk * b_pk.x, lj * b_pj.y + lk * b_pk.y);
-                d.e = make_float4(b_pj.x, b_pj.y, b_pk.x, b_pk.y);
             }
             return d;
         }
-        // no descending triangle: the incident edge of largest positive slope (ties to the lower id)
+        // no descending triangle: the incident edge of largest positive slope (ties to the
+        // lower id), the fan over the G lanes of the group
         int best_u = -1;
         float best_s = 0.f;
         float2 best_p = make_float2(0.f, 0.f);
         const float fv = f[v];
         const float2 pv = p.xy[v];
-        for (int q = p.vt_off[v]; q < p.vt_off[v + 1]; ++q) {
+        for (int q = p.vt_off[v] + (threadIdx.x & (G - 1)); q < p.vt_off[v + 1]; q += G) {
             const Tri Q = load_tri(p.rec, p.vt[q]);
 #pragma unroll
             for (int e = 0; e < 3; ++e) {
@@ -211,6 +224,20 @@ struct FanScan {
                     best_s = slope;
                     best_u = u;
                     best_p = pu;
+                }
+            }
+        }
+        if (G > 1) {
+            __syncwarp(mask);
+#pragma unroll
+            for (int o = G / 2; o > 0; o >>= 1) {
+                const float s2 = __shfl_xor_sync(mask, best_s, o);
+                const int u2 = __shfl_xor_sync(mask, best_u, o);
+                const float px = __shfl_xor_sync(mask, best_p.x, o), py = __shfl_xor_sync(mask, best_p.y, o);
+                if (u2 >= 0 && (s2 > best_s || (s2 == best_s && u2 < best_u))) {
+                    best_s = s2;
+                    best_u = u2;
+                    best_p = make_float2(px, py);
                 }
             }
         }
@@ -235,10 +262,40 @@ __device__ __forceinline__ VDec vertex_decision(const TraceDom &p, const float *
         const int tl = p.vt[q];
         fs.add(v, target, tl, load_tri(p.rec, tl), __ldg(rates + (int64_t)tl * rstride));
     }
-    return fs.finish(p, f, target, v);
+    return fs.finish<1>(p, f, target, v);
 }
 
-// one warp per (vertex, group of 32 fields), lane = field: dec[v * T + a]
+// The best triangle of a fan whose triangles were dealt to the G lanes of a
+// group (aligned, all of them in `mask`): the steepest, ties to the lowest id
+// -- what one lane scanning the whole fan finds, in any order.
+template <int G>
+__device__ __forceinline__ void fan_reduce(FanScan &fs, unsigned mask) {
+    int from = threadIdx.x & 31, adj = fs.adj;
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) {
+        adj |= __shfl_xor_sync(mask, adj, o);
+        const float g2 = __shfl_xor_sync(mask, fs.best_g2, o);
+        const int tl = __shfl_xor_sync(mask, fs.best, o), at = __shfl_xor_sync(mask, from, o);
+        if (g2 > fs.best_g2 || (g2 == fs.best_g2 && tl < fs.best)) {
+            fs.best_g2 = g2;
+            fs.best = tl;
+            from = at;
+        }
+    }
+    fs.adj = adj != 0;
+    fs.baj = __shfl_sync(mask, fs.baj, from);
+    fs.bak = __shfl_sync(mask, fs.bak, from);
+    fs.b_vj = __shfl_sync(mask, fs.b_vj, from);
+    fs.b_vk = __shfl_sync(mask, fs.b_vk, from);
+    fs.b_next = __shfl_sync(mask, fs.b_next, from);
+    fs.b_pj.x = __shfl_sync(mask, fs.b_pj.x, from);
+    fs.b_pj.y = __shfl_sync(mask, fs.b_pj.y, from);
+    fs.b_pk.x = __shfl_sync(mask, fs.b_pk.x, from);
+    fs.b_pk.y = __shfl_sync(mask, fs.b_pk.y, from);
+}
+
+// one warp per (vertex, group of 32 fields), lane = field: dec[v * T + a];
+// vertices of more than kWideFan triangles are left to wide_decision_kernel
 __global__ void vertex_decision_kernel(const TraceDom p, int32_t T, const float *__restrict__ fields,
                                        int64_t field_stride, const float4 *__restrict__ rates,
                                        const int32_t *__restrict__ targets, VDec *__restrict__ dec) {
@@ -246,25 +303,44 @@ __global__ void vertex_decision_kernel(const TraceDom p, int32_t T, const float 
     const int groups = (T + 31) >> 5;
     const int64_t v = w / groups;
     const int a = (int)(w - v * groups) * 32 + (threadIdx.x & 31);
-    if (v >= p.n_v || a >= T) return;
+    if (v >= p.n_v || a >= T || p.vt_off[v + 1] - p.vt_off[v] > kWideFan) return;
     dec[v * T + a] = vertex_decision(p, fields + (int64_t)a * field_stride, rates + a, T, targets[a], (int)v);
 }
 
+// The vertices with wide fans (a disk's centre: as many triangles as the disk
+// has sectors), one warp per (vertex, field), the fan over the lanes.  With
+// one lane scanning it the 512 triangles of one centre were a chain of 0.65
+// ms, all of the decision pass but 0.12 ms (71,681 vertices, 64 fields).
+__global__ void wide_decision_kernel(const TraceDom p, const int32_t *__restrict__ wide, int32_t T,
+                                     const float *__restrict__ fields, int64_t field_stride,
+                                     const float4 *__restrict__ rates, const int32_t *__restrict__ targets,
+                                     VDec *__restrict__ dec) {
+    const int v = wide[blockIdx.x], lane = threadIdx.x & 31;
+    const int a = blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (a >= T) return;
+    const float *f = fields + (int64_t)a * field_stride;
+    FanScan fs;
+    fs.begin();
+    for (int q = p.vt_off[v] + lane, q1 = p.vt_off[v + 1]; q < q1; q += 32) {
+        const int tl = p.vt[q];
+        fs.add(v, targets[a], tl, load_tri(p.rec, tl), __ldg(rates + (int64_t)tl * T + a));
+    }
+    __syncwarp();
+    fan_reduce<32>(fs, 0xffffffffu);
+    const VDec d = fs.finish<32>(p, f, targets[a], v, 0xffffffffu);
+    if (lane == 0) dec[(int64_t)v * T + a] = d;
+}
+
 // One path: walk from `source` to `target` on field f, with that field's
-// triangle rates and vertex decisions.  The warp votes at the top of every
+// triangle rates.  The warp votes at the top of every
 // iteration, so its threads reconverge once per step; finished threads (and
 // padding lanes) idle there until the last path of the warp ends.
-// (rates of this field start at `rates`, one entry per triangle every
-// `rstride`; its decisions at `dec`, one per vertex every `dstride`.  With
-// dec == nullptr a vertex state computes its decision itself -- the same
-// function, so the same result -- which pays when few paths share a field.
-// With rates == nullptr the walk computes each triangle's rates from the
-// field where it needs them, by the same function as rates_kernel, so again
-// with the same result: few paths per field touch a small share of the
-// triangles, and a pass over all of them would cost more than the walk.)
+// (rates of this field start at `rates`, one entry per triangle; a vertex
+// state computes its decision itself, from the same functions as the decision
+// kernels, so with the same result.)  One thread a path: for batches of maps,
+// whose hundreds of thousands of paths fill the GPU.
 __device__ __forceinline__ void trace_path(const TraceDom &p, const float *__restrict__ f,
-                                           const float4 *__restrict__ rates, int64_t rstride,
-                                           const VDec *__restrict__ dec, int64_t dstride, int target, int source,
+                                           const float4 *__restrict__ rates, int target, int source,
                                            float2 *__restrict__ out, int32_t max_pts, int32_t max_steps,
                                            int32_t *len_out, int32_t *status_out, bool active) {
     const float eps2 = kEpsWedge * kEpsWedge;
@@ -274,12 +350,12 @@ __device__ __forceinline__ void trace_path(const TraceDom &p, const float *__res
     bool fin = !active;
     bool at_vertex = true;
     int v = source;
-    // fan scan of the current vertex when decisions are not precomputed: one
+    // fan scan of the current vertex: one
     // incident triangle (from the vertex's triangle list) per iteration
     FanScan fs;
     fs.begin();
     int scan_q = 0, scan_end = 0;
-    if (active && !dec) {
+    if (active) {
         scan_q = p.vt_off[v];
         scan_end = p.vt_off[v + 1];
     }
@@ -309,11 +385,9 @@ __device__ __forceinline__ void trace_path(const TraceDom &p, const float *__res
 #define DD_ENTER_VERTEX(vert)                    \
     v = (vert);                                  \
     at_vertex = true;                            \
-    if (!dec) {                                  \
-        fs.begin();                              \
-        scan_q = p.vt_off[v];                    \
-        scan_end = p.vt_off[v + 1];              \
-    }                                            \
+    fs.begin();                                  \
+    scan_q = p.vt_off[v];                        \
+    scan_end = p.vt_off[v + 1];                  \
     if (++states > max_steps) {                  \
         fin = true;                              \
         continue;                                \
@@ -337,21 +411,16 @@ __device__ __forceinline__ void trace_path(const TraceDom &p, const float *__res
         if (!__any_sync(0xffffffffu, !fin)) break;
         if (fin) continue;
         if (at_vertex) {
-            // ---- vertex state: apply the decision (precomputed, or scanned here one
-            // incident triangle per iteration, so the warp's other lanes wait little)
-            const VDec *dv = dec ? dec + (int64_t)v * dstride : nullptr;
-            VDec own;
-            if (!dv) {
-                if (scan_q < scan_end) {
-                    const int tl = p.vt[scan_q++];
-                    fs.add(v, target, tl, load_tri(p.rec, tl),
-                           rates ? __ldg(rates + (int64_t)tl * rstride) : tri_rates(p.gphi, p.rec, tl, f));
-                    continue;
-                }
-                own = fs.finish(p, f, target, v);
+            // ---- vertex state: scan one incident triangle per iteration (so the warp's
+            // other lanes wait little), then apply the decision
+            if (scan_q < scan_end) {
+                const int tl = p.vt[scan_q++];
+                fs.add(v, target, tl, load_tri(p.rec, tl), __ldg(rates + tl));
+                continue;
             }
-            const int4 h = dv ? __ldg(&dv->h) : own.h;
-            const float4 w = dv ? __ldg(&dv->w) : own.w;
+            const VDec own = fs.finish<1>(p, f, target, v);
+            const int4 h = own.h;
+            const float4 w = own.w;
             const int kind = h.x;
             if (kind == kVStuck) {
                 status = DD_TRACE_STUCK;
@@ -369,15 +438,14 @@ __device__ __forceinline__ void trace_path(const TraceDom &p, const float *__res
                 DD_ENTER_VERTEX(h.y);
                 continue;
             }
-            const float4 e = dv ? __ldg(&dv->e) : own.e;
             at_vertex = false;
             ea = h.y;
             eb = h.z;
             t_next = h.w;
             la = w.x;
             lb = w.y;
-            pa = make_float2(e.x, e.y);
-            pb = make_float2(e.z, e.w);
+            pa = fs.b_pj;
+            pb = fs.b_pk;
             if (++states > max_steps) fin = true;
             continue;
         }
@@ -389,7 +457,7 @@ __device__ __forceinline__ void trace_path(const TraceDom &p, const float *__res
         // eb is local vertex L, ea is X, and the opposite vertex is Y
         const int tl = t_next;
         const Tri T = load_tri(p.rec, tl);
-        const float4 Rt = rates ? __ldg(rates + (int64_t)tl * rstride) : tri_rates(p.gphi, p.rec, tl, f);
+        const float4 Rt = __ldg(rates + tl);
         const int L = local_of(T, eb), X = L == 2 ? 0 : L + 1, Y = L == 0 ? 2 : L - 1;
         const float ra = sel3f(X, Rt.x, Rt.y, Rt.z), rb = sel3f(L, Rt.x, Rt.y, Rt.z), rc = sel3f(Y, Rt.x, Rt.y, Rt.z);
         const float qY = sel3f(Y, T.q0, T.q1, T.q2);
@@ -460,9 +528,270 @@ __device__ __forceinline__ void trace_path(const TraceDom &p, const float *__res
     }
 }
 
+// A crossing as the walk meets it, 48 bytes for each triangle and entry edge
+// (4 t + L, L the local vertex that is the entry edge's second end b; a is the
+// next vertex counter-clockwise and Y the one across): no choice among local
+// vertices is left but the order in which the rates are formed.
+//   (g0x, g0y, g1x, g1y)  (Y, position of Y, |grad phi_Y|^2)
+//   (na, nb, oa, ob): the crossing after leaving through the edge opposite a
+//   or b (-1 on the boundary) and the vertex beyond that edge
+__global__ void crossings_kernel(const int4 *__restrict__ rec, const float4 *__restrict__ gphi, int64_t n_t,
+                                 int4 *__restrict__ hrec) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t t = i >> 2;
+    const int L = (int)(i & 3);
+    if (t >= n_t) return;
+    int4 *h = hrec + 3 * i;
+    if (L == 3) {
+        h[0] = h[1] = h[2] = make_int4(0, 0, 0, 0);
+        return;
+    }
+    const Tri T = load_tri(rec, (int)t);
+    const int X = L == 2 ? 0 : L + 1, Y = L == 0 ? 2 : L - 1;
+    const int vb = vid(T, L), vY = vid(T, Y);
+    const float2 pY = pos(T, Y);
+    // through the edge opposite a = (Y, b): b stays second; opposite b = (a, Y): Y is
+    auto next = [&](int tn, int second, int &n, int &o) {
+        n = -1;
+        o = -1;
+        if (tn < 0) return;
+        const Tri Q = load_tri(rec, tn);
+        const int l = local_of(Q, second);
+        n = 4 * tn + l;
+        o = vid(Q, l == 0 ? 2 : l - 1);
+    };
+    int4 w;
+    next(sel3i(X, T.n0, T.n1, T.n2), vb, w.x, w.z);
+    next(sel3i(L, T.n0, T.n1, T.n2), vY, w.y, w.w);
+    const float4 g = gphi[2 * t];
+    h[0] = make_int4(__float_as_int(g.x), __float_as_int(g.y), __float_as_int(g.z), __float_as_int(g.w));
+    h[1] = make_int4(vY, __float_as_int(pY.x), __float_as_int(pY.y), __float_as_int(sel3f(Y, T.q0, T.q1, T.q2)));
+    h[2] = w;
+}
+
+// One path, walked by a group of G lanes (aligned within the warp, `mask`).
+// The walk is trace_path's, decision by decision and operation by operation;
+// what differs is what a step costs and when things are read, for a step's
+// chain is what a path waits for:
+//  * crossings come ready-made (crossings_kernel): a step took 300
+//    instructions on triangle records, most of them choosing among local
+//    vertices;
+//  * at the start of a crossing the two that can follow it and the field at
+//    the vertices beyond are read, and arrive while it is decided; with the
+//    edge's field values carried along, no read of a step waits for another;
+//  * every lane of the group carries the whole state (reads of one address by
+//    a group are one access) and its first lane writes the points;
+//  * a vertex state without precomputed decisions deals the fan's triangles
+//    to the lanes.
+// Fewer paths to a warp also mean fewer of them waiting for another's branch.
+template <int G>
+__device__ __forceinline__ void walk_path(const TraceDom &p, const float *__restrict__ f,
+                                          const VDec *__restrict__ dec, int64_t dstride, int target, int source,
+                                          float2 *__restrict__ out, int32_t max_pts, int32_t max_steps,
+                                          int32_t *len_out, int32_t *status_out, bool active, unsigned mask) {
+    const float eps2 = kEpsWedge * kEpsWedge;
+    const int gl = threadIdx.x & (G - 1);
+    struct Crossing {
+        float4 g, y;
+        int4 n;
+    };
+    auto read = [&](int h) {
+        Crossing c;
+        const int4 *r = p.hrec + 3 * (int64_t)h;
+        c.g = __ldg(reinterpret_cast<const float4 *>(r));
+        c.y = __ldg(reinterpret_cast<const float4 *>(r + 1));
+        c.n = __ldg(r + 2);
+        return c;
+    };
+    int len = 0;
+    int status = DD_TRACE_STEP_LIMIT;
+    int states = 1;
+    bool fin = !active;
+    bool at_vertex = true;
+    int v = source;
+    // edge state: edge (ea, eb) at weights (la, lb), its ends' field values and
+    // positions; the crossing h (4 t + L, -1 on the boundary) and the field at its Y
+    int h = -1, ea = 0, eb = 0;
+    float la = 0.f, lb = 0.f, fa = 0.f, fb = 0.f, fc = 0.f;
+    float2 pa = make_float2(0.f, 0.f), pb = pa;
+    Crossing c = {};
+    if (active) {
+        if (gl == 0) out[len] = p.xy[v];
+        ++len;
+        if (v == target) {
+            status = DD_TRACE_OK;
+            fin = true;
+        }
+    }
+#define DD_PUSH(pt)                              \
+    if (len >= max_pts) {                        \
+        status = DD_TRACE_TRUNCATED;             \
+        fin = true;                              \
+        continue;                                \
+    }                                            \
+    if (gl == 0) out[len] = (pt);                \
+    ++len;
+#define DD_ENTER_VERTEX(vert)                    \
+    v = (vert);                                  \
+    at_vertex = true;                            \
+    if (++states > max_steps) {                  \
+        fin = true;                              \
+        continue;                                \
+    }                                            \
+    if (v == target) {                           \
+        status = DD_TRACE_OK;                    \
+        fin = true;                              \
+        continue;                                \
+    }
+#define DD_SLIDE()                                                     \
+    {                                                                  \
+        const bool a_low = fa < fb || (fa == fb && ea < eb);           \
+        DD_PUSH(a_low ? pa : pb);                                      \
+        DD_ENTER_VERTEX(a_low ? ea : eb);                              \
+    }
+
+    for (;;) {
+        // (one path to a warp: its lanes agree)
+        if (G == 32 ? fin : !__any_sync(0xffffffffu, !fin)) break;
+        if (fin) continue;
+        if (at_vertex) {
+            VDec d;
+            if (dec) {
+                const VDec *dv = dec + (int64_t)v * dstride;
+                d.h = __ldg(&dv->h);
+                d.w = __ldg(&dv->w);
+            } else {
+                FanScan fs;
+                fs.begin();
+                for (int q = p.vt_off[v] + gl, q1 = p.vt_off[v + 1]; q < q1; q += G) {
+                    const int tl = p.vt[q];
+                    fs.add(v, target, tl, load_tri(p.rec, tl), tri_rates(p.gphi, p.rec, tl, f));
+                }
+                if (G > 1) {
+                    __syncwarp(mask);
+                    fan_reduce<G>(fs, mask);
+                }
+                d = fs.finish<G>(p, f, target, v, mask);
+            }
+            const int kind = d.h.x;
+            if (kind == kVStuck) {
+                status = DD_TRACE_STUCK;
+                fin = true;
+                continue;
+            }
+            const bool cross = kind == kVCross;
+            DD_PUSH(make_float2(cross ? d.w.z : d.w.x, cross ? d.w.w : d.w.y));
+            if (kind == kVAdjacent) {
+                status = DD_TRACE_OK;
+                fin = true;
+                continue;
+            }
+            if (!cross) {
+                DD_ENTER_VERTEX(d.h.y);
+                continue;
+            }
+            at_vertex = false;
+            ea = d.h.y;
+            eb = d.h.z;
+            la = d.w.x;
+            lb = d.w.y;
+            pa = p.xy[ea];
+            pb = p.xy[eb];
+            fa = f[ea];
+            fb = f[eb];
+            h = -1;
+            if (d.h.w >= 0) {
+                const int4 q = __ldg(p.rec + 4 * (int64_t)d.h.w);
+                h = 4 * d.h.w + (q.x == eb ? 0 : (q.y == eb ? 1 : 2));
+                c = read(h);
+                fc = f[__float_as_int(c.y.x)];
+            }
+            if (++states > max_steps) fin = true;
+            continue;
+        }
+        if (h < 0) {                     // boundary edge: slide to the lower endpoint
+            DD_SLIDE();
+            continue;
+        }
+        // edge state: crossing the triangle from (ea, eb) to one of its other edges
+        const int ha = c.n.x, hb = c.n.y;
+        const float foa = f[max(c.n.z, 0)], fob = f[max(c.n.w, 0)];
+        const Crossing ca = read(max(ha, 0)), cb = read(max(hb, 0));
+        const bool l0 = (h & 3) == 0, l1 = (h & 3) == 1;       // b is local vertex 0, 1 (or 2)
+        const float4 Rt = rates_of(c.g, l0 ? fb : (l1 ? fc : fa), l0 ? fa : (l1 ? fb : fc), l0 ? fc : (l1 ? fa : fb));
+        const float ra = l0 ? Rt.y : (l1 ? Rt.z : Rt.x), rb = l0 ? Rt.x : (l1 ? Rt.y : Rt.z),
+                    rc = l0 ? Rt.z : (l1 ? Rt.x : Rt.y);
+        const bool enters = rc > 0.f && rc * rc > eps2 * Rt.w * c.y.w;
+        const float sa = ra < 0.f ? __fdividef(la, -ra) : INFINITY;
+        const float sb = rb < 0.f ? __fdividef(lb, -rb) : INFINITY;
+        if (!enters || !(fminf(sa, sb) < INFINITY)) {   // valley edge (or no exit): lower endpoint
+            DD_SLIDE();
+            continue;
+        }
+        const int vY = __float_as_int(c.y.x);
+        const float2 pY = make_float2(c.y.y, c.y.z);
+        const bool via_a = sa <= sb;                      // exit through the edge opposite a (the Y-b edge)
+        const float s = via_a ? sa : sb;
+        float lkeep = fmaxf(via_a ? lb + s * rb : la + s * ra, 0.f);
+        float lc2 = fmaxf(s * rc, 0.f);
+        const float inv = __fdividef(1.0f, lkeep + lc2);
+        lkeep *= inv;
+        lc2 *= inv;
+        const int keep_v = via_a ? eb : ea;
+        const float2 keep_p = via_a ? pb : pa;
+        if (lkeep <= kEpsBary) {
+            DD_PUSH(pY);
+            DD_ENTER_VERTEX(vY);
+            continue;
+        }
+        if (lc2 <= kEpsBary) {
+            DD_PUSH(keep_p);
+            DD_ENTER_VERTEX(keep_v);
+            continue;
+        }
+        DD_PUSH(make_float2(lkeep * keep_p.x + lc2 * pY.x, lkeep * keep_p.y + lc2 * pY.y));
+        // new edge, counter-clockwise: via a -> (Y, b); via b -> (a, Y)
+        if (via_a) {
+            h = ha;
+            c = ca;
+            ea = vY;
+            pa = pY;
+            fa = fc;
+            fc = foa;
+            la = lc2;
+            lb = lkeep;
+        } else {
+            h = hb;
+            c = cb;
+            eb = vY;
+            pb = pY;
+            fb = fc;
+            fc = fob;
+            la = lkeep;
+            lb = lc2;
+        }
+        if (++states > max_steps) {
+            fin = true;
+            continue;
+        }
+        if (vY == target || keep_v == target) {   // an edge incident on the target
+            DD_PUSH(p.xy[target]);
+            status = DD_TRACE_OK;
+            fin = true;
+            continue;
+        }
+    }
+#undef DD_PUSH
+#undef DD_ENTER_VERTEX
+#undef DD_SLIDE
+    if (active && gl == 0) {
+        *len_out = len;
+        *status_out = status;
+    }
+}
+
 struct TraceParams {
     TraceDom d;
-    const float4 *rates;           // [n_t][T]
     const VDec *dec;               // [n_v][T]
     const float *fields;
     int64_t field_stride;
@@ -473,15 +802,17 @@ struct TraceParams {
     int32_t *out_len, *out_status;
 };
 
-__global__ void __launch_bounds__(128) trace_kernel(const TraceParams p) {
-    const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool active = gid < p.total;       // padding lanes stay in the warp's walk loop, idle
+// G lanes a path
+template <int G>
+__global__ void __launch_bounds__(64) trace_group_kernel(const TraceParams p) {
+    const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
+    const bool active = gid < p.total;
     const int64_t id = active ? gid : 0;
     const int a = (int)(id / p.S);
-    trace_path(p.d, p.fields + (int64_t)a * p.field_stride, p.rates ? p.rates + a : nullptr, p.T,
-               p.dec ? p.dec + a : nullptr, p.T,
-               p.targets[a], p.sources[id], p.out_xy + id * p.max_pts, p.max_pts, p.max_steps, p.out_len + id,
-               p.out_status + id, active);
+    const unsigned mask = G == 32 ? 0xffffffffu : (((1u << (G & 31)) - 1u) << (threadIdx.x & 31 & ~(G - 1)));
+    walk_path<G>(p.d, p.fields + (int64_t)a * p.field_stride, p.dec ? p.dec + a : nullptr, p.T, p.targets[a],
+                 p.sources[id], p.out_xy + id * p.max_pts, p.max_pts, p.max_steps, p.out_len + id, p.out_status + id,
+                 active, mask);
 }
 
 // ---- several meshes in one launch: global target g belongs to domain tdom[g] (local index tloc[g])
@@ -517,13 +848,14 @@ __global__ void __launch_bounds__(64) batch_trace_kernel(const BatchTraceDom *__
     const int g = path_target ? path_target[id] : (int)(id / S);
     const BatchTraceDom q = doms[tdom[g]];
     const int a = tloc[g];
-    trace_path(q.d, q.fields + (int64_t)a * q.d.n_v, q.rates + (int64_t)a * q.d.n_t, 1, nullptr, 0, targets[g],
-               sources[id], out_xy + id * max_pts, max_pts, q.max_steps, out_len + id, out_status + id, active);
+    trace_path(q.d, q.fields + (int64_t)a * q.d.n_v, q.rates + (int64_t)a * q.d.n_t, targets[g], sources[id],
+               out_xy + id * max_pts, max_pts, q.max_steps, out_len + id, out_status + id, active);
 }
 
 TraceDom make_dom(const DevMesh &m) {
     TraceDom d;
     d.rec = m.trec;
+    d.hrec = m.hrec;
     d.gphi = m.gphi;
     d.xy = m.xy;
     d.vt_off = m.vt_off;
@@ -548,22 +880,25 @@ size_t trace_scratch_bytes(const DevMesh &m, int32_t T, bool decisions) {
 }
 
 // Vertex decisions for every (field, vertex) before the walk pay off when
-// many paths share a field (they are reused); with few paths each vertex
-// state computes its own.  DD_TRACE_DECISIONS=dense|lazy overrides the choice
-// (for measurements).
-bool trace_dense_decisions(int32_t S) {
+// many paths share a field (they are reused) and share warps (a group that
+// scans a fan holds up the others of its warp); with few each vertex state
+// computes its own.  grid140, one target, 256 paths: the walk takes 119 us
+// either way and the two passes 24; 71,681 vertices, 64 x 256 paths: 476 + 340
+// us against 1,155.  DD_TRACE_DECISIONS=dense|lazy overrides the choice (for
+// measurements).
+bool trace_dense_decisions(int32_t T, int32_t S) {
     static int mode = -1;
     if (mode < 0) {
         const char *e = getenv("DD_TRACE_DECISIONS");
         mode = (e && !strcmp(e, "dense")) ? 1 : (e && !strcmp(e, "lazy")) ? 0 : 2;
     }
-    return mode == 2 ? S >= kDenseMinPaths : mode == 1;
+    return mode == 2 ? S >= kDenseMinPaths && (int64_t)T * S > kWarpPaths : mode == 1;
 }
 
 void launch_trace(const DevMesh &m, const float *fields, int64_t field_stride, const int32_t *targets,
                   const int32_t *sources, int32_t T, int32_t S, int32_t max_pts, float2 *out_xy, int32_t *out_len,
                   int32_t *out_status, void *scratch, cudaStream_t s) {
-    const bool dense = trace_dense_decisions(S);
+    const bool dense = trace_dense_decisions(T, S);
     TraceParams p;
     // the rates of every triangle only where vertex decisions are precomputed (many
     // paths per field); with few, the walk forms the rates it needs itself
@@ -572,7 +907,6 @@ void launch_trace(const DevMesh &m, const float *fields, int64_t field_stride, c
                                                  align256((size_t)T * m.n_t * sizeof(float4)))
                       : nullptr;
     p.d = make_dom(m);
-    p.rates = rates;
     p.dec = dec;
     p.fields = fields;
     p.field_stride = field_stride;
@@ -599,11 +933,31 @@ void launch_trace(const DevMesh &m, const float *fields, int64_t field_stride, c
             vertex_decision_kernel<<<(unsigned)((warps + 3) / 4), 128, 0, s>>>(p.d, T, fields, field_stride, rates,
                                                                                 targets, dec);
         }
+        if (m.n_wide > 0) {
+            KMark km_("wide_decision_kernel", s);
+            wide_decision_kernel<<<dim3((unsigned)m.n_wide, (unsigned)((T + 3) / 4)), 128, 0, s>>>(
+                p.d, m.wide, T, fields, field_stride, rates, targets, dec);
+        }
     }
-    {
+    auto groups = [&](auto kern, int G) {
         KMark km_("trace_kernel", s);
-        trace_kernel<<<(unsigned)((p.total + 127) / 128), 128, 0, s>>>(p);   // 128: measured best of 64/128/256
-    }
+        kern<<<(unsigned)((p.total * G + 63) / 64), 64, 0, s>>>(p);
+    };
+    // Lanes a path: a warp each while that leaves every scheduler at most four
+    // warps (a path alone in its warp never waits for another's branch: 256
+    // paths of grid140 119 us, against 134 with eight lanes and 153 with one),
+    // then four (16,384 paths: 476 us; 1,340 with a warp each, issue-bound;
+    // 493 with one lane), one where there are warps enough without
+    if (p.total <= kWarpPaths)
+        groups(trace_group_kernel<32>, 32);
+    else if (p.total <= 16 * kWarpPaths)
+        groups(trace_group_kernel<4>, 4);
+    else
+        groups(trace_group_kernel<1>, 1);
+}
+
+void launch_crossings(const DevMesh &m, cudaStream_t s) {
+    if (m.n_t > 0) crossings_kernel<<<(unsigned)((4 * m.n_t + 255) / 256), 256, 0, s>>>(m.trec, m.gphi, m.n_t, m.hrec);
 }
 
 size_t batch_trace_dom_bytes() { return sizeof(BatchTraceDom); }
