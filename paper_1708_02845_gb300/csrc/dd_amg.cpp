@@ -191,6 +191,28 @@ AmgCsr smoothed_prolongator(const AmgCsr &A, const std::vector<double> &d, const
     return P;
 }
 
+// The level's fused operators (AmgLevel): Q = P - w D^-1 (A P) on the pattern
+// of A P, which holds P's (A has its diagonal), Qt its transpose, and G on A's.
+void fuse_level(AmgLevel &L, const AmgCsr &A, AmgCsr &&AP) {
+    L.Q = std::move(AP);
+    for (int64_t i = 0; i < A.rows; ++i) {
+        const double w = L.omega * L.dinv[i];
+        int64_t q = L.P.off[i];
+        for (int64_t p = L.Q.off[i]; p < L.Q.off[i + 1]; ++p) {
+            double v = -w * L.Q.val[p];
+            if (q < L.P.off[i + 1] && L.P.col[q] == L.Q.col[p]) v += L.P.val[q++];
+            L.Q.val[p] = v;
+        }
+    }
+    L.Qt = transpose(L.Q);
+    L.G = A;
+    for (int64_t i = 0; i < A.rows; ++i)
+        for (int64_t p = A.off[i]; p < A.off[i + 1]; ++p) {
+            const int32_t j = A.col[p];
+            L.G.val[p] = L.omega * L.dinv[i] * ((j == (int32_t)i ? 2.0 : 0.0) - A.val[p] * L.omega * L.dinv[j]);
+        }
+}
+
 // dense inverse of an SPD matrix by Cholesky; false if not positive definite
 bool dense_spd_inverse(const AmgCsr &A, std::vector<double> &inv) {
     const int64_t n = A.rows;
@@ -271,7 +293,9 @@ bool build_amg(const AmgCsr &A0, AmgHierarchy &H, std::string &err) {
         }
         L.P = smoothed_prolongator(A, d, agg, na, L.omega);
         L.R = transpose(L.P);
-        AmgCsr Ac = spgemm(L.R, spgemm(A, L.P));
+        AmgCsr AP = spgemm(A, L.P);
+        AmgCsr Ac = spgemm(L.R, AP);
+        fuse_level(L, A, std::move(AP));
         L.A = std::move(A);
         H.levels.push_back(std::move(L));
         A = std::move(Ac);

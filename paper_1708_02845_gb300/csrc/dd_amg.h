@@ -17,8 +17,17 @@ struct AmgCsr {
 // One level: its operator A, the inverse diagonal, the Jacobi weight omega
 // (also the prolongator-smoothing weight) and, except on the coarsest level,
 // the prolongator P to it from the next coarser level and R = P^T.
+//
+// With one Jacobi sweep before and after the coarse correction, and the
+// prolongator smoothed with the same weight, the level's V-cycle z = V(b) is
+//   b_c = Q^T b,   z = G b + Q V_c(b_c),
+//   Q = (I - w D^-1 A) P,   G = w D^-1 (2 I - A w D^-1)
+// (write S = I - w D^-1 A; the sweep before gives x = w D^-1 b with residual
+// S^T b, the coarse right-hand side is P^T S^T b = Q^T b, and the sweep after
+// turns x + P e into S x + Q e + w D^-1 b): two sparse products a level
+// instead of seven passes.
 struct AmgLevel {
-    AmgCsr A, P, R;
+    AmgCsr A, P, R, Q, Qt, G;
     std::vector<double> dinv;
     double omega = 0.0;
 };

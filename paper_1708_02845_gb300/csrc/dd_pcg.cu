@@ -18,9 +18,11 @@
 #include <cstdio>
 #include <cstring>
 #include <cstdlib>
-#include <functional>
+#include <utility>
+#include <vector>
 
 #include "dd_amg.h"
+#include "dd_f32x2.cuh"
 #include "dd_internal.h"
 
 namespace {
@@ -97,7 +99,10 @@ __global__ void update_p_kernel(int64_t m, int64_t kc, const double *__restrict_
     }
 }
 
-// Sum the [nrb][kc] partials of each column: blockDim (32, 8)
+// Sum the [nrb][kc] partials of each column: blockDim (32, 32) (with 8 rows of
+// threads the two sums of beta took 28 us an iteration on grid140, a chain of
+// loads on 33 blocks)
+constexpr int kSumRows = 32;
 __device__ __forceinline__ double column_sum(const double *part, int64_t nrb, int64_t kc, int64_t c,
                                              double (*sh)[33]) {
     double s = 0.0;
@@ -115,7 +120,7 @@ __device__ __forceinline__ double column_sum(const double *part, int64_t nrb, in
 __global__ void alpha_kernel(int64_t nrb, int64_t kc, const double *__restrict__ part,
                              const double *__restrict__ rz, const int *__restrict__ done,
                              double *__restrict__ alpha) {
-    __shared__ double sh[8][33];
+    __shared__ double sh[kSumRows][33];
     const int64_t c = (int64_t)blockIdx.x * 32 + threadIdx.x;
     double pAp = column_sum(part, nrb, kc, c, sh);
     if (threadIdx.y == 0 && c < kc) alpha[c] = (!done[c] && pAp > 0.0) ? rz[c] / pAp : 0.0;
@@ -125,7 +130,7 @@ __global__ void beta_kernel(int64_t nrb, int64_t kc, const double *__restrict__ 
                             const double *__restrict__ part_rr, const double *__restrict__ bnorm,
                             double *__restrict__ rz, const int *__restrict__ done,
                             double *__restrict__ beta, unsigned long long *__restrict__ maxres) {
-    __shared__ double sh[8][33];
+    __shared__ double sh[kSumRows][33];
     const int64_t c = (int64_t)blockIdx.x * 32 + threadIdx.x;
     double rz_new = column_sum(part_rz, nrb, kc, c, sh);
     double rr = column_sum(part_rr, nrb, kc, c, sh);
@@ -180,7 +185,7 @@ __global__ void init_p_kernel(int64_t m, int64_t kc, const double *__restrict__ 
 __global__ void init_scalars_kernel(int64_t nrb, int64_t kc, const double *__restrict__ part_rz,
                                     const double *__restrict__ part_rr, double *__restrict__ rz,
                                     double *__restrict__ bnorm, int *__restrict__ done) {
-    __shared__ double sh[8][33];
+    __shared__ double sh[kSumRows][33];
     const int64_t c = (int64_t)blockIdx.x * 32 + threadIdx.x;
     double s_rz = column_sum(part_rz, nrb, kc, c, sh);
     double s_rr = column_sum(part_rr, nrb, kc, c, sh);
@@ -222,60 +227,223 @@ __global__ void store_host_p_kernel(int64_t n_v, int64_t k, int64_t k_pad, const
 }
 
 // ---------------------------------------------------------------- multigrid V-cycle kernels
-// Row-major [rows][kc] FP64 blocks, one thread per column, CTAs over row blocks.
-enum { kSpmmSet = 0, kSpmmResidual = 1, kSpmmAdd = 2 };
+// The V-cycle's two sparse products a level (dd_amg.h: AmgLevel).  This part
+// does about one FP64 multiply-add for every 60 in FP32, and in FP64 the
+// cycle's 17 to 21 multiply-adds per fine entry took two thirds of the solve.
+// It is the preconditioner, a fixed symmetric operator that only steers the
+// iteration, so its numbers are unevaluated sums of two floats (about 48
+// bits) and its sums compensated in the same form (Dekker, "A floating-point
+// technique for extending the available precision", Numerische Mathematik
+// 1971); the iteration itself -- residual, products, steps, stopping test --
+// stays in FP64.  One term costs 12 FP32 operations, packed over the two
+// columns of a thread.
+//
+// A block [rows][kc] of such numbers keeps the columns of a pair side by
+// side: (hi0, hi1, lo0, lo1) in 16 bytes (kc is even).
+struct Df2 {
+    f2_t hi, lo;
+};
 
-// MODE kSpmmSet: Y = M X;  kSpmmResidual: Y = B - M X;  kSpmmAdd: Y += M X
-template <int MODE>
-__global__ void csr_spmm_kernel(int64_t rows, int64_t kc, const int64_t *__restrict__ off,
-                                const int32_t *__restrict__ col, const double *__restrict__ val,
-                                const double *__restrict__ X, const double *__restrict__ B, double *__restrict__ Y,
-                                int rpb) {
-    const int64_t c = (int64_t)blockIdx.y * kColsPerBlock + threadIdx.x;
-    if (c >= kc) return;
+__device__ __forceinline__ Df2 df_load(const float4 *p) {
+    const float4 v = *p;
+    return Df2{pk(v.x, v.y), pk(v.z, v.w)};
+}
+__device__ __forceinline__ f2_t sub2(f2_t a, f2_t b) { return fma2(b, pk(-1.0f, -1.0f), a); }
+
+// (s, c) += a x: the product's leading part with its rounding error, added by a two-sum
+__device__ __forceinline__ void df_fma(f2_t &s, f2_t &c, float2 a, const Df2 &x) {
+    const f2_t ah = pk(a.x, a.x), al = pk(a.y, a.y);
+    const f2_t p = mul2(ah, x.hi);
+    f2_t e = fma2(ah, x.hi, p ^ 0x8000000080000000ULL);
+    e = fma2(ah, x.lo, e);
+    e = fma2(al, x.hi, e);
+    const f2_t t = add2(s, p), b = sub2(t, s);
+    const f2_t err = add2(sub2(s, sub2(t, b)), sub2(p, b));
+    s = t;
+    c = add2(c, add2(err, e));
+}
+// the sum as a normalised pair
+__device__ __forceinline__ Df2 df_norm(f2_t s, f2_t c) {
+    const f2_t h = add2(s, c);
+    return Df2{h, sub2(c, sub2(h, s))};
+}
+__device__ __forceinline__ float4 df_pack(const Df2 &v) {
+    float4 r;
+    upk(v.hi, r.x, r.y);
+    upk(v.lo, r.z, r.w);
+    return r;
+}
+
+// A double as an unevaluated sum of two floats, by integer operations on its
+// bits (this part converts FP64 no faster than it multiplies it): the leading
+// 24 bits of the significand, and the 29 that follow as an integer scaled.
+// Magnitudes outside 2^-90 .. 2^120 come out as 0 or as 2^120 (residuals of
+// the solve start below 2^30 and stop 1e-15 lower).
+__device__ __forceinline__ void df_split(double d, float &hi, float &lo) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(d);
+    const unsigned sign = (unsigned)(u >> 32) & 0x80000000u;
+    const int e = (int)((u >> 52) & 0x7ff) - 1023;
+    const int ec = min(e, 120);
+    const unsigned top = (unsigned)(u >> 29) & 0x7fffffu;
+    const float l = (float)(int)((unsigned)u & 0x1fffffffu);               // < 2^29
+    const float scale = __uint_as_float((unsigned)(ec - 29 + 127) << 23);  // 2^(e - 29); times 2^-23 below
+    const bool tiny = e < -90;
+    hi = tiny ? 0.0f : __uint_as_float(sign | ((unsigned)(ec + 127) << 23) | top);
+    lo = tiny ? 0.0f : __uint_as_float(sign ^ __float_as_uint(l * scale * 0x1p-23f));
+}
+// float to double by its bits (subnormals as 0)
+__device__ __forceinline__ double widen(float f) {
+    const unsigned u = __float_as_uint(f);
+    const unsigned m = u & 0x7fffffffu;
+    const unsigned h = m < 0x00800000u ? 0u : (m >> 3) + (896u << 20);
+    return __hiloint2double((int)((u & 0x80000000u) | h), (int)(m < 0x00800000u ? 0u : m << 29));
+}
+
+constexpr int kPairs = 64;      // column pairs (threads) of one CTA
+
+// Y = M X
+__global__ void __launch_bounds__(kPairs) df_spmm_kernel(int64_t rows, int64_t kp, const int32_t *__restrict__ off,
+                                                         const int32_t *__restrict__ col,
+                                                         const float2 *__restrict__ val, const float4 *__restrict__ X,
+                                                         float4 *__restrict__ Y, int rpb) {
+    const int64_t c = (int64_t)blockIdx.y * kPairs + threadIdx.x;
+    if (c >= kp) return;
     const int64_t r0 = (int64_t)blockIdx.x * rpb;
     const int64_t r1 = r0 + rpb < rows ? r0 + rpb : rows;
     for (int64_t r = r0; r < r1; ++r) {
-        double s = 0.0;
-        for (int64_t q = off[r]; q < off[r + 1]; ++q) s += val[q] * X[(int64_t)col[q] * kc + c];
-        const int64_t i = r * kc + c;
-        if (MODE == kSpmmSet) Y[i] = s;
-        if (MODE == kSpmmResidual) Y[i] = B[i] - s;
-        if (MODE == kSpmmAdd) Y[i] += s;
+        f2_t s = 0ULL, cc = 0ULL;
+#pragma unroll 4
+        for (int q = off[r]; q < off[r + 1]; ++q) df_fma(s, cc, val[q], df_load(X + (int64_t)col[q] * kp + c));
+        Y[r * kp + c] = df_pack(df_norm(s, cc));
     }
 }
 
-// X = omega D^-1 B (one Jacobi sweep from zero)
-__global__ void jacobi0_kernel(int64_t rows, int64_t kc, double omega, const double *__restrict__ dinv,
-                               const double *__restrict__ B, double *__restrict__ X, int rpb) {
-    const int64_t c = (int64_t)blockIdx.y * kColsPerBlock + threadIdx.x;
-    if (c >= kc) return;
+// Z = G B + Q E (E: rows of the next level).  FINE: Z in FP64, with partial
+// column sums of R . Z; else Z in pairs like B.
+template <bool FINE>
+__global__ void __launch_bounds__(kPairs) df_up_kernel(int64_t rows, int64_t kp, const int32_t *__restrict__ goff,
+                                                       const int32_t *__restrict__ gcol,
+                                                       const float2 *__restrict__ gval,
+                                                       const int32_t *__restrict__ qoff,
+                                                       const int32_t *__restrict__ qcol,
+                                                       const float2 *__restrict__ qval, const float4 *__restrict__ B,
+                                                       const float4 *__restrict__ E, const double2 *__restrict__ R,
+                                                       void *__restrict__ Z, double2 *__restrict__ part, int rpb) {
+    const int64_t c = (int64_t)blockIdx.y * kPairs + threadIdx.x;
+    if (c >= kp) return;
     const int64_t r0 = (int64_t)blockIdx.x * rpb;
     const int64_t r1 = r0 + rpb < rows ? r0 + rpb : rows;
-    for (int64_t r = r0; r < r1; ++r) X[r * kc + c] = omega * dinv[r] * B[r * kc + c];
-}
-
-// X += omega D^-1 Res; with DOT, also partial column sums of Rp . X (the
-// preconditioned residual's inner product, on the fine level)
-template <bool DOT>
-__global__ void jacobi_add_kernel(int64_t rows, int64_t kc, double omega, const double *__restrict__ dinv,
-                                  const double *__restrict__ Res, double *__restrict__ X,
-                                  const double *__restrict__ Rp, double *__restrict__ part, int rpb) {
-    const int64_t c = (int64_t)blockIdx.y * kColsPerBlock + threadIdx.x;
-    if (c >= kc) return;
-    const int64_t r0 = (int64_t)blockIdx.x * rpb;
-    const int64_t r1 = r0 + rpb < rows ? r0 + rpb : rows;
-    double acc = 0.0;
+    double d0 = 0.0, d1 = 0.0;
     for (int64_t r = r0; r < r1; ++r) {
-        const int64_t i = r * kc + c;
-        const double x = X[i] + omega * dinv[r] * Res[i];
-        X[i] = x;
-        if (DOT) acc += Rp[i] * x;
+        f2_t s = 0ULL, cc = 0ULL;
+#pragma unroll 4
+        for (int q = goff[r]; q < goff[r + 1]; ++q) df_fma(s, cc, gval[q], df_load(B + (int64_t)gcol[q] * kp + c));
+#pragma unroll 4
+        for (int q = qoff[r]; q < qoff[r + 1]; ++q) df_fma(s, cc, qval[q], df_load(E + (int64_t)qcol[q] * kp + c));
+        const float4 z = df_pack(df_norm(s, cc));
+        if (FINE) {
+            const double2 v = R[r * kp + c];
+            const double z0 = widen(z.x) + widen(z.z), z1 = widen(z.y) + widen(z.w);
+            static_cast<double2 *>(Z)[r * kp + c] = make_double2(z0, z1);
+            d0 += v.x * z0;
+            d1 += v.y * z1;
+        } else {
+            static_cast<float4 *>(Z)[r * kp + c] = z;
+        }
     }
-    if (DOT) part[(int64_t)blockIdx.x * kc + c] = acc;
+    if (FINE) part[(int64_t)blockIdx.x * kp + c] = make_double2(d0, d1);
 }
 
 // X = Ainv B on the coarsest level (Ainv dense n x n, row-major)
+__global__ void __launch_bounds__(kPairs) df_coarse_kernel(int64_t n, int64_t kp, const float2 *__restrict__ ainv,
+                                                           const float4 *__restrict__ B, float4 *__restrict__ X) {
+    const int64_t c = (int64_t)blockIdx.x * kPairs + threadIdx.x;
+    const int64_t i = blockIdx.y;
+    if (c >= kp || i >= n) return;
+    f2_t s = 0ULL, cc = 0ULL;
+#pragma unroll 4
+    for (int64_t j = 0; j < n; ++j) df_fma(s, cc, ainv[i * n + j], df_load(B + j * kp + c));
+    X[i * kp + c] = df_pack(df_norm(s, cc));
+}
+
+// a block as pairs (the first V-cycle's right-hand side), with partial column sums of R . R
+__global__ void __launch_bounds__(kPairs) df_first_kernel(int64_t rows, int64_t kp, const double2 *__restrict__ R,
+                                                          float4 *__restrict__ B, double2 *__restrict__ part,
+                                                          int rpb) {
+    const int64_t c = (int64_t)blockIdx.y * kPairs + threadIdx.x;
+    if (c >= kp) return;
+    const int64_t r0 = (int64_t)blockIdx.x * rpb;
+    const int64_t r1 = r0 + rpb < rows ? r0 + rpb : rows;
+    double d0 = 0.0, d1 = 0.0;
+    for (int64_t r = r0; r < r1; ++r) {
+        const double2 v = R[r * kp + c];
+        float4 b;
+        df_split(v.x, b.x, b.z);
+        df_split(v.y, b.y, b.w);
+        B[r * kp + c] = b;
+        d0 += v.x * v.x;
+        d1 += v.y * v.y;
+    }
+    part[(int64_t)blockIdx.x * kp + c] = make_double2(d0, d1);
+}
+
+// R -= alpha AP, also as pairs into B; partial column sums of R . R (a column
+// with alpha = 0 keeps its residual)
+__global__ void __launch_bounds__(kPairs) update_r_kernel(int64_t rows, int64_t kp,
+                                                          const double2 *__restrict__ alpha,
+                                                          double2 *__restrict__ R, const double2 *__restrict__ AP,
+                                                          float4 *__restrict__ B, double2 *__restrict__ part,
+                                                          int rpb) {
+    const int64_t c = (int64_t)blockIdx.y * kPairs + threadIdx.x;
+    if (c >= kp) return;
+    const int64_t r0 = (int64_t)blockIdx.x * rpb;
+    const int64_t r1 = r0 + rpb < rows ? r0 + rpb : rows;
+    const double2 a = alpha[c];
+    double d0 = 0.0, d1 = 0.0;
+#pragma unroll 2
+    for (int64_t r = r0; r < r1; ++r) {
+        const int64_t i = r * kp + c;
+        double2 v = R[i];
+        const double2 w = AP[i];
+        v.x -= a.x * w.x;
+        v.y -= a.y * w.y;
+        R[i] = v;
+        float4 b;
+        df_split(v.x, b.x, b.z);
+        df_split(v.y, b.y, b.w);
+        B[i] = b;
+        d0 += v.x * v.x;
+        d1 += v.y * v.y;
+    }
+    part[(int64_t)blockIdx.x * kp + c] = make_double2(d0, d1);
+}
+
+// X += alpha Pd, then Pd = Z + beta Pd: one read of Pd for both
+__global__ void __launch_bounds__(kPairs) update_xp_kernel(int64_t rows, int64_t kp,
+                                                           const double2 *__restrict__ alpha,
+                                                           const double2 *__restrict__ beta,
+                                                           const double2 *__restrict__ Z, double2 *__restrict__ X,
+                                                           double2 *__restrict__ Pd, int rpb) {
+    const int64_t c = (int64_t)blockIdx.y * kPairs + threadIdx.x;
+    if (c >= kp) return;
+    const int64_t r0 = (int64_t)blockIdx.x * rpb;
+    const int64_t r1 = r0 + rpb < rows ? r0 + rpb : rows;
+    const double2 a = alpha[c], b = beta[c];
+#pragma unroll 2
+    for (int64_t r = r0; r < r1; ++r) {
+        const int64_t i = r * kp + c;
+        double2 x = X[i], p = Pd[i];
+        const double2 z = Z[i];
+        x.x += a.x * p.x;
+        x.y += a.y * p.y;
+        p.x = z.x + b.x * p.x;
+        p.y = z.y + b.y * p.y;
+        X[i] = x;
+        Pd[i] = p;
+    }
+}
+
+// X = Ainv B in FP64, where the whole problem is the coarsest level
 __global__ void coarse_solve_kernel(int64_t n, int64_t kc, const double *__restrict__ ainv,
                                     const double *__restrict__ B, double *__restrict__ X) {
     const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -286,61 +454,11 @@ __global__ void coarse_solve_kernel(int64_t n, int64_t kc, const double *__restr
     X[i * kc + c] = s;
 }
 
-// X += alpha Pd, R -= alpha AP; partial column sums of R.R
-__global__ void update_xr_plain_kernel(int64_t m, int64_t kc, const double *__restrict__ alpha,
-                                       double *__restrict__ X, double *__restrict__ R,
-                                       const double *__restrict__ Pd, const double *__restrict__ AP,
-                                       double *__restrict__ part_rr, int rpb) {
-    const int64_t c = (int64_t)blockIdx.y * kColsPerBlock + threadIdx.x;
-    if (c >= kc) return;
-    const int64_t r0 = (int64_t)blockIdx.x * rpb;
-    const int64_t r1 = r0 + rpb < m ? r0 + rpb : m;
-    const double a = alpha[c];
-    double srr = 0.0;
-    for (int64_t r = r0; r < r1; ++r) {
-        const int64_t i = r * kc + c;
-        double rr = R[i];
-        if (a != 0.0) {
-            X[i] += a * Pd[i];
-            rr -= a * AP[i];
-            R[i] = rr;
-        }
-        srr += rr * rr;
-    }
-    part_rr[(int64_t)blockIdx.x * kc + c] = srr;
-}
-
-// partial column sums of R.R
-__global__ void dot_rr_kernel(int64_t m, int64_t kc, const double *__restrict__ R, double *__restrict__ part,
-                              int rpb) {
-    const int64_t c = (int64_t)blockIdx.y * kColsPerBlock + threadIdx.x;
-    if (c >= kc) return;
-    const int64_t r0 = (int64_t)blockIdx.x * rpb;
-    const int64_t r1 = r0 + rpb < m ? r0 + rpb : m;
-    double acc = 0.0;
-    for (int64_t r = r0; r < r1; ++r) acc += R[r * kc + c] * R[r * kc + c];
-    part[(int64_t)blockIdx.x * kc + c] = acc;
-}
-
-// Pd = Z + beta Pd (beta = 0 on the first iteration)
-__global__ void update_p_z_kernel(int64_t m, int64_t kc, const double *__restrict__ beta,
-                                  const double *__restrict__ Z, double *__restrict__ Pd, int first, int rpb) {
-    const int64_t c = (int64_t)blockIdx.y * kColsPerBlock + threadIdx.x;
-    if (c >= kc) return;
-    const int64_t r0 = (int64_t)blockIdx.x * rpb;
-    const int64_t r1 = r0 + rpb < m ? r0 + rpb : m;
-    const double b = first ? 0.0 : beta[c];
-    for (int64_t r = r0; r < r1; ++r) {
-        const int64_t i = r * kc + c;
-        Pd[i] = first ? Z[i] : Z[i] + b * Pd[i];
-    }
-}
-
 // rz = column sums of part_rz, bnorm from part_rr, done flags (first iteration)
 __global__ void amg_init_scalars_kernel(int64_t nrb, int64_t kc, const double *__restrict__ part_rz,
                                         const double *__restrict__ part_rr, double *__restrict__ rz,
                                         double *__restrict__ bnorm, int *__restrict__ done) {
-    __shared__ double sh[8][33];
+    __shared__ double sh[kSumRows][33];
     const int64_t c = (int64_t)blockIdx.x * 32 + threadIdx.x;
     double s_rz = column_sum(part_rz, nrb, kc, c, sh);
     double s_rr = column_sum(part_rr, nrb, kc, c, sh);
@@ -370,11 +488,14 @@ int rows_per_block(int64_t rows, int64_t kc) {
 }
 
 struct DevCsr {
-    int64_t rows = 0;
-    int64_t *off = nullptr;
-    int32_t *col = nullptr;
-    double *val = nullptr;
+    int32_t *off = nullptr, *col = nullptr;
+    float2 *val = nullptr;         // (hi, lo)
 };
+
+float2 split_pair(double v) {
+    const float h = (float)v;
+    return make_float2(h, (float)(v - (double)h));
+}
 
 // Block CG with the smoothed-aggregation V-cycle as preconditioner (one
 // Jacobi pre- and post-sweep per level, exact coarsest solve): symmetric and
@@ -403,136 +524,138 @@ dd_status run_pcg_amg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s,
     }
     const int nl = (int)H.levels.size();
 
-    std::vector<void *> tmp;
-    cudaError_t ce = cudaSuccess;
-    auto dalloc = [&](void **p, size_t bytes) {
-        if (ce != cudaSuccess) return;
-        ce = cudaMalloc(p, bytes > 0 ? bytes : 8);
-        if (ce == cudaSuccess) tmp.push_back(*p);
-    };
-    auto upload = [&](void *dst, const void *src, size_t bytes) {
-        if (ce == cudaSuccess && bytes > 0) ce = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s);
-    };
-    auto up_csr = [&](const AmgCsr &h, DevCsr &d) {
-        d.rows = h.rows;
-        dalloc((void **)&d.off, h.off.size() * sizeof(int64_t));
-        dalloc((void **)&d.col, h.col.size() * sizeof(int32_t));
-        dalloc((void **)&d.val, h.val.size() * sizeof(double));
-        upload(d.off, h.off.data(), h.off.size() * sizeof(int64_t));
-        upload(d.col, h.col.data(), h.col.size() * sizeof(int32_t));
-        upload(d.val, h.val.data(), h.val.size() * sizeof(double));
-    };
-    std::vector<DevCsr> dA(nl), dP(nl), dR(nl);
-    std::vector<double *> dinv(nl, nullptr);
-    for (int l = 0; l < nl; ++l) {
-        const AmgLevel &L = H.levels[l];
-        if (l == 0) {
-            dA[0].rows = m;
-            dA[0].off = M.a_off;
-            dA[0].col = M.a_col;
-            dA[0].val = M.a_val;
-        } else {
-            up_csr(L.A, dA[l]);
-        }
-        dalloc((void **)&dinv[l], L.dinv.size() * sizeof(double));
-        upload(dinv[l], L.dinv.data(), L.dinv.size() * sizeof(double));
-        if (l + 1 < nl) {
-            up_csr(L.P, dP[l]);
-            up_csr(L.R, dR[l]);
-        }
-    }
-    double *ainv = nullptr;
-    dalloc((void **)&ainv, H.coarse_inv.size() * sizeof(double));
-    upload(ainv, H.coarse_inv.data(), H.coarse_inv.size() * sizeof(double));
-
-    // chunk width: six FP64 [m][kc] vectors on the fine level, three per coarser
-    // level, within a 24 GB workspace budget
+    // chunk width: six FP64 [m][kc] vectors on the fine level (five and the
+    // pairs), two of pairs per coarser level, within a 24 GB workspace budget
     double per_col = 6.0 * 8.0 * (double)m;
-    for (int l = 1; l < nl; ++l) per_col += 3.0 * 8.0 * (double)H.levels[l].A.rows;
+    for (int l = 1; l < nl; ++l) per_col += 2.0 * 8.0 * (double)H.levels[l].A.rows;
     int64_t kc = (int64_t)(24e9 / per_col);
     kc = kc / 128 * 128;
     if (kc < 128) kc = 128;
     if (kc > ((k + 3) / 4) * 4) kc = ((k + 3) / 4) * 4;
+    const int64_t kp = kc / 2;
     const int rpb0 = rows_per_block(m, kc);
     const int64_t nrb = (m + rpb0 - 1) / rpb0;
     std::vector<int> rpb(nl);
     for (int l = 0; l < nl; ++l) rpb[l] = rows_per_block(H.levels[l].A.rows, kc);
-    const size_t vec = (size_t)m * kc * sizeof(double);
-    double *X = nullptr, *R = nullptr, *Z = nullptr, *Pd = nullptr, *AP = nullptr;
-    double *part0 = nullptr, *part1 = nullptr, *alpha = nullptr, *beta = nullptr, *rz = nullptr, *bnorm = nullptr;
-    int *done = nullptr;
-    unsigned long long *maxres = nullptr;
-    dalloc((void **)&X, vec);
-    dalloc((void **)&R, vec);
-    dalloc((void **)&Z, vec);
-    dalloc((void **)&Pd, vec);
-    dalloc((void **)&AP, vec);
-    std::vector<double *> lb(nl, nullptr), lx(nl, nullptr), lr(nl, nullptr);
-    for (int l = 0; l < nl; ++l) {
-        const size_t lv = (size_t)H.levels[l].A.rows * kc * sizeof(double);
-        dalloc((void **)&lr[l], lv);
-        if (l > 0) {
-            dalloc((void **)&lb[l], lv);
-            dalloc((void **)&lx[l], lv);
+
+    // one device allocation for the hierarchy and the workspace (a solve has
+    // dozens of arrays; allocated and freed one by one they cost 2 ms), the
+    // hierarchy's part filled from one host buffer in one copy
+    size_t total = 0;
+    auto take = [&](size_t bytes) {
+        const size_t o = total;
+        total += (bytes + 255) / 256 * 256;
+        return o;
+    };
+    struct Plan {
+        const AmgCsr *h;
+        DevCsr *d;
+        size_t off, col, val;
+    };
+    std::vector<DevCsr> dG(nl), dQ(nl), dQt(nl);
+    std::vector<Plan> plans;
+    for (int l = 0; l + 1 < nl; ++l) {
+        AmgLevel &L = H.levels[l];
+        for (auto pr : {std::make_pair(&L.G, &dG[l]), std::make_pair(&L.Q, &dQ[l]), std::make_pair(&L.Qt, &dQt[l])}) {
+            if (pr.first->col.size() > (size_t)INT32_MAX) {
+                *fallback = true;
+                err = "multigrid operators exceed 32-bit offsets";
+                return DD_ENOMEM;
+            }
+            const size_t o = take((size_t)(pr.first->rows + 1) * sizeof(int32_t));
+            const size_t cl = take(pr.first->col.size() * sizeof(int32_t));
+            plans.push_back(Plan{pr.first, pr.second, o, cl, take(pr.first->val.size() * sizeof(float2))});
         }
     }
-    dalloc((void **)&part0, (size_t)nrb * kc * sizeof(double));
-    dalloc((void **)&part1, (size_t)nrb * kc * sizeof(double));
-    dalloc((void **)&alpha, kc * sizeof(double));
-    dalloc((void **)&beta, kc * sizeof(double));
-    dalloc((void **)&rz, kc * sizeof(double));
-    dalloc((void **)&bnorm, kc * sizeof(double));
-    dalloc((void **)&done, kc * sizeof(int));
-    dalloc((void **)&maxres, sizeof(unsigned long long));
-    auto release = [&]() {
-        cudaStreamSynchronize(s);
-        for (void *p : tmp) cudaFree(p);
-        tmp.clear();
-    };
+    const size_t o_ainv = take(H.coarse_inv.size() * sizeof(double));
+    const size_t filled = total;
+    const size_t vec = (size_t)m * kc * sizeof(double);
+    const size_t o_X = take(vec), o_R = take(vec), o_Z = take(vec), o_Pd = take(vec), o_AP = take(vec);
+    std::vector<size_t> o_b(nl), o_x(nl);
+    for (int l = 0; l < nl; ++l) {
+        const size_t lv = (size_t)H.levels[l].A.rows * kc * sizeof(float2);
+        o_b[l] = take(lv);
+        if (l > 0) o_x[l] = take(lv);
+    }
+    const size_t o_p0 = take((size_t)nrb * kc * sizeof(double)), o_p1 = take((size_t)nrb * kc * sizeof(double));
+    const size_t o_al = take(kc * sizeof(double)), o_be = take(kc * sizeof(double)), o_rz = take(kc * sizeof(double));
+    const size_t o_bn = take(kc * sizeof(double)), o_dn = take(kc * sizeof(int));
+    const size_t o_mr = take(sizeof(unsigned long long));
+    std::vector<uint8_t> host(filled);
+    for (const Plan &q : plans) {
+        int32_t *off = reinterpret_cast<int32_t *>(host.data() + q.off);
+        for (int64_t i = 0; i <= q.h->rows; ++i) off[i] = (int32_t)q.h->off[i];
+        std::memcpy(host.data() + q.col, q.h->col.data(), q.h->col.size() * sizeof(int32_t));
+        float2 *val = reinterpret_cast<float2 *>(host.data() + q.val);
+        for (size_t i = 0; i < q.h->val.size(); ++i) val[i] = split_pair(q.h->val[i]);
+    }
+    // the coarsest inverse: FP64 where it solves the whole problem, else pairs
+    if (nl == 1) {
+        std::memcpy(host.data() + o_ainv, H.coarse_inv.data(), H.coarse_inv.size() * sizeof(double));
+    } else {
+        float2 *val = reinterpret_cast<float2 *>(host.data() + o_ainv);
+        for (size_t i = 0; i < H.coarse_inv.size(); ++i) val[i] = split_pair(H.coarse_inv[i]);
+    }
+    uint8_t *ws = nullptr;
+    cudaError_t ce = cudaMalloc((void **)&ws, total);
+    if (ce == cudaSuccess) ce = cudaMemcpyAsync(ws, host.data(), filled, cudaMemcpyHostToDevice, s);
     if (ce != cudaSuccess) {
-        release();
+        if (ws) cudaFree(ws);
         cudaGetLastError();
         *fallback = true;
         err = std::string("multigrid workspace allocation failed: ") + cudaGetErrorString(ce);
         return DD_ENOMEM;
     }
+    auto release = [&]() {
+        cudaStreamSynchronize(s);
+        cudaFree(ws);
+    };
+    for (const Plan &q : plans)
+        *q.d = DevCsr{reinterpret_cast<int32_t *>(ws + q.off), reinterpret_cast<int32_t *>(ws + q.col),
+                      reinterpret_cast<float2 *>(ws + q.val)};
+    auto at = [&](size_t o) { return reinterpret_cast<double *>(ws + o); };
+    double *X = at(o_X), *R = at(o_R), *Z = at(o_Z), *Pd = at(o_Pd), *AP = at(o_AP);
+    double *part0 = at(o_p0), *part1 = at(o_p1), *alpha = at(o_al), *beta = at(o_be), *rz = at(o_rz), *bnorm = at(o_bn);
+    int *done = reinterpret_cast<int *>(ws + o_dn);
+    unsigned long long *maxres = reinterpret_cast<unsigned long long *>(ws + o_mr);
+    auto lb = [&](int l) { return reinterpret_cast<float4 *>(ws + o_b[l]); };
+    auto lx = [&](int l) { return reinterpret_cast<float4 *>(ws + o_x[l]); };
+    auto d2 = [](double *p) { return reinterpret_cast<double2 *>(p); };
 
     auto grid = [&](int64_t rows, int rb) {
         return dim3((unsigned)((rows + rb - 1) / rb), (unsigned)((kc + kColsPerBlock - 1) / kColsPerBlock));
     };
-    // z = V(b) on level l (x must not alias b); dot: partial sums of b.x into part0 (fine level)
-    std::function<void(int, const double *, double *, bool)> vcycle = [&](int l, const double *b, double *x,
-                                                                          bool dot) {
-        const int64_t n = H.levels[l].A.rows;
-        if (l == nl - 1) {   // coarsest level (never the fine one here: nl >= 2)
-            coarse_solve_kernel<<<dim3((unsigned)((kc + 127) / 128), (unsigned)n), 128, 0, s>>>(n, kc, ainv, b, x);
-            return;
+    auto grid2 = [&](int64_t rows, int rb) {
+        return dim3((unsigned)((rows + rb - 1) / rb), (unsigned)((kp + kPairs - 1) / kPairs));
+    };
+    // Z = V(the fine level's pairs lb(0)), partial sums of R . Z into part0
+    auto vcycle = [&]() {
+        for (int l = 0; l + 1 < nl; ++l) {
+            const int64_t nc = H.levels[l + 1].A.rows;
+            df_spmm_kernel<<<grid2(nc, rpb[l + 1]), kPairs, 0, s>>>(nc, kp, dQt[l].off, dQt[l].col, dQt[l].val, lb(l),
+                                                                    lb(l + 1), rpb[l + 1]);
         }
-        const double w = H.levels[l].omega;
-        const dim3 g = grid(n, rpb[l]);
-        const int64_t nc = H.levels[l + 1].A.rows;
-        jacobi0_kernel<<<g, kColsPerBlock, 0, s>>>(n, kc, w, dinv[l], b, x, rpb[l]);
-        csr_spmm_kernel<kSpmmResidual><<<g, kColsPerBlock, 0, s>>>(n, kc, dA[l].off, dA[l].col, dA[l].val, x, b,
-                                                                    lr[l], rpb[l]);
-        csr_spmm_kernel<kSpmmSet><<<grid(nc, rpb[l + 1]), kColsPerBlock, 0, s>>>(
-            nc, kc, dR[l].off, dR[l].col, dR[l].val, lr[l], nullptr, lb[l + 1], rpb[l + 1]);
-        vcycle(l + 1, lb[l + 1], lx[l + 1], false);
-        csr_spmm_kernel<kSpmmAdd><<<g, kColsPerBlock, 0, s>>>(n, kc, dP[l].off, dP[l].col, dP[l].val, lx[l + 1],
-                                                               nullptr, x, rpb[l]);
-        csr_spmm_kernel<kSpmmResidual><<<g, kColsPerBlock, 0, s>>>(n, kc, dA[l].off, dA[l].col, dA[l].val, x, b,
-                                                                    lr[l], rpb[l]);
-        if (dot)
-            jacobi_add_kernel<true><<<g, kColsPerBlock, 0, s>>>(n, kc, w, dinv[l], lr[l], x, b, part0, rpb[l]);
-        else
-            jacobi_add_kernel<false><<<g, kColsPerBlock, 0, s>>>(n, kc, w, dinv[l], lr[l], x, nullptr, nullptr,
-                                                                  rpb[l]);
+        const int64_t nc = H.levels[nl - 1].A.rows;
+        df_coarse_kernel<<<dim3((unsigned)((kp + kPairs - 1) / kPairs), (unsigned)nc), kPairs, 0, s>>>(
+            nc, kp, reinterpret_cast<const float2 *>(ws + o_ainv), lb(nl - 1), lx(nl - 1));
+        for (int l = nl - 2; l >= 0; --l) {
+            const int64_t n = H.levels[l].A.rows;
+            if (l > 0)
+                df_up_kernel<false><<<grid2(n, rpb[l]), kPairs, 0, s>>>(
+                    n, kp, dG[l].off, dG[l].col, dG[l].val, dQ[l].off, dQ[l].col, dQ[l].val, lb(l), lx(l + 1), nullptr,
+                    lx(l), nullptr, rpb[l]);
+            else
+                df_up_kernel<true><<<grid2(n, rpb[l]), kPairs, 0, s>>>(
+                    n, kp, dG[l].off, dG[l].col, dG[l].val, dQ[l].off, dQ[l].col, dQ[l].val, lb(l), lx(l + 1), d2(R), Z,
+                    d2(part0), rpb[l]);
+        }
     };
 
     dd_status st = DD_OK;
     int32_t iters_max = 0;
     double res_max = 0.0;
     const int check_every = 4;
-    const dim3 g0 = grid(m, rpb0), gc((unsigned)((kc + 31) / 32)), bc(32, 8);
+    const dim3 g0 = grid(m, rpb0), gc((unsigned)((kc + 31) / 32)), bc(32, kSumRows);
     for (int64_t c0 = 0; c0 < k && st == DD_OK; c0 += kc) {
         const int64_t kcur = (k - c0) < kc ? (k - c0) : kc;
         cudaMemsetAsync(X, 0, vec, s);
@@ -541,26 +664,26 @@ dd_status run_pcg_amg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s,
             scatter_rhs_kernel<<<(unsigned)((M.n_rb + 255) / 256), 256, 0, s>>>(M.n_rb, M.rb_row, M.rb_col, M.rb_val,
                                                                                 c0, kcur, kc, R);
         if (nl == 1) {   // the whole problem is the coarsest level: one exact solve
-            coarse_solve_kernel<<<dim3((unsigned)((kc + 127) / 128), (unsigned)m), 128, 0, s>>>(m, kc, ainv, R, X);
+            coarse_solve_kernel<<<dim3((unsigned)((kc + 127) / 128), (unsigned)m), 128, 0, s>>>(m, kc, at(o_ainv), R, X);
             pack_chunk_kernel<<<dim3((unsigned)nrb, (unsigned)((kcur + kColsPerBlock - 1) / kColsPerBlock)),
                                 kColsPerBlock, 0, s>>>(m, kcur, kc, c0, M.k_pad, M.interior, X, M.P, rpb0);
             iters_max = std::max(iters_max, 1);
             continue;
         }
-        vcycle(0, R, Z, true);
-        dot_rr_kernel<<<g0, kColsPerBlock, 0, s>>>(m, kc, R, part1, rpb0);
+        df_first_kernel<<<grid2(m, rpb0), kPairs, 0, s>>>(m, kp, d2(R), lb(0), d2(part1), rpb0);
+        vcycle();
         amg_init_scalars_kernel<<<gc, bc, 0, s>>>(nrb, kc, part0, part1, rz, bnorm, done);
-        update_p_z_kernel<<<g0, kColsPerBlock, 0, s>>>(m, kc, beta, Z, Pd, 1, rpb0);
+        cudaMemcpyAsync(Pd, Z, vec, cudaMemcpyDeviceToDevice, s);
         int32_t it = 0;
         double res = 1.0;
         for (it = 1; it <= max_iter; ++it) {
             spmm_dot_kernel<<<g0, kColsPerBlock, 0, s>>>(m, kc, M.a_off, M.a_col, M.a_val, Pd, AP, part0, rpb0);
             alpha_kernel<<<gc, bc, 0, s>>>(nrb, kc, part0, rz, done, alpha);
-            update_xr_plain_kernel<<<g0, kColsPerBlock, 0, s>>>(m, kc, alpha, X, R, Pd, AP, part1, rpb0);
-            vcycle(0, R, Z, true);
+            update_r_kernel<<<grid2(m, rpb0), kPairs, 0, s>>>(m, kp, d2(alpha), d2(R), d2(AP), lb(0), d2(part1), rpb0);
+            vcycle();
             cudaMemsetAsync(maxres, 0, sizeof(unsigned long long), s);
             beta_kernel<<<gc, bc, 0, s>>>(nrb, kc, part0, part1, bnorm, rz, done, beta, maxres);
-            update_p_z_kernel<<<g0, kColsPerBlock, 0, s>>>(m, kc, beta, Z, Pd, 0, rpb0);
+            update_xp_kernel<<<grid2(m, rpb0), kPairs, 0, s>>>(m, kp, d2(alpha), d2(beta), d2(Z), d2(X), d2(Pd), rpb0);
             if (it % check_every == 0 || it == max_iter) {
                 unsigned long long bits = 0;
                 cudaError_t e1 = cudaMemcpyAsync(&bits, maxres, sizeof bits, cudaMemcpyDeviceToHost, s);
@@ -697,7 +820,7 @@ dd_status run_pcg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s, int
         // vectors keep pitch kc; columns beyond kcur stay zero and converge at once
         dim3 g2((unsigned)w.nrb, (unsigned)((kc + kColsPerBlock - 1) / kColsPerBlock));
         dim3 gc((unsigned)((kc + 31) / 32));
-        dim3 bc(32, 8);
+        dim3 bc(32, kSumRows);
         cudaMemsetAsync(w.X, 0, vec * sizeof(double), s);
         cudaMemsetAsync(w.R, 0, vec * sizeof(double), s);
         if (M.n_rb > 0)
