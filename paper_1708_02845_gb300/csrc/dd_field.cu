@@ -14,7 +14,7 @@
 // r_j = 1/c_j and log c_j over [1, 2) indexed by the top 7 mantissa bits,
 // u = m r_j - 1 (|u| <= 2^-8, one rounding) and log(1 + u) from its degree-3
 // Taylor polynomial (truncation |u|^4/4 <= 2^-34, far below the final
-// rounding of lm).  The table is computed in FP64 by each CTA.  Every step
+// rounding of lm).  Every step
 // uses explicit round-to-nearest operations so all call sites produce
 // bit-identical values.  Target-side arguments below FLT_MIN are evaluated
 // at FLT_MIN; row-side terms with P[x,b] = 0 contribute 0 (the 0 log 0 rule).
@@ -75,8 +75,7 @@ __device__ __forceinline__ void accumulate_kl(float px, float lmx, float ex, flo
 
 // stage_P / stage_L / stage_E / stage_F: [T][k_pad] target row, its mantissa
 // log (table), biased exponent and mantissa log2 (hardware), the target-side
-// arguments clamped at FLT_MIN.  One CTA per target, so that the log table
-// (FP64, slow on this part) is built once per target row.  A target id
+// arguments clamped at FLT_MIN.  One CTA per target.  A target id
 // outside [0, n_v) reads nothing: its staged rows are zero-filled and
 // *bad_id (when given) is set to 1.
 __global__ void stage_targets_kernel(const float *__restrict__ P, int64_t n_v, int64_t k_pad,
@@ -784,28 +783,37 @@ __device__ __forceinline__ void pipe_store(const float (&kl)[4][4], const float 
     }
 }
 
-template <bool KL, bool TV, int H, int PB, int PS, int UNR>
-__global__ void __launch_bounds__(256 * H, 2 / H) field_tile_pipe_kernel(const float *__restrict__ PT,
+// R rows x 64 targets a CTA: 128 or 64 (whole row tiles), or 32 (half of one,
+// of which it then brings in both halves).
+template <bool KL, bool TV, int R, int PB, int PS>
+constexpr size_t pipe_smem() {
+    return (size_t)PS * ((KL ? 2 : 1) * (R >= 64 ? R / 64 : 1) + (KL ? 1 : 0) + (TV ? 1 : 0)) * PB * kTiledRows *
+           sizeof(float);
+}
+template <bool KL, bool TV, int R, int PB, int PS, int UNR>
+__global__ void __launch_bounds__(4 * R, 128 / R) field_tile_pipe_kernel(const float *__restrict__ PT,
                                                                       const float *__restrict__ LT, int64_t n_v,
                                                                       int64_t kt, const float *__restrict__ TQ,
                                                                       const float *__restrict__ TL, int32_t T,
                                                                       float *__restrict__ out_kl,
                                                                       float *__restrict__ out_tv,
                                                                       int *__restrict__ err) {
-    constexpr int RM = 4, CN = 4, NW = 8 * H;
+    constexpr int H = R >= 64 ? R / 64 : 1;         // row tiles brought in
+    constexpr int RM = 4, CN = 4, NW = R / 8;
     constexpr int TCH = PB * kTiledRows;            // floats per array, stage and 64-row (or target) tile
     constexpr int RCH = H * TCH;
-    constexpr int SST = 2 * RCH + 2 * TCH;          // floats per stage
+    constexpr int OQ = (KL ? 2 : 1) * RCH, OT = OQ + (TV ? TCH : 0);
+    constexpr int SST = OT + (KL ? TCH : 0);        // floats per stage
     extern __shared__ __align__(128) float psm[];   // [stage][P rows, log2 rows, P targets, log2 targets]
     __shared__ __align__(8) uint64_t full[PS], empty[PS];
     const int tid = threadIdx.x, lane = tid & 31;
     const int tx = tid % (kTiledRows / CN), ty = tid / (kTiledRows / CN);
     // target tiles vary fastest over the grid: the CTAs that read one pair of
     // row tiles run together and share it through L2
-    const int64_t x0 = (int64_t)blockIdx.y * H * kTiledRows;
+    const int64_t x0 = (int64_t)blockIdx.y * R;
     const int a0 = blockIdx.x * kTiledRows;
-    const float *gP = PT + (int64_t)blockIdx.y * H * kt * kTiledRows;
-    const float *gL = LT + (int64_t)blockIdx.y * H * kt * kTiledRows;
+    const float *gP = PT + x0 / kTiledRows * kt * kTiledRows;
+    const float *gL = LT + x0 / kTiledRows * kt * kTiledRows;
     const float *gQ = TQ + (int64_t)blockIdx.x * kt * kTiledRows;
     const float *gT = TL + (int64_t)blockIdx.x * kt * kTiledRows;
     const int nch = (int)(kt / PB);
@@ -821,8 +829,8 @@ __global__ void __launch_bounds__(256 * H, 2 / H) field_tile_pipe_kernel(const f
             bulk_g2s(st + h * TCH, gP + (int64_t)h * kt * kTiledRows + go, kArr, &full[s]);
             if (KL) bulk_g2s(st + RCH + h * TCH, gL + (int64_t)h * kt * kTiledRows + go, kArr, &full[s]);
         }
-        if (TV) bulk_g2s(st + 2 * RCH, gQ + go, kArr, &full[s]);
-        if (KL) bulk_g2s(st + 2 * RCH + TCH, gT + go, kArr, &full[s]);
+        if (TV) bulk_g2s(st + OQ, gQ + go, kArr, &full[s]);
+        if (KL) bulk_g2s(st + OT, gT + go, kArr, &full[s]);
     };
     if (tid == 0) {
         for (int s = 0; s < PS; ++s) {
@@ -842,7 +850,7 @@ __global__ void __launch_bounds__(256 * H, 2 / H) field_tile_pipe_kernel(const f
 #pragma unroll
         for (int c = 0; c < CN; ++c) kl[r][c] = tv[r][c] = klc[r][c] = ckl[r][c] = ctv[r][c] = 0.0f;
     // this thread's rows within the stage: 64-row half ty / 16, rows (ty % 16) * 4 ..
-    const int roff = (ty / 16) * TCH + (ty % 16) * RM;
+    const int roff = (ty / 16) * TCH + (ty % 16) * RM + (int)(x0 % kTiledRows);
     bool ok = true;
     int c = 0;
     for (; c < nch; ++c) {
@@ -861,8 +869,8 @@ __global__ void __launch_bounds__(256 * H, 2 / H) field_tile_pipe_kernel(const f
             break;
         }
         const float *cP = psm + s * SST + roff;
-        const float *cQ = psm + s * SST + 2 * RCH + tx * CN;
-        pipe_stage<KL, TV, PB, UNR>(cP, cP + RCH, cQ, cQ + TCH, ckl, ctv);
+        const float *cS = psm + s * SST + tx * CN;
+        pipe_stage<KL, TV, PB, UNR>(cP, cP + RCH, cS + OQ, cS + OT, ckl, ctv);
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[s]);
         // 64-column partial sums, merged at the end of every 64 columns
@@ -1343,24 +1351,33 @@ constexpr int kPipeShape = 3;      // the pipelined tile on the tiled layout (si
 
 // the pipelined tile: 128 rows x 64 targets per CTA of 512 threads (one CTA per
 // SM), two stages of 64 columns (192 KB of shared memory); the column loop is
-// unrolled 16 deep for KL+TV and 32 deep for one field
+// unrolled 16 deep for KL+TV and 32 deep for one field.  TV alone (the FP32
+// pass of maps whose KL the tensor cores form) takes 64 or 32 rows a CTA
+// where that shortens the fullest SM's share: grid140 with 64 targets has 154
+// tiles of 128 rows for 152 SMs, and two of them took as long again (125 us;
+// 85 us with 32 rows).
 void launch_pipe(const TiledArgs &ta, int64_t n_v, int32_t T, float *out_kl, float *out_tv, int *err,
                  cudaStream_t s) {
-    constexpr int H = 2, PB = 64, PS = 2;
-    const dim3 g((unsigned)((T + kTiledRows - 1) / kTiledRows),
-                 (unsigned)((n_v + H * kTiledRows - 1) / (H * kTiledRows)));
-    auto go = [&](auto kern) {
-        const size_t smem = (size_t)PS * (2 * H + 2) * PB * kTiledRows * sizeof(float);
+    const int nat = (T + kTiledRows - 1) / kTiledRows;
+    auto go = [&](auto kern, int R, size_t smem) {
+        const dim3 g((unsigned)nat, (unsigned)((n_v + R - 1) / R));
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         KMark km_("field_tile_kernel", s);
-        kern<<<g, 256 * H, smem, s>>>(ta.PT, ta.LT, n_v, ta.kt, ta.TQ, ta.TL, T, out_kl, out_tv, err);
+        kern<<<g, 4 * R, smem, s>>>(ta.PT, ta.LT, n_v, ta.kt, ta.TQ, ta.TL, T, out_kl, out_tv, err);
     };
     if (out_kl && out_tv)
-        go(field_tile_pipe_kernel<true, true, H, PB, PS, 16>);
-    else if (out_kl)
-        go(field_tile_pipe_kernel<true, false, H, PB, PS, 32>);
+        return go(field_tile_pipe_kernel<true, true, 128, 64, 2, 16>, 128, pipe_smem<true, true, 128, 64, 2>());
+    if (out_kl)
+        return go(field_tile_pipe_kernel<true, false, 128, 64, 2, 32>, 128, pipe_smem<true, false, 128, 64, 2>());
+    // rows of the fullest SM, smaller tiles charged for their share of the copies
+    auto share = [&](int R) { return (((n_v + R - 1) / R * nat + num_sms() - 1) / num_sms()) * R; };
+    const int64_t c128 = share(128) * 100, c64 = share(64) * 103, c32 = share(32) * 108;
+    if (c128 <= c64 && c128 <= c32)
+        go(field_tile_pipe_kernel<false, true, 128, 64, 2, 32>, 128, pipe_smem<false, true, 128, 64, 2>());
+    else if (c64 <= c32)
+        go(field_tile_pipe_kernel<false, true, 64, 64, 2, 32>, 64, pipe_smem<false, true, 64, 64, 2>());
     else
-        go(field_tile_pipe_kernel<false, true, H, PB, PS, 32>);
+        go(field_tile_pipe_kernel<false, true, 32, 32, 3, 32>, 32, pipe_smem<false, true, 32, 32, 3>());
 }
 
 void launch_variant(int v, const float *P, int64_t n_v, int64_t k_pad, const float *sP, const float *sL,
