@@ -55,6 +55,7 @@
 #include "dd_bulk.cuh"
 #include "dd_f32x2.cuh"
 #include "dd_internal.h"
+#include "dd_logtable.cuh"
 
 namespace {
 
@@ -309,11 +310,9 @@ struct Log2Tab {
 };
 __device__ __forceinline__ void build_log2_table(Log2Tab &t) {
     for (int j = threadIdx.x; j < kTab; j += blockDim.x) {
-        const float r = (float)(1.0 / (1.0 + (j + 0.5) / kTab));
-        const double l = -log2((double)r), h = rint(l * 4096.0) / 4096.0;
-        t.r[j] = r;
-        t.h[j] = (float)h;
-        t.l[j] = (float)(l - h);
+        t.r[j] = __uint_as_float(kLogTableBits[j]);
+        t.h[j] = __uint_as_float(kLogTableBits[2 * kTab + j]);
+        t.l[j] = __uint_as_float(kLogTableBits[3 * kTab + j]);
     }
 }
 __device__ __forceinline__ float2 log2_pair(float p, const Log2Tab &t) {
