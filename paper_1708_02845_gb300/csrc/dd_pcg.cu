@@ -126,13 +126,14 @@ __global__ void alpha_kernel(int64_t nrb, int64_t kc, const double *__restrict__
     if (threadIdx.y == 0 && c < kc) alpha[c] = (!done[c] && pAp > 0.0) ? rz[c] / pAp : 0.0;
 }
 
-__global__ void beta_kernel(int64_t nrb, int64_t kc, const double *__restrict__ part_rz,
+// (nrz, nrb: how many partials part_rz and part_rr hold a column)
+__global__ void beta_kernel(int64_t nrz, int64_t nrb, int64_t kc, const double *__restrict__ part_rz,
                             const double *__restrict__ part_rr, const double *__restrict__ bnorm,
                             double *__restrict__ rz, const int *__restrict__ done,
                             double *__restrict__ beta, unsigned long long *__restrict__ maxres) {
     __shared__ double sh[kSumRows][33];
     const int64_t c = (int64_t)blockIdx.x * 32 + threadIdx.x;
-    double rz_new = column_sum(part_rz, nrb, kc, c, sh);
+    double rz_new = column_sum(part_rz, nrz, kc, c, sh);
     double rr = column_sum(part_rr, nrb, kc, c, sh);
     if (threadIdx.y == 0 && c < kc) {
         double res = bnorm[c] > 0.0 ? sqrt(rr) / bnorm[c] : 0.0;
@@ -301,16 +302,23 @@ __device__ __forceinline__ double widen(float f) {
 
 constexpr int kPairs = 64;      // column pairs (threads) of one CTA
 
+// The sparse products' CTAs: 16 pairs of columns (256 bytes of a row) x 32
+// rows at a time, down a band of consecutive rows.  A row of X is read by
+// every row of its stencil, grid lines apart; a CTA that holds 64 pairs and
+// eight rows reads most of them from L2 again (Q^T of grid140's finest level
+// 180 us, L2's bandwidth), a narrow band keeps the last few lines in L1
+// (the four Q^T of grid140 together 238 -> 117 us a cycle).
+constexpr int kBandPairs = 16, kBandRows = 32;
+
 // Y = M X
-__global__ void __launch_bounds__(kPairs) df_spmm_kernel(int64_t rows, int64_t kp, const int32_t *__restrict__ off,
-                                                         const int32_t *__restrict__ col,
-                                                         const float2 *__restrict__ val, const float4 *__restrict__ X,
-                                                         float4 *__restrict__ Y, int rpb) {
-    const int64_t c = (int64_t)blockIdx.y * kPairs + threadIdx.x;
+__global__ void __launch_bounds__(kBandPairs *kBandRows, 2)
+    df_spmm_kernel(int64_t rows, int64_t kp, const int32_t *__restrict__ off, const int32_t *__restrict__ col,
+                   const float2 *__restrict__ val, const float4 *__restrict__ X, float4 *__restrict__ Y, int band) {
+    const int64_t c = (int64_t)blockIdx.y * kBandPairs + threadIdx.x;
     if (c >= kp) return;
-    const int64_t r0 = (int64_t)blockIdx.x * rpb;
-    const int64_t r1 = r0 + rpb < rows ? r0 + rpb : rows;
-    for (int64_t r = r0; r < r1; ++r) {
+    const int64_t r0 = (int64_t)blockIdx.x * band;
+    const int64_t r1 = r0 + band < rows ? r0 + band : rows;
+    for (int64_t r = r0 + threadIdx.y; r < r1; r += kBandRows) {
         f2_t s = 0ULL, cc = 0ULL;
 #pragma unroll 4
         for (int q = off[r]; q < off[r + 1]; ++q) df_fma(s, cc, val[q], df_load(X + (int64_t)col[q] * kp + c));
@@ -321,37 +329,48 @@ __global__ void __launch_bounds__(kPairs) df_spmm_kernel(int64_t rows, int64_t k
 // Z = G B + Q E (E: rows of the next level).  FINE: Z in FP64, with partial
 // column sums of R . Z; else Z in pairs like B.
 template <bool FINE>
-__global__ void __launch_bounds__(kPairs) df_up_kernel(int64_t rows, int64_t kp, const int32_t *__restrict__ goff,
-                                                       const int32_t *__restrict__ gcol,
-                                                       const float2 *__restrict__ gval,
-                                                       const int32_t *__restrict__ qoff,
-                                                       const int32_t *__restrict__ qcol,
-                                                       const float2 *__restrict__ qval, const float4 *__restrict__ B,
-                                                       const float4 *__restrict__ E, const double2 *__restrict__ R,
-                                                       void *__restrict__ Z, double2 *__restrict__ part, int rpb) {
-    const int64_t c = (int64_t)blockIdx.y * kPairs + threadIdx.x;
-    if (c >= kp) return;
-    const int64_t r0 = (int64_t)blockIdx.x * rpb;
-    const int64_t r1 = r0 + rpb < rows ? r0 + rpb : rows;
+__global__ void __launch_bounds__(kBandPairs *kBandRows, 2)
+    df_up_kernel(int64_t rows, int64_t kp, const int32_t *__restrict__ goff, const int32_t *__restrict__ gcol,
+                 const float2 *__restrict__ gval, const int32_t *__restrict__ qoff, const int32_t *__restrict__ qcol,
+                 const float2 *__restrict__ qval, const float4 *__restrict__ B, const float4 *__restrict__ E,
+                 const double2 *__restrict__ R, void *__restrict__ Z, double2 *__restrict__ part, int band) {
+    __shared__ double2 sum[FINE ? kBandRows : 1][kBandPairs];
+    const int64_t c = (int64_t)blockIdx.y * kBandPairs + threadIdx.x;
+    const int64_t r0 = (int64_t)blockIdx.x * band;
+    const int64_t r1 = r0 + band < rows ? r0 + band : rows;
     double d0 = 0.0, d1 = 0.0;
-    for (int64_t r = r0; r < r1; ++r) {
-        f2_t s = 0ULL, cc = 0ULL;
+    if (c < kp) {
+        for (int64_t r = r0 + threadIdx.y; r < r1; r += kBandRows) {
+            f2_t s = 0ULL, cc = 0ULL;
 #pragma unroll 4
-        for (int q = goff[r]; q < goff[r + 1]; ++q) df_fma(s, cc, gval[q], df_load(B + (int64_t)gcol[q] * kp + c));
+            for (int q = goff[r]; q < goff[r + 1]; ++q)
+                df_fma(s, cc, gval[q], df_load(B + (int64_t)gcol[q] * kp + c));
 #pragma unroll 4
-        for (int q = qoff[r]; q < qoff[r + 1]; ++q) df_fma(s, cc, qval[q], df_load(E + (int64_t)qcol[q] * kp + c));
-        const float4 z = df_pack(df_norm(s, cc));
-        if (FINE) {
-            const double2 v = R[r * kp + c];
-            const double z0 = widen(z.x) + widen(z.z), z1 = widen(z.y) + widen(z.w);
-            static_cast<double2 *>(Z)[r * kp + c] = make_double2(z0, z1);
-            d0 += v.x * z0;
-            d1 += v.y * z1;
-        } else {
-            static_cast<float4 *>(Z)[r * kp + c] = z;
+            for (int q = qoff[r]; q < qoff[r + 1]; ++q)
+                df_fma(s, cc, qval[q], df_load(E + (int64_t)qcol[q] * kp + c));
+            const float4 z = df_pack(df_norm(s, cc));
+            if (FINE) {
+                const double2 v = R[r * kp + c];
+                const double z0 = widen(z.x) + widen(z.z), z1 = widen(z.y) + widen(z.w);
+                static_cast<double2 *>(Z)[r * kp + c] = make_double2(z0, z1);
+                d0 += v.x * z0;
+                d1 += v.y * z1;
+            } else {
+                static_cast<float4 *>(Z)[r * kp + c] = z;
+            }
         }
     }
-    if (FINE) part[(int64_t)blockIdx.x * kp + c] = make_double2(d0, d1);
+    if (FINE) {
+        sum[threadIdx.y][threadIdx.x] = make_double2(d0, d1);
+        __syncthreads();
+        if (threadIdx.y == 0 && c < kp) {
+            for (int y = 1; y < kBandRows; ++y) {
+                d0 += sum[y][threadIdx.x].x;
+                d1 += sum[y][threadIdx.x].y;
+            }
+            part[(int64_t)blockIdx.x * kp + c] = make_double2(d0, d1);
+        }
+    }
 }
 
 // X = Ainv B on the coarsest level (Ainv dense n x n, row-major)
@@ -455,12 +474,12 @@ __global__ void coarse_solve_kernel(int64_t n, int64_t kc, const double *__restr
 }
 
 // rz = column sums of part_rz, bnorm from part_rr, done flags (first iteration)
-__global__ void amg_init_scalars_kernel(int64_t nrb, int64_t kc, const double *__restrict__ part_rz,
+__global__ void amg_init_scalars_kernel(int64_t nrz, int64_t nrb, int64_t kc, const double *__restrict__ part_rz,
                                         const double *__restrict__ part_rr, double *__restrict__ rz,
                                         double *__restrict__ bnorm, int *__restrict__ done) {
     __shared__ double sh[kSumRows][33];
     const int64_t c = (int64_t)blockIdx.x * 32 + threadIdx.x;
-    double s_rz = column_sum(part_rz, nrb, kc, c, sh);
+    double s_rz = column_sum(part_rz, nrz, kc, c, sh);
     double s_rr = column_sum(part_rr, nrb, kc, c, sh);
     if (threadIdx.y == 0 && c < kc) {
         rz[c] = s_rz;
@@ -475,11 +494,14 @@ cudaError_t alloc(T **p, size_t count) {
 }
 
 // rows per CTA for a [rows][kc] block: enough CTAs (about 16 per SM), at most 256 rows
-int rows_per_block(int64_t rows, int64_t kc) {
+int sm_count() {
     int sms = 0, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (sms <= 0) sms = 1;
+    return sms > 0 ? sms : 1;
+}
+int rows_per_block(int64_t rows, int64_t kc) {
+    const int sms = sm_count();
     const int64_t colblocks = (kc + kColsPerBlock - 1) / kColsPerBlock;
     const int64_t want = rows * colblocks / (16LL * sms);
     int rpb = 256;
@@ -535,8 +557,14 @@ dd_status run_pcg_amg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s,
     const int64_t kp = kc / 2;
     const int rpb0 = rows_per_block(m, kc);
     const int64_t nrb = (m + rpb0 - 1) / rpb0;
-    std::vector<int> rpb(nl);
-    for (int l = 0; l < nl; ++l) rpb[l] = rows_per_block(H.levels[l].A.rows, kc);
+    // rows of a sparse product's band: two CTAs an SM over all columns, at least 32 rows
+    std::vector<int> band(nl);
+    const int64_t colb = (kp + kBandPairs - 1) / kBandPairs;
+    for (int l = 0; l < nl; ++l) {
+        const int64_t nb = std::max<int64_t>(1, 2LL * sm_count() / colb), rows = H.levels[l].A.rows;
+        band[l] = (int)std::max<int64_t>(kBandRows, (rows + nb - 1) / nb);
+    }
+    const int64_t nbands = (m + band[0] - 1) / band[0];
 
     // one device allocation for the hierarchy and the workspace (a solve has
     // dozens of arrays; allocated and freed one by one they cost 2 ms), the
@@ -577,7 +605,7 @@ dd_status run_pcg_amg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s,
         o_b[l] = take(lv);
         if (l > 0) o_x[l] = take(lv);
     }
-    const size_t o_p0 = take((size_t)nrb * kc * sizeof(double)), o_p1 = take((size_t)nrb * kc * sizeof(double));
+    const size_t o_p0 = take((size_t)std::max(nrb, nbands) * kc * sizeof(double)), o_p1 = take((size_t)nrb * kc * sizeof(double));
     const size_t o_al = take(kc * sizeof(double)), o_be = take(kc * sizeof(double)), o_rz = take(kc * sizeof(double));
     const size_t o_bn = take(kc * sizeof(double)), o_dn = take(kc * sizeof(int));
     const size_t o_mr = take(sizeof(unsigned long long));
@@ -628,26 +656,28 @@ dd_status run_pcg_amg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s,
     auto grid2 = [&](int64_t rows, int rb) {
         return dim3((unsigned)((rows + rb - 1) / rb), (unsigned)((kp + kPairs - 1) / kPairs));
     };
+    auto bands = [&](int l) {
+        return dim3((unsigned)((H.levels[l].A.rows + band[l] - 1) / band[l]), (unsigned)colb);
+    };
+    const dim3 bb(kBandPairs, kBandRows);
     // Z = V(the fine level's pairs lb(0)), partial sums of R . Z into part0
     auto vcycle = [&]() {
-        for (int l = 0; l + 1 < nl; ++l) {
-            const int64_t nc = H.levels[l + 1].A.rows;
-            df_spmm_kernel<<<grid2(nc, rpb[l + 1]), kPairs, 0, s>>>(nc, kp, dQt[l].off, dQt[l].col, dQt[l].val, lb(l),
-                                                                    lb(l + 1), rpb[l + 1]);
-        }
+        for (int l = 0; l + 1 < nl; ++l)
+            df_spmm_kernel<<<bands(l + 1), bb, 0, s>>>(H.levels[l + 1].A.rows, kp, dQt[l].off, dQt[l].col, dQt[l].val,
+                                                      lb(l), lb(l + 1), band[l + 1]);
         const int64_t nc = H.levels[nl - 1].A.rows;
         df_coarse_kernel<<<dim3((unsigned)((kp + kPairs - 1) / kPairs), (unsigned)nc), kPairs, 0, s>>>(
             nc, kp, reinterpret_cast<const float2 *>(ws + o_ainv), lb(nl - 1), lx(nl - 1));
         for (int l = nl - 2; l >= 0; --l) {
             const int64_t n = H.levels[l].A.rows;
             if (l > 0)
-                df_up_kernel<false><<<grid2(n, rpb[l]), kPairs, 0, s>>>(
-                    n, kp, dG[l].off, dG[l].col, dG[l].val, dQ[l].off, dQ[l].col, dQ[l].val, lb(l), lx(l + 1), nullptr,
-                    lx(l), nullptr, rpb[l]);
+                df_up_kernel<false><<<bands(l), bb, 0, s>>>(n, kp, dG[l].off, dG[l].col, dG[l].val, dQ[l].off,
+                                                            dQ[l].col, dQ[l].val, lb(l), lx(l + 1), nullptr, lx(l),
+                                                            nullptr, band[l]);
             else
-                df_up_kernel<true><<<grid2(n, rpb[l]), kPairs, 0, s>>>(
-                    n, kp, dG[l].off, dG[l].col, dG[l].val, dQ[l].off, dQ[l].col, dQ[l].val, lb(l), lx(l + 1), d2(R), Z,
-                    d2(part0), rpb[l]);
+                df_up_kernel<true><<<bands(l), bb, 0, s>>>(n, kp, dG[l].off, dG[l].col, dG[l].val, dQ[l].off,
+                                                           dQ[l].col, dQ[l].val, lb(l), lx(l + 1), d2(R), Z, d2(part0),
+                                                           band[l]);
         }
     };
 
@@ -672,7 +702,7 @@ dd_status run_pcg_amg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s,
         }
         df_first_kernel<<<grid2(m, rpb0), kPairs, 0, s>>>(m, kp, d2(R), lb(0), d2(part1), rpb0);
         vcycle();
-        amg_init_scalars_kernel<<<gc, bc, 0, s>>>(nrb, kc, part0, part1, rz, bnorm, done);
+        amg_init_scalars_kernel<<<gc, bc, 0, s>>>(nbands, nrb, kc, part0, part1, rz, bnorm, done);
         cudaMemcpyAsync(Pd, Z, vec, cudaMemcpyDeviceToDevice, s);
         int32_t it = 0;
         double res = 1.0;
@@ -682,7 +712,7 @@ dd_status run_pcg_amg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s,
             update_r_kernel<<<grid2(m, rpb0), kPairs, 0, s>>>(m, kp, d2(alpha), d2(R), d2(AP), lb(0), d2(part1), rpb0);
             vcycle();
             cudaMemsetAsync(maxres, 0, sizeof(unsigned long long), s);
-            beta_kernel<<<gc, bc, 0, s>>>(nrb, kc, part0, part1, bnorm, rz, done, beta, maxres);
+            beta_kernel<<<gc, bc, 0, s>>>(nbands, nrb, kc, part0, part1, bnorm, rz, done, beta, maxres);
             update_xp_kernel<<<grid2(m, rpb0), kPairs, 0, s>>>(m, kp, d2(alpha), d2(beta), d2(Z), d2(X), d2(Pd), rpb0);
             if (it % check_every == 0 || it == max_iter) {
                 unsigned long long bits = 0;
@@ -836,7 +866,7 @@ dd_status run_pcg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s, int
             update_xr_kernel<<<g2, kColsPerBlock, 0, s>>>(m, kc, w.alpha, w.dinv, w.X, w.R, w.Pd, w.AP, w.part0,
                                                           w.part1, rpb);
             cudaMemsetAsync(w.maxres, 0, sizeof(unsigned long long), s);
-            beta_kernel<<<gc, bc, 0, s>>>(w.nrb, kc, w.part0, w.part1, w.bnorm, w.rz, w.done, w.beta,
+            beta_kernel<<<gc, bc, 0, s>>>(w.nrb, w.nrb, kc, w.part0, w.part1, w.bnorm, w.rz, w.done, w.beta,
                                           w.maxres);
             update_p_kernel<<<g2, kColsPerBlock, 0, s>>>(m, kc, w.beta, w.dinv, w.R, w.Pd, rpb);
             if (it % check_every == 0 || it == max_iter) {
