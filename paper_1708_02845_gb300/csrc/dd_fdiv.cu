@@ -33,6 +33,7 @@
 #include <algorithm>
 #include <cfloat>
 #include <cmath>
+#include <type_traits>
 
 #include "dd_f32x2.cuh"
 #include "dd_internal.h"
@@ -140,15 +141,15 @@ __device__ __forceinline__ float klrev_logp_term(float pt, float lmt, float Ebt,
 // rows whose first-pass value is below q.below = max(DD_EXACT_BELOW,
 // 2e5 |lin| / |e| 2^-22) are recomputed in the exact form, and every other
 // value is within 1e-5 / 2 of exact, relatively.  The entries with P_x = 0 or
-// P_t = 0 take their limits by selection, evaluated only when a lane of the
-// warp holds one; every lane of the warp must call it (padding entries pass
-// P_x = P_t = 0 and give 0).
+// P_t = 0 take their limits by selection (ZEROS), for the chunks that hold one
+// (padding entries pass P_x = P_t = 0 and give 0).
 // Four entries of a row as every target of a pass reads them: the entries,
 // their hardware mantissa logs and biased exponents, packed by pairs.
 struct Row4 {
     f2_t p[2], lf[2], eb[2];
-    bool zero;                   // an entry is 0
 };
+// whether an entry is 0 (entries are not negative)
+__device__ __forceinline__ bool has_zero(const float4 &v) { return fminf(fminf(v.x, v.y), fminf(v.z, v.w)) == 0.0f; }
 __device__ __forceinline__ Row4 row_side(const float4 &v) {
     const float px[4] = {v.x, v.y, v.z, v.w};
     Row4 r;
@@ -161,12 +162,12 @@ __device__ __forceinline__ Row4 row_side(const float4 &v) {
         r.eb[h] = pk(__int_as_float((int)__funnelshift_r((unsigned)b0, (unsigned)kMagicHi, 23)),
                      __int_as_float((int)__funnelshift_r((unsigned)b1, (unsigned)kMagicHi, 23)));
     }
-    r.zero = fminf(fminf(px[0], px[1]), fminf(px[2], px[3])) == 0.0f;      // entries are not negative
     return r;
 }
 
+template <bool ZEROS>
 __device__ __forceinline__ void alpha_fast4(const Row4 &x, const f2_t (&pe)[2], const float4 &p4, const float4 &f4,
-                                            const float4 &e4, bool t_zero, const FdParams &q, f2_t &sum) {
+                                            const float4 &e4, const FdParams &q, f2_t &sum) {
     // the adds and multiplies two entries at a time in packed FP32x2 (each half
     // rounds exactly as the scalar operation: a product is fma(a, b, 0));
     // pe = -P_x / e, which every target of the pass shares
@@ -185,9 +186,7 @@ __device__ __forceinline__ void alpha_fast4(const Row4 &x, const f2_t (&pe)[2], 
         const f2_t um1 = add2(pk(ex2_hw(y0), ex2_hw(y1)), mone);                    // 2^(e L2) - 1
         t[h] = fma2(fma2(pe[h], um1, fma2(x.p[h], mone, pt2)), lin2, zero);         // (P_t - P_x) - P_x um1 / e
     }
-    // a zero entry on either side takes its limit; the warp looks only where one
-    // of its 128 row entries or target entries is 0
-    if (__any_sync(0xffffffffu, x.zero) || t_zero) {
+    if (ZEROS) {      // an entry 0 on either side takes its limit
         const float at_px0 = q.alpha_gt1 ? INFINITY : q.lin;
         const float pt[4] = {p4.x, p4.y, p4.z, p4.w};
         float px[4], v[4];
@@ -342,7 +341,7 @@ __global__ void __launch_bounds__(256) fdiv_kernel(const float *__restrict__ P, 
 // TT targets a CTA (blockIdx.y: which TT of them): P is read, and its entries'
 // logarithms formed, once for both.  One target at a time, the alpha
 // divergence of two targets (300 x 300 cells) took 424 us, bound by the
-// hardware log2 and exp2 and the instructions around them; 352 us with two.
+// hardware log2 and exp2 and the instructions around them; 323 us with two.
 template <int FAM, int TT>
 __global__ void __launch_bounds__(256 * TT, 2 / TT) two_pass_kernel(const float *__restrict__ P, int64_t n_v,
                                                                int64_t k_pad, const float *__restrict__ sP,
@@ -353,12 +352,12 @@ __global__ void __launch_bounds__(256 * TT, 2 / TT) two_pass_kernel(const float 
     constexpr int U = TT == 1 ? 8 : 4;       // float4 per lane and buffer: 4 KB per warp and target in flight
     extern __shared__ __align__(16) float fsm[];
     __shared__ float tab[2 * kLogTab];
-    __shared__ unsigned char tz[TT][kMaxGroups];      // a group of the target's entries (32 float4) holds a 0
+    __shared__ unsigned char tz[kMaxGroups];      // a target's group of entries (32 float4) holds a 0
     // the staged rows zero-padded to whole groups of 32 float4 (two_pass_pitch):
     // every lane of a group reads its target entries without a test
     const int64_t kp = two_pass_pitch(k_pad);
     const int a = a0 + blockIdx.y * TT;
-    for (int i = threadIdx.x; i < TT * kMaxGroups; i += blockDim.x) (&tz[0][0])[i] = 0;
+    for (int i = threadIdx.x; i < kMaxGroups; i += blockDim.x) tz[i] = 0;
     __syncthreads();
     for (int i = 0; i < TT; ++i)
         for (int64_t b = threadIdx.x; b < kp; b += blockDim.x) {
@@ -367,7 +366,7 @@ __global__ void __launch_bounds__(256 * TT, 2 / TT) two_pass_kernel(const float 
             float *t = fsm + 4 * i * kp + b;
             const float p = in ? sP[o] : 0.0f;
             t[0] = p;
-            if (p == 0.0f) tz[i][b >> 7] = 1;
+            if (p == 0.0f) tz[b >> 7] = 1;
             t[kp] = in ? sL[o] : 0.0f;
             t[2 * kp] = in ? sE[o] : 0.0f;
             t[3 * kp] = in ? sF[o] : 0.0f;
@@ -383,35 +382,55 @@ __global__ void __launch_bounds__(256 * TT, 2 / TT) two_pass_kernel(const float 
     f2_t sums[TT];
 #pragma unroll
     for (int i = 0; i < TT; ++i) sums[i] = zero2;
-    auto chunk = [&](const float4(&v)[U], int64_t, int c0) {
+    // one float4 of the row against every target of the pass
+    auto group = [&](const float4 &v, int c, auto zeros) {
+        float4 w = v;
+        if (FAM == kKlRev)                    // a row entry 0 is taken at FLT_MIN
+            w = make_float4(fmaxf(w.x, FLT_MIN), fmaxf(w.y, FLT_MIN), fmaxf(w.z, FLT_MIN), fmaxf(w.w, FLT_MIN));
+        const Row4 x = row_side(w);
+        f2_t pe[2] = {zero2, zero2};
+        if (FAM == kAlpha) {
+            pe[0] = fma2(x.p[0], nie2, zero2);
+            pe[1] = fma2(x.p[1], nie2, zero2);
+        }
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (c0 + u * 32 >= nvec) break;      // the same for the whole warp
-            const int c = c0 + u * 32 + lane;
-            float4 w = v[u];
-            if (FAM == kKlRev)                    // a row entry 0 is taken at FLT_MIN
-                w = make_float4(fmaxf(w.x, FLT_MIN), fmaxf(w.y, FLT_MIN), fmaxf(w.z, FLT_MIN), fmaxf(w.w, FLT_MIN));
-            const Row4 x = row_side(w);
-            f2_t pe[2] = {zero2, zero2};
+        for (int i = 0; i < TT; ++i) {
+            // past the row's end P and the padded target row are 0, and so is the term
+            const float4 p4 = tg[4 * i * kv + c], f4 = tg[(4 * i + 3) * kv + c], e4 = tg[(4 * i + 2) * kv + c];
             if (FAM == kAlpha) {
-                pe[0] = fma2(x.p[0], nie2, zero2);
-                pe[1] = fma2(x.p[1], nie2, zero2);
-            }
+                alpha_fast4<decltype(zeros)::value>(x, pe, p4, f4, e4, q, sums[i]);
+            } else {
 #pragma unroll
-            for (int i = 0; i < TT; ++i) {
-                // past the row's end P and the padded target row are 0, and so is the term
-                const float4 p4 = tg[4 * i * kv + c], f4 = tg[(4 * i + 3) * kv + c], e4 = tg[(4 * i + 2) * kv + c];
-                if (FAM == kAlpha) {
-                    alpha_fast4(x, pe, p4, f4, e4, tz[i][(c0 >> 5) + u] != 0, q, sums[i]);
-                } else {
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const f2_t pt2 = h ? pk(p4.z, p4.w) : pk(p4.x, p4.y);
-                        const f2_t ft2 = h ? pk(f4.z, f4.w) : pk(f4.x, f4.y);
-                        const f2_t et2 = h ? pk(e4.z, e4.w) : pk(e4.x, e4.y);
-                        sums[i] = fma2(pt2, add2(fma2(x.lf[h], mone, ft2), fma2(x.eb[h], mone, et2)), sums[i]);
-                    }
+                for (int h = 0; h < 2; ++h) {
+                    const f2_t pt2 = h ? pk(p4.z, p4.w) : pk(p4.x, p4.y);
+                    const f2_t ft2 = h ? pk(f4.z, f4.w) : pk(f4.x, f4.y);
+                    const f2_t et2 = h ? pk(e4.z, e4.w) : pk(e4.x, e4.y);
+                    sums[i] = fma2(pt2, add2(fma2(x.lf[h], mone, ft2), fma2(x.eb[h], mone, et2)), sums[i]);
                 }
+            }
+        }
+    };
+    // whole chunks without a zero run straight through (a test and a branch for
+    // every float4 and target left one of them in flight at a time)
+    auto chunk = [&](const float4(&v)[U], int64_t, int c0) {
+        bool plain = c0 + 32 * U <= nvec;
+        if (FAM == kAlpha) {
+            bool z = false;
+#pragma unroll
+            for (int u = 0; u < U; ++u) z |= has_zero(v[u]) || tz[min((c0 >> 5) + u, kMaxGroups - 1)];
+            plain = !__any_sync(0xffffffffu, z) && plain;
+        }
+        if (plain) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) group(v[u], c0 + u * 32 + lane, std::false_type());
+        } else {
+#pragma unroll 1
+            for (int u = 0; u < U && c0 + u * 32 < nvec; ++u) {      // the same for the whole warp
+                float4 w = v[0];
+#pragma unroll
+                for (int j = 1; j < U; ++j)
+                    if (u == j) w = v[j];
+                group(w, c0 + u * 32 + lane, std::true_type());
             }
         }
     };
