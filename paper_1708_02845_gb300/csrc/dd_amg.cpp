@@ -21,6 +21,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <future>
 #include <string>
 #include <vector>
 
@@ -32,12 +33,28 @@ constexpr double kTheta = 0.08;
 constexpr int64_t kCoarsest = 64;
 constexpr int kMaxLevels = 16;
 
+// ascending; the rows here touch a dozen columns
+void sort_short(std::vector<int32_t> &v) {
+    if (v.size() > 32) {
+        std::sort(v.begin(), v.end());
+        return;
+    }
+    for (size_t i = 1; i < v.size(); ++i) {
+        const int32_t x = v[i];
+        size_t j = i;
+        for (; j > 0 && v[j - 1] > x; --j) v[j] = v[j - 1];
+        v[j] = x;
+    }
+}
+
 // C = A B (Gustavson: one dense accumulator row with a touched list)
 AmgCsr spgemm(const AmgCsr &A, const AmgCsr &B) {
     AmgCsr C;
     C.rows = A.rows;
     C.cols = B.cols;
     C.off.assign(A.rows + 1, 0);
+    C.col.reserve(A.col.size() + B.col.size());
+    C.val.reserve(A.col.size() + B.col.size());
     std::vector<double> acc(B.cols, 0.0);
     std::vector<int32_t> mark(B.cols, -1), touched;
     for (int64_t i = 0; i < A.rows; ++i) {
@@ -45,7 +62,7 @@ AmgCsr spgemm(const AmgCsr &A, const AmgCsr &B) {
         for (int64_t p = A.off[i]; p < A.off[i + 1]; ++p) {
             const int32_t k = A.col[p];
             const double a = A.val[p];
-            for (int64_t q = B.off[k]; q < B.off[k + 1]; ++q) {
+            for (int64_t q = B.off[k], qe = B.off[k + 1]; q < qe; ++q) {
                 const int32_t j = B.col[q];
                 if (mark[j] != (int32_t)i) {
                     mark[j] = (int32_t)i;
@@ -55,7 +72,7 @@ AmgCsr spgemm(const AmgCsr &A, const AmgCsr &B) {
                 acc[j] += a * B.val[q];
             }
         }
-        std::sort(touched.begin(), touched.end());
+        sort_short(touched);
         for (int32_t j : touched) {
             C.col.push_back(j);
             C.val.push_back(acc[j]);
@@ -166,6 +183,8 @@ AmgCsr smoothed_prolongator(const AmgCsr &A, const std::vector<double> &d, const
     P.rows = A.rows;
     P.cols = na;
     P.off.assign(A.rows + 1, 0);
+    P.col.reserve(3 * A.rows);
+    P.val.reserve(3 * A.rows);
     std::vector<double> acc(na, 0.0);
     std::vector<int32_t> mark(na, -1), touched;
     for (int64_t i = 0; i < A.rows; ++i) {
@@ -180,7 +199,7 @@ AmgCsr smoothed_prolongator(const AmgCsr &A, const std::vector<double> &d, const
         };
         add(agg[i], 1.0);
         for (int64_t p = A.off[i]; p < A.off[i + 1]; ++p) add(agg[A.col[p]], -w * A.val[p] / d[i]);
-        std::sort(touched.begin(), touched.end());
+        sort_short(touched);
         for (int32_t g : touched) {
             if (acc[g] == 0.0) continue;
             P.col.push_back(g);
@@ -191,10 +210,10 @@ AmgCsr smoothed_prolongator(const AmgCsr &A, const std::vector<double> &d, const
     return P;
 }
 
-// The level's fused operators (AmgLevel): Q = P - w D^-1 (A P) on the pattern
-// of A P, which holds P's (A has its diagonal), Qt its transpose, and G on A's.
-void fuse_level(AmgLevel &L, const AmgCsr &A, AmgCsr &&AP) {
-    L.Q = std::move(AP);
+// The level's fused operators (AmgLevel): Q, which holds A P, becomes
+// P - w D^-1 (A P) on the pattern of A P, which holds P's (A has its diagonal), Qt its transpose, and G on A's.
+void fuse_level(AmgLevel &L) {
+    const AmgCsr &A = L.A;
     for (int64_t i = 0; i < A.rows; ++i) {
         const double w = L.omega * L.dinv[i];
         int64_t q = L.P.off[i];
@@ -251,9 +270,11 @@ bool dense_spd_inverse(const AmgCsr &A, std::vector<double> &inv) {
 
 }  // namespace
 
-bool build_amg(const AmgCsr &A0, AmgHierarchy &H, std::string &err) {
+bool build_amg(const AmgCsr &A0, AmgHierarchy &H, std::string &err, double rho0) {
     H = AmgHierarchy();
+    H.levels.reserve(kMaxLevels);      // a level's fused operators are formed while the next are built
     AmgCsr A = A0;
+    std::vector<std::future<void>> fused;      // waited for on every way out (their destructors do)
     for (int lev = 0; lev < kMaxLevels; ++lev) {
         const std::vector<double> d = diagonal(A);
         for (double v : d)
@@ -273,9 +294,10 @@ bool build_amg(const AmgCsr &A0, AmgHierarchy &H, std::string &err) {
             L.A = std::move(A);
             L.omega = 0.0;
             H.levels.push_back(std::move(L));
+            for (auto &f : fused) f.get();
             return true;
         }
-        const double rho = spectral_radius(A, d);
+        const double rho = lev == 0 && rho0 > 0.0 ? rho0 : spectral_radius(A, d);
         L.omega = 4.0 / (3.0 * rho);
         std::vector<int64_t> agg;
         const int64_t na = aggregate(A, d, agg);
@@ -286,6 +308,7 @@ bool build_amg(const AmgCsr &A0, AmgHierarchy &H, std::string &err) {
                 L.A = std::move(A);
                 L.omega = 0.0;
                 H.levels.push_back(std::move(L));
+                for (auto &f : fused) f.get();
                 return true;
             }
             err = "multigrid setup: aggregation did not coarsen";
@@ -295,9 +318,12 @@ bool build_amg(const AmgCsr &A0, AmgHierarchy &H, std::string &err) {
         L.R = transpose(L.P);
         AmgCsr AP = spgemm(A, L.P);
         AmgCsr Ac = spgemm(L.R, AP);
-        fuse_level(L, A, std::move(AP));
         L.A = std::move(A);
+        L.Q = std::move(AP);
         H.levels.push_back(std::move(L));
+        AmgLevel *last = &H.levels.back();
+        fused.push_back(std::async(lev == 0 ? std::launch::async | std::launch::deferred : std::launch::deferred,
+                                   [last] { fuse_level(*last); }));
         A = std::move(Ac);
     }
     err = "multigrid setup: too many levels";

@@ -39,8 +39,9 @@ struct AmgHierarchy {
 };
 
 // Build the hierarchy for the SPD matrix A0; false (with a message) when a
-// step fails.
-bool build_amg(const AmgCsr &A0, AmgHierarchy &H, std::string &err);
+// step fails.  rho0: the finest level's spectral radius of D^-1 A where the
+// caller has it (the power iteration's result), else 0.
+bool build_amg(const AmgCsr &A0, AmgHierarchy &H, std::string &err, double rho0 = 0.0);
 
 // The device solver's multigrid-preconditioned CG for one right-hand side, on
 // the host (a check of the hierarchy and the V-cycle without a GPU): solves

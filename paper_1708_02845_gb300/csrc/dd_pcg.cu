@@ -488,6 +488,71 @@ __global__ void amg_init_scalars_kernel(int64_t nrz, int64_t nrb, int64_t kc, co
     }
 }
 
+// One step of the power iteration for the largest eigenvalue of D^-1 A
+// (dd_amg.cpp: spectral_radius, from the same start), the fine level's: y =
+// D^-1 A x / |x|, with y's squared norm as one partial a CTA.  On
+// the host its 24 steps took a third of the hierarchy's setup (3 ms on
+// grid140).  part_x null: x is the start vector, formed here.
+constexpr int kPowerCtas = 128, kPowerSteps = 24;
+__device__ __forceinline__ double power_start(int64_t i) { return 1.0 + 0.5 * sin(0.7 * (double)i); }
+__global__ void __launch_bounds__(256) power_kernel(int64_t m, const int64_t *__restrict__ off,
+                                                    const int32_t *__restrict__ col, const double *__restrict__ val,
+                                                    const double *__restrict__ diag, const double *__restrict__ x,
+                                                    const double *__restrict__ part_x, double *__restrict__ y,
+                                                    double *__restrict__ part_y) {
+    __shared__ double sh[8];
+    const int tid = threadIdx.x, lane = tid & 31;
+    auto block_sum = [&](double v) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        __syncthreads();
+        if (lane == 0) sh[tid >> 5] = v;
+        __syncthreads();
+        double t = 0.0;
+        for (int w = 0; w < 8; ++w) t += sh[w];
+        return t;
+    };
+    double scale = 1.0;
+    if (part_x) scale = rsqrt(block_sum(tid < kPowerCtas ? part_x[tid] : 0.0));
+    double ny = 0.0;
+    for (int64_t i = (int64_t)blockIdx.x * 256 + tid; i < m; i += (int64_t)gridDim.x * 256) {
+        double s = 0.0;
+        for (int64_t p = off[i]; p < off[i + 1]; ++p) s += val[p] * (part_x ? x[col[p]] : power_start(col[p]));
+        const double v = s * scale / diag[i];
+        y[i] = v;
+        ny += v * v;
+    }
+    ny = block_sum(ny);
+    if (tid == 0) part_y[blockIdx.x] = ny;
+}
+
+// rho(D^-1 A) of the mesh's operator, or 0 where that fails (the host then forms it)
+double device_spectral_radius(const DevMesh &M, cudaStream_t s) {
+    double *w = nullptr;
+    const size_t n = (size_t)M.m;
+    if (cudaMalloc((void **)&w, (2 * n + 2 * kPowerCtas) * sizeof(double)) != cudaSuccess) {
+        cudaGetLastError();
+        return 0.0;
+    }
+    double *part = w + 2 * n, h[kPowerCtas];
+    for (int it = 0; it < kPowerSteps; ++it)
+        power_kernel<<<kPowerCtas, 256, 0, s>>>(M.m, M.a_off, M.a_col, M.a_val, M.a_diag, w + (it & 1 ? 0 : n),
+                                                it ? part + (it & 1 ? 0 : kPowerCtas) : nullptr, w + (it & 1 ? n : 0),
+                                                part + (it & 1 ? kPowerCtas : 0));
+    // the last step's x has norm 1, so |y| is the estimate
+    const bool ok = cudaMemcpyAsync(h, part + ((kPowerSteps - 1) & 1 ? kPowerCtas : 0), sizeof h,
+                                    cudaMemcpyDeviceToHost, s) == cudaSuccess &&
+                    cudaStreamSynchronize(s) == cudaSuccess;
+    cudaFree(w);
+    if (!ok) {
+        cudaGetLastError();
+        return 0.0;
+    }
+    double t = 0.0;
+    for (double v : h) t += v;
+    return t > 0.0 && std::isfinite(t) ? std::sqrt(t) : 0.0;
+}
+
 template <typename T>
 cudaError_t alloc(T **p, size_t count) {
     return cudaMalloc((void **)p, count * sizeof(T));
@@ -539,7 +604,7 @@ dd_status run_pcg_amg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s,
     DD_CUDA_TRY(cudaMemcpy(A0.val.data(), M.a_val, nnz * sizeof(double), cudaMemcpyDeviceToHost), err);
     AmgHierarchy H;
     std::string why;
-    if (!build_amg(A0, H, why)) {
+    if (!build_amg(A0, H, why, device_spectral_radius(M, s))) {
         *fallback = true;
         err = why;
         return DD_ENOTCONV;
