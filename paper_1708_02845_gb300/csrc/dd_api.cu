@@ -1301,8 +1301,28 @@ dd_status dd_query_batch(dd_ctx *ctx, int32_t n_items, const int32_t *mesh_ids, 
                                  return x.first > y.first;
                              });
         }
+        // the pipelined TV pass alone: a problem's last target tile of at most 32 or
+        // 16 targets in items of that many and more rows (twelve uneven maps of 28 to
+        // 246 targets: 13 % of padded sums instead of 25 %, the tile pass 861 -> 855 us)
+        std::vector<std::pair<int64_t, BatchItem>> order_tv;
+        if (pipe_ok && !tile_kl) {
+            for (int i = 0; i < n_items; ++i) {
+                const int nat = (T_per[i] + 63) / 64, rem = T_per[i] - 64 * (nat - 1);
+                const int last = rem <= 16 ? 2 : rem <= 32 ? 1 : 0;
+                for (int at = 0; at < nat; ++at) {
+                    const int shape = at == nat - 1 ? last : 0;
+                    for (int64_t xt = 0; xt * (128 << shape) < ms[i]->n_v; ++xt)
+                        order_tv.push_back({tiled_k32(ms[i]->k_pad), BatchItem{i, (int32_t)xt, at, shape}});
+                }
+            }
+            std::stable_sort(order_tv.begin(), order_tv.end(),
+                             [](const std::pair<int64_t, BatchItem> &x, const std::pair<int64_t, BatchItem> &y) {
+                                 return x.first > y.first;
+                             });
+        }
         const size_t o_items_pipe = o_items + align256(order.size() * sizeof(BatchItem));
-        meta.resize(o_items_pipe + order_pipe.size() * sizeof(BatchItem));
+        const size_t o_items_tv = o_items_pipe + align256(order_pipe.size() * sizeof(BatchItem));
+        meta.resize(o_items_tv + order_tv.size() * sizeof(BatchItem));
         std::memcpy(meta.data() + o_probs, probs.data(), n_items * sizeof(BatchProblem));
         // trace domains; gradients per item in consecutive blocks [T_i][n_t_i]
         {
@@ -1318,6 +1338,8 @@ dd_status dd_query_batch(dd_ctx *ctx, int32_t n_items, const int32_t *mesh_ids, 
             std::memcpy(meta.data() + o_items + j * sizeof(BatchItem), &order[j].second, sizeof(BatchItem));
         for (size_t j = 0; j < order_pipe.size(); ++j)
             std::memcpy(meta.data() + o_items_pipe + j * sizeof(BatchItem), &order_pipe[j].second, sizeof(BatchItem));
+        for (size_t j = 0; j < order_tv.size(); ++j)
+            std::memcpy(meta.data() + o_items_tv + j * sizeof(BatchItem), &order_tv[j].second, sizeof(BatchItem));
         if ((st = upload(ctx, S_META, meta.data(), meta.size())) != DD_OK) return st;
         dmeta = reinterpret_cast<uint8_t *>(ctx->scratch[S_META]);
         int64_t fix_blocks = 0, work = 0;
@@ -1335,7 +1357,10 @@ dd_status dd_query_batch(dd_ctx *ctx, int32_t n_items, const int32_t *mesh_ids, 
                                 (int32_t)order.size(), dcounter, ctx->stream, fix_blocks, klp);
         };
         auto pipelined = [&]() {
-            launch_batch_fields_pipe(dprobs, (int32_t)n_items, ditems_pipe, (int32_t)order_pipe.size(), dcounter,
+            const bool narrow = !order_tv.empty();
+            launch_batch_fields_pipe(dprobs, (int32_t)n_items,
+                                     narrow ? reinterpret_cast<const BatchItem *>(dmeta + o_items_tv) : ditems_pipe,
+                                     (int32_t)(narrow ? order_tv.size() : order_pipe.size()), dcounter,
                                      ctx->d_err, ctx->stream, fix_blocks, max_tiles, (f_mask & DD_F_KL) != 0,
                                      (f_mask & DD_F_TV) != 0, klp);
         };

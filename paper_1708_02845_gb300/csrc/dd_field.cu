@@ -786,23 +786,26 @@ __device__ __forceinline__ void pipe_store(const float (&kl)[4][4], const float 
     }
 }
 
-// R rows x 64 targets a CTA: 128 or 64 (whole row tiles), or 32 (half of one,
-// of which it then brings in both halves).
+// R rows x TN targets a CTA, 4 x 4 a thread: R a multiple of 64 (whole row
+// tiles), or 32 (half of one, of which it then brings in both halves); TN 64, or
+// the first 32 or 16 targets of a last tile that holds no more (with as many
+// more rows), from target tile at0 on.
+constexpr int pipe_threads(int R, int TN) { return R * TN / 16; }
 template <bool KL, bool TV, int R, int PB, int PS>
 constexpr size_t pipe_smem() {
     return (size_t)PS * ((KL ? 2 : 1) * (R >= 64 ? R / 64 : 1) + (KL ? 1 : 0) + (TV ? 1 : 0)) * PB * kTiledRows *
            sizeof(float);
 }
-template <bool KL, bool TV, int R, int PB, int PS, int UNR>
-__global__ void __launch_bounds__(4 * R, 128 / R) field_tile_pipe_kernel(const float *__restrict__ PT,
+template <bool KL, bool TV, int R, int TN, int PB, int PS, int UNR>
+__global__ void __launch_bounds__(pipe_threads(R, TN), 512 / pipe_threads(R, TN)) field_tile_pipe_kernel(const float *__restrict__ PT,
                                                                       const float *__restrict__ LT, int64_t n_v,
                                                                       int64_t kt, const float *__restrict__ TQ,
-                                                                      const float *__restrict__ TL, int32_t T,
+                                                                      const float *__restrict__ TL, int32_t T, int at0,
                                                                       float *__restrict__ out_kl,
                                                                       float *__restrict__ out_tv,
                                                                       int *__restrict__ err) {
     constexpr int H = R >= 64 ? R / 64 : 1;         // row tiles brought in
-    constexpr int RM = 4, CN = 4, NW = R / 8;
+    constexpr int RM = 4, CN = 4, NW = pipe_threads(R, TN) / 32;
     constexpr int TCH = PB * kTiledRows;            // floats per array, stage and 64-row (or target) tile
     constexpr int RCH = H * TCH;
     constexpr int OQ = (KL ? 2 : 1) * RCH, OT = OQ + (TV ? TCH : 0);
@@ -810,15 +813,14 @@ __global__ void __launch_bounds__(4 * R, 128 / R) field_tile_pipe_kernel(const f
     extern __shared__ __align__(128) float psm[];   // [stage][P rows, log2 rows, P targets, log2 targets]
     __shared__ __align__(8) uint64_t full[PS], empty[PS];
     const int tid = threadIdx.x, lane = tid & 31;
-    const int tx = tid % (kTiledRows / CN), ty = tid / (kTiledRows / CN);
+    const int tx = tid % (TN / CN), ty = tid / (TN / CN);
     // target tiles vary fastest over the grid: the CTAs that read one pair of
     // row tiles run together and share it through L2
     const int64_t x0 = (int64_t)blockIdx.y * R;
-    const int a0 = blockIdx.x * kTiledRows;
-    const float *gP = PT + x0 / kTiledRows * kt * kTiledRows;
-    const float *gL = LT + x0 / kTiledRows * kt * kTiledRows;
-    const float *gQ = TQ + (int64_t)blockIdx.x * kt * kTiledRows;
-    const float *gT = TL + (int64_t)blockIdx.x * kt * kTiledRows;
+    const int at = at0 + (int)blockIdx.x, a0 = at * kTiledRows;
+    const int64_t tile = kt * kTiledRows, t0 = x0 / kTiledRows, t1 = (n_v - 1) / kTiledRows;   // (t1: the last row tile)
+    const float *gQ = TQ + at * tile;
+    const float *gT = TL + at * tile;
     const int nch = (int)(kt / PB);
     constexpr uint32_t kArr = TCH * sizeof(float);
     constexpr uint32_t kStageBytes = kArr * (H * (KL ? 2 : 1) + (KL ? 1 : 0) + (TV ? 1 : 0));
@@ -829,8 +831,10 @@ __global__ void __launch_bounds__(4 * R, 128 / R) field_tile_pipe_kernel(const f
         mbar_expect_tx(&full[s], kStageBytes);
 #pragma unroll
         for (int h = 0; h < H; ++h) {
-            bulk_g2s(st + h * TCH, gP + (int64_t)h * kt * kTiledRows + go, kArr, &full[s]);
-            if (KL) bulk_g2s(st + RCH + h * TCH, gL + (int64_t)h * kt * kTiledRows + go, kArr, &full[s]);
+            // (past the last row tile: it again, for rows that are not written)
+            const int64_t ro = (t0 + h < t1 ? t0 + h : t1) * tile + go;
+            bulk_g2s(st + h * TCH, PT + ro, kArr, &full[s]);
+            if (KL) bulk_g2s(st + RCH + h * TCH, LT + ro, kArr, &full[s]);
         }
         if (TV) bulk_g2s(st + OQ, gQ + go, kArr, &full[s]);
         if (KL) bulk_g2s(st + OT, gT + go, kArr, &full[s]);
@@ -891,8 +895,9 @@ __global__ void __launch_bounds__(4 * R, 128 / R) field_tile_pipe_kernel(const f
 }
 
 // Many problems in one persistent launch, on the tiled layouts: one CTA of
-// 512 threads per SM takes (problem, pair of row tiles, target tile) items
-// from an atomic counter, largest first.  One thread streams the chunks of
+// 512 threads per SM takes (problem, rows, target tile) items of 128 rows x 64
+// targets -- TV alone also 256 x 32 and 512 x 16, for a problem's last target
+// tile of no more targets than that -- from an atomic counter, largest first.  One thread streams the chunks of
 // the items it takes, item after item, through the two stages, and records
 // with each stage the item and chunk it holds; the CTA's warps start an item
 // at its first chunk (the problem's sizes and outputs, zero sums) and write
@@ -900,24 +905,32 @@ __global__ void __launch_bounds__(4 * R, 128 / R) field_tile_pipe_kernel(const f
 // the sums of the previous item's last.  The stage that follows the last item
 // carries no copy and the item -1: the CTA ends there.  Every wait is bounded
 // (error flag, no output from the CTA that gave up).
+constexpr int kBatchPB = 32, kBatchPS = 3;
+template <bool KL, bool TV>
+constexpr int batch_stage_arrays() {      // most 64-row (or target) arrays of a stage
+    return KL ? (TV ? 6 : 5) : 9;
+}
+template <bool KL, bool TV>
+constexpr size_t batch_pipe_smem() {
+    return (size_t)kBatchPS * batch_stage_arrays<KL, TV>() * kBatchPB * kTiledRows * sizeof(float);
+}
 template <bool KL, bool TV>
 __global__ void __launch_bounds__(512, 1) batch_pipe_kernel(const BatchProblem *__restrict__ probs,
                                                          const BatchItem *__restrict__ items, int32_t n_items,
                                                          int32_t *__restrict__ counter, int *__restrict__ err) {
-    constexpr int H = 2, PB = 64, PS = 2, RM = 4, CN = 4, NW = 16;
-    constexpr int TCH = PB * kTiledRows, RCH = H * TCH, SST = 2 * RCH + 2 * TCH;
+    constexpr int PB = kBatchPB, PS = kBatchPS, RM = 4, CN = 4, NW = 16;
+    constexpr int TCH = PB * kTiledRows, SST = batch_stage_arrays<KL, TV>() * TCH;
     constexpr uint32_t kArr = TCH * sizeof(float);
-    constexpr uint32_t kStageBytes = kArr * (H * (KL ? 2 : 1) + (KL ? 1 : 0) + (TV ? 1 : 0));
     extern __shared__ __align__(128) float psm[];
     __shared__ __align__(8) uint64_t full[PS], empty[PS];
     __shared__ int slot_item[PS], slot_chunk[PS];
     const int tid = threadIdx.x, lane = tid & 31;
-    const int tx = tid % (kTiledRows / CN), ty = tid / (kTiledRows / CN);
 
     // producer state (thread 0)
     int p_item = -1, p_ch = 0, p_nch = 0, produced = 0;
     bool p_done = false;
-    int64_t p_kt = 0;
+    int64_t p_tile = 0, t0 = 0, t1 = 0;     // floats of a row or target tile; first and last row tile
+    int p_H = 2;                            // row tiles of the item
     const float *gP = nullptr, *gL = nullptr, *gQ = nullptr, *gT = nullptr;
     auto produce = [&](int s) {
         if (p_ch >= p_nch) {
@@ -933,25 +946,29 @@ __global__ void __launch_bounds__(512, 1) batch_pipe_kernel(const BatchProblem *
             const BatchProblem &q = probs[w.prob];
             p_item = it;
             p_ch = 0;
-            p_kt = q.kt;
+            p_tile = q.kt * kTiledRows;
+            if (!KL) p_H = 2 << w.shape;
+            t0 = (int64_t)w.x_tile * p_H;
+            t1 = (q.n_v - 1) / kTiledRows;
             p_nch = (int)(q.kt / PB);
-            gP = q.PT + (int64_t)w.x_tile * H * q.kt * kTiledRows;
-            gL = q.LT + (int64_t)w.x_tile * H * q.kt * kTiledRows;
-            gQ = q.TQ + (int64_t)w.a_tile * q.kt * kTiledRows;
-            gT = q.TL + (int64_t)w.a_tile * q.kt * kTiledRows;
+            gP = q.PT;
+            gL = q.LT;
+            gQ = q.TQ + w.a_tile * p_tile;
+            gT = q.TL + w.a_tile * p_tile;
         }
         slot_item[s] = p_item;
         slot_chunk[s] = p_ch;
         float *st = psm + s * SST;
         const int64_t go = (int64_t)p_ch * TCH;
-        mbar_expect_tx(&full[s], kStageBytes);
-#pragma unroll
-        for (int h = 0; h < H; ++h) {
-            bulk_g2s(st + h * TCH, gP + (int64_t)h * p_kt * kTiledRows + go, kArr, &full[s]);
-            if (KL) bulk_g2s(st + RCH + h * TCH, gL + (int64_t)h * p_kt * kTiledRows + go, kArr, &full[s]);
+        const int RCH = p_H * TCH, OQ = (KL ? 2 : 1) * RCH, OT = OQ + (TV ? TCH : 0);
+        mbar_expect_tx(&full[s], kArr * (p_H * (KL ? 2 : 1) + (KL ? 1 : 0) + (TV ? 1 : 0)));
+        for (int h = 0; h < p_H; ++h) {
+            const int64_t ro = (t0 + h < t1 ? t0 + h : t1) * p_tile + go;
+            bulk_g2s(st + h * TCH, gP + ro, kArr, &full[s]);
+            if (KL) bulk_g2s(st + RCH + h * TCH, gL + ro, kArr, &full[s]);
         }
-        if (TV) bulk_g2s(st + 2 * RCH, gQ + go, kArr, &full[s]);
-        if (KL) bulk_g2s(st + 2 * RCH + TCH, gT + go, kArr, &full[s]);
+        if (TV) bulk_g2s(st + OQ, gQ + go, kArr, &full[s]);
+        if (KL) bulk_g2s(st + OT, gT + go, kArr, &full[s]);
         ++p_ch;
         ++produced;
     };
@@ -971,7 +988,8 @@ __global__ void __launch_bounds__(512, 1) batch_pipe_kernel(const BatchProblem *
     int32_t T = 0;
     int ar = 0, nch = 0;
     float *okl = nullptr, *otv = nullptr;
-    const int roff = (ty / 16) * TCH + (ty % 16) * RM;
+    // this thread's rows and targets within a stage; floats of an item's rows
+    int tx = tid % 16, ty = tid / 16, RCH = 2 * TCH, ro4 = (ty / 16) * TCH + (ty % 16) * RM;
     bool ok = true;
     int c = 0;
     for (;; ++c) {
@@ -999,19 +1017,26 @@ __global__ void __launch_bounds__(512, 1) batch_pipe_kernel(const BatchProblem *
             okl = q.out_kl;
             otv = q.out_tv;
             nch = (int)(q.kt / PB);
-            xr = (int64_t)w.x_tile * H * kTiledRows + ty * RM;
+            if (!KL) {       // (with KL every item is 128 x 64)
+                const int lg = 4 - w.shape;
+                tx = tid & ((1 << lg) - 1);
+                ty = tid >> lg;
+                RCH = (2 << w.shape) * TCH;
+                ro4 = (ty / 16) * TCH + (ty % 16) * RM;
+            }
+            xr = (int64_t)w.x_tile * (2 * kTiledRows << (KL ? 0 : w.shape)) + ty * RM;
             ar = w.a_tile * kTiledRows + tx * CN;
 #pragma unroll
             for (int r = 0; r < RM; ++r)
 #pragma unroll
                 for (int q2 = 0; q2 < CN; ++q2) kl[r][q2] = tv[r][q2] = klc[r][q2] = ckl[r][q2] = ctv[r][q2] = 0.0f;
         }
-        const float *cP = psm + s * SST + roff;
-        const float *cQ = psm + s * SST + 2 * RCH + tx * CN;
-        pipe_stage<KL, TV, PB, 16>(cP, cP + RCH, cQ, cQ + TCH, ckl, ctv);
+        const float *cP = psm + s * SST + ro4;
+        const float *cQ = psm + s * SST + (KL ? 2 : 1) * RCH + tx * CN;
+        pipe_stage<KL, TV, PB, 16>(cP, cP + RCH, cQ, cQ + (TV ? TCH : 0), ckl, ctv);
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[s]);
-        pipe_merge(kl, klc, tv, ckl, ctv);           // every stage is one 64-column block
+        if (((ch + 1) * PB) % 64 == 0) pipe_merge(kl, klc, tv, ckl, ctv);     // 64-column partial sums (kt is a multiple)
         if (ch == nch - 1) pipe_store<KL, TV>(kl, tv, xr, ar, n_v, T, okl, otv);
     }
     if (!ok && tid == 0) {
@@ -1359,28 +1384,68 @@ constexpr int kPipeShape = 3;      // the pipelined tile on the tiled layout (si
 // where that shortens the fullest SM's share: grid140 with 64 targets has 154
 // tiles of 128 rows for 152 SMs, and two of them took as long again (125 us;
 // 85 us with 32 rows).
+//
+// A last target tile of at most 32 or 16 targets goes to a launch of its own
+// with that many and more rows a CTA, where that takes less: 333 targets are
+// five tiles and 13 targets, not six tiles (300 x 300 cells: 4.44 -> 4.02 ms).
 void launch_pipe(const TiledArgs &ta, int64_t n_v, int32_t T, float *out_kl, float *out_tv, int *err,
                  cudaStream_t s) {
     const int nat = (T + kTiledRows - 1) / kTiledRows;
-    auto go = [&](auto kern, int R, size_t smem) {
-        const dim3 g((unsigned)nat, (unsigned)((n_v + R - 1) / R));
+    auto go = [&](auto kern, int R, int TN, size_t smem, int at0, int count) {
+        const dim3 g((unsigned)count, (unsigned)((n_v + R - 1) / R));
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         KMark km_("field_tile_kernel", s);
-        kern<<<g, 4 * R, smem, s>>>(ta.PT, ta.LT, n_v, ta.kt, ta.TQ, ta.TL, T, out_kl, out_tv, err);
+        kern<<<g, pipe_threads(R, TN), smem, s>>>(ta.PT, ta.LT, n_v, ta.kt, ta.TQ, ta.TL, T, at0, out_kl, out_tv, err);
     };
     if (out_kl && out_tv)
-        return go(field_tile_pipe_kernel<true, true, 128, 64, 2, 16>, 128, pipe_smem<true, true, 128, 64, 2>());
+        return go(field_tile_pipe_kernel<true, true, 128, 64, 64, 2, 16>, 128, 64, pipe_smem<true, true, 128, 64, 2>(),
+                  0, nat);
     if (out_kl)
-        return go(field_tile_pipe_kernel<true, false, 128, 64, 2, 32>, 128, pipe_smem<true, false, 128, 64, 2>());
-    // rows of the fullest SM, smaller tiles charged for their share of the copies
-    auto share = [&](int R) { return (((n_v + R - 1) / R * nat + num_sms() - 1) / num_sms()) * R; };
-    const int64_t c128 = share(128) * 100, c64 = share(64) * 103, c32 = share(32) * 108;
-    if (c128 <= c64 && c128 <= c32)
-        go(field_tile_pipe_kernel<false, true, 128, 64, 2, 32>, 128, pipe_smem<false, true, 128, 64, 2>());
-    else if (c64 <= c32)
-        go(field_tile_pipe_kernel<false, true, 64, 64, 2, 32>, 64, pipe_smem<false, true, 64, 64, 2>());
-    else
-        go(field_tile_pipe_kernel<false, true, 32, 32, 3, 32>, 32, pipe_smem<false, true, 32, 32, 3>());
+        return go(field_tile_pipe_kernel<true, false, 128, 64, 64, 2, 32>, 128, 64,
+                  pipe_smem<true, false, 128, 64, 2>(), 0, nat);
+    // (row, target) sums of the fullest SM; smaller tiles are charged for their share of the copies
+    auto share = [&](int R, int TN, int count) {
+        return (((n_v + R - 1) / R * count + num_sms() - 1) / num_sms()) * R * TN;
+    };
+    auto wide_cost = [&](int count) {
+        return count ? std::min(share(128, 64, count) * 100, std::min(share(64, 64, count) * 103,
+                                                                      share(32, 64, count) * 108)) : 0;
+    };
+    auto wide = [&](int count) {
+        const int64_t c128 = share(128, 64, count) * 100, c64 = share(64, 64, count) * 103,
+                      c32 = share(32, 64, count) * 108;
+        if (c128 <= c64 && c128 <= c32)
+            go(field_tile_pipe_kernel<false, true, 128, 64, 64, 2, 32>, 128, 64, pipe_smem<false, true, 128, 64, 2>(),
+               0, count);
+        else if (c64 <= c32)
+            go(field_tile_pipe_kernel<false, true, 64, 64, 64, 2, 32>, 64, 64, pipe_smem<false, true, 64, 64, 2>(), 0,
+               count);
+        else
+            go(field_tile_pipe_kernel<false, true, 32, 64, 32, 3, 32>, 32, 64, pipe_smem<false, true, 32, 32, 3>(), 0,
+               count);
+    };
+    const int rem = T - (nat - 1) * kTiledRows;
+    const int64_t n32 = std::min(share(256, 32, 1) * 104, share(128, 32, 1) * 106);
+    const int64_t n16 = std::min(share(512, 16, 1) * 108, share(128, 16, 1) * 112);
+    const int64_t narrow = rem <= 16 ? n16 : rem <= 32 ? n32 : INT64_MAX / 2;
+    // (a launch of its own costs about as much as an eighth of a 128 x 64 tile)
+    if (wide_cost(nat - 1) + narrow + (nat > 1 ? 100 * 1024 : 0) >= wide_cost(nat)) return wide(nat);
+    if (nat > 1) wide(nat - 1);
+    if (rem <= 16) {
+        if (share(512, 16, 1) * 108 <= share(128, 16, 1) * 112)
+            go(field_tile_pipe_kernel<false, true, 512, 16, 32, 2, 32>, 512, 16,
+               pipe_smem<false, true, 512, 32, 2>(), nat - 1, 1);
+        else
+            go(field_tile_pipe_kernel<false, true, 128, 16, 32, 3, 32>, 128, 16,
+               pipe_smem<false, true, 128, 32, 3>(), nat - 1, 1);
+    } else {
+        if (share(256, 32, 1) * 104 <= share(128, 32, 1) * 106)
+            go(field_tile_pipe_kernel<false, true, 256, 32, 64, 2, 32>, 256, 32,
+               pipe_smem<false, true, 256, 64, 2>(), nat - 1, 1);
+        else
+            go(field_tile_pipe_kernel<false, true, 128, 32, 64, 2, 32>, 128, 32,
+               pipe_smem<false, true, 128, 64, 2>(), nat - 1, 1);
+    }
 }
 
 void launch_variant(int v, const float *P, int64_t n_v, int64_t k_pad, const float *sP, const float *sL,
@@ -1646,20 +1711,19 @@ void launch_batch_fields_pipe(const BatchProblem *d_probs, int32_t n_probs, cons
             KMark km_("tiled_targets_kernel", s);
             batch_tiled_targets_kernel<<<dim3((unsigned)max_tiles, (unsigned)n_probs), 256, 0, s>>>(d_probs);
         }
-        constexpr size_t smem = (size_t)2 * 6 * 64 * kTiledRows * sizeof(float);
         cudaMemsetAsync(d_counter, 0, sizeof(int32_t), s);
         const unsigned grid = (unsigned)std::min<int64_t>(num_sms(), n_items);
-        auto go = [&](auto kern) {
+        auto go = [&](auto kern, size_t smem) {
             cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             KMark km_("batch_tile_kernel", s);
             kern<<<grid, 512, smem, s>>>(d_probs, d_items, n_items, d_counter, err);
         };
         if (f_kl && f_tv)
-            go(batch_pipe_kernel<true, true>);
+            go(batch_pipe_kernel<true, true>, batch_pipe_smem<true, true>());
         else if (f_kl)
-            go(batch_pipe_kernel<true, false>);
+            go(batch_pipe_kernel<true, false>, batch_pipe_smem<true, false>());
         else
-            go(batch_pipe_kernel<false, true>);
+            go(batch_pipe_kernel<false, true>, batch_pipe_smem<false, true>());
     }
     if (kl_mma) launch_batch_kl_mma(d_probs, n_probs, kl_mma->items, kl_mma->n_items, kl_mma->max_T, kl_mma->err, s);
     launch_batch_fix(d_probs, n_probs, fix_blocks, kl_mma ? kMmaExactBelow : kTileExactBelow, s);

@@ -164,7 +164,8 @@ struct BatchProblem {
     int32_t knch;
 };
 struct BatchItem {
-    int32_t prob, x_tile, a_tile, pad;
+    int32_t prob, x_tile, a_tile;
+    int32_t shape;               // the pipelined TV pass: 0: 128 rows x 64 targets, 1: 256 x 32, 2: 512 x 16
 };
 // autotuned tile shape for one problem (may run timed launches the first time)
 int tile_variant_for(const float *P, int64_t n_v, int64_t k_pad, const float *sP, const float *sL, const float *sE,
@@ -185,8 +186,8 @@ struct BatchKlMma {
 void launch_batch_fields(const BatchProblem *d_probs, int32_t n_probs, const BatchItem *d_items, int32_t n_items,
                          int32_t *d_counter, cudaStream_t s, int64_t fix_blocks, const BatchKlMma *kl_mma = nullptr);
 // The pipelined multi-domain launch: every problem carries its tiled arrays
-// (PT, LT, TQ, TL, kt) and the items are 128-row x 64-target tiles (BatchItem
-// x_tile counts pairs of 64-row tiles); the targets are first put into the
+// (PT, LT, TQ, TL, kt) and the items are 128-row x 64-target tiles, for TV
+// alone also the narrower ones of BatchItem::shape (x_tile counts an item's rows); the targets are first put into the
 // tiled layout (max_tiles: the largest ceil(T / 64) * kt / 32 of the problems),
 // then one persistent launch computes every tile (f_kl / f_tv: which fields
 // all problems ask for), then the exact recompute.

@@ -90,3 +90,27 @@ def test_replaced_kernel(env, scale):
     for a in (0, 7, 19):
         assert field_error(out[0, a], kl_field_fast(P2, P2[targets[a]])) <= TOL_FP32
         assert field_error(out[1, a], tv_field(P2, P2[targets[a]])) <= TOL_FP32
+
+
+@pytest.mark.parametrize("T", [7, 16, 17, 32, 33, 72, 96])
+def test_tv_pass_of_narrow_last_tiles(env, monkeypatch, T):
+    """The pipelined TV pass (every shape of its last target tile) has the
+    staged shapes' sums bit for bit, alone and in a batch."""
+    dd, ctx, mesh, po, P, mid = env
+    targets = targets_of(po, T)
+    ref = None
+    for shape in ("0", "3"):
+        monkeypatch.setenv("DD_TILE_SHAPE", shape)
+        got = fields(dd, ctx, mid, mesh.n_v, targets, dd.DD_F_TV)[0]
+        ref = got if ref is None else ref
+        assert np.array_equal(got, ref)
+    monkeypatch.delenv("DD_TILE_SHAPE")
+    n = mesh.n_v
+    both = fields(dd, ctx, mid, n, targets, 3)
+    for pipe in ("0", "1"):
+        monkeypatch.setenv("DD_BATCH_PIPE", pipe)
+        out = torch.full((2 * (T + 64) * n,), float("nan"), dtype=torch.float32, device="cuda")
+        dd.dd_query_batch(ctx, [mid, mid], [T, 64], np.concatenate([targets, targets_of(po, 64)]).astype(np.int32),
+                          None, 0, 3, 1, 2, out)
+        dd.dd_sync(ctx)
+        assert np.array_equal(out[:2 * T * n].reshape(2, T, n).cpu().numpy(), both)
