@@ -1206,7 +1206,7 @@ dd_status dd_query_batch(dd_ctx *ctx, int32_t n_items, const int32_t *mesh_ids, 
             std::string err;
             mma = kl_mma_wanted(*ms[i]);
             if (mma && (st = prepare_kl_mma(*ms[i], ctx->stream, &mma, err)) != DD_OK) return set_err(ctx, st, err);
-            kb_bytes += kl_mma_target_bytes(ms[i]->k_pad, T_per[i], 64);
+            kb_bytes += kl_mma_target_bytes(ms[i]->k_pad, T_per[i], kl_mma_batch_tile(T_per[i]));
             max_T = std::max(max_T, T_per[i]);
         }
         if (mma && ensure_scratch(ctx, S_KLMMA, kb_bytes) != DD_OK) {
@@ -1222,7 +1222,8 @@ dd_status dd_query_batch(dd_ctx *ctx, int32_t n_items, const int32_t *mesh_ids, 
                 q.kex = ms[i]->kl_ex;
                 q.KB = kb;
                 q.knch = kl_mma_chunks(ms[i]->k_pad);
-                kb += kl_mma_target_bytes(ms[i]->k_pad, T_per[i], 64);
+                q.ktile = kl_mma_batch_tile(T_per[i]);
+                kb += kl_mma_target_bytes(ms[i]->k_pad, T_per[i], q.ktile);
             }
         }
         const bool tile_kl = (f_mask & DD_F_KL) && !mma;      // KL in the tile pass
@@ -1264,7 +1265,7 @@ dd_status dd_query_batch(dd_ctx *ctx, int32_t n_items, const int32_t *mesh_ids, 
         // the pipelined launch: every mesh's tiled copy of P (built once per
         // mesh; without room for it the batch stays staged), every problem's
         // targets in the tiled layout, items of 128 rows x 64 targets
-        bool pipe_ok = true;
+        bool pipe_ok = tile_kl || (f_mask & DD_F_TV);      // (a tile pass is needed)
         int64_t tstage_bytes = 0, max_tiles = 0;
         for (int i = 0; i < n_items && pipe_ok; ++i) {
             std::string err;
@@ -1276,30 +1277,46 @@ dd_status dd_query_batch(dd_ctx *ctx, int32_t n_items, const int32_t *mesh_ids, 
             cudaGetLastError();
             pipe_ok = false;
         }
-        // (the tensor-core KL takes the same 128 x 64 items, with or without the tiled copies)
-        std::vector<std::pair<int64_t, BatchItem>> order_pipe;
-        if (pipe_ok || mma) {
-            float *ts = pipe_ok ? reinterpret_cast<float *>(ctx->scratch[S_TSTAGE]) : nullptr;
-            for (int i = 0; i < n_items; ++i) {
-                BatchProblem &q = probs[i];
-                const DevMesh &m = *ms[i];
-                if (pipe_ok) {
-                    const int64_t half = (int64_t)tiled_target_bytes(m.k_pad, T_per[i]) / (2 * sizeof(float));
-                    q.PT = m.pt_p;
-                    q.LT = m.pt_l;
-                    q.kt = m.pt_kt;
-                    q.TQ = ts;
-                    q.TL = ts + half;
-                    ts += 2 * half;
-                }
-                for (int64_t xt = 0; xt * 128 < m.n_v; ++xt)
-                    for (int at = 0; at * 64 < T_per[i]; ++at)
-                        order_pipe.push_back({tiled_k32(m.k_pad), BatchItem{i, (int32_t)xt, at, 0}});
-            }
-            std::stable_sort(order_pipe.begin(), order_pipe.end(),
+        auto costliest_first = [](std::vector<std::pair<int64_t, BatchItem>> &v) {
+            std::stable_sort(v.begin(), v.end(),
                              [](const std::pair<int64_t, BatchItem> &x, const std::pair<int64_t, BatchItem> &y) {
                                  return x.first > y.first;
                              });
+        };
+        std::vector<std::pair<int64_t, BatchItem>> order_pipe;
+        if (pipe_ok) {
+            float *ts = reinterpret_cast<float *>(ctx->scratch[S_TSTAGE]);
+            for (int i = 0; i < n_items; ++i) {
+                BatchProblem &q = probs[i];
+                const DevMesh &m = *ms[i];
+                const int64_t half = (int64_t)tiled_target_bytes(m.k_pad, T_per[i]) / (2 * sizeof(float));
+                q.PT = m.pt_p;
+                q.LT = m.pt_l;
+                q.kt = m.pt_kt;
+                q.TQ = ts;
+                q.TL = ts + half;
+                ts += 2 * half;
+                if (!tile_kl) continue;      // TV alone: order_tv
+                for (int64_t xt = 0; xt * 128 < m.n_v; ++xt)
+                    for (int at = 0; at * 64 < T_per[i]; ++at)
+                        order_pipe.push_back({m.pt_kt, BatchItem{i, (int32_t)xt, at, 0}});
+            }
+            costliest_first(order_pipe);
+        }
+        // the tensor-core KL's items, those of 128 targets first
+        std::vector<std::pair<int64_t, BatchItem>> order_kl;
+        int32_t kl_wide = 0;
+        for (int tile = 128; mma && tile >= 64; tile -= 64) {
+            std::vector<std::pair<int64_t, BatchItem>> part;
+            for (int i = 0; i < n_items; ++i) {
+                if (probs[i].ktile != tile) continue;
+                for (int64_t xt = 0; xt * 128 < ms[i]->n_v; ++xt)
+                    for (int at = 0; at * tile < T_per[i]; ++at)
+                        part.push_back({probs[i].knch, BatchItem{i, (int32_t)xt, at, 0}});
+            }
+            costliest_first(part);
+            order_kl.insert(order_kl.end(), part.begin(), part.end());
+            if (tile == 128) kl_wide = (int32_t)order_kl.size();
         }
         // the pipelined TV pass alone: a problem's last target tile of at most 32 or
         // 16 targets in items of that many and more rows (twelve uneven maps of 28 to
@@ -1315,14 +1332,12 @@ dd_status dd_query_batch(dd_ctx *ctx, int32_t n_items, const int32_t *mesh_ids, 
                         order_tv.push_back({tiled_k32(ms[i]->k_pad), BatchItem{i, (int32_t)xt, at, shape}});
                 }
             }
-            std::stable_sort(order_tv.begin(), order_tv.end(),
-                             [](const std::pair<int64_t, BatchItem> &x, const std::pair<int64_t, BatchItem> &y) {
-                                 return x.first > y.first;
-                             });
+            costliest_first(order_tv);
         }
         const size_t o_items_pipe = o_items + align256(order.size() * sizeof(BatchItem));
         const size_t o_items_tv = o_items_pipe + align256(order_pipe.size() * sizeof(BatchItem));
-        meta.resize(o_items_tv + order_tv.size() * sizeof(BatchItem));
+        const size_t o_items_kl = o_items_tv + align256(order_tv.size() * sizeof(BatchItem));
+        meta.resize(o_items_kl + order_kl.size() * sizeof(BatchItem));
         std::memcpy(meta.data() + o_probs, probs.data(), n_items * sizeof(BatchProblem));
         // trace domains; gradients per item in consecutive blocks [T_i][n_t_i]
         {
@@ -1340,6 +1355,8 @@ dd_status dd_query_batch(dd_ctx *ctx, int32_t n_items, const int32_t *mesh_ids, 
             std::memcpy(meta.data() + o_items_pipe + j * sizeof(BatchItem), &order_pipe[j].second, sizeof(BatchItem));
         for (size_t j = 0; j < order_tv.size(); ++j)
             std::memcpy(meta.data() + o_items_tv + j * sizeof(BatchItem), &order_tv[j].second, sizeof(BatchItem));
+        for (size_t j = 0; j < order_kl.size(); ++j)
+            std::memcpy(meta.data() + o_items_kl + j * sizeof(BatchItem), &order_kl[j].second, sizeof(BatchItem));
         if ((st = upload(ctx, S_META, meta.data(), meta.size())) != DD_OK) return st;
         dmeta = reinterpret_cast<uint8_t *>(ctx->scratch[S_META]);
         int64_t fix_blocks = 0, work = 0;
@@ -1350,7 +1367,8 @@ dd_status dd_query_batch(dd_ctx *ctx, int32_t n_items, const int32_t *mesh_ids, 
         const BatchProblem *dprobs = reinterpret_cast<const BatchProblem *>(dmeta + o_probs);
         int32_t *dcounter = reinterpret_cast<int32_t *>(dmeta + o_counter);
         const BatchItem *ditems_pipe = reinterpret_cast<const BatchItem *>(dmeta + o_items_pipe);
-        const BatchKlMma kl{ditems_pipe, (int32_t)order_pipe.size(), max_T, ctx->d_err, (f_mask & DD_F_TV) != 0};
+        const BatchKlMma kl{reinterpret_cast<const BatchItem *>(dmeta + o_items_kl), kl_wide, (int32_t)order_kl.size(),
+                            max_T, ctx->d_err, (f_mask & DD_F_TV) != 0};
         const BatchKlMma *klp = mma ? &kl : nullptr;
         auto staged = [&]() {
             launch_batch_fields(dprobs, (int32_t)n_items, reinterpret_cast<const BatchItem *>(dmeta + o_items),

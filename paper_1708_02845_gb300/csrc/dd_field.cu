@@ -1697,7 +1697,7 @@ void launch_batch_fields(const BatchProblem *d_probs, int32_t n_probs, const Bat
         tile(batch_tile_kernel<true>);
     else if (kl_mma->tv)
         tile(batch_tile_kernel<false>);
-    if (kl_mma) launch_batch_kl_mma(d_probs, n_probs, kl_mma->items, kl_mma->n_items, kl_mma->max_T, kl_mma->err, s);
+    if (kl_mma) launch_batch_kl_mma(d_probs, n_probs, *kl_mma, s);
     launch_batch_fix(d_probs, n_probs, fix_blocks, kl_mma ? kMmaExactBelow : kTileExactBelow, s);
 }
 
@@ -1725,7 +1725,7 @@ void launch_batch_fields_pipe(const BatchProblem *d_probs, int32_t n_probs, cons
         else
             go(batch_pipe_kernel<false, true>, batch_pipe_smem<false, true>());
     }
-    if (kl_mma) launch_batch_kl_mma(d_probs, n_probs, kl_mma->items, kl_mma->n_items, kl_mma->max_T, kl_mma->err, s);
+    if (kl_mma) launch_batch_kl_mma(d_probs, n_probs, *kl_mma, s);
     launch_batch_fix(d_probs, n_probs, fix_blocks, kl_mma ? kMmaExactBelow : kTileExactBelow, s);
 }
 

@@ -157,11 +157,11 @@ struct BatchProblem {
     float *TQ, *TL;
     int64_t kt;
     // the tensor-core KL: the mesh's row slices and e_x, this problem's target
-    // slices (tiles of 64), chunks of 64 columns (null: KL in the tile pass)
+    // slices (tiles of ktile), chunks of 64 columns (null: KL in the tile pass)
     const uint8_t *KA;
     uint8_t *KB;
     const float2 *kex;
-    int32_t knch;
+    int32_t knch, ktile;
 };
 struct BatchItem {
     int32_t prob, x_tile, a_tile;
@@ -178,8 +178,8 @@ void launch_batch_stage(const BatchProblem *d_probs, const int32_t *d_tprob, con
 // problem with KL output (fix_blocks: the sum of their fix_row_blocks(n_v))
 // (kl_mma: KL comes from launch_batch_kl_mma before the recompute; the tile pass sums TV alone)
 struct BatchKlMma {
-    const BatchItem *items;      // 128 rows x 64 targets
-    int32_t n_items, max_T;
+    const BatchItem *items;      // 128 rows x ktile targets: first those of problems with ktile 128
+    int32_t n_wide, n_items, max_T;
     int *err;
     bool tv;                     // TV is asked for
 };
@@ -211,15 +211,15 @@ struct KlMmaArgs {
 bool kl_mma_wanted(const DevMesh &m);
 int32_t kl_mma_chunks(int64_t k_pad);
 int kl_mma_tile(int32_t T);
+int kl_mma_batch_tile(int32_t T);      // a batch has tiles of 128 and 64 (one launch each)
 size_t kl_mma_target_bytes(int64_t k_pad, int32_t T, int N);
 size_t kl_mma_row_bytes(const DevMesh &m);
 size_t kl_mma_ex_bytes(const DevMesh &m);
 dd_status prepare_kl_mma(DevMesh &m, cudaStream_t s, bool *usable, std::string &err);
 void launch_kl_mma(const KlMmaArgs &args, const float *sP, int64_t n_v, int64_t k_pad, int32_t T, float *out_kl,
                    int *err, cudaStream_t s);
-// every problem's KL (KA, KB, kex, knch set; items of 128 rows x 64 targets)
-void launch_batch_kl_mma(const BatchProblem *d_probs, int32_t n_probs, const BatchItem *d_items, int32_t n_items,
-                         int32_t max_T, int *err, cudaStream_t s);
+// every problem's KL (KA, KB, kex, knch, ktile set)
+void launch_batch_kl_mma(const BatchProblem *d_probs, int32_t n_probs, const BatchKlMma &batch, cudaStream_t s);
 // The autotuner's choice between the staged (0) and the pipelined (1)
 // multi-domain launch: the first time a class of batches is seen (the fields
 // asked for, problems and n k T work in powers of two) both run (a warm-up

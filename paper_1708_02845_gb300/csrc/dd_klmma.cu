@@ -448,15 +448,15 @@ __global__ void __launch_bounds__(256) kl_targets_kernel(const float *__restrict
     for (int c = threadIdx.x >> 5; c < nch; c += 8) kl_targets_chunk(sP, T, k_pad, N, blockIdx.x, c, nch, B, tab);
 }
 
-// blockIdx.y a problem, blockIdx.x one of its targets (tiles of 64)
+// blockIdx.y a problem, blockIdx.x one of its targets (tiles of q.ktile)
 __global__ void __launch_bounds__(256) kl_batch_targets_kernel(const BatchProblem *__restrict__ probs) {
     __shared__ Log2Tab tab;
     const BatchProblem &q = probs[blockIdx.y];
-    if ((int)blockIdx.x >= (q.T + 63) / 64 * 64) return;
+    if ((int)blockIdx.x >= (q.T + q.ktile - 1) / q.ktile * q.ktile) return;
     build_log2_table(tab);
     __syncthreads();
     for (int c = threadIdx.x >> 5; c < q.knch; c += 8)
-        kl_targets_chunk(q.sP, q.T, q.k_pad, 64, blockIdx.x, c, q.knch, q.KB, tab);
+        kl_targets_chunk(q.sP, q.T, q.k_pad, q.ktile, blockIdx.x, c, q.knch, q.KB, tab);
 }
 
 int sm_count() {
@@ -481,6 +481,8 @@ int32_t kl_mma_chunks(int64_t k_pad) { return (int32_t)((k_pad + BK - 1) / BK); 
 // memory bound N = 64 at about two thirds of it, N = 16 at a fifth), narrower
 // ones waste less on padding.
 int kl_mma_tile(int32_t T) { return T <= 16 ? 16 : T <= 64 ? 64 : 128; }
+
+int kl_mma_batch_tile(int32_t T) { return T <= 64 ? 64 : 128; }
 
 size_t kl_mma_target_bytes(int64_t k_pad, int32_t T, int N) {
     return (size_t)((T + N - 1) / N) * kl_mma_chunks(k_pad) * b_bytes(N);
@@ -563,15 +565,18 @@ void launch_kl_mma(const KlMmaArgs &ka, const float *sP, int64_t n_v, int64_t k_
         go(kl_mma_kernel<128, false>, smem_bytes(128));
 }
 
-void launch_batch_kl_mma(const BatchProblem *d_probs, int32_t n_probs, const BatchItem *d_items, int32_t n_items,
-                         int32_t max_T, int *err, cudaStream_t s) {
-    if (n_items <= 0) return;
+void launch_batch_kl_mma(const BatchProblem *d_probs, int32_t n_probs, const BatchKlMma &b, cudaStream_t s) {
     {
         KMark km_("kl_targets_kernel", s);
-        kl_batch_targets_kernel<<<dim3((unsigned)((max_T + 63) / 64 * 64), (unsigned)n_probs), 256, 0, s>>>(d_probs);
+        kl_batch_targets_kernel<<<dim3((unsigned)((b.max_T + 127) / 128 * 128), (unsigned)n_probs), 256, 0, s>>>(
+            d_probs);
     }
-    cudaFuncSetAttribute(kl_mma_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(64));
-    KMark km_("kl_mma_kernel", s);
-    kl_mma_kernel<64, true><<<(unsigned)std::min<int64_t>(n_items, sm_count()), 320, smem_bytes(64), s>>>(
-        KlOne{}, d_probs, d_items, n_items, err);
+    auto go = [&](auto kern, int smem, const BatchItem *items, int32_t n) {
+        if (n <= 0) return;
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        KMark km_("kl_mma_kernel", s);
+        kern<<<(unsigned)std::min<int64_t>(n, sm_count()), 320, smem, s>>>(KlOne{}, d_probs, items, n, b.err);
+    };
+    go(kl_mma_kernel<128, true>, smem_bytes(128), b.items, b.n_wide);
+    go(kl_mma_kernel<64, true>, smem_bytes(64), b.items + b.n_wide, b.n_items - b.n_wide);
 }
