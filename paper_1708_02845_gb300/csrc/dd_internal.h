@@ -270,7 +270,7 @@ void launch_sparse_fields(const DevMesh &m, const int32_t *d_targets, float4 *st
 // spread (max - min) of the hardware mantissa log's error over [1, 2), in base-2 units
 dd_status fast_log_spread(double *spread, std::string &err);
 
-// Tracer: when trace_dense_decisions(T, S), per-field triangle rates and vertex
+// Tracer: when trace_dense_decisions(T, S), the fields by vertex and the vertex
 // decisions into `scratch` (trace_scratch_bytes(m, T, true) bytes), then T*S
 // paths; otherwise the walk forms the rates and decisions it needs itself and
 // `scratch` is unused.

@@ -164,9 +164,22 @@ __global__ void __launch_bounds__(320, 1) kl_mma_kernel(const KlOne one, const B
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
 
+    // Few targets: the copies of the rows bound the pass, and a last round of a
+    // few tiles takes as long as a full one (201 x 201 cells: 317 tiles on 152
+    // SMs, 73 us).  Its tiles are cut into quarters of 32 rows, an item each:
+    // only those rows are copied (the MMA's others hold what was there, and
+    // their results are not stored) (III us).
+    constexpr bool kQuarters = !BATCH && N == 16;
+    const int rounds = n_items / (int)gridDim.x * (int)gridDim.x;
+    const bool cut = kQuarters && rounds > 0 && 2 * (n_items - rounds) <= (int)gridDim.x;
+    const int n_whole = cut ? rounds : n_items, n_work = n_whole + 4 * (n_items - n_whole);
+    // the quarter of its tile that work item i is, or -1: the whole of it
+    auto quarter = [&](int i) { return i < n_whole ? -1 : (i - n_whole) & 3; };
+
     // item i: its operands and sizes.  One problem: the target tiles vary
     // fastest, so the CTAs that work at one time share their row tiles in L2
     auto problem = [&](int i, int &xt, int &at) {
+        if (i > n_whole) i = n_whole + ((i - n_whole) >> 2);
         if (BATCH) {
             const BatchItem w = items[i];
             const BatchProblem &q = probs[w.prob];
@@ -183,16 +196,26 @@ __global__ void __launch_bounds__(320, 1) kl_mma_kernel(const KlOne one, const B
     if (warp == 0) {
         if (lane == 0) {
             int g = 0;
-            for (int i = blockIdx.x; i < n_items && !*abort; i += gridDim.x) {
+            for (int i = blockIdx.x; i < n_work && !*abort; i += gridDim.x) {
                 int xt, at;
                 const KlOne q = problem(i, xt, at);
+                const int part = quarter(i);
                 const uint8_t *a = q.A + (int64_t)xt * q.nch * A_BYTES, *b = q.B + (int64_t)at * q.nch * b_bytes(N);
                 for (int c = 0; c < q.nch; ++c, ++g) {
                     const int s = g % ST, round = g / ST;
                     if (round > 0 && !wait_or_abort(&empty[s], (round - 1) & 1, err, abort)) break;
                     uint8_t *st = smem + s * SB;
-                    mbar_expect_tx(&full[s], SB);
-                    bulk_g2s(st, a + (int64_t)c * A_BYTES, A_BYTES, &full[s]);
+                    const uint8_t *ac = a + (int64_t)c * A_BYTES;
+                    if (part < 0) {
+                        mbar_expect_tx(&full[s], SB);
+                        bulk_g2s(st, ac, A_BYTES, &full[s]);
+                    } else {
+                        constexpr int kPart = 32 * ROW_B;      // of each slice
+                        mbar_expect_tx(&full[s], NSA * kPart + b_bytes(N));
+                        for (int k = 0; k < NSA; ++k)
+                            bulk_g2s(st + k * BM * ROW_B + part * kPart, ac + k * BM * ROW_B + part * kPart, kPart,
+                                     &full[s]);
+                    }
                     bulk_g2s(st + A_BYTES, b + (int64_t)c * b_bytes(N), b_bytes(N), &full[s]);
                 }
             }
@@ -204,7 +227,7 @@ __global__ void __launch_bounds__(320, 1) kl_mma_kernel(const KlOne one, const B
         if (lane == 0) {
             int g = 0;
             bool ok = true;
-            for (int i = blockIdx.x; i < n_items && ok && !*abort; i += gridDim.x) {
+            for (int i = blockIdx.x; i < n_work && ok && !*abort; i += gridDim.x) {
                 int xt, at;
                 const int nch = problem(i, xt, at).nch;
                 for (int c = 0; c < nch; ++c, ++g) {
@@ -242,7 +265,7 @@ __global__ void __launch_bounds__(320, 1) kl_mma_kernel(const KlOne one, const B
         const f2_t split = pk(kSplit, kSplit), nsplit = pk(-kSplit, -kSplit), mone = pk(-1.0f, -1.0f);
         int g = 0;
         bool ok = true;
-        for (int i = blockIdx.x; i < n_items && ok; i += gridDim.x) {
+        for (int i = blockIdx.x; i < n_work && ok; i += gridDim.x) {
             int xt, at;
             const KlOne q = problem(i, xt, at);
             f2_t hi[CW / 2], lo[CW / 2];
@@ -276,7 +299,8 @@ __global__ void __launch_bounds__(320, 1) kl_mma_kernel(const KlOne one, const B
             }
             if (!ok) break;
             const int64_t row = (int64_t)xt * BM + quad * 32 + lane;
-            if (row < q.n_v) {
+            const int part = quarter(i);
+            if (row < q.n_v && (part < 0 || part == quad)) {
                 const float2 e = q.ex[row];
                 const int a0 = at * N + half * CW;
 #pragma unroll

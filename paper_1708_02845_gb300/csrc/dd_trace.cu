@@ -24,10 +24,10 @@
 // order in which the incident triangles are examined does not matter).  Where
 // many paths share a field it is computed for every vertex of every field
 // before the walk (vertex_decision_kernel; wide fans in wide_decision_kernel),
-// after the barycentric rates of every triangle (rates_kernel).  Both are
-// stored field-minor ([triangle][field], [vertex][field]): a warp of the
-// decision kernel handles one vertex for 32 fields, so the triangle records it
-// reads are shared by all its lanes and the rates it reads are contiguous.
+// from the fields vertex by vertex (fields_by_vertex_kernel), into decisions
+// stored [vertex][field]: a warp of the decision kernel handles one vertex for
+// 32 fields, so the triangle records it reads are shared by all its lanes and
+// the values it reads are contiguous.
 // The walk (walk_path) then does one thing per iteration: cross one triangle
 // from an edge, apply one vertex decision, or slide along a valley or
 // boundary edge.  Batches of several maps walk one path per thread on stored
@@ -37,7 +37,7 @@
 // us (a call with its fields, results in host buffers, 362 -> 222 us); 142
 // points, 32 paths on the 2,049-vertex disk 250 -> 47 us (a call 240 -> 68 us);
 // 941 points, 64 x 256 paths on the 71,681-vertex disk 953 -> 476 us and the
-// decisions 778 -> 270 us (a call 1,760 -> 829 us).
+// decisions 778 -> 253 us (a call 1,735 -> 732 us).
 #include <cfloat>
 #include <cstring>
 #include <cstdlib>
@@ -107,14 +107,20 @@ __device__ __forceinline__ float4 tri_rates(const float4 *__restrict__ gphi, con
     return rates_of(__ldg(gphi + 2 * t), f[a.x], f[a.y], f[a.z]);
 }
 
-// rates[t * T + a] for every triangle t and field a (field-minor)
-__global__ void rates_kernel(const float4 *__restrict__ gphi, const int4 *__restrict__ rec, int64_t n_t, int32_t T,
-                             const float *__restrict__ fields, int64_t field_stride, float4 *__restrict__ rates) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_t * T) return;
-    const int64_t t = i / T;
-    const int a = (int)(i - t * T);
-    rates[i] = tri_rates(gphi, rec, t, fields + (int64_t)a * field_stride);
+// ft[v * T + a] = field a at vertex v: the fields vertex by vertex, so that a
+// warp of the decision kernel reads 32 fields of a vertex at once
+__global__ void __launch_bounds__(256) fields_by_vertex_kernel(const float *__restrict__ fields, int64_t field_stride,
+                                                               int64_t n_v, int32_t T, float *__restrict__ ft) {
+    __shared__ float tile[32][33];
+    const int64_t v0 = (int64_t)blockIdx.x * 32;
+    const int a0 = blockIdx.y * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = ty; i < 32; i += 8)
+        if (a0 + i < T && v0 + tx < n_v) tile[i][tx] = fields[(int64_t)(a0 + i) * field_stride + v0 + tx];
+    __syncthreads();
+#pragma unroll
+    for (int i = ty; i < 32; i += 8)
+        if (v0 + i < n_v && a0 + tx < T) ft[(v0 + i) * T + a0 + tx] = tile[tx][i];
 }
 
 // What the walk does at a vertex (32 bytes)
@@ -252,19 +258,6 @@ struct FanScan {
     }
 };
 
-// the vertex state's decision at v for field f (rates of that field at
-// `rates`, one entry per triangle every `rstride`)
-__device__ __forceinline__ VDec vertex_decision(const TraceDom &p, const float *__restrict__ f,
-                                                const float4 *__restrict__ rates, int64_t rstride, int target, int v) {
-    FanScan fs;
-    fs.begin();
-    for (int q = p.vt_off[v], q1 = p.vt_off[v + 1]; q < q1; ++q) {
-        const int tl = p.vt[q];
-        fs.add(v, target, tl, load_tri(p.rec, tl), __ldg(rates + (int64_t)tl * rstride));
-    }
-    return fs.finish<1>(p, f, target, v);
-}
-
 // The best triangle of a fan whose triangles were dealt to the G lanes of a
 // group (aligned, all of them in `mask`): the steepest, ties to the lowest id
 // -- what one lane scanning the whole fan finds, in any order.
@@ -294,17 +287,32 @@ __device__ __forceinline__ void fan_reduce(FanScan &fs, unsigned mask) {
     fs.b_pk.y = __shfl_sync(mask, fs.b_pk.y, from);
 }
 
-// one warp per (vertex, group of 32 fields), lane = field: dec[v * T + a];
-// vertices of more than kWideFan triangles are left to wide_decision_kernel
-__global__ void vertex_decision_kernel(const TraceDom p, int32_t T, const float *__restrict__ fields,
-                                       int64_t field_stride, const float4 *__restrict__ rates,
-                                       const int32_t *__restrict__ targets, VDec *__restrict__ dec) {
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int groups = (T + 31) >> 5;
-    const int64_t v = w / groups;
-    const int a = (int)(w - v * groups) * 32 + (threadIdx.x & 31);
-    if (v >= p.n_v || a >= T || p.vt_off[v + 1] - p.vt_off[v] > kWideFan) return;
-    dec[v * T + a] = vertex_decision(p, fields + (int64_t)a * field_stride, rates + a, T, targets[a], (int)v);
+// one warp per vertex and 32 fields (blockIdx.y), lane = field: dec[v * T + a];
+// vertices of more than kWideFan triangles are left to wide_decision_kernel.
+// The rates of a fan's triangles are formed here from the fields by vertex:
+// 64 fields of 71,681 vertices, the rates of every triangle stored first (147
+// MB written, read three times) took 68 + 230 us, this 8 + 216.
+__global__ void __launch_bounds__(128) vertex_decision_kernel(const TraceDom p, int32_t T,
+                                                              const float *__restrict__ fields, int64_t field_stride,
+                                                              const float *__restrict__ ft,
+                                                              const int32_t *__restrict__ targets,
+                                                              VDec *__restrict__ dec) {
+    const int64_t v = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
+    const int a = blockIdx.y * 32 + (threadIdx.x & 31);
+    if (v >= p.n_v || a >= T) return;
+    const int q0 = p.vt_off[v], q1 = p.vt_off[v + 1];
+    if (q1 - q0 > kWideFan) return;
+    const int target = targets[a];
+    FanScan fs;
+    fs.begin();
+    for (int q = q0; q < q1; ++q) {
+        const int tl = p.vt[q];
+        const Tri t = load_tri(p.rec, tl);
+        const float4 r = rates_of(__ldg(p.gphi + 2 * (int64_t)tl), ft[(int64_t)t.v0 * T + a], ft[(int64_t)t.v1 * T + a],
+                                  ft[(int64_t)t.v2 * T + a]);
+        fs.add((int)v, target, tl, t, r);
+    }
+    dec[v * T + a] = fs.finish<1>(p, fields + (int64_t)a * field_stride, target, (int)v);
 }
 
 // The vertices with wide fans (a disk's centre: as many triangles as the disk
@@ -313,8 +321,7 @@ __global__ void vertex_decision_kernel(const TraceDom p, int32_t T, const float 
 // ms, all of the decision pass but 0.12 ms (71,681 vertices, 64 fields).
 __global__ void wide_decision_kernel(const TraceDom p, const int32_t *__restrict__ wide, int32_t T,
                                      const float *__restrict__ fields, int64_t field_stride,
-                                     const float4 *__restrict__ rates, const int32_t *__restrict__ targets,
-                                     VDec *__restrict__ dec) {
+                                     const int32_t *__restrict__ targets, VDec *__restrict__ dec) {
     const int v = wide[blockIdx.x], lane = threadIdx.x & 31;
     const int a = blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (a >= T) return;
@@ -323,7 +330,7 @@ __global__ void wide_decision_kernel(const TraceDom p, const int32_t *__restrict
     fs.begin();
     for (int q = p.vt_off[v] + lane, q1 = p.vt_off[v + 1]; q < q1; q += 32) {
         const int tl = p.vt[q];
-        fs.add(v, targets[a], tl, load_tri(p.rec, tl), __ldg(rates + (int64_t)tl * T + a));
+        fs.add(v, targets[a], tl, load_tri(p.rec, tl), tri_rates(p.gphi, p.rec, tl, f));
     }
     __syncwarp();
     fan_reduce<32>(fs, 0xffffffffu);
@@ -875,8 +882,8 @@ int32_t step_cap(const DevMesh &m) {
 }  // namespace
 
 size_t trace_scratch_bytes(const DevMesh &m, int32_t T, bool decisions) {
-    return align256((size_t)T * m.n_t * sizeof(float4)) +
-           (decisions ? align256((size_t)T * m.n_v * sizeof(VDec)) : 0);
+    return decisions ? align256((size_t)T * m.n_v * sizeof(float)) + align256((size_t)T * m.n_v * sizeof(VDec))
+                     : align256((size_t)T * m.n_t * sizeof(float4));
 }
 
 // Vertex decisions for every (field, vertex) before the walk pay off when
@@ -900,11 +907,9 @@ void launch_trace(const DevMesh &m, const float *fields, int64_t field_stride, c
                   int32_t *out_status, void *scratch, cudaStream_t s) {
     const bool dense = trace_dense_decisions(T, S);
     TraceParams p;
-    // the rates of every triangle only where vertex decisions are precomputed (many
-    // paths per field); with few, the walk forms the rates it needs itself
-    float4 *rates = dense ? reinterpret_cast<float4 *>(scratch) : nullptr;
+    float *ft = dense ? reinterpret_cast<float *>(scratch) : nullptr;
     VDec *dec = dense ? reinterpret_cast<VDec *>(reinterpret_cast<char *>(scratch) +
-                                                 align256((size_t)T * m.n_t * sizeof(float4)))
+                                                 align256((size_t)T * m.n_v * sizeof(float)))
                       : nullptr;
     p.d = make_dom(m);
     p.dec = dec;
@@ -922,21 +927,21 @@ void launch_trace(const DevMesh &m, const float *fields, int64_t field_stride, c
     p.out_status = out_status;
     if (p.total == 0) return;
     if (dense) {
+        const unsigned groups32 = (unsigned)((T + 31) / 32);
         {
-            KMark km_("rates_kernel", s);
-            rates_kernel<<<(unsigned)((m.n_t * T + 255) / 256), 256, 0, s>>>(m.gphi, m.trec, m.n_t, T, fields,
-                                                                              field_stride, rates);
+            KMark km_("fields_by_vertex_kernel", s);
+            fields_by_vertex_kernel<<<dim3((unsigned)((m.n_v + 31) / 32), groups32), 256, 0, s>>>(fields, field_stride,
+                                                                                                 m.n_v, T, ft);
         }
-        const int64_t warps = m.n_v * ((T + 31) / 32);
         {
             KMark km_("vertex_decision_kernel", s);
-            vertex_decision_kernel<<<(unsigned)((warps + 3) / 4), 128, 0, s>>>(p.d, T, fields, field_stride, rates,
-                                                                                targets, dec);
+            vertex_decision_kernel<<<dim3((unsigned)((m.n_v + 3) / 4), groups32), 128, 0, s>>>(
+                p.d, T, fields, field_stride, ft, targets, dec);
         }
         if (m.n_wide > 0) {
             KMark km_("wide_decision_kernel", s);
             wide_decision_kernel<<<dim3((unsigned)m.n_wide, (unsigned)((T + 3) / 4)), 128, 0, s>>>(
-                p.d, m.wide, T, fields, field_stride, rates, targets, dec);
+                p.d, m.wide, T, fields, field_stride, targets, dec);
         }
     }
     auto groups = [&](auto kern, int G) {
