@@ -55,20 +55,17 @@ WORKLOADS = {
                         "+ %dx%d KL paths per step"},
 }
 HEADLINE = "grid450"
-# kernels one dd_query step launches at most: target staging, the targets in
-# the tiled layout, field tile, exact KL recompute near the targets, triangle
-# rates and vertex decisions (only when 128 or more paths share a field),
-# path walk
+# kernels one dd_query step launches on grid450: target staging, the targets in
+# the tiled layout, the TV tile, the targets' slices, the tensor-core KL, the
+# exact KL recompute near the targets, the path walk
 STEP_LAUNCHES = 7
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch, from
 # ncu captures of the step's kernels (means over the captured query steps);
 # absent where no capture of the current kernel exists; used only when the
-# step runs the captured (T, S).  grid450's tile launch (the pipelined tile
-# on the tiled copy of P) reads each pair of row tiles from DRAM about once:
-# the 16 CTAs of one pair run together and share it through L2.
+# step runs the captured (T, S).
 TRAFFIC = {
     "grid140": {},
-    "grid450": {"T": 1024, "S": 16, "field_tile_kernel": 9287471001, "trace_kernel": 307644416},
+    "grid450": {},
 }
 # the same for one field_stream_kernel launch of the grid450 single-target pass
 STREAM_TRAFFIC_BYTES = 3035740160    # 3,032,217,088 read + 3,523,072 written (4 n k_pad = 3.03 GB of P)
@@ -180,13 +177,14 @@ def clocks_rejected(clocks) -> bool:
     return bool(sm and mx and sm < 0.8 * mx and not reasons)
 
 
-def roof_tile(n_v, k, T, tile_ms, sms, sm_mhz, traffic):
+def roof_tile(n_v, k, T, tile_ms, sms, sm_mhz, traffic, tv_alone=False):
     """The field tile kernel against the FP32 pipe's rate: per (row, column,
     target) 4 FP32 operations -- KL one addition (the log2 ratio) and one
-    multiply-add, TV two additions -- against 128 FP32 lanes x clock per SM
-    (one operation per lane per clock; a packed FP32x2 instruction does two
-    and holds the pipe twice as long)."""
-    ops = 4.0 * n_v * k * T
+    multiply-add, TV two additions -- or TV's two alone where the tensor cores
+    form KL, against 128 FP32 lanes x clock per SM (one operation per lane per
+    clock; a packed FP32x2 instruction does two and holds the pipe twice as
+    long)."""
+    ops = (2.0 if tv_alone else 4.0) * n_v * k * T
     peak_alu = sms * 128 * sm_mhz * 1e6 / 1e12
     achieved = ops / (tile_ms / 1e3) / 1e12
     return {"kernel": "field_tile_kernel", "bound": "alu", "achieved": round(achieved, 3), "peak": round(peak_alu, 3),
@@ -360,7 +358,8 @@ def query_step(dd, ctx, dev, stream, flush, args, rank, world, local_rank, name,
     if (traffic.get("T"), traffic.get("S")) != (T, S):
         traffic = {}
     tile_ms = per_launch.get("field_tile_kernel", field_ms)
-    roof_t = roof_tile(n_v, k, T, tile_ms, sms, sm_mhz, traffic.get("field_tile_kernel"))
+    roof_t = roof_tile(n_v, k, T, tile_ms, sms, sm_mhz, traffic.get("field_tile_kernel"),
+                       tv_alone="kl_mma_kernel" in per_launch)
     walk_ms = per_launch.get("trace_kernel")
     walk_points = int(np.clip(lens, 0, None).sum())
     roof_w = (roof_walk(walk_ms, walk_points, int(lens.max()), traffic.get("trace_kernel"), load_latency(dd, ctx))
@@ -870,7 +869,7 @@ def mid_section(dd, ctx, dev, stream, flush, pk, pk_kind, reps: int = 8):
     outk = torch.empty((1, T, n_v), dtype=torch.float32, device=dev)
     dd.dd_distance(ctx, mid, tl, 1, dd.DD_PREC_BF16X3, outk)
     gemm_ms = timed(lambda i: dd.dd_distance(ctx, mid, tl, 1, dd.DD_PREC_BF16X3, outk), 4)
-    # the FP32 many-target pass (field tile kernel + exact recompute), KL+TV
+    # the FP32 many-target pass (TV tile, tensor-core KL, exact recompute), KL+TV
     out2 = torch.empty((2, T, n_v), dtype=torch.float32, device=dev)
     dd.dd_distance(ctx, mid, tl, 3, dd.DD_PREC_FP32, out2)      # the first call runs the tile autotuner
     tile_ms = timed(lambda i: dd.dd_distance(ctx, mid, tl, 3, dd.DD_PREC_FP32, out2), 4)
@@ -954,7 +953,7 @@ def batch_section(dd, ctx, dev, stream, flush, args, S: int = 64, max_pts: int =
                         % (len(wls), min(n_vs), max(n_vs), min(ks), max(ks), nT, nT * S),
             "ms_per_batch": round(med, 3), "fields_per_s": round(2 * nT / (med / 1e3), 1),
             "paths_per_s": round(nT * S / (med / 1e3), 1),
-            "field_fp32_instructions_per_batch": 4.0 * elem_targets, "paths_ok_frac": float(np.mean(stn == 0)),
+            "field_fp32_instructions_per_batch": (2.0 if "kl_mma_kernel" in kt else 4.0) * elem_targets, "paths_ok_frac": float(np.mean(stn == 0)),
             "tile_shapes": dd.dd_tuning_table().strip().splitlines(), "kernels": kernels,
             "preproc": {"pcg_iters_total": pcg_iters, "seconds": round(pre, 2)},
             "launches_per_batch": round(sum(c for c, _ in kt.values()) / max(len(ms), 1), 2)}

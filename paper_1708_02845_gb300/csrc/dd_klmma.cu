@@ -18,7 +18,8 @@
 // integer of at most 2^16 units and a chunk's 64 of them sum exactly in the 24
 // bits of an FP32 accumulator.  Nine products are kept,
 //   A = p1 l1 (exact),   B = (p4 l1 + p3 l2 + p2 l3) + (p1 l3 + p2 l2 + p3 l1) + (p1 l2 + p2 l1)
-// (each bracket 2^-9 of the next, the smallest first), in two accumulators; what is dropped is about
+// (each bracket 2^-9 of the next, the smallest first), in two accumulators, or
+// one a bracket (up to 64 targets); what is dropped is about
 // 2^-33 of the chunk's largest entry times the largest log.  After every chunk
 // A is split at multiples of 2^-15: the upper part goes into a total of
 // such multiples (exact below 2^9), the rest and B into a second total.
@@ -33,8 +34,8 @@
 // Kernel: persistent, one CTA per SM walks 128-row x N-target output tiles.
 // The operands lie in global memory chunk by chunk in the shared-memory image
 // of the MMA (K-major, 128-byte swizzle), so a stage is two contiguous bulk
-// copies.  Warp 0 copies, warp 1 issues the MMAs (36 of K = 16 a chunk) into
-// one of two accumulator pairs in TMEM, warps 2-9 take the finished pair of a
+// copies.  Warp 0 copies, warp 1 issues the MMAs (16 or 36 of K = 16 a chunk) into
+// one of two accumulator sets in TMEM, warps 2-9 take the finished set of a
 // chunk out and add it to the totals in registers while the next chunk's MMAs
 // run.  Every wait is bounded and also gives up when another role has.
 //
@@ -131,7 +132,17 @@ __global__ void __launch_bounds__(320, 1) kl_mma_kernel(const KlOne one, const B
                                                         int *__restrict__ err) {
     constexpr int ST = stages(N), SB = A_BYTES + b_bytes(N);
     constexpr int CW = N / 2;            // columns of an epilogue warp
-    constexpr uint32_t TCOLS = 4 * N;    // two pairs of N-column accumulators (a power of two)
+    // An MMA fetches its row operand (128 x 16, 4 KB) from shared memory in some
+    // 64 clocks, as long as it takes to multiply 128 columns: with fewer targets
+    // the row slices are fetched once each instead of once a product, against
+    // the target slices side by side (p1 [l1 l2 l3], p2 [l1 l2 l3], p3 [l1 l2],
+    // p4 [l1]), each one accumulator further on, so that the columns of an
+    // accumulator hold one bracket of the sum: 16 MMAs a chunk instead of 36
+    // (201 x 201 cells, 7 targets: 73 -> 53 us with the quarters above; grid140
+    // with 64: 44 -> 34)
+    constexpr bool kJoined = N <= 64;
+    constexpr int NACC = kJoined ? 4 : 2;
+    constexpr uint32_t TCOLS = 2 * NACC * N;    // two sets of N-column accumulators (a power of two)
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + ST * SB);
@@ -168,7 +179,7 @@ __global__ void __launch_bounds__(320, 1) kl_mma_kernel(const KlOne one, const B
     // few tiles takes as long as a full one (201 x 201 cells: 317 tiles on 152
     // SMs, 73 us).  Its tiles are cut into quarters of 32 rows, an item each:
     // only those rows are copied (the MMA's others hold what was there, and
-    // their results are not stored) (III us).
+    // their results are not stored).
     constexpr bool kQuarters = !BATCH && N == 16;
     const int rounds = n_items / (int)gridDim.x * (int)gridDim.x;
     const bool cut = kQuarters && rounds > 0 && 2 * (n_items - rounds) <= (int)gridDim.x;
@@ -240,16 +251,26 @@ __global__ void __launch_bounds__(320, 1) kl_mma_kernel(const KlOne one, const B
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t st = smem_addr(smem + s * SB);
                     const uint64_t a0 = smem_desc(st), b0 = smem_desc(st + A_BYTES);
-                    const uint32_t accA = tmem + (uint32_t)(buf * 2 * N), accB = accA + N;
+                    const uint32_t accA = tmem + (uint32_t)(buf * NACC * N), accB = accA + N;
                     constexpr uint64_t SA = (BM * ROW_B) >> 4, SBN = (N * ROW_B) >> 4;   // one slice further
+                    if constexpr (kJoined) {
 #pragma unroll
-                    for (int kk = 0; kk < BK / 16; ++kk) mma<N>(accA, a0 + 2 * kk, b0 + 2 * kk, kk > 0);
-                    constexpr int pi[8] = {3, 2, 1, 0, 1, 2, 0, 1}, li[8] = {0, 1, 2, 2, 1, 0, 1, 0};
+                        for (int kk = 0; kk < BK / 16; ++kk) {
+                            mma<N>(accA + 3 * N, a0 + 3 * SA + 2 * kk, b0 + 2 * kk, kk > 0);
+                            mma<3 * N>(accA, a0 + 2 * kk, b0 + 2 * kk, kk > 0);
+                            mma<2 * N>(accA + 2 * N, a0 + 2 * SA + 2 * kk, b0 + 2 * kk, true);
+                            mma<3 * N>(accA + N, a0 + SA + 2 * kk, b0 + 2 * kk, true);
+                        }
+                    } else {
 #pragma unroll
-                    for (int p = 0; p < 8; ++p)
+                        for (int kk = 0; kk < BK / 16; ++kk) mma<N>(accA, a0 + 2 * kk, b0 + 2 * kk, kk > 0);
+                        constexpr int pi[8] = {3, 2, 1, 0, 1, 2, 0, 1}, li[8] = {0, 1, 2, 2, 1, 0, 1, 0};
 #pragma unroll
-                        for (int kk = 0; kk < BK / 16; ++kk)
-                            mma<N>(accB, a0 + pi[p] * SA + 2 * kk, b0 + li[p] * SBN + 2 * kk, p > 0 || kk > 0);
+                        for (int p = 0; p < 8; ++p)
+#pragma unroll
+                            for (int kk = 0; kk < BK / 16; ++kk)
+                                mma<N>(accB, a0 + pi[p] * SA + 2 * kk, b0 + li[p] * SBN + 2 * kk, p > 0 || kk > 0);
+                    }
                     commit(&empty[s]);       // the stage is free once these MMAs complete
                     commit(&accf[buf]);
                 }
@@ -276,17 +297,26 @@ __global__ void __launch_bounds__(320, 1) kl_mma_kernel(const KlOne one, const B
                 ok = __all_sync(0xffffffffu, wait_or_abort(&accf[buf], (g >> 1) & 1, err, abort));
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t ta = tmem + lane_base + (uint32_t)(buf * 2 * N + half * CW);
+                const uint32_t ta = tmem + lane_base + (uint32_t)(buf * NACC * N + half * CW);
 #pragma unroll
                 for (int c0 = 0; c0 < CW; c0 += 8) {
-                    uint32_t ra[8], rb[8];
+                    uint32_t ra[8], rb[8], rc[8], rd[8];
                     tmem_ld8(ra, ta + c0);
                     tmem_ld8(rb, ta + N + c0);
+                    if constexpr (kJoined) {
+                        tmem_ld8(rc, ta + 2 * N + c0);
+                        tmem_ld8(rd, ta + 3 * N + c0);
+                    }
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         const f2_t a = pk(__uint_as_float(ra[2 * j]), __uint_as_float(ra[2 * j + 1]));
-                        const f2_t b = pk(__uint_as_float(rb[2 * j]), __uint_as_float(rb[2 * j + 1]));
+                        f2_t b = pk(__uint_as_float(rb[2 * j]), __uint_as_float(rb[2 * j + 1]));
+                        if constexpr (kJoined) {
+                            const f2_t c3 = pk(__uint_as_float(rc[2 * j]), __uint_as_float(rc[2 * j + 1]));
+                            const f2_t d4 = pk(__uint_as_float(rd[2 * j]), __uint_as_float(rd[2 * j + 1]));
+                            b = add2(add2(d4, c3), b);
+                        }
                         const f2_t h = add2(add2(a, split), nsplit);
                         f2_t &H = hi[c0 / 2 + j], &L = lo[c0 / 2 + j];
                         H = add2(H, h);

@@ -59,9 +59,11 @@ def test_tile_edges(env, T):
         assert field_error(both[0, a], kl_field_fast(P, P[t])) <= TOL_FP32
         assert field_error(both[1, a], tv_field(P, P[t])) <= TOL_FP32
         assert both[0, a, t] == 0.0 and both[1, a, t] == 0.0
-    # a target's field does not depend on the tile and column it falls in
-    single = fields(dd, ctx, mid, mesh.n_v, targets[:3], dd.DD_F_KL)
-    assert np.array_equal(single[0], both[0, :3])
+    # a target's field does not depend on the tile and column it falls in (up to
+    # 64 targets share one order of the small products, more another)
+    few = targets[:3] if T <= 64 else targets[:65]
+    single = fields(dd, ctx, mid, mesh.n_v, few, dd.DD_F_KL)
+    assert np.array_equal(single[0], both[0, :len(few)])
 
 
 def test_batch_has_the_fields_of_single_calls(env, monkeypatch):
