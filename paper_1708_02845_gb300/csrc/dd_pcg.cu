@@ -631,9 +631,11 @@ dd_status run_pcg_amg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s,
     }
     const int64_t nbands = (m + band[0] - 1) / band[0];
 
-    // one device allocation for the hierarchy and the workspace (a solve has
-    // dozens of arrays; allocated and freed one by one they cost 2 ms), the
-    // hierarchy's part filled from one host buffer in one copy
+    // one device allocation for the hierarchy and the small arrays (a solve has
+    // dozens; allocated and freed one by one they cost 2 ms), the hierarchy's
+    // part filled from one host buffer in one copy; the six fine-level blocks
+    // apart (as one block with the rest, its release left the next
+    // allocations, and the first pass over P, up to 2 ms slower)
     size_t total = 0;
     auto take = [&](size_t bytes) {
         const size_t o = total;
@@ -663,12 +665,11 @@ dd_status run_pcg_amg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s,
     const size_t o_ainv = take(H.coarse_inv.size() * sizeof(double));
     const size_t filled = total;
     const size_t vec = (size_t)m * kc * sizeof(double);
-    const size_t o_X = take(vec), o_R = take(vec), o_Z = take(vec), o_Pd = take(vec), o_AP = take(vec);
     std::vector<size_t> o_b(nl), o_x(nl);
-    for (int l = 0; l < nl; ++l) {
+    for (int l = 1; l < nl; ++l) {
         const size_t lv = (size_t)H.levels[l].A.rows * kc * sizeof(float2);
         o_b[l] = take(lv);
-        if (l > 0) o_x[l] = take(lv);
+        o_x[l] = take(lv);
     }
     const size_t o_p0 = take((size_t)std::max(nrb, nbands) * kc * sizeof(double)), o_p1 = take((size_t)nrb * kc * sizeof(double));
     const size_t o_al = take(kc * sizeof(double)), o_be = take(kc * sizeof(double)), o_rz = take(kc * sizeof(double));
@@ -690,10 +691,18 @@ dd_status run_pcg_amg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s,
         for (size_t i = 0; i < H.coarse_inv.size(); ++i) val[i] = split_pair(H.coarse_inv[i]);
     }
     uint8_t *ws = nullptr;
+    double *fine[6] = {};
     cudaError_t ce = cudaMalloc((void **)&ws, total);
+    for (double *&v : fine)
+        if (ce == cudaSuccess) ce = cudaMalloc((void **)&v, vec);
     if (ce == cudaSuccess) ce = cudaMemcpyAsync(ws, host.data(), filled, cudaMemcpyHostToDevice, s);
-    if (ce != cudaSuccess) {
+    auto drop = [&]() {
         if (ws) cudaFree(ws);
+        for (double *v : fine)
+            if (v) cudaFree(v);
+    };
+    if (ce != cudaSuccess) {
+        drop();
         cudaGetLastError();
         *fallback = true;
         err = std::string("multigrid workspace allocation failed: ") + cudaGetErrorString(ce);
@@ -701,17 +710,19 @@ dd_status run_pcg_amg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s,
     }
     auto release = [&]() {
         cudaStreamSynchronize(s);
-        cudaFree(ws);
+        drop();
     };
     for (const Plan &q : plans)
         *q.d = DevCsr{reinterpret_cast<int32_t *>(ws + q.off), reinterpret_cast<int32_t *>(ws + q.col),
                       reinterpret_cast<float2 *>(ws + q.val)};
     auto at = [&](size_t o) { return reinterpret_cast<double *>(ws + o); };
-    double *X = at(o_X), *R = at(o_R), *Z = at(o_Z), *Pd = at(o_Pd), *AP = at(o_AP);
+    double *X = fine[0], *R = fine[1], *Z = fine[2], *Pd = fine[3], *AP = fine[4];
     double *part0 = at(o_p0), *part1 = at(o_p1), *alpha = at(o_al), *beta = at(o_be), *rz = at(o_rz), *bnorm = at(o_bn);
     int *done = reinterpret_cast<int *>(ws + o_dn);
     unsigned long long *maxres = reinterpret_cast<unsigned long long *>(ws + o_mr);
-    auto lb = [&](int l) { return reinterpret_cast<float4 *>(ws + o_b[l]); };
+    auto lb = [&](int l) {
+        return l == 0 ? reinterpret_cast<float4 *>(fine[5]) : reinterpret_cast<float4 *>(ws + o_b[l]);
+    };
     auto lx = [&](int l) { return reinterpret_cast<float4 *>(ws + o_x[l]); };
     auto d2 = [](double *p) { return reinterpret_cast<double2 *>(p); };
 
