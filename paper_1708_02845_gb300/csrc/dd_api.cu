@@ -20,6 +20,8 @@
 
 namespace {
 
+std::atomic<int> g_kt_on{0};      // contexts with per-kernel timing on
+
 dd_status set_err(dd_ctx *c, dd_status s, const std::string &msg) {
     if (c) c->err = msg;
     return s;
@@ -104,11 +106,16 @@ void *mapped_alias(const void *p) {
 
 dd_status ensure_side(dd_ctx *ctx) {
     if (ctx->side) return DD_OK;
-    if (cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ctx->side_ev[0], cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ctx->side_ev[1], cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ctx->side_ev[2], cudaEventDisableTiming) != cudaSuccess) {
+    bool ok = cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking) == cudaSuccess;
+    for (cudaEvent_t &e : ctx->side_ev) ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) {
         cudaGetLastError();
+        for (cudaEvent_t &e : ctx->side_ev) {
+            if (e) cudaEventDestroy(e);
+            e = nullptr;
+        }
+        if (ctx->side) cudaStreamDestroy(ctx->side);
+        ctx->side = nullptr;
         return set_err(ctx, DD_ECUDA, "side stream creation failed");
     }
     return DD_OK;
@@ -252,8 +259,15 @@ dd_status fields_into(dd_ctx *ctx, DevMesh &m, const int32_t *d_targets, int32_t
         if ((st = ensure_scratch(ctx, S_STAGE, sparse_stage_bytes(m.k_pad, T))) != DD_OK) return st;
         float4 *stage = reinterpret_cast<float4 *>(ctx->scratch[S_STAGE]);
         launch_stage_targets(m.P, m.n_v, m.k_pad, d_targets, T, stage, ctx->stream);
+        // (per-kernel timing is by stream: with it on, everything stays on the caller's)
+        SideStream side{};
+        const bool fork = klt && (kl || tv) && g_kt_on.load(std::memory_order_relaxed) == 0;
+        if (fork) {
+            if ((st = ensure_side(ctx)) != DD_OK) return st;
+            side = SideStream{ctx->side, ctx->side_ev[3], ctx->side_ev[4]};
+        }
         launch_sparse_fields(m, d_targets, stage, T, kl, tv, klt, prec == DD_PREC_SPARSE_MERGED, ctx->d_err,
-                             ctx->stream);
+                             ctx->stream, fork ? &side : nullptr);
         CK(cudaGetLastError(), "sparse field kernel launch");
         return DD_OK;
     }
@@ -329,7 +343,6 @@ struct KTimer {
 
 std::mutex g_kt_mutex;
 std::map<cudaStream_t, KTimer> g_kt;
-std::atomic<int> g_kt_on{0};
 
 cudaEvent_t kt_event(KTimer &t) {
     if (!t.pool.empty()) {

@@ -265,8 +265,15 @@ size_t sparse_stage_bytes(int64_t k_pad, int32_t T);
 size_t sparse_field_smem(int64_t k_pad);
 dd_status build_sparse_rows(DevMesh &m, double theta, cudaStream_t s, int64_t *kept_out, int64_t *bytes_out,
                             std::string &err);
+// side: null, or a second stream of the caller's and two events, on which KLT~
+// may run beside the CSR pass (s waits for it before the call returns).
+struct SideStream {
+    cudaStream_t stream;
+    cudaEvent_t fork, join;
+};
 void launch_sparse_fields(const DevMesh &m, const int32_t *d_targets, float4 *stage, int32_t T, float *out_kl,
-                          float *out_tv, float *out_klt, bool merged, int *err_flag, cudaStream_t s);
+                          float *out_tv, float *out_klt, bool merged, int *err_flag, cudaStream_t s,
+                          const SideStream *side = nullptr);
 // spread (max - min) of the hardware mantissa log's error over [1, 2), in base-2 units
 dd_status fast_log_spread(double *spread, std::string &err);
 
@@ -321,7 +328,7 @@ struct dd_ctx {
     size_t pinned_cap[S_COUNT] = {};
     cudaEvent_t pinned_free[S_COUNT] = {};    // recorded after the last upload from pinned[id]
     cudaStream_t side = nullptr;              // copies that overlap the main stream's kernels
-    cudaEvent_t side_ev[3] = {};             // fields ready, fields copied, tile pass done
+    cudaEvent_t side_ev[5] = {};             // fields ready, fields copied, tile pass done; sparse fork, join
 };
 
 // Per-kernel device time (dd_kernel_timing): while timing is enabled for a

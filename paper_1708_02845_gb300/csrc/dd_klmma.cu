@@ -43,8 +43,8 @@
 // TFLOP/s = 93 % of the measured burst rate of 1,931), with the TV tile pass
 // (45.3 ms) and a recompute of fewer pairs (1.6 against 4.1 ms) in place of
 // the 94.5 ms KL+TV tile pass: a call 98.9 -> 54.9 ms.  grid140, 64 targets:
-// 44 us (N = 64; the slices' 158 MB from memory bound it), a call 324 -> 241
-// us.  KL alone, 201 x 201 cells, 7 targets: a call 228 -> 131 us.
+// 34 us (N = 64; the slices' 131 MB from memory bound it), a call 321 -> 181
+// us.  KL alone, 201 x 201 cells, 7 targets: a call 228 -> 104 us.
 #include <cuda_bf16.h>
 
 #include <algorithm>

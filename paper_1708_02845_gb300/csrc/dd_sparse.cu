@@ -222,7 +222,7 @@ __global__ void sparse_stage_kernel(const float *__restrict__ P, float *__restri
                                     const float *__restrict__ sF, int64_t k_pad, float theta,
                                     uint16_t *__restrict__ list, int64_t lp, int32_t *__restrict__ count,
                                     const long long *__restrict__ rowsum, const int32_t *__restrict__ targets,
-                                    double *__restrict__ mt_out) {
+                                    double *__restrict__ mt_out) {      // mt_out null: M_t is not asked for
     __shared__ float red[32];
     __shared__ int wsum[32];
     const int a = blockIdx.x;
@@ -274,7 +274,7 @@ __global__ void sparse_stage_kernel(const float *__restrict__ P, float *__restri
     if (threadIdx.x == 0) count[a] = base;
     // the target's mass outside S_t, by the routine and lane order the field
     // kernel uses for every row (so that it reproduces this value at x = t)
-    if (threadIdx.x < 32) {
+    if (mt_out && threadIdx.x < 32) {
         const double mt = total62(rowsum[targets[a]]) -
                           kept_mass(P, targets[a], k_pad, L, base, reinterpret_cast<const float4 *>(row),
                                     reinterpret_cast<const float4 *>(sF + (int64_t)a * k_pad),
@@ -830,7 +830,8 @@ dd_status build_sparse_rows(DevMesh &m, double theta, cudaStream_t s, int64_t *k
 }
 
 void launch_sparse_fields(const DevMesh &m, const int32_t *d_targets, float4 *stage, int32_t T, float *out_kl,
-                          float *out_tv, float *out_klt, bool merged, int *err_flag, cudaStream_t s) {
+                          float *out_tv, float *out_klt, bool merged, int *err_flag, cudaStream_t s,
+                          const SideStream *side) {
     float *sP = reinterpret_cast<float *>(stage);
     const float *sL = sP + (int64_t)T * m.k_pad;
     const float *sE = sL + (int64_t)T * m.k_pad;
@@ -842,7 +843,7 @@ void launch_sparse_fields(const DevMesh &m, const int32_t *d_targets, float4 *st
     {
         KMark km_("sparse_stage_kernel", s);
         sparse_stage_kernel<<<(unsigned)T, 256, 0, s>>>(m.P, sP, sE, sF, m.k_pad, m.sp_theta, sList, lp, sCount,
-                                                         m.sp_rowsum, d_targets, sMt);
+                                                         m.sp_rowsum, d_targets, merged ? sMt : nullptr);
     }
     const int64_t row_blocks = (m.n_v + 7) / 8;
     auto grid_x = [&](auto kern, size_t smem) {
@@ -855,12 +856,19 @@ void launch_sparse_fields(const DevMesh &m, const int32_t *d_targets, float4 *st
         if (gx > row_blocks) gx = row_blocks;
         return (unsigned)gx;
     };
+    // KLT~ beside KL~ / TV~ on the side stream: both passes wait for memory and
+    // shared memory most of their time, and a CTA of each fits an SM (300 x 300
+    // cells, all three fields: 84 + 42 us one after the other, a call 8 % shorter
+    // together).
+    // Not for small copies, whose passes take as long as the two events.
+    const bool beside = side && out_klt && (out_kl || out_tv) && !merged && m.sp_kept >= (1 << 22);
+    cudaStream_t klt_stream = beside ? side->stream : s;
     // the dense rows at the target's blocks: KLT~ (or the merged-bin fields)
     auto go = [&](auto kern) {
         const size_t smem = sparse_field_smem(m.k_pad);
         const unsigned gx = grid_x(kern, smem);
-        KMark km_("sparse_field_kernel", s);
-        kern<<<dim3(gx, (unsigned)T), 256, smem, s>>>(m.P, m.n_v, m.k_pad, sP, sL, sE, sF, sList, lp, sCount, sMt,
+        KMark km_("sparse_field_kernel", klt_stream);
+        kern<<<dim3(gx, (unsigned)T), 256, smem, klt_stream>>>(m.P, m.n_v, m.k_pad, sP, sL, sE, sF, sList, lp, sCount, sMt,
                                                        m.sp_rowsum, out_kl, out_tv, out_klt, err_flag);
     };
     // the CSR rows: KL~ and TV~.  The deepest pipeline whose buffers fit next
@@ -906,6 +914,10 @@ void launch_sparse_fields(const DevMesh &m, const int32_t *d_targets, float4 *st
     }
     using Yes = std::true_type;
     using No = std::false_type;
+    if (beside) {
+        cudaEventRecord(side->fork, s);
+        cudaStreamWaitEvent(klt_stream, side->fork, 0);
+    }
     if (out_kl && out_tv)
         csr(Yes{}, Yes{});
     else if (out_kl)
@@ -913,4 +925,8 @@ void launch_sparse_fields(const DevMesh &m, const int32_t *d_targets, float4 *st
     else if (out_tv)
         csr(No{}, Yes{});
     if (out_klt) go(sparse_field_kernel<2, false, false, true, false>);
+    if (beside) {
+        cudaEventRecord(side->join, klt_stream);
+        cudaStreamWaitEvent(s, side->join, 0);
+    }
 }
