@@ -37,7 +37,7 @@
 // us (a call with its fields, results in host buffers, 362 -> 222 us); 142
 // points, 32 paths on the 2,049-vertex disk 250 -> 47 us (a call 240 -> 68 us);
 // 941 points, 64 x 256 paths on the 71,681-vertex disk 953 -> 476 us and the
-// decisions 778 -> 253 us (a call 1,735 -> 732 us).
+// decisions 778 -> 221 us (a call 1,749 -> 689 us).
 #include <cfloat>
 #include <cstring>
 #include <cstdlib>
@@ -158,15 +158,12 @@ struct FanScan {
         b_pj = b_pk = make_float2(0.f, 0.f);
     }
 
-    // triangle tl (record T, rates R of the field) incident on v
-    __device__ __forceinline__ void add(int v, int target, int tl, const Tri &T, const float4 &R) {
+    // triangle tl (record T, rates R of the field), v its local vertex L, then X
+    // and Y counter-clockwise (rates rX, rY; vertices and positions): the exit
+    // edge is X-Y
+    __device__ __forceinline__ void consider(int target, int tl, float rX, float rY, float qX, float qY, float gg, int vX,
+                                             int vY, float2 pX, float2 pY, int next) {
         const float eps2 = kEpsWedge * kEpsWedge;
-        // rotated view: v is local vertex L, then X and Y counter-clockwise; the exit edge is X-Y
-        const int L = local_of(T, v), X = L == 2 ? 0 : L + 1, Y = L == 0 ? 2 : L - 1;
-        const float rX = sel3f(X, R.x, R.y, R.z), rY = sel3f(Y, R.x, R.y, R.z);
-        const float qX = sel3f(X, T.q0, T.q1, T.q2), qY = sel3f(Y, T.q0, T.q1, T.q2);
-        const int vX = sel3i(X, T.v0, T.v1, T.v2), vY = sel3i(Y, T.v0, T.v1, T.v2);
-        const float gg = R.w;
         adj |= (vX == target) | (vY == target);
         const float tol2 = eps2 * gg * fmaxf(qX, qY);
         const bool in_x = rX >= 0.f || rX * rX <= tol2;
@@ -178,10 +175,28 @@ struct FanScan {
             bak = fmaxf(rY, 0.f);
             b_vj = vX;
             b_vk = vY;
-            b_pj = pos(T, X);
-            b_pk = pos(T, Y);
-            b_next = sel3i(L, T.n0, T.n1, T.n2);
+            b_pj = pX;
+            b_pk = pY;
+            b_next = next;
         }
+    }
+
+    // triangle tl (record T, rates R of the field) incident on v
+    __device__ __forceinline__ void add(int v, int target, int tl, const Tri &T, const float4 &R) {
+        const int L = local_of(T, v), X = L == 2 ? 0 : L + 1, Y = L == 0 ? 2 : L - 1;
+        consider(target, tl, sel3f(X, R.x, R.y, R.z), sel3f(Y, R.x, R.y, R.z), sel3f(X, T.q0, T.q1, T.q2),
+                 sel3f(Y, T.q0, T.q1, T.q2), R.w, sel3i(X, T.v0, T.v1, T.v2), sel3i(Y, T.v0, T.v1, T.v2), pos(T, X),
+                 pos(T, Y), sel3i(L, T.n0, T.n1, T.n2));
+    }
+    // the same where the whole warp looks at one triangle and vertex: a branch
+    // on the local vertex instead of a choice for every operand
+    __device__ __forceinline__ void add_same(int v, int target, int tl, const Tri &T, const float4 &R) {
+        if (T.v0 == v)
+            consider(target, tl, R.y, R.z, T.q1, T.q2, R.w, T.v1, T.v2, T.p1, T.p2, T.n0);
+        else if (T.v1 == v)
+            consider(target, tl, R.z, R.x, T.q2, T.q0, R.w, T.v2, T.v0, T.p2, T.p0, T.n1);
+        else
+            consider(target, tl, R.x, R.y, T.q0, T.q1, R.w, T.v0, T.v1, T.p0, T.p1, T.n2);
     }
 
     // (G lanes of `mask` hold the same scan and share the fallback's fan)
@@ -291,7 +306,8 @@ __device__ __forceinline__ void fan_reduce(FanScan &fs, unsigned mask) {
 // vertices of more than kWideFan triangles are left to wide_decision_kernel.
 // The rates of a fan's triangles are formed here from the fields by vertex:
 // 64 fields of 71,681 vertices, the rates of every triangle stored first (147
-// MB written, read three times) took 68 + 230 us, this 8 + 216.
+// MB written, read three times) took 68 + 230 us, this 8 + 183 (216 with a
+// choice among the local vertices for every operand).
 __global__ void __launch_bounds__(128) vertex_decision_kernel(const TraceDom p, int32_t T,
                                                               const float *__restrict__ fields, int64_t field_stride,
                                                               const float *__restrict__ ft,
@@ -310,7 +326,7 @@ __global__ void __launch_bounds__(128) vertex_decision_kernel(const TraceDom p, 
         const Tri t = load_tri(p.rec, tl);
         const float4 r = rates_of(__ldg(p.gphi + 2 * (int64_t)tl), ft[(int64_t)t.v0 * T + a], ft[(int64_t)t.v1 * T + a],
                                   ft[(int64_t)t.v2 * T + a]);
-        fs.add((int)v, target, tl, t, r);
+        fs.add_same((int)v, target, tl, t, r);
     }
     dec[v * T + a] = fs.finish<1>(p, fields + (int64_t)a * field_stride, target, (int)v);
 }
