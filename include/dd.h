@@ -518,7 +518,10 @@ void dd_server_destroy(dd_server *sv);
  *   out      device float32 [nf][T][n_v], layout as in dd_distance, 4-byte
  *            aligned
  *   cuda_stream  stream for the work (NULL = legacy default stream)
- * The fields equal dd_distance's bit for bit.  Nothing is timed or tuned:
+ * The fields equal dd_distance's bit for bit, but for KL of more than two
+ * targets on maps with n_v k_pad >= 2^20: there dd_distance forms KL on the
+ * tensor cores from operands that this call has no room for, and the two agree
+ * to FP32 rounding (both within 1e-5 relative).  Nothing is timed or tuned:
  * for T > 2 the tile shape is a fixed function of T (dd_distance's autotuner
  * would run timed launches the first time it meets a size class).
  * Scratch: one fixed device array per GPU (16 MiB, held until the process
