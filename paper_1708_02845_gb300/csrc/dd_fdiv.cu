@@ -141,8 +141,50 @@ __device__ __forceinline__ float klrev_logp_term(float pt, float lmt, float Ebt,
 // rows whose first-pass value is below q.below = max(DD_EXACT_BELOW,
 // 2e5 |lin| / |e| 2^-22) are recomputed in the exact form, and every other
 // value is within 1e-5 / 2 of exact, relatively.  The entries with P_x = 0 or
-// P_t = 0 take their limits by selection (ZEROS), for the chunks that hold one
-// (padding entries pass P_x = P_t = 0 and give 0).
+// P_t = 0 take their limits by selection, evaluated only when a lane of the
+// warp holds one; every lane of the warp must call it (padding entries pass
+// P_x = P_t = 0 and give 0).
+__device__ __forceinline__ void alpha_fast4(const float (&px)[4], const float (&pt)[4], const float (&ft)[4],
+                                            const float (&et)[4], const FdParams &q, float (&t)[4]) {
+    // the adds and multiplies two entries at a time in packed FP32x2 (each half
+    // rounds exactly as the scalar operation: a product is fma(a, b, 0))
+    const f2_t mone = pk(-1.0f, -1.0f), zero = pk(0.0f, 0.0f);
+    const f2_t e2 = pk(q.p, q.p), nie2 = pk(-q.inv_e, -q.inv_e), lin2 = pk(q.lin, q.lin);
+    bool special = false;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int j0 = 2 * h, j1 = 2 * h + 1;
+        // no clamp: P holds no subnormals, and a zero entry takes its limit below
+        const int b0 = __float_as_int(px[j0]), b1 = __float_as_int(px[j1]);
+        const f2_t lf = pk(lg2_mant(b0), lg2_mant(b1));
+        const f2_t eb = pk(__int_as_float((int)__funnelshift_r((unsigned)b0, (unsigned)kMagicHi, 23)),
+                           __int_as_float((int)__funnelshift_r((unsigned)b1, (unsigned)kMagicHi, 23)));
+        const f2_t px2 = pk(px[j0], px[j1]), pt2 = pk(pt[j0], pt[j1]);
+        // L2 = (lg2 m_t - lg2 m_x) + (E_t - E_x)
+        const f2_t L2 = add2(fma2(lf, mone, pk(ft[j0], ft[j1])), fma2(eb, mone, pk(et[j0], et[j1])));
+        float y0, y1;
+        upk(fma2(L2, e2, zero), y0, y1);
+        const f2_t um1 = add2(pk(ex2_hw(y0), ex2_hw(y1)), mone);                    // 2^(e L2) - 1
+        const f2_t r = fma2(fma2(px2, nie2, zero), um1, fma2(px2, mone, pt2));      // (P_t - P_x) - P_x um1 / e
+        upk(fma2(r, lin2, zero), t[j0], t[j1]);
+        // a zero factor among P_x, P_t (a product that underflows only sends the
+        // warp through the selection, which leaves every other entry as it is)
+        float z0, z1;
+        upk(fma2(px2, pt2, zero), z0, z1);
+        special |= (z0 == 0.0f) | (z1 == 0.0f);
+    }
+    if (__any_sync(0xffffffffu, special)) {
+        const float at_px0 = q.alpha_gt1 ? INFINITY : q.lin;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float v = pt[j] == 0.0f ? px[j] * q.inv_e : t[j];                   // u = 0: lin P_x (1/e - 1) = P_x / e
+            v = px[j] == 0.0f ? (pt[j] == 0.0f ? 0.0f : at_px0 * pt[j]) : v;    // P_x = 0: lin P_t, or +inf for a > 1
+            t[j] = v;
+        }
+    }
+}
+
+// The same for the pair kernel, split into a row's side and a target's.
 // Four entries of a row as every target of a pass reads them: the entries,
 // their hardware mantissa logs and biased exponents, packed by pairs.
 struct Row4 {
@@ -166,7 +208,7 @@ __device__ __forceinline__ Row4 row_side(const float4 &v) {
 }
 
 template <bool ZEROS>
-__device__ __forceinline__ void alpha_fast4(const Row4 &x, const f2_t (&pe)[2], const float4 &p4, const float4 &f4,
+__device__ __forceinline__ void alpha_pair4(const Row4 &x, const f2_t (&pe)[2], const float4 &p4, const float4 &f4,
                                             const float4 &e4, const FdParams &q, f2_t &sum) {
     // the adds and multiplies two entries at a time in packed FP32x2 (each half
     // rounds exactly as the scalar operation: a product is fma(a, b, 0));
@@ -254,10 +296,14 @@ __device__ __forceinline__ void stream_rows(const float *__restrict__ P, int64_t
     }
 }
 
-// floats per staged row of two_pass_kernel: k_pad rounded up to whole groups
+// floats per staged row of two_pass_pair_kernel: k_pad rounded up to whole groups
 // of 32 lanes x one float4
 constexpr int kMaxGroups = 104;      // 200 KB of staged rows of one target
-__host__ __device__ constexpr int64_t two_pass_pitch(int64_t k_pad) { return (k_pad + 127) / 128 * 128; }
+__host__ __device__ constexpr int64_t two_pass_pair_pitch(int64_t k_pad) { return (k_pad + 127) / 128 * 128; }
+
+// floats per staged row of two_pass_kernel: k_pad rounded up to whole
+// chunks of 32 lanes x 8 float4
+__host__ __device__ constexpr int64_t two_pass_pitch(int64_t k_pad) { return (k_pad + 1023) / 1024 * 1024; }
 
 // LP (reverse KL only, may be null): log2 P; an entry whose FP32 value is 0
 // takes log P[x,b] from it instead of the clamp at FLT_MIN
@@ -336,27 +382,125 @@ __global__ void __launch_bounds__(256) fdiv_kernel(const float *__restrict__ P, 
 // around the target, x = t among them -- recomputed by its warp with the
 // table logarithm (fterm), so every value keeps 1e-5 relative accuracy.  A
 // row entry P[x,b] = 0 is taken at FLT_MIN on both passes (reverse KL).
-// Shared memory: each target's P, table mantissa log, biased exponent and
+// Shared memory: the target's P, table mantissa log, biased exponent and
 // hardware mantissa log2.
-// TT targets a CTA (blockIdx.y: which TT of them): P is read, and its entries'
-// logarithms formed, once for both.  One target at a time, the alpha
-// divergence of two targets (300 x 300 cells) took 424 us, bound by the
-// hardware log2 and exp2 and the instructions around them; 323 us with two.
-template <int FAM, int TT>
-__global__ void __launch_bounds__(256 * TT, 2 / TT) two_pass_kernel(const float *__restrict__ P, int64_t n_v,
+template <int FAM>
+__global__ void __launch_bounds__(256) two_pass_kernel(const float *__restrict__ P, int64_t n_v, int64_t k_pad,
+                                                       const float *__restrict__ sP, const float *__restrict__ sL,
+                                                       const float *__restrict__ sE, const float *__restrict__ sF,
+                                                       FdParams q, float *__restrict__ out) {
+    constexpr int U = 8;       // float4 per lane and buffer: 2 x 4 KB per warp in flight
+    extern __shared__ __align__(16) float fsm[];
+    __shared__ float tab[2 * kLogTab];
+    // alpha: the staged rows zero-padded to whole chunks (two_pass_pitch), so
+    // that every lane of a chunk reads its target entries without a test
+    const int64_t kp = FAM == kAlpha ? two_pass_pitch(k_pad) : k_pad;
+    float *tP = fsm, *tL = fsm + kp, *tE = fsm + 2 * kp, *tF = fsm + 3 * kp;
+    const int a = blockIdx.y;
+    for (int64_t b = threadIdx.x; b < kp; b += blockDim.x) {
+        const bool in = b < k_pad;
+        tP[b] = in ? sP[(int64_t)a * k_pad + b] : 0.0f;
+        tL[b] = in ? sL[(int64_t)a * k_pad + b] : 0.0f;
+        tE[b] = in ? sE[(int64_t)a * k_pad + b] : 0.0f;
+        tF[b] = in ? sF[(int64_t)a * k_pad + b] : 0.0f;
+    }
+    build_log_table(tab);
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int nvec = (int)(k_pad >> 2);
+    float s0 = 0.0f, s1 = 0.0f;
+    auto chunk = [&](const float4(&v)[U], int64_t, int c0) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int c = c0 + u * 32 + lane;
+            if (FAM == kAlpha) {
+                // every lane takes part (the first pass votes per group of four
+                // entries); past the row's end P and the padded target row are 0
+                const float4 p4 = reinterpret_cast<const float4 *>(tP)[c];
+                const float4 f4 = reinterpret_cast<const float4 *>(tF)[c];
+                const float4 e4 = reinterpret_cast<const float4 *>(tE)[c];
+                const float px[4] = {v[u].x, v[u].y, v[u].z, v[u].w}, pt[4] = {p4.x, p4.y, p4.z, p4.w};
+                const float ft[4] = {f4.x, f4.y, f4.z, f4.w}, et[4] = {e4.x, e4.y, e4.z, e4.w};
+                float t[4];
+                alpha_fast4(px, pt, ft, et, q, t);
+                s0 += t[0];
+                s1 += t[1];
+                s0 += t[2];
+                s1 += t[3];
+                continue;
+            }
+            if (c >= nvec) break;
+            const float4 p4 = reinterpret_cast<const float4 *>(tP)[c];
+            const float4 f4 = reinterpret_cast<const float4 *>(tF)[c];
+            const float4 e4 = reinterpret_cast<const float4 *>(tE)[c];
+            const float px[4] = {v[u].x, v[u].y, v[u].z, v[u].w}, pt[4] = {p4.x, p4.y, p4.z, p4.w};
+            const float ft[4] = {f4.x, f4.y, f4.z, f4.w}, et[4] = {e4.x, e4.y, e4.z, e4.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int bits = __float_as_int(fmaxf(px[e], FLT_MIN));
+                const float lf = lg2_mant(bits);
+                const float eb = __int_as_float((int)__funnelshift_r((unsigned)bits, (unsigned)kMagicHi, 23));
+                const float t = pt[e] * __fadd_rn(__fadd_rn(ft[e], -lf), __fadd_rn(et[e], -eb));
+                if (e & 1)
+                    s1 += t;
+                else
+                    s0 += t;
+            }
+        }
+    };
+    auto done = [&](int64_t x) {
+        float sum = s0 + s1;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (FAM == kKlRev) sum *= kLn2f;
+        if (sum < q.below) {                    // warp-uniform: the exact (table) form
+            const float4 *row = reinterpret_cast<const float4 *>(P + x * k_pad);
+            float r0 = 0.0f, r1 = 0.0f;
+            for (int c = lane; c < nvec; c += 32) {
+                const float4 vx = __ldcg(row + c);
+                const float4 p4 = reinterpret_cast<const float4 *>(tP)[c];
+                const float4 l4 = reinterpret_cast<const float4 *>(tL)[c];
+                const float4 e4 = reinterpret_cast<const float4 *>(tE)[c];
+                r0 += fterm<FAM>(vx.x, p4.x, l4.x, e4.x, q, tab);
+                r1 += fterm<FAM>(vx.y, p4.y, l4.y, e4.y, q, tab);
+                r0 += fterm<FAM>(vx.z, p4.z, l4.z, e4.z, q, tab);
+                r1 += fterm<FAM>(vx.w, p4.w, l4.w, e4.w, q, tab);
+            }
+            sum = r0 + r1;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        }
+        if (lane == 0) out[(int64_t)a * n_v + x] = sum;
+        s0 = s1 = 0.0f;
+    };
+    stream_rows<U>(P, n_v, k_pad, warp, nwarps, lane, chunk, done);
+}
+
+// Two targets a CTA of 512 threads: P is read, and its entries' logarithms
+// formed, once for both, and chunks without a zero run without branches (the
+// two take 125 registers: one CTA an SM).  For two targets of a map well
+// beyond L2: alpha 0.5 on 300 x 300 cells 442 -> 332 us a call, reverse KL 194
+// -> 181.  For a P that L2 holds, one target, or three and more, whose blocks
+// share what one of them has read, the kernel above is the better one (177 x
+// 177 cells, two targets: 83 us against 108; 300 x 300, three: 470 against 539
+// with a pair and one).
+template <int FAM>
+__global__ void __launch_bounds__(512, 1) two_pass_pair_kernel(const float *__restrict__ P, int64_t n_v,
                                                                int64_t k_pad, const float *__restrict__ sP,
                                                                const float *__restrict__ sL,
                                                                const float *__restrict__ sE,
-                                                               const float *__restrict__ sF, int a0, FdParams q,
+                                                               const float *__restrict__ sF, FdParams q,
                                                                float *__restrict__ out) {
-    constexpr int U = TT == 1 ? 8 : 4;       // float4 per lane and buffer: 4 KB per warp and target in flight
+    constexpr int TT = 2, U = 4;             // targets; float4 per lane and buffer
     extern __shared__ __align__(16) float fsm[];
     __shared__ float tab[2 * kLogTab];
     __shared__ unsigned char tz[kMaxGroups];      // a target's group of entries (32 float4) holds a 0
-    // the staged rows zero-padded to whole groups of 32 float4 (two_pass_pitch):
+    // the staged rows zero-padded to whole groups of 32 float4 (two_pass_pair_pitch):
     // every lane of a group reads its target entries without a test
-    const int64_t kp = two_pass_pitch(k_pad);
-    const int a = a0 + blockIdx.y * TT;
+    const int64_t kp = two_pass_pair_pitch(k_pad);
+    const int a = 0;
     for (int i = threadIdx.x; i < kMaxGroups; i += blockDim.x) tz[i] = 0;
     __syncthreads();
     for (int i = 0; i < TT; ++i)
@@ -398,7 +542,7 @@ __global__ void __launch_bounds__(256 * TT, 2 / TT) two_pass_kernel(const float 
             // past the row's end P and the padded target row are 0, and so is the term
             const float4 p4 = tg[4 * i * kv + c], f4 = tg[(4 * i + 3) * kv + c], e4 = tg[(4 * i + 2) * kv + c];
             if (FAM == kAlpha) {
-                alpha_fast4<decltype(zeros)::value>(x, pe, p4, f4, e4, q, sums[i]);
+                alpha_pair4<decltype(zeros)::value>(x, pe, p4, f4, e4, q, sums[i]);
             } else {
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
@@ -519,38 +663,30 @@ dd_status launch_fdiv(const float *P, int64_t n_v, int64_t k_pad, const float4 *
     if ((family == DD_DIV_KL_REVERSE && !LP) || alpha_fast) {
         // two passes (hardware mantissa logs, then the table form near the target)
         const float *sF = sE + (int64_t)T * k_pad;
-        const size_t smem4 = 4 * (size_t)two_pass_pitch(k_pad) * sizeof(float);
-        // pairs of targets while two targets' rows fit beside the log table
-        // (k up to about 6,900), a last odd one by itself
-        const int pairs = 2 * smem4 <= 220 * 1024 ? T / 2 : 0;
-        auto pass = [&](auto kern, int a0, int count, int tt) {
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(tt * smem4));
+        // two targets of a P of 256 MB or more: both in one pass
+        const size_t smem_pair = 8 * (size_t)two_pass_pair_pitch(k_pad) * sizeof(float);
+        if (T == 2 && n_v * k_pad * (int64_t)sizeof(float) >= (int64_t)256 << 20 && smem_pair <= 200 * 1024) {
+            auto kern = family == DD_DIV_ALPHA ? two_pass_pair_kernel<kAlpha> : two_pass_pair_kernel<kKlRev>;
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_pair);
+            const int64_t blocks = std::min<int64_t>(sms, (n_v + 15) / 16);
+            KMark km_("two_pass_kernel", s);
+            kern<<<(unsigned)blocks, 512, smem_pair, s>>>(P, n_v, k_pad, sP, sL, sE, sF, q, out);
+            return DD_OK;
+        }
+        const size_t smem4 =
+            4 * (size_t)(family == DD_DIV_ALPHA ? two_pass_pitch(k_pad) : k_pad) * sizeof(float);
+        if (smem4 <= 200 * 1024) {
+            auto kern = family == DD_DIV_ALPHA ? two_pass_kernel<kAlpha> : two_pass_kernel<kKlRev>;
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem4);
             int per_sm = 0;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256 * tt, tt * smem4);
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem4);
             if (per_sm < 1) per_sm = 1;
-            int64_t gx = (int64_t)sms * per_sm / count;
-            const int64_t rows_blocks = (n_v + 8 * tt - 1) / (8 * tt);
+            int64_t gx = (int64_t)sms * per_sm / (T > 0 ? T : 1);
+            const int64_t rows_blocks = (n_v + 7) / 8;
             if (gx < 1) gx = 1;
             if (gx > rows_blocks) gx = rows_blocks;
             KMark km_("two_pass_kernel", s);
-            kern<<<dim3((unsigned)gx, (unsigned)count), 256 * tt, tt * smem4, s>>>(P, n_v, k_pad, sP, sL, sE, sF, a0,
-                                                                                  q, out);
-        };
-        const bool alpha = family == DD_DIV_ALPHA;
-        // (the exact form throughout beyond, alpha in whole units of 1,024 columns)
-        if ((alpha ? 16 * (size_t)((k_pad + 1023) / 1024 * 1024) : smem4) <= 200 * 1024) {
-            if (pairs > 0) {
-                if (alpha)
-                    pass(two_pass_kernel<kAlpha, 2>, 0, pairs, 2);
-                else
-                    pass(two_pass_kernel<kKlRev, 2>, 0, pairs, 2);
-            }
-            if (T > 2 * pairs) {
-                if (alpha)
-                    pass(two_pass_kernel<kAlpha, 1>, 2 * pairs, T - 2 * pairs, 1);
-                else
-                    pass(two_pass_kernel<kKlRev, 1>, 2 * pairs, T - 2 * pairs, 1);
-            }
+            kern<<<dim3((unsigned)gx, (unsigned)T), 256, smem4, s>>>(P, n_v, k_pad, sP, sL, sE, sF, q, out);
             return DD_OK;
         }
     }

@@ -106,3 +106,27 @@ def test_fdiv_end_to_end_grid140(env):
         dd.dd_divergence(ctx, mid, t, const, prm, host)
         assert field_error(host[0], fdiv.field(P, P[t[0]], fam, prm)) <= TOL_FP32
     dd.dd_unload_mesh(ctx, mid)
+
+
+@pytest.mark.parametrize("const,prm", [("DD_DIV_ALPHA", 0.5), ("DD_DIV_ALPHA", 3.0), ("DD_DIV_KL_REVERSE", 0.0)])
+def test_two_targets_of_a_large_map(env, const, prm):
+    """Two targets of a P beyond 256 MB share one pass: the fields of two
+    single calls (the same terms in the same order; boundary rows, whose
+    entries are 0, among them)."""
+    dd, ctx = env
+    wl = workloads.small_grid(260, 4, T=2, S=1, seed=260)
+    mid = load(dd, ctx, wl.mesh)
+    dd.dd_poisson_kernel(ctx, mid, 1e-15, 20000)
+    info = dd.dd_mesh_info(ctx, mid)
+    assert info["n_v"] * info["k_pad"] * 4 >= 256 << 20
+    targets = [int(t) for t in wl.targets[:2]]
+    two = torch.empty((2, wl.mesh.n_v), dtype=torch.float32, device="cuda")
+    one = torch.empty((2, wl.mesh.n_v), dtype=torch.float32, device="cuda")
+    dd.dd_divergence(ctx, mid, targets, getattr(dd, const), prm, two)
+    for a in range(2):
+        dd.dd_divergence(ctx, mid, targets[a:a + 1], getattr(dd, const), prm, one[a:a + 1])
+    dd.dd_sync(ctx)
+    got, ref = two.cpu().numpy(), one.cpu().numpy()
+    assert np.array_equal(np.isfinite(got), np.isfinite(ref)) and got[0, targets[0]] == 0.0
+    assert field_error(got[np.isfinite(ref)], ref[np.isfinite(ref)]) <= TOL_FP32
+    dd.dd_unload_mesh(ctx, mid)
