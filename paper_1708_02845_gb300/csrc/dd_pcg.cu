@@ -126,11 +126,24 @@ __global__ void alpha_kernel(int64_t nrb, int64_t kc, const double *__restrict__
     if (threadIdx.y == 0 && c < kc) alpha[c] = (!done[c] && pAp > 0.0) ? rz[c] / pAp : 0.0;
 }
 
-// (nrz, nrb: how many partials part_rz and part_rr hold a column)
+// The exponents that a column's numbers gain on their way into the V-cycle and
+// lose on their way out (df_split, widen).  The residual's norm then lies
+// near 2^60: a factor 2^-150 below it is kept and one of 2^58 above it fits,
+// whatever the size of the column's right-hand side and however far the column
+// has converged.
+constexpr int kShiftTop = 60, kShiftMin = -452, kShiftMax = 572;
+// from the squared norm (0, subnormal and infinite numbers included)
+__device__ __forceinline__ int shift_of_square(double rr) {
+    return kShiftTop - ((((int)((unsigned long long)__double_as_longlong(rr) >> 52) & 0x7ff) - 1023) >> 1);
+}
+
+// (nrz, nrb: how many partials part_rz and part_rr hold a column; shift: null, or
+// the columns' exponents for the next residual)
 __global__ void beta_kernel(int64_t nrz, int64_t nrb, int64_t kc, const double *__restrict__ part_rz,
                             const double *__restrict__ part_rr, const double *__restrict__ bnorm,
                             double *__restrict__ rz, const int *__restrict__ done,
-                            double *__restrict__ beta, unsigned long long *__restrict__ maxres) {
+                            double *__restrict__ beta, unsigned long long *__restrict__ maxres,
+                            int *__restrict__ shift) {
     __shared__ double sh[kSumRows][33];
     const int64_t c = (int64_t)blockIdx.x * 32 + threadIdx.x;
     double rz_new = column_sum(part_rz, nrz, kc, c, sh);
@@ -143,19 +156,29 @@ __global__ void beta_kernel(int64_t nrz, int64_t nrb, int64_t kc, const double *
         const int d = done[c];
         beta[c] = (!d && rz[c] > 0.0) ? rz_new / rz[c] : 0.0;
         rz[c] = rz_new;
+        if (shift) shift[c] = shift_of_square(rr);
         atomicMax(maxres, (unsigned long long)__double_as_longlong(res));
     }
 }
 
-// R = L_IB[:, c0:c0+kc] (scatter of the edge weights to boundary columns)
+// R = L_IB[:, c0:c0+kc] (scatter of the edge weights to boundary columns); top:
+// null, or the largest biased exponent of each column's entries (0 before)
 __global__ void scatter_rhs_kernel(int64_t n_rb, const int32_t *__restrict__ rb_row,
                                    const int32_t *__restrict__ rb_col, const double *__restrict__ rb_val,
-                                   int64_t c0, int64_t ncols, int64_t ld, double *__restrict__ R) {
+                                   int64_t c0, int64_t ncols, int64_t ld, double *__restrict__ R,
+                                   int *__restrict__ top) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_rb) return;
     int64_t c = (int64_t)rb_col[i] - c0;
     if (c < 0 || c >= ncols) return;
     R[(int64_t)rb_row[i] * ld + c] += rb_val[i];   // one edge per (row, column): no race
+    if (top) atomicMax(top + c, (int)((unsigned long long)__double_as_longlong(rb_val[i]) >> 52) & 0x7ff);
+}
+
+// the right-hand side's exponents (beta_kernel) from the largest biased one, in place
+__global__ void first_shift_kernel(int64_t kc, int *__restrict__ shift) {
+    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (c < kc) shift[c] = max(kShiftMin, min(kShiftMax, kShiftTop + 1023 - shift[c]));
 }
 
 __global__ void dinv_kernel(int64_t m, const double *__restrict__ diag, double *__restrict__ dinv) {
@@ -275,15 +298,19 @@ __device__ __forceinline__ float4 df_pack(const Df2 &v) {
     return r;
 }
 
-// A double as an unevaluated sum of two floats, by integer operations on its
-// bits (this part converts FP64 no faster than it multiplies it): the leading
-// 24 bits of the significand, and the 29 that follow as an integer scaled.
-// Magnitudes outside 2^-90 .. 2^120 come out as 0 or as 2^120 (residuals of
-// the solve start below 2^30 and stop 1e-15 lower).
-__device__ __forceinline__ void df_split(double d, float &hi, float &lo) {
+// A double times 2^shift as an unevaluated sum of two floats, by integer
+// operations on its bits (this part converts FP64 no faster than it multiplies
+// it): the leading 24 bits of the significand, and the 29 that follow as an
+// integer scaled.  Magnitudes outside 2^-90 .. 2^120 come out as 0 or as 2^120:
+// the column's exponent (shift_of_square) keeps what matters between them.  A
+// residual is relative to its own right-hand side, which may be 1e-17 (a
+// corner that meets the interior by a right-angled cell's diagonal alone,
+// rotated) or far above 1, and falls by 1e-15 and more; without the shift
+// such columns stopped at 1e-9 of theirs.
+__device__ __forceinline__ void df_split(double d, int shift, float &hi, float &lo) {
     const unsigned long long u = (unsigned long long)__double_as_longlong(d);
     const unsigned sign = (unsigned)(u >> 32) & 0x80000000u;
-    const int e = (int)((u >> 52) & 0x7ff) - 1023;
+    const int e = (int)((u >> 52) & 0x7ff) - 1023 + shift;
     const int ec = min(e, 120);
     const unsigned top = (unsigned)(u >> 29) & 0x7fffffu;
     const float l = (float)(int)((unsigned)u & 0x1fffffffu);               // < 2^29
@@ -292,11 +319,11 @@ __device__ __forceinline__ void df_split(double d, float &hi, float &lo) {
     hi = tiny ? 0.0f : __uint_as_float(sign | ((unsigned)(ec + 127) << 23) | top);
     lo = tiny ? 0.0f : __uint_as_float(sign ^ __float_as_uint(l * scale * 0x1p-23f));
 }
-// float to double by its bits (subnormals as 0)
-__device__ __forceinline__ double widen(float f) {
+// float times 2^-shift to double by its bits (subnormals as 0)
+__device__ __forceinline__ double widen(float f, int shift) {
     const unsigned u = __float_as_uint(f);
     const unsigned m = u & 0x7fffffffu;
-    const unsigned h = m < 0x00800000u ? 0u : (m >> 3) + (896u << 20);
+    const unsigned h = m < 0x00800000u ? 0u : (m >> 3) + ((unsigned)(896 - shift) << 20);
     return __hiloint2double((int)((u & 0x80000000u) | h), (int)(m < 0x00800000u ? 0u : m << 29));
 }
 
@@ -326,20 +353,22 @@ __global__ void __launch_bounds__(kBandPairs *kBandRows, 2)
     }
 }
 
-// Z = G B + Q E (E: rows of the next level).  FINE: Z in FP64, with partial
-// column sums of R . Z; else Z in pairs like B.
+// Z = G B + Q E (E: rows of the next level).  FINE: Z in FP64 without the
+// columns' exponents, with partial column sums of R . Z; else Z in pairs like B.
 template <bool FINE>
 __global__ void __launch_bounds__(kBandPairs *kBandRows, 2)
     df_up_kernel(int64_t rows, int64_t kp, const int32_t *__restrict__ goff, const int32_t *__restrict__ gcol,
                  const float2 *__restrict__ gval, const int32_t *__restrict__ qoff, const int32_t *__restrict__ qcol,
                  const float2 *__restrict__ qval, const float4 *__restrict__ B, const float4 *__restrict__ E,
-                 const double2 *__restrict__ R, void *__restrict__ Z, double2 *__restrict__ part, int band) {
+                 const double2 *__restrict__ R, const int2 *__restrict__ shift, void *__restrict__ Z,
+                 double2 *__restrict__ part, int band) {
     __shared__ double2 sum[FINE ? kBandRows : 1][kBandPairs];
     const int64_t c = (int64_t)blockIdx.y * kBandPairs + threadIdx.x;
     const int64_t r0 = (int64_t)blockIdx.x * band;
     const int64_t r1 = r0 + band < rows ? r0 + band : rows;
     double d0 = 0.0, d1 = 0.0;
     if (c < kp) {
+        const int2 sh = FINE ? shift[c] : make_int2(0, 0);
         for (int64_t r = r0 + threadIdx.y; r < r1; r += kBandRows) {
             f2_t s = 0ULL, cc = 0ULL;
 #pragma unroll 4
@@ -351,7 +380,7 @@ __global__ void __launch_bounds__(kBandPairs *kBandRows, 2)
             const float4 z = df_pack(df_norm(s, cc));
             if (FINE) {
                 const double2 v = R[r * kp + c];
-                const double z0 = widen(z.x) + widen(z.z), z1 = widen(z.y) + widen(z.w);
+                const double z0 = widen(z.x, sh.x) + widen(z.z, sh.x), z1 = widen(z.y, sh.y) + widen(z.w, sh.y);
                 static_cast<double2 *>(Z)[r * kp + c] = make_double2(z0, z1);
                 d0 += v.x * z0;
                 d1 += v.y * z1;
@@ -387,18 +416,19 @@ __global__ void __launch_bounds__(kPairs) df_coarse_kernel(int64_t n, int64_t kp
 
 // a block as pairs (the first V-cycle's right-hand side), with partial column sums of R . R
 __global__ void __launch_bounds__(kPairs) df_first_kernel(int64_t rows, int64_t kp, const double2 *__restrict__ R,
-                                                          float4 *__restrict__ B, double2 *__restrict__ part,
+                                                          const int2 *__restrict__ shift, float4 *__restrict__ B, double2 *__restrict__ part,
                                                           int rpb) {
     const int64_t c = (int64_t)blockIdx.y * kPairs + threadIdx.x;
     if (c >= kp) return;
     const int64_t r0 = (int64_t)blockIdx.x * rpb;
     const int64_t r1 = r0 + rpb < rows ? r0 + rpb : rows;
+    const int2 sh = shift[c];
     double d0 = 0.0, d1 = 0.0;
     for (int64_t r = r0; r < r1; ++r) {
         const double2 v = R[r * kp + c];
         float4 b;
-        df_split(v.x, b.x, b.z);
-        df_split(v.y, b.y, b.w);
+        df_split(v.x, sh.x, b.x, b.z);
+        df_split(v.y, sh.y, b.y, b.w);
         B[r * kp + c] = b;
         d0 += v.x * v.x;
         d1 += v.y * v.y;
@@ -411,13 +441,14 @@ __global__ void __launch_bounds__(kPairs) df_first_kernel(int64_t rows, int64_t 
 __global__ void __launch_bounds__(kPairs) update_r_kernel(int64_t rows, int64_t kp,
                                                           const double2 *__restrict__ alpha,
                                                           double2 *__restrict__ R, const double2 *__restrict__ AP,
-                                                          float4 *__restrict__ B, double2 *__restrict__ part,
+                                                          const int2 *__restrict__ shift, float4 *__restrict__ B, double2 *__restrict__ part,
                                                           int rpb) {
     const int64_t c = (int64_t)blockIdx.y * kPairs + threadIdx.x;
     if (c >= kp) return;
     const int64_t r0 = (int64_t)blockIdx.x * rpb;
     const int64_t r1 = r0 + rpb < rows ? r0 + rpb : rows;
     const double2 a = alpha[c];
+    const int2 sh = shift[c];
     double d0 = 0.0, d1 = 0.0;
 #pragma unroll 2
     for (int64_t r = r0; r < r1; ++r) {
@@ -428,8 +459,8 @@ __global__ void __launch_bounds__(kPairs) update_r_kernel(int64_t rows, int64_t 
         v.y -= a.y * w.y;
         R[i] = v;
         float4 b;
-        df_split(v.x, b.x, b.z);
-        df_split(v.y, b.y, b.w);
+        df_split(v.x, sh.x, b.x, b.z);
+        df_split(v.y, sh.y, b.y, b.w);
         B[i] = b;
         d0 += v.x * v.x;
         d1 += v.y * v.y;
@@ -674,7 +705,7 @@ dd_status run_pcg_amg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s,
     const size_t o_p0 = take((size_t)std::max(nrb, nbands) * kc * sizeof(double)), o_p1 = take((size_t)nrb * kc * sizeof(double));
     const size_t o_al = take(kc * sizeof(double)), o_be = take(kc * sizeof(double)), o_rz = take(kc * sizeof(double));
     const size_t o_bn = take(kc * sizeof(double)), o_dn = take(kc * sizeof(int));
-    const size_t o_mr = take(sizeof(unsigned long long));
+    const size_t o_mr = take(sizeof(unsigned long long)), o_sh = take(kc * sizeof(int));
     std::vector<uint8_t> host(filled);
     for (const Plan &q : plans) {
         int32_t *off = reinterpret_cast<int32_t *>(host.data() + q.off);
@@ -718,7 +749,8 @@ dd_status run_pcg_amg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s,
     auto at = [&](size_t o) { return reinterpret_cast<double *>(ws + o); };
     double *X = fine[0], *R = fine[1], *Z = fine[2], *Pd = fine[3], *AP = fine[4];
     double *part0 = at(o_p0), *part1 = at(o_p1), *alpha = at(o_al), *beta = at(o_be), *rz = at(o_rz), *bnorm = at(o_bn);
-    int *done = reinterpret_cast<int *>(ws + o_dn);
+    int *done = reinterpret_cast<int *>(ws + o_dn), *shift = reinterpret_cast<int *>(ws + o_sh);
+    const int2 *shift2 = reinterpret_cast<const int2 *>(shift);
     unsigned long long *maxres = reinterpret_cast<unsigned long long *>(ws + o_mr);
     auto lb = [&](int l) {
         return l == 0 ? reinterpret_cast<float4 *>(fine[5]) : reinterpret_cast<float4 *>(ws + o_b[l]);
@@ -748,12 +780,12 @@ dd_status run_pcg_amg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s,
             const int64_t n = H.levels[l].A.rows;
             if (l > 0)
                 df_up_kernel<false><<<bands(l), bb, 0, s>>>(n, kp, dG[l].off, dG[l].col, dG[l].val, dQ[l].off,
-                                                            dQ[l].col, dQ[l].val, lb(l), lx(l + 1), nullptr, lx(l),
-                                                            nullptr, band[l]);
+                                                            dQ[l].col, dQ[l].val, lb(l), lx(l + 1), nullptr, nullptr,
+                                                            lx(l), nullptr, band[l]);
             else
                 df_up_kernel<true><<<bands(l), bb, 0, s>>>(n, kp, dG[l].off, dG[l].col, dG[l].val, dQ[l].off,
-                                                           dQ[l].col, dQ[l].val, lb(l), lx(l + 1), d2(R), Z, d2(part0),
-                                                           band[l]);
+                                                           dQ[l].col, dQ[l].val, lb(l), lx(l + 1), d2(R), shift2, Z,
+                                                           d2(part0), band[l]);
         }
     };
 
@@ -765,10 +797,11 @@ dd_status run_pcg_amg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s,
     for (int64_t c0 = 0; c0 < k && st == DD_OK; c0 += kc) {
         const int64_t kcur = (k - c0) < kc ? (k - c0) : kc;
         cudaMemsetAsync(X, 0, vec, s);
+        cudaMemsetAsync(shift, 0, kc * sizeof(int), s);
         cudaMemsetAsync(R, 0, vec, s);
         if (M.n_rb > 0)
             scatter_rhs_kernel<<<(unsigned)((M.n_rb + 255) / 256), 256, 0, s>>>(M.n_rb, M.rb_row, M.rb_col, M.rb_val,
-                                                                                c0, kcur, kc, R);
+                                                                                c0, kcur, kc, R, shift);
         if (nl == 1) {   // the whole problem is the coarsest level: one exact solve
             coarse_solve_kernel<<<dim3((unsigned)((kc + 127) / 128), (unsigned)m), 128, 0, s>>>(m, kc, at(o_ainv), R, X);
             pack_chunk_kernel<<<dim3((unsigned)nrb, (unsigned)((kcur + kColsPerBlock - 1) / kColsPerBlock)),
@@ -776,7 +809,8 @@ dd_status run_pcg_amg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s,
             iters_max = std::max(iters_max, 1);
             continue;
         }
-        df_first_kernel<<<grid2(m, rpb0), kPairs, 0, s>>>(m, kp, d2(R), lb(0), d2(part1), rpb0);
+        first_shift_kernel<<<(unsigned)((kc + 255) / 256), 256, 0, s>>>(kc, shift);
+        df_first_kernel<<<grid2(m, rpb0), kPairs, 0, s>>>(m, kp, d2(R), shift2, lb(0), d2(part1), rpb0);
         vcycle();
         amg_init_scalars_kernel<<<gc, bc, 0, s>>>(nbands, nrb, kc, part0, part1, rz, bnorm, done);
         cudaMemcpyAsync(Pd, Z, vec, cudaMemcpyDeviceToDevice, s);
@@ -785,10 +819,11 @@ dd_status run_pcg_amg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s,
         for (it = 1; it <= max_iter; ++it) {
             spmm_dot_kernel<<<g0, kColsPerBlock, 0, s>>>(m, kc, M.a_off, M.a_col, M.a_val, Pd, AP, part0, rpb0);
             alpha_kernel<<<gc, bc, 0, s>>>(nrb, kc, part0, rz, done, alpha);
-            update_r_kernel<<<grid2(m, rpb0), kPairs, 0, s>>>(m, kp, d2(alpha), d2(R), d2(AP), lb(0), d2(part1), rpb0);
+            update_r_kernel<<<grid2(m, rpb0), kPairs, 0, s>>>(m, kp, d2(alpha), d2(R), d2(AP), shift2, lb(0), d2(part1),
+                                                              rpb0);
             vcycle();
             cudaMemsetAsync(maxres, 0, sizeof(unsigned long long), s);
-            beta_kernel<<<gc, bc, 0, s>>>(nbands, nrb, kc, part0, part1, bnorm, rz, done, beta, maxres);
+            beta_kernel<<<gc, bc, 0, s>>>(nbands, nrb, kc, part0, part1, bnorm, rz, done, beta, maxres, shift);
             update_xp_kernel<<<grid2(m, rpb0), kPairs, 0, s>>>(m, kp, d2(alpha), d2(beta), d2(Z), d2(X), d2(Pd), rpb0);
             if (it % check_every == 0 || it == max_iter) {
                 unsigned long long bits = 0;
@@ -931,7 +966,7 @@ dd_status run_pcg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s, int
         cudaMemsetAsync(w.R, 0, vec * sizeof(double), s);
         if (M.n_rb > 0)
             scatter_rhs_kernel<<<(unsigned)((M.n_rb + 255) / 256), 256, 0, s>>>(M.n_rb, M.rb_row, M.rb_col,
-                                                                                M.rb_val, c0, kcur, kc, w.R);
+                                                                                M.rb_val, c0, kcur, kc, w.R, nullptr);
         init_p_kernel<<<g2, kColsPerBlock, 0, s>>>(m, kc, w.dinv, w.R, w.Pd, w.part0, w.part1, rpb);
         init_scalars_kernel<<<gc, bc, 0, s>>>(w.nrb, kc, w.part0, w.part1, w.rz, w.bnorm, w.done);
         int32_t it = 0;
@@ -943,7 +978,7 @@ dd_status run_pcg(DevMesh &M, double rtol, int32_t max_iter, cudaStream_t s, int
                                                           w.part1, rpb);
             cudaMemsetAsync(w.maxres, 0, sizeof(unsigned long long), s);
             beta_kernel<<<gc, bc, 0, s>>>(w.nrb, w.nrb, kc, w.part0, w.part1, w.bnorm, w.rz, w.done, w.beta,
-                                          w.maxres);
+                                          w.maxres, nullptr);
             update_p_kernel<<<g2, kColsPerBlock, 0, s>>>(m, kc, w.beta, w.dinv, w.R, w.Pd, rpb);
             if (it % check_every == 0 || it == max_iter) {
                 unsigned long long bits = 0;
