@@ -77,15 +77,15 @@ enum { DD_F_KL = 1, DD_F_TV = 2, DD_F_KLT = 4 };
  *                 more than two targets on a map with n_v k_pad >= 2^20 (and
  *                 without dd_log_poisson_kernel) KL is formed on the tensor
  *                 cores from BF16 slices of P and log2 P that sum exactly, as
- *                 e_x - sum_b P[x,b] log P[t,b]; it is as accurate (against
- *                 64 bits two to three times more, above 0.25), and the
- *                 pairs below 0.07 are recomputed in the exact form.  The
- *                 slices (8 bytes an entry of P) are built on the first such
+ *                 e_x - sum_b P[x,b] log P[t,b]; against 64 bits it is two to
+ *                 three times as accurate, and the pairs below 0.07 are
+ *                 recomputed in the exact form.  The slices (8 bytes an entry
+ *                 of P, rounded up to whole tiles) are built on the first such
  *                 call, which synchronizes, and kept with the map; a P with
  *                 entries outside [0, 2] or row sums above 1.01, or no room
- *                 for them, keeps the FP32 sums.  In all cases the rows near the target (x = t among them) come
- *                 from the exact form and every value keeps 1e-5 relative
- *                 accuracy.
+ *                 for them, keeps the FP32 sums.  In all cases the rows near
+ *                 the target (x = t among them) come from the exact form and
+ *                 every value keeps 1e-5 relative accuracy.
  *  DD_PREC_BF16X3 KL cross term sum_b P[x,b] log P[t,b] as a tensor-core GEMM
  *                 of split BF16 hi/lo operands (hi*hi + hi*lo + lo*hi, FP32
  *                 accumulation); TV and KLT are always FP32

@@ -1381,7 +1381,7 @@ dd_status dd_query_batch(dd_ctx *ctx, int32_t n_items, const int32_t *mesh_ids, 
         int32_t *dcounter = reinterpret_cast<int32_t *>(dmeta + o_counter);
         const BatchItem *ditems_pipe = reinterpret_cast<const BatchItem *>(dmeta + o_items_pipe);
         const BatchKlMma kl{reinterpret_cast<const BatchItem *>(dmeta + o_items_kl), kl_wide, (int32_t)order_kl.size(),
-                            max_T, ctx->d_err, (f_mask & DD_F_TV) != 0};
+                            max_T, max_k, ctx->d_err, (f_mask & DD_F_TV) != 0};
         const BatchKlMma *klp = mma ? &kl : nullptr;
         auto staged = [&]() {
             launch_batch_fields(dprobs, (int32_t)n_items, reinterpret_cast<const BatchItem *>(dmeta + o_items),

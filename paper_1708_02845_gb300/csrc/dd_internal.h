@@ -180,6 +180,7 @@ void launch_batch_stage(const BatchProblem *d_probs, const int32_t *d_tprob, con
 struct BatchKlMma {
     const BatchItem *items;      // 128 rows x ktile targets: first those of problems with ktile 128
     int32_t n_wide, n_items, max_T;
+    int64_t max_k;               // largest k_pad of the problems
     int *err;
     bool tv;                     // TV is asked for
 };

@@ -13,23 +13,34 @@
 // multiples of q = 2^-7 of their largest entry's power of two, the remainder
 // to multiples of 2^-9 q, and so on (four slices), and the target's log2 P
 // the same way (three slices; entries below -32 keep their own BF16 grid, so
-// that one near-empty column does not coarsen its chunk).  Slices are integers
+// that one near-empty column does not coarsen its chunk).  The logs are taken
+// from a whole number in the middle of their chunk's, c, which counts with the
+// chunk's sum of P:  sum_b P l = sum_b P (l - c) + c sum_b P.  Along a boundary
+// log2 P varies little, so l - c is several times smaller than l, and so is
+// what three slices of it leave.  The second term is summed like the first, by
+// columns of their own behind the map's: the chunks' sums of P, exact, on the
+// rows' side and c on the targets'.  Slices are integers
 // of at most 2^8 times their grid, so a product of two leading slices is an
 // integer of at most 2^16 units and a chunk's 64 of them sum exactly in the 24
 // bits of an FP32 accumulator.  Nine products are kept,
 //   A = p1 l1 (exact),   B = (p4 l1 + p3 l2 + p2 l3) + (p1 l3 + p2 l2 + p3 l1) + (p1 l2 + p2 l1)
 // (each bracket 2^-9 of the next, the smallest first), in two accumulators, or
-// one a bracket (up to 64 targets); what is dropped is about
-// 2^-33 of the chunk's largest entry times the largest log.  After every chunk
+// one a bracket (up to 64 targets); what is dropped is 2^-36 of the chunk's
+// largest entry times the logs, and P times what the three slices leave of
+// l - c: at most 2^-26 of its largest power of two.  After every chunk
 // A is split at multiples of 2^-15: the upper part goes into a total of
 // such multiples (exact below 2^9), the rest and B into a second total.
 // e_x is summed once per mesh in pairs of floats and kept in the same two parts.
 //
-// Against 64 bits (KL above 0.07, three obstacle grids of 60 to 140 cells a
-// side) the relative error is 3e-8 .. 7e-8 in the root mean square and at most
-// 7.3e-7, against 1.1e-7 .. 2.5e-7 and 1.4e-6 for the FP32 sums of the tile
-// kernels; the pairs below kMmaExactBelow are recomputed in the exact form as
-// there.
+// Against 64 bits (KL above 0.07, solved kernels of obstacle grids of 64 to 201
+// cells a side) the relative error is 3.5e-8 .. 6.2e-8 in the root mean square
+// of every range of KL and at most 3.6e-7, against 6.9e-8 .. 1.7e-7 and 1.4e-6
+// for the FP32 sums of the tile kernels and their recompute below 0.25 (slices
+// of l itself: up to 1.6e-7 below 0.25).  For target rows of equal entries,
+// where what the slices leave does not average out: below 8e-8, against 1.6e-7
+// (4.4e-7).  The pairs below kMmaExactBelow are recomputed in the exact form as
+// there.  The extra columns cost 0.3 % of a call with a chunk more (grid450,
+// 1,024 targets: 54.95 -> 55.13 ms) and up to 1 % of small ones.
 //
 // Kernel: persistent, one CTA per SM walks 128-row x N-target output tiles.
 // The operands lie in global memory chunk by chunk in the shared-memory image
@@ -42,13 +53,14 @@
 // Measured: grid450, 1,024 targets: 7.8 ms (N = 128; 14.0 TFLOP issued, 1,790
 // TFLOP/s = 93 % of the measured burst rate of 1,931), with the TV tile pass
 // (45.3 ms) and a recompute of fewer pairs (1.6 against 4.1 ms) in place of
-// the 94.5 ms KL+TV tile pass: a call 98.9 -> 54.9 ms.  grid140, 64 targets:
+// the 94.5 ms KL+TV tile pass: a call 98.9 -> 55.1 ms.  grid140, 64 targets:
 // 34 us (N = 64; the slices' 131 MB from memory bound it), a call 321 -> 181
 // us.  KL alone, 201 x 201 cells, 7 targets: a call 228 -> 104 us.
 #include <cuda_bf16.h>
 
 #include <algorithm>
 #include <cfloat>
+#include <climits>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -64,6 +76,7 @@ constexpr int BM = 128, BK = 64;              // rows of a tile, columns of a ch
 constexpr int NSA = 4, NSB = 3;               // slices of P and of log2 P
 constexpr int ROW_B = BK * 2;                 // bytes of a slice row in a chunk
 constexpr int A_BYTES = NSA * BM * ROW_B;     // 64 KB
+constexpr int64_t kMaxColumns = 1 << 17;
 constexpr float kLn2 = 0.693147180559945309f;
 constexpr float kSplit = 384.0f;              // 1.5 * 2^8: adding it rounds |A| < 128 to multiples of 2^-15
 
@@ -389,23 +402,52 @@ __device__ __forceinline__ void pair_add(float &s, float &c, float a) {
     s = t;
 }
 
+// Columns: the k_pad of P in chunks of BK, then one for each of those chunks
+// (its sum of P; its c), then zeros to whole chunks.
+__host__ __device__ constexpr int data_chunks(int64_t k_pad) { return (int)((k_pad + BK - 1) / BK); }
+__host__ __device__ constexpr int all_chunks(int64_t k_pad) {
+    return (int)((k_pad + data_chunks(k_pad) + BK - 1) / BK);
+}
+
+// a + b = s + t
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &t) {
+    s = __fadd_rn(a, b);
+    const float v = __fsub_rn(s, a);
+    t = __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(b, v));
+}
+
+// the grid of a chunk of P: 2^-7 of its largest entry's power of two (chunks below 2^-87: of that)
+__device__ __forceinline__ int row_grid(float x, float y) {
+    // entries are not negative: their bit patterns order as the numbers do
+    const unsigned mx = __reduce_max_sync(0xffffffffu, max(__float_as_uint(x), __float_as_uint(y)));
+    return min(max((int)(mx >> 23), 40), 200) - 7;
+}
+
 // The slices of P's rows and e_x, one warp per row (rows past n_v: zeros), two
 // columns a lane.  Rows that the exactness argument does not cover (an entry
 // that is negative, infinite or NaN, or a sum above 1.01) raise *bad.
 __global__ void __launch_bounds__(256) kl_rows_kernel(const float *__restrict__ P, int64_t n_v, int64_t n_pad,
-                                                      int64_t k_pad, int32_t nch, uint8_t *__restrict__ A,
+                                                      int64_t k_pad, uint8_t *__restrict__ A,
                                                       float2 *__restrict__ ex, int *__restrict__ bad) {
     __shared__ Log2Tab tab;
+    extern __shared__ float2 sums[];     // [8][chunks of P]: a row's sums of P, pairs
     build_log2_table(tab);
     __syncthreads();
     const int lane = threadIdx.x & 31;
+    const int nb = data_chunks(k_pad), nch = all_chunks(k_pad), whole = (int)(k_pad / BK);
+    float2 *rs = sums + (threadIdx.x >> 5) * nb;
     const int64_t nw = (int64_t)gridDim.x * 8;
     for (int64_t x = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); x < n_pad; x += nw) {
         float es = 0.0f, ec = 0.0f;      // this lane's part of e_x, a pair
         float sum = 0.0f;
         bool wrong = false;
         uint8_t *img = A + (x / BM) * nch * A_BYTES + image_at((int)(x % BM), 2 * lane);
-        for (int c = 0; c < nch; ++c, img += A_BYTES) {
+        auto store = [&](int s, float rx, float ry) {
+            *reinterpret_cast<__nv_bfloat162 *>(img + s * BM * ROW_B) =
+                __nv_bfloat162(__float2bfloat16_rn(rx), __float2bfloat16_rn(ry));
+        };
+        float2 last = make_float2(0.f, 0.f);      // the entries of a last chunk that is not whole
+        for (int c = 0; c < nb; ++c) {
             const int64_t b = (int64_t)c * BK + 2 * lane;
             float2 p = make_float2(0.f, 0.f);
             if (x < n_v && b < k_pad) p = *reinterpret_cast<const float2 *>(P + x * k_pad + b);   // k_pad is a multiple of 4
@@ -421,18 +463,45 @@ __global__ void __launch_bounds__(256) kl_rows_kernel(const float *__restrict__ 
                     pair_add(es, ec, a);
                 }
             }
-            // entries are not negative: their bit patterns order as the numbers do
-            unsigned mx = __reduce_max_sync(0xffffffffu, max(__float_as_uint(p.x), __float_as_uint(p.y)));
-            // grid 2^-7 of the largest entry's power of two (chunks below 2^-87: of that)
-            const int eb = min(max((int)(mx >> 23), 40), 200);
-            float q = __int_as_float((eb - 7) << 23), iq = __int_as_float((254 - (eb - 7)) << 23);
+            last = p;
+            const int g = row_grid(p.x, p.y);
+            float q = __int_as_float(g << 23), iq = __int_as_float((254 - g) << 23);
+            float n[NSA];
 #pragma unroll
             for (int s = 0; s < NSA; ++s) {
-                const float rx = rintf(p.x * iq) * q, ry = rintf(p.y * iq) * q;
-                *reinterpret_cast<__nv_bfloat162 *>(img + s * BM * ROW_B) =
-                    __nv_bfloat162(__float2bfloat16_rn(rx), __float2bfloat16_rn(ry));
+                const float nx = rintf(p.x * iq), ny = rintf(p.y * iq), rx = nx * q, ry = ny * q;
+                n[s] = q * (float)__reduce_add_sync(0xffffffffu, (int)(nx + ny));    // below 2^14 of the grid
+                if (c < whole) store(s, rx, ry);
                 p.x -= rx;
                 p.y -= ry;
+                q *= 0x1p-9f;
+                iq *= 0x1p9f;
+            }
+            if (c < whole) img += A_BYTES;
+            if (lane == 0) rs[c] = make_float2(n[0] + n[1], n[2] + n[3]);      // both exact
+        }
+        __syncwarp();
+        // the rest: entries of P behind the whole chunks, then the sums
+        for (int c = whole; c < nch; ++c, img += A_BYTES) {
+            float h[2], l[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int64_t b = (int64_t)c * BK + 2 * lane + i, j = b - k_pad;
+                h[i] = j < 0 ? (i ? last.y : last.x) : 0.0f;
+                l[i] = 0.0f;
+                if (j >= 0 && j < nb) two_sum(rs[j].x, rs[j].y, h[i], l[i]);
+            }
+            const int g = row_grid(h[0], h[1]);
+            float q = __int_as_float(g << 23), iq = __int_as_float((254 - g) << 23);
+#pragma unroll
+            for (int s = 0; s < NSA; ++s) {
+                float r[2];
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    r[i] = rintf(h[i] * iq) * q;
+                    two_sum(h[i] - r[i], l[i], h[i], l[i]);
+                }
+                store(s, r[0], r[1]);
                 q *= 0x1p-9f;
                 iq *= 0x1p9f;
             }
@@ -448,69 +517,119 @@ __global__ void __launch_bounds__(256) kl_rows_kernel(const float *__restrict__ 
             ex[x] = make_float2(h, (float)(e - (double)h));
             if (wrong) atomicExch(bad, 1);
         }
+        __syncwarp();
     }
 }
 
-// The slices of log2 max(P[t,b], FLT_MIN), one warp per (target, chunk); rows
-// past T and columns past k_pad are zeros.  N targets to a tile.
-__device__ __forceinline__ void kl_targets_chunk(const float *__restrict__ sP, int32_t T, int64_t k_pad, int N, int a,
-                                                 int c, int32_t nch, uint8_t *__restrict__ B, const Log2Tab &tab) {
-    const int lane = threadIdx.x & 31;
-    const int64_t b = (int64_t)c * BK + 2 * lane;
-    // log2 as a normalised sum of two floats: the slices reach 2^-19 of the
-    // chunk's grid (2^-23 and up), above the pair's error
-    float l[2] = {0.f, 0.f}, t[2] = {0.f, 0.f};
-    if (a < T && b < k_pad) {
-        const float2 p = *reinterpret_cast<const float2 *>(sP + (int64_t)a * k_pad + b);
-        const float pv[2] = {p.x, p.y};
+// The slices of log2 max(P[t,b], FLT_MIN) - c, a CTA per target, a warp per
+// chunk; rows past T and columns past the last are zeros.  N targets to a tile.
+// cs: c of every chunk of P (shared memory).
+__device__ __forceinline__ void kl_target_slices(const float *__restrict__ sP, int32_t T, int64_t k_pad, int N, int a,
+                                                 uint8_t *__restrict__ B, int *cs, const Log2Tab &tab) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nb = data_chunks(k_pad), nch = all_chunks(k_pad), whole = (int)(k_pad / BK);
+    uint8_t *row = B + (int64_t)(a / N) * nch * b_bytes(N) + image_at(a % N, 2 * lane);
+    // log2 of this lane's entry i of chunk c, exponent and table part apart; false past the columns of P
+    auto log2_at = [&](int c, int i, float2 &d) {
+        const int64_t b = (int64_t)c * BK + 2 * lane + i;
+        if (a >= T || b >= k_pad) return false;
+        d = log2_pair(fmaxf(sP[(int64_t)a * k_pad + b], FLT_MIN), tab);
+        return true;
+    };
+    // The chunk c with the numbers h + t (|t| within h's rounding; grid: whether an
+    // entry counts for the chunk's grid, 2^-7 of the largest magnitude's power of
+    // two, at least that of `least`); an entry's own BF16 grid where that is coarser
+    auto slices = [&](int c, float (&h)[2], float (&t)[2], const bool (&grid)[2], float least) {
+        float mag = least;
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            if (grid[i]) mag = fmaxf(mag, fabsf(h[i]));
+        const unsigned mx = __reduce_max_sync(0xffffffffu, __float_as_uint(mag));
+        int qe = max((int)(mx >> 23), 100) - 7;          // biased exponent of the grid
+        uint8_t *img = row + (int64_t)c * b_bytes(N);
+#pragma unroll
+        for (int s = 0; s < NSB; ++s, qe -= 9) {
+            __nv_bfloat16 v[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int e = max(qe, ((__float_as_int(h[i]) >> 23) & 255) - 7);
+                float r = rintf(h[i] * __int_as_float((254 - e) << 23)) * __int_as_float(e << 23);
+                if (s == NSB - 1) r = h[i];              // the last need not lie on a grid
+                v[i] = __float2bfloat16_rn(r);
+                h[i] = __fadd_rn(__fsub_rn(h[i], r), t[i]);      // h - r is exact
+                t[i] = 0.f;
+            }
+            *reinterpret_cast<__nv_bfloat162 *>(img + s * N * ROW_B) = __nv_bfloat162(v[0], v[1]);
+        }
+    };
+    // entries of P less c: a normalised pair (above its error of 2^-31: the slices reach 2^-18 of the grid)
+    auto data = [&](int c, int ci, float (&h)[2], float (&t)[2], bool (&grid)[2]) {
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-            const float2 d = log2_pair(fmaxf(pv[i], FLT_MIN), tab);
-            l[i] = __fadd_rn(d.x, d.y);
-            t[i] = __fsub_rn(d.y, __fsub_rn(l[i], d.x));
+            float2 d;
+            if (log2_at(c, i, d)) {
+                grid[i] = d.x >= -32.0f;
+                two_sum(d.x - (float)ci, d.y, h[i], t[i]);       // d.x is a multiple of 2^-12: exact
+            }
         }
+    };
+    for (int c = warp; c < nb; c += 8) {
+        // the whole number in the middle of the logs down to -32
+        int lo = INT_MAX, hi = INT_MIN;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            float2 d;
+            if (log2_at(c, i, d) && d.x >= -32.0f) {
+                const int v = __float2int_rn(d.x);
+                lo = min(lo, v);
+                hi = max(hi, v);
+            }
+        }
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        const int ci = lo <= hi ? (lo + hi) >> 1 : 0;
+        if (lane == 0) cs[c] = ci;
+        if (c >= whole) continue;
+        float h[2] = {0.f, 0.f}, t[2] = {0.f, 0.f};
+        bool grid[2] = {false, false};
+        data(c, ci, h, t, grid);
+        slices(c, h, t, grid, 0.0f);
     }
-    // the chunk's grid, 2^-7 of the largest magnitude's power of two among those up to 32
-    float mag = 0.0f;
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-        if (fabsf(l[i]) <= 32.0f) mag = fmaxf(mag, fabsf(l[i]));
-    const unsigned mx = __reduce_max_sync(0xffffffffu, __float_as_uint(mag));
-    int qe = max((int)(mx >> 23), 100) - 7;          // biased exponent of the grid
-    uint8_t *img = B + ((int64_t)(a / N) * nch + c) * b_bytes(N) + image_at(a % N, 2 * lane);
-#pragma unroll
-    for (int s = 0; s < NSB; ++s, qe -= 9) {
-        __nv_bfloat16 v[2];
+    __syncthreads();
+    // The rest.  A chunk that also holds c columns keeps a grid of 2^-7 or more, so
+    // that their products with sums of P (a row's largest is at least 1 / nb) and
+    // those of its entries still sum within 24 bits.
+    for (int c = whole + warp; c < nch; c += 8) {
+        float h[2] = {0.f, 0.f}, t[2] = {0.f, 0.f};
+        bool grid[2] = {false, false};
+        if (c < nb) data(c, cs[c], h, t, grid);
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-            // the chunk's grid, or the entry's own BF16 grid where that is coarser
-            const int e = max(qe, ((__float_as_int(l[i]) >> 23) & 255) - 7);
-            const float r = rintf(l[i] * __int_as_float((254 - e) << 23)) * __int_as_float(e << 23);
-            v[i] = __float2bfloat16_rn(r);
-            l[i] = __fadd_rn(__fsub_rn(l[i], r), t[i]);      // l - r is exact
-            t[i] = 0.f;
+            const int64_t j = (int64_t)c * BK + 2 * lane + i - k_pad;
+            if (j >= 0 && j < nb) h[i] = (float)cs[j];
         }
-        *reinterpret_cast<__nv_bfloat162 *>(img + s * N * ROW_B) = __nv_bfloat162(v[0], v[1]);
+        slices(c, h, t, grid, 1.0f);
     }
 }
 
 __global__ void __launch_bounds__(256) kl_targets_kernel(const float *__restrict__ sP, int32_t T, int64_t k_pad, int N,
-                                                         int32_t nch, uint8_t *__restrict__ B) {
+                                                         uint8_t *__restrict__ B) {
     __shared__ Log2Tab tab;
+    extern __shared__ int cs[];
     build_log2_table(tab);
     __syncthreads();
-    for (int c = threadIdx.x >> 5; c < nch; c += 8) kl_targets_chunk(sP, T, k_pad, N, blockIdx.x, c, nch, B, tab);
+    kl_target_slices(sP, T, k_pad, N, blockIdx.x, B, cs, tab);
 }
 
 // blockIdx.y a problem, blockIdx.x one of its targets (tiles of q.ktile)
 __global__ void __launch_bounds__(256) kl_batch_targets_kernel(const BatchProblem *__restrict__ probs) {
     __shared__ Log2Tab tab;
+    extern __shared__ int cs[];
     const BatchProblem &q = probs[blockIdx.y];
     if ((int)blockIdx.x >= (q.T + q.ktile - 1) / q.ktile * q.ktile) return;
     build_log2_table(tab);
     __syncthreads();
-    for (int c = threadIdx.x >> 5; c < q.knch; c += 8)
-        kl_targets_chunk(q.sP, q.T, q.k_pad, q.ktile, blockIdx.x, c, q.knch, q.KB, tab);
+    kl_target_slices(q.sP, q.T, q.k_pad, q.ktile, blockIdx.x, q.KB, cs, tab);
 }
 
 int sm_count() {
@@ -526,9 +645,12 @@ int sm_count() {
 // tile pass takes a few microseconds and the slicing of the targets as much.
 // A refined log2 P (dd_log_poisson_kernel) reaches far below log2 FLT_MIN,
 // beyond the totals' range: its KL stays in the tile pass.
-bool kl_mma_wanted(const DevMesh &m) { return !m.LP && m.n_v * m.k_pad >= (1 << 20); }
+// (2^17 columns: the sums of a row's chunks, eight rows a CTA, take 128 KB of shared memory.)
+bool kl_mma_wanted(const DevMesh &m) {
+    return !m.LP && m.n_v * m.k_pad >= (1 << 20) && m.k_pad <= kMaxColumns;
+}
 
-int32_t kl_mma_chunks(int64_t k_pad) { return (int32_t)((k_pad + BK - 1) / BK); }
+int32_t kl_mma_chunks(int64_t k_pad) { return all_chunks(k_pad); }
 
 // Target tile: wider tiles share one read of the row slices among more
 // targets and use more of the MMA rate (an MMA's operand reads from shared
@@ -564,7 +686,9 @@ dd_status prepare_kl_mma(DevMesh &m, cudaStream_t s, bool *usable, std::string &
     if (ce == cudaSuccess) {
         KMark km_("kl_rows_kernel", s);
         const int64_t blocks = std::min<int64_t>((nt * BM + 7) / 8, 8LL * sm_count());
-        kl_rows_kernel<<<(unsigned)blocks, 256, 0, s>>>(m.P, m.n_v, nt * BM, m.k_pad, nch, a, (float2 *)e, bad);
+        const int smem = 8 * data_chunks(m.k_pad) * (int)sizeof(float2);
+        cudaFuncSetAttribute(kl_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        kl_rows_kernel<<<(unsigned)blocks, 256, smem, s>>>(m.P, m.n_v, nt * BM, m.k_pad, a, (float2 *)e, bad);
         ce = cudaGetLastError();
     }
     if (ce == cudaSuccess) ce = cudaMemcpyAsync(&flag, bad, sizeof flag, cudaMemcpyDeviceToHost, s);
@@ -601,7 +725,7 @@ void launch_kl_mma(const KlMmaArgs &ka, const float *sP, int64_t n_v, int64_t k_
     const int nat = (T + N - 1) / N;
     {
         KMark km_("kl_targets_kernel", s);
-        kl_targets_kernel<<<(unsigned)(nat * N), 256, 0, s>>>(sP, T, k_pad, N, nch, ka.B);
+        kl_targets_kernel<<<(unsigned)(nat * N), 256, data_chunks(k_pad) * sizeof(int), s>>>(sP, T, k_pad, N, ka.B);
     }
     const KlOne one{ka.A, ka.B, ka.ex, out_kl, n_v, T, nch};
     const int64_t n_items = (n_v + BM - 1) / BM * nat;
@@ -622,8 +746,8 @@ void launch_kl_mma(const KlMmaArgs &ka, const float *sP, int64_t n_v, int64_t k_
 void launch_batch_kl_mma(const BatchProblem *d_probs, int32_t n_probs, const BatchKlMma &b, cudaStream_t s) {
     {
         KMark km_("kl_targets_kernel", s);
-        kl_batch_targets_kernel<<<dim3((unsigned)((b.max_T + 127) / 128 * 128), (unsigned)n_probs), 256, 0, s>>>(
-            d_probs);
+        kl_batch_targets_kernel<<<dim3((unsigned)((b.max_T + 127) / 128 * 128), (unsigned)n_probs), 256,
+                                  data_chunks(b.max_k) * sizeof(int), s>>>(d_probs);
     }
     auto go = [&](auto kern, int smem, const BatchItem *items, int32_t n) {
         if (n <= 0) return;
