@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "dd_amg.h"
+#include "dd_pairs.h"
 
 namespace {
 
@@ -342,29 +343,67 @@ void csr_apply(const AmgCsr &A, const std::vector<double> &x, std::vector<double
     }
 }
 
-// the V-cycle of the device solver, on the host: x = V(b) on level l
-void host_vcycle(const AmgHierarchy &H, size_t l, const std::vector<double> &b, std::vector<double> &x) {
-    const AmgLevel &L = H.levels[l];
-    const int64_t n = L.A.rows;
-    x.assign(n, 0.0);
-    if (l + 1 == H.levels.size()) {
-        for (int64_t i = 0; i < n; ++i) {
-            double s = 0.0;
-            for (int64_t j = 0; j < n; ++j) s += H.coarse_inv[i * n + j] * b[j];
-            x[i] = s;
-        }
+struct Df {
+    float hi, lo;
+};
+Df df_pair(double v) {
+    const float h = (float)v;
+    return Df{h, (float)(v - (double)h)};
+}
+// (s, c) += a x, as the device's df_fma
+void df_fma(float &s, float &c, Df a, Df x) {
+    const float p = std::fmaf(a.hi, x.hi, 0.0f);      // (not contracted with the sum below)
+    float e = std::fmaf(a.hi, x.hi, -p);
+    e = std::fmaf(a.hi, x.lo, e);
+    e = std::fmaf(a.lo, x.hi, e);
+    const float t = s + p, b = t - s;
+    c += ((s - (t - b)) + (p - b)) + e;
+    s = t;
+}
+Df df_norm(float s, float c) {
+    const float h = s + c;
+    return Df{h, c - (h - s)};
+}
+
+// y = M x (+ M2 x2)
+void df_apply(const AmgCsr &M, const std::vector<Df> &x, const AmgCsr *M2, const std::vector<Df> *x2,
+              std::vector<Df> &y) {
+    y.resize(M.rows);
+    for (int64_t i = 0; i < M.rows; ++i) {
+        float s = 0.0f, c = 0.0f;
+        for (int64_t p = M.off[i]; p < M.off[i + 1]; ++p) df_fma(s, c, df_pair(M.val[p]), x[M.col[p]]);
+        if (M2)
+            for (int64_t p = M2->off[i]; p < M2->off[i + 1]; ++p) df_fma(s, c, df_pair(M2->val[p]), (*x2)[M2->col[p]]);
+        y[i] = df_norm(s, c);
+    }
+}
+
+// z = V(r), the device solver's V-cycle: the fused products Q^T, G and Q in pairs
+// of floats, r and z with the column's exponent (one level: the exact solve)
+void host_vcycle(const AmgHierarchy &H, const std::vector<double> &r, int shift, std::vector<double> &z) {
+    const size_t nl = H.levels.size();
+    const int64_t n = H.levels[0].A.rows, nc = H.coarse_n;
+    z.assign(n, 0.0);
+    if (nl == 1) {
+        for (int64_t i = 0; i < n; ++i)
+            for (int64_t j = 0; j < n; ++j) z[i] += H.coarse_inv[i * n + j] * r[j];
         return;
     }
-    for (int64_t i = 0; i < n; ++i) x[i] = L.omega * L.dinv[i] * b[i];
-    std::vector<double> t, r(n), bc, xc;
-    csr_apply(L.A, x, t);
-    for (int64_t i = 0; i < n; ++i) r[i] = b[i] - t[i];
-    csr_apply(L.R, r, bc);
-    host_vcycle(H, l + 1, bc, xc);
-    csr_apply(L.P, xc, t);
-    for (int64_t i = 0; i < n; ++i) x[i] += t[i];
-    csr_apply(L.A, x, t);
-    for (int64_t i = 0; i < n; ++i) x[i] += L.omega * L.dinv[i] * (b[i] - t[i]);
+    std::vector<std::vector<Df>> b(nl);
+    b[0].resize(n);
+    for (int64_t i = 0; i < n; ++i) df_split(r[i], shift, b[0][i].hi, b[0][i].lo);
+    for (size_t l = 0; l + 1 < nl; ++l) df_apply(H.levels[l].Qt, b[l], nullptr, nullptr, b[l + 1]);
+    std::vector<Df> x(nc), y;
+    for (int64_t i = 0; i < nc; ++i) {
+        float s = 0.0f, c = 0.0f;
+        for (int64_t j = 0; j < nc; ++j) df_fma(s, c, df_pair(H.coarse_inv[i * nc + j]), b[nl - 1][j]);
+        x[i] = df_norm(s, c);
+    }
+    for (size_t l = nl - 1; l-- > 0;) {
+        df_apply(H.levels[l].G, b[l], &H.levels[l].Q, &x, y);
+        x.swap(y);
+    }
+    for (int64_t i = 0; i < n; ++i) z[i] = widen(x[i].hi, shift) + widen(x[i].lo, shift);
 }
 
 }  // namespace
@@ -382,7 +421,10 @@ bool amg_host_solve(const AmgCsr &A, const std::vector<double> &b, std::vector<d
     bn = std::sqrt(bn);
     *iters = 0;
     if (!(bn > 0.0)) return true;
-    host_vcycle(H, 0, r, z);
+    int top = 0;
+    for (double v : r) top = std::max(top, (int)(bits_as<uint64_t>(v) >> 52 & 0x7ff));
+    int shift = shift_of_top(top);
+    host_vcycle(H, r, shift, z);
     p = z;
     double rz = 0.0;
     for (int64_t i = 0; i < n; ++i) rz += r[i] * z[i];
@@ -399,7 +441,8 @@ bool amg_host_solve(const AmgCsr &A, const std::vector<double> &b, std::vector<d
         }
         *iters = it;
         if (std::sqrt(rr) <= rtol * bn) return true;
-        host_vcycle(H, 0, r, z);
+        host_vcycle(H, r, shift, z);
+        shift = shift_of_square(rr);
         double rz2 = 0.0;
         for (int64_t i = 0; i < n; ++i) rz2 += r[i] * z[i];
         const double beta = rz2 / rz;

@@ -24,6 +24,7 @@
 #include "dd_amg.h"
 #include "dd_f32x2.cuh"
 #include "dd_internal.h"
+#include "dd_pairs.h"
 
 namespace {
 
@@ -126,17 +127,6 @@ __global__ void alpha_kernel(int64_t nrb, int64_t kc, const double *__restrict__
     if (threadIdx.y == 0 && c < kc) alpha[c] = (!done[c] && pAp > 0.0) ? rz[c] / pAp : 0.0;
 }
 
-// The exponents that a column's numbers gain on their way into the V-cycle and
-// lose on their way out (df_split, widen).  The residual's norm then lies
-// near 2^60: a factor 2^-150 below it is kept and one of 2^58 above it fits,
-// whatever the size of the column's right-hand side and however far the column
-// has converged.
-constexpr int kShiftTop = 60, kShiftMin = -452, kShiftMax = 572;
-// from the squared norm (0, subnormal and infinite numbers included)
-__device__ __forceinline__ int shift_of_square(double rr) {
-    return kShiftTop - ((((int)((unsigned long long)__double_as_longlong(rr) >> 52) & 0x7ff) - 1023) >> 1);
-}
-
 // (nrz, nrb: how many partials part_rz and part_rr hold a column; shift: null, or
 // the columns' exponents for the next residual)
 __global__ void beta_kernel(int64_t nrz, int64_t nrb, int64_t kc, const double *__restrict__ part_rz,
@@ -178,7 +168,7 @@ __global__ void scatter_rhs_kernel(int64_t n_rb, const int32_t *__restrict__ rb_
 // the right-hand side's exponents (beta_kernel) from the largest biased one, in place
 __global__ void first_shift_kernel(int64_t kc, int *__restrict__ shift) {
     const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < kc) shift[c] = max(kShiftMin, min(kShiftMax, kShiftTop + 1023 - shift[c]));
+    if (c < kc) shift[c] = shift_of_top(shift[c]);
 }
 
 __global__ void dinv_kernel(int64_t m, const double *__restrict__ diag, double *__restrict__ dinv) {
@@ -296,35 +286,6 @@ __device__ __forceinline__ float4 df_pack(const Df2 &v) {
     upk(v.hi, r.x, r.y);
     upk(v.lo, r.z, r.w);
     return r;
-}
-
-// A double times 2^shift as an unevaluated sum of two floats, by integer
-// operations on its bits (this part converts FP64 no faster than it multiplies
-// it): the leading 24 bits of the significand, and the 29 that follow as an
-// integer scaled.  Magnitudes outside 2^-90 .. 2^120 come out as 0 or as 2^120:
-// the column's exponent (shift_of_square) keeps what matters between them.  A
-// residual is relative to its own right-hand side, which may be 1e-17 (a
-// corner that meets the interior by a right-angled cell's diagonal alone,
-// rotated) or far above 1, and falls by 1e-15 and more; without the shift
-// such columns stopped at 1e-9 of theirs.
-__device__ __forceinline__ void df_split(double d, int shift, float &hi, float &lo) {
-    const unsigned long long u = (unsigned long long)__double_as_longlong(d);
-    const unsigned sign = (unsigned)(u >> 32) & 0x80000000u;
-    const int e = (int)((u >> 52) & 0x7ff) - 1023 + shift;
-    const int ec = min(e, 120);
-    const unsigned top = (unsigned)(u >> 29) & 0x7fffffu;
-    const float l = (float)(int)((unsigned)u & 0x1fffffffu);               // < 2^29
-    const float scale = __uint_as_float((unsigned)(ec - 29 + 127) << 23);  // 2^(e - 29); times 2^-23 below
-    const bool tiny = e < -90;
-    hi = tiny ? 0.0f : __uint_as_float(sign | ((unsigned)(ec + 127) << 23) | top);
-    lo = tiny ? 0.0f : __uint_as_float(sign ^ __float_as_uint(l * scale * 0x1p-23f));
-}
-// float times 2^-shift to double by its bits (subnormals as 0)
-__device__ __forceinline__ double widen(float f, int shift) {
-    const unsigned u = __float_as_uint(f);
-    const unsigned m = u & 0x7fffffffu;
-    const unsigned h = m < 0x00800000u ? 0u : (m >> 3) + ((unsigned)(896 - shift) << 20);
-    return __hiloint2double((int)((u & 0x80000000u) | h), (int)(m < 0x00800000u ? 0u : m << 29));
 }
 
 constexpr int kPairs = 64;      // column pairs (threads) of one CTA
