@@ -110,10 +110,11 @@ __device__ __forceinline__ float4 tri_rates(const float4 *__restrict__ gphi, con
 // ft[v * T + a] = field a at vertex v: the fields vertex by vertex, so that a
 // warp of the decision kernel reads 32 fields of a vertex at once
 __global__ void __launch_bounds__(256) fields_by_vertex_kernel(const float *__restrict__ fields, int64_t field_stride,
-                                                               int64_t n_v, int32_t T, float *__restrict__ ft) {
+                                                               int64_t n_v, int32_t T, int32_t first,
+                                                               float *__restrict__ ft) {
     __shared__ float tile[32][33];
     const int64_t v0 = (int64_t)blockIdx.x * 32;
-    const int a0 = blockIdx.y * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int a0 = first + blockIdx.y * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
 #pragma unroll
     for (int i = ty; i < 32; i += 8)
         if (a0 + i < T && v0 + tx < n_v) tile[i][tx] = fields[(int64_t)(a0 + i) * field_stride + v0 + tx];
@@ -302,19 +303,19 @@ __device__ __forceinline__ void fan_reduce(FanScan &fs, unsigned mask) {
     fs.b_pk.y = __shfl_sync(mask, fs.b_pk.y, from);
 }
 
-// one warp per vertex and 32 fields (blockIdx.y), lane = field: dec[v * T + a];
+// one warp per vertex and 32 fields (blockIdx.y, from field `first` on), lane = field: dec[v * T + a];
 // vertices of more than kWideFan triangles are left to wide_decision_kernel.
 // The rates of a fan's triangles are formed here from the fields by vertex:
 // 64 fields of 71,681 vertices, the rates of every triangle stored first (147
 // MB written, read three times) took 68 + 230 us, this 8 + 183 (216 with a
 // choice among the local vertices for every operand).
-__global__ void __launch_bounds__(128) vertex_decision_kernel(const TraceDom p, int32_t T,
+__global__ void __launch_bounds__(128) vertex_decision_kernel(const TraceDom p, int32_t T, int32_t first,
                                                               const float *__restrict__ fields, int64_t field_stride,
                                                               const float *__restrict__ ft,
                                                               const int32_t *__restrict__ targets,
                                                               VDec *__restrict__ dec) {
     const int64_t v = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
-    const int a = blockIdx.y * 32 + (threadIdx.x & 31);
+    const int a = first + blockIdx.y * 32 + (threadIdx.x & 31);
     if (v >= p.n_v || a >= T) return;
     const int q0 = p.vt_off[v], q1 = p.vt_off[v + 1];
     if (q1 - q0 > kWideFan) return;
@@ -335,11 +336,11 @@ __global__ void __launch_bounds__(128) vertex_decision_kernel(const TraceDom p, 
 // has sectors), one warp per (vertex, field), the fan over the lanes.  With
 // one lane scanning it the 512 triangles of one centre were a chain of 0.65
 // ms, all of the decision pass but 0.12 ms (71,681 vertices, 64 fields).
-__global__ void wide_decision_kernel(const TraceDom p, const int32_t *__restrict__ wide, int32_t T,
+__global__ void wide_decision_kernel(const TraceDom p, const int32_t *__restrict__ wide, int32_t T, int32_t first,
                                      const float *__restrict__ fields, int64_t field_stride,
                                      const int32_t *__restrict__ targets, VDec *__restrict__ dec) {
     const int v = wide[blockIdx.x], lane = threadIdx.x & 31;
-    const int a = blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int a = first + blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (a >= T) return;
     const float *f = fields + (int64_t)a * field_stride;
     FanScan fs;
@@ -943,22 +944,28 @@ void launch_trace(const DevMesh &m, const float *fields, int64_t field_stride, c
     p.out_status = out_status;
     if (p.total == 0) return;
     if (dense) {
-        const unsigned groups32 = (unsigned)((T + 31) / 32);
-        {
+        // (a grid has at most 65,535 rows; here each has up to 65,504 groups of fields)
+        auto by_fields = [&](int per_group, auto launch) {
+            constexpr int64_t kRows = 65504;
+            for (int64_t first = 0; first < T; first += kRows * per_group)
+                launch((int32_t)first, (unsigned)std::min<int64_t>(kRows, (T - first + per_group - 1) / per_group));
+        };
+        by_fields(32, [&](int32_t first, unsigned rows) {
             KMark km_("fields_by_vertex_kernel", s);
-            fields_by_vertex_kernel<<<dim3((unsigned)((m.n_v + 31) / 32), groups32), 256, 0, s>>>(fields, field_stride,
-                                                                                                 m.n_v, T, ft);
-        }
-        {
+            fields_by_vertex_kernel<<<dim3((unsigned)((m.n_v + 31) / 32), rows), 256, 0, s>>>(fields, field_stride,
+                                                                                             m.n_v, T, first, ft);
+        });
+        by_fields(32, [&](int32_t first, unsigned rows) {
             KMark km_("vertex_decision_kernel", s);
-            vertex_decision_kernel<<<dim3((unsigned)((m.n_v + 3) / 4), groups32), 128, 0, s>>>(
-                p.d, T, fields, field_stride, ft, targets, dec);
-        }
-        if (m.n_wide > 0) {
-            KMark km_("wide_decision_kernel", s);
-            wide_decision_kernel<<<dim3((unsigned)m.n_wide, (unsigned)((T + 3) / 4)), 128, 0, s>>>(
-                p.d, m.wide, T, fields, field_stride, targets, dec);
-        }
+            vertex_decision_kernel<<<dim3((unsigned)((m.n_v + 3) / 4), rows), 128, 0, s>>>(
+                p.d, T, first, fields, field_stride, ft, targets, dec);
+        });
+        if (m.n_wide > 0)
+            by_fields(4, [&](int32_t first, unsigned rows) {
+                KMark km_("wide_decision_kernel", s);
+                wide_decision_kernel<<<dim3((unsigned)m.n_wide, rows), 128, 0, s>>>(p.d, m.wide, T, first, fields,
+                                                                                   field_stride, targets, dec);
+            });
     }
     auto groups = [&](auto kern, int G) {
         KMark km_("trace_kernel", s);
