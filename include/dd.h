@@ -83,9 +83,11 @@ enum { DD_F_KL = 1, DD_F_TV = 2, DD_F_KLT = 4 };
  *                 of P, rounded up to whole tiles) are built on the first such
  *                 call, which synchronizes, and kept with the map; a P with
  *                 entries outside [0, 2] or row sums above 1.01, or no room
- *                 for them, keeps the FP32 sums.  In all cases the rows near
- *                 the target (x = t among them) come from the exact form and
- *                 every value keeps 1e-5 relative accuracy.
+ *                 for them (tried again once P changes or the library has
+ *                 given device memory back), keeps the FP32 sums.  The last
+ *                 bits of KL depend on whether T is above 64.  In all cases
+ *                 the rows near the target (x = t among them) come from the
+ *                 exact form and every value keeps 1e-5 relative accuracy.
  *  DD_PREC_BF16X3 KL cross term sum_b P[x,b] log P[t,b] as a tensor-core GEMM
  *                 of split BF16 hi/lo operands (hi*hi + hi*lo + lo*hi, FP32
  *                 accumulation); TV and KLT are always FP32

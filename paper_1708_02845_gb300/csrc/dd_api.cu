@@ -21,6 +21,7 @@
 namespace {
 
 std::atomic<int> g_kt_on{0};      // contexts with per-kernel timing on
+std::atomic<int64_t> g_releases{0};      // device arrays given back so far (memory_releases)
 
 dd_status set_err(dd_ctx *c, dd_status s, const std::string &msg) {
     if (c) c->err = msg;
@@ -50,7 +51,10 @@ dd_status ensure_scratch(dd_ctx *ctx, int id, size_t bytes) {
     if (bytes == 0) bytes = 16;
     if (ctx->scratch_cap[id] >= bytes) return DD_OK;
     CK(cudaStreamSynchronize(ctx->stream), "synchronize before scratch growth");
-    if (ctx->scratch[id]) cudaFree(ctx->scratch[id]);
+    if (ctx->scratch[id]) {
+        cudaFree(ctx->scratch[id]);
+        ++g_releases;
+    }
     ctx->scratch[id] = nullptr;
     ctx->scratch_cap[id] = 0;
     size_t cap = bytes + bytes / 4;
@@ -145,6 +149,7 @@ dd_status dev_copy(dd_ctx *ctx, DevMesh &m, T **dst, const T *src, size_t count)
 
 void free_mesh(DevMesh &m) {
     for (void *p : m.owned) cudaFree(p);
+    ++g_releases;
     m = DevMesh();
 }
 
@@ -153,6 +158,7 @@ template <typename T>
 void release(DevMesh &m, T *&p, int64_t bytes) {
     if (!p) return;
     cudaFree((void *)p);
+    ++g_releases;
     m.owned.erase(std::remove(m.owned.begin(), m.owned.end(), (void *)p), m.owned.end());
     m.bytes -= bytes;
     p = nullptr;
@@ -180,6 +186,7 @@ void drop_kl_mma(DevMesh &m) {
     release(m, m.kl_a, (int64_t)kl_mma_row_bytes(m));
     release(m, m.kl_ex, (int64_t)kl_mma_ex_bytes(m));
     m.kl_state = 0;
+    m.kl_no_room = -1;
 }
 
 // what was derived from the stored P (the BF16 split, the row entropies, the
@@ -376,6 +383,8 @@ void kt_fold(KTimer &t) {
 }
 
 }  // namespace
+
+int64_t memory_releases() { return g_releases.load(std::memory_order_relaxed); }
 
 KMark::KMark(const char *n, cudaStream_t s) {
     if (!g_kt_on.load(std::memory_order_relaxed)) return;

@@ -83,6 +83,7 @@ struct DevMesh {
     uint8_t *kl_a = nullptr;
     float2 *kl_ex = nullptr;
     int kl_state = 0;
+    int64_t kl_no_room = -1;   // memory_releases() when there was no room for them
     // sparse fields (dd_sparsify): the threshold relative to the row maximum,
     // the sparsified P as CSR (each row's kept entries in column order), and
     // the exact total of every stored row (for the merged-bin extension)
@@ -199,7 +200,8 @@ int64_t fix_row_blocks(int64_t n_v);
 
 // The KL fields of more than two targets on the tensor cores, as accurate as
 // FP32 sums (dd_klmma.cu).  prepare_kl_mma builds the mesh's operands once;
-// *usable is false where there is no room for them or P does not qualify.
+// *usable is false where P does not qualify or there is no room for them (which
+// is not tried again before P or some other array of the library is given back).
 // launch_kl_mma: the targets' slices into args.B (kl_mma_target_bytes with
 // kl_mma_tile's N), then out_kl [T][n_v]; the values below kMmaExactBelow are
 // then for the exact recompute.
@@ -217,6 +219,7 @@ size_t kl_mma_target_bytes(int64_t k_pad, int32_t T, int N);
 size_t kl_mma_row_bytes(const DevMesh &m);
 size_t kl_mma_ex_bytes(const DevMesh &m);
 dd_status prepare_kl_mma(DevMesh &m, cudaStream_t s, bool *usable, std::string &err);
+int64_t memory_releases();      // how many device arrays the library has given back
 void launch_kl_mma(const KlMmaArgs &args, const float *sP, int64_t n_v, int64_t k_pad, int32_t T, float *out_kl,
                    int *err, cudaStream_t s);
 // every problem's KL (KA, KB, kex, knch, ktile set)

@@ -666,7 +666,7 @@ size_t kl_mma_target_bytes(int64_t k_pad, int32_t T, int N) {
 
 dd_status prepare_kl_mma(DevMesh &m, cudaStream_t s, bool *usable, std::string &err) {
     *usable = m.kl_state == 1;
-    if (m.kl_state != 0) return DD_OK;
+    if (m.kl_state != 0 || m.kl_no_room == memory_releases()) return DD_OK;
     const int32_t nch = kl_mma_chunks(m.k_pad);
     const int64_t nt = (m.n_v + BM - 1) / BM;
     const size_t abytes = (size_t)nt * nch * A_BYTES, ebytes = (size_t)nt * BM * sizeof(float2);
@@ -678,6 +678,7 @@ dd_status prepare_kl_mma(DevMesh &m, cudaStream_t s, bool *usable, std::string &
     if (cudaMalloc((void **)&a, abytes) != cudaSuccess || cudaMalloc((void **)&e, ebytes + sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
         drop();
+        m.kl_no_room = memory_releases();
         return DD_OK;      // no room: the FP32 tile kernels, which need none, run instead
     }
     int *bad = reinterpret_cast<int *>(e + ebytes);
