@@ -401,8 +401,9 @@ dd_status dd_query(dd_ctx *ctx, int32_t mesh, const int32_t *targets, int32_t T,
  * bytes times n_v k_pad per mesh, kept with the mesh; without room for them the
  * launch stays staged), whichever the autotuner measured faster for the
  * class of the batch (dd_tuning_table).  Same arithmetic as dd_query with
- * FP32 (KL on the tensor cores when every map qualifies): both launches give
- * the same fields, bit for bit.
+ * FP32, item by item (KL on the tensor cores for the maps that qualify; the
+ * others in launches of their own): both launches give the same fields, bit
+ * for bit, whatever the other items are.
  *   n_items   number of items (>= 1)
  *   mesh_ids  host [n_items] loaded meshes with a Poisson kernel
  *   T_per     host [n_items] targets per item (>= 1)

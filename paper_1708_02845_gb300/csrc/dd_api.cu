@@ -1182,12 +1182,6 @@ dd_status dd_query_batch(dd_ctx *ctx, int32_t n_items, const int32_t *mesh_ids, 
         if (st != DD_OK) return st;
 
         // metadata block: tprob, tloc, problems, items, trace domains, counter
-        std::vector<int32_t> tprob(nT), tloc(nT);
-        for (int i = 0; i < n_items; ++i)
-            for (int a = 0; a < T_per[i]; ++a) {
-                tprob[toff[i] + a] = i;
-                tloc[toff[i] + a] = a;
-            }
         if ((st = upload(ctx, S_TARGETS, targets, (size_t)nT * sizeof(int32_t))) != DD_OK) return st;
         if (S > 0 && (st = upload(ctx, S_SOURCES, sources, (size_t)nT * S * sizeof(int32_t))) != DD_OK) return st;
         const size_t out_bytes = (size_t)foff[n_items] * sizeof(float);
@@ -1201,10 +1195,60 @@ dd_status dd_query_batch(dd_ctx *ctx, int32_t n_items, const int32_t *mesh_ids, 
         float *stage = reinterpret_cast<float *>(ctx->scratch[S_STAGE]);
         char *grads = reinterpret_cast<char *>(ctx->scratch[S_GRAD]);
 
+        // KL of an item comes from the tensor cores where its map qualifies and has room
+        // for the operands, as in dd_distance, else from the tile pass: an item's fields
+        // do not depend on the other items' maps.  The problems of either kind follow one
+        // another, and each kind has launches of its own.
+        std::vector<char> mma(n_items, 0);
+        size_t kb_bytes = 0;
+        for (int i = 0; i < n_items && (f_mask & DD_F_KL); ++i) {
+            if (!kl_mma_wanted(*ms[i])) continue;
+            std::string err;
+            bool ok = false;
+            if ((st = prepare_kl_mma(*ms[i], ctx->stream, &ok, err)) != DD_OK) return set_err(ctx, st, err);
+            if (!ok) continue;
+            mma[i] = 1;
+            kb_bytes += kl_mma_target_bytes(ms[i]->k_pad, T_per[i], kl_mma_batch_tile(T_per[i]));
+        }
+        if (kb_bytes && ensure_scratch(ctx, S_KLMMA, kb_bytes) != DD_OK) {
+            cudaGetLastError();
+            ctx->err.clear();
+            mma.assign(n_items, 0);
+        }
+        struct Kind {
+            bool mma = false, tile_kl = false, tile = false;      // KL in the tile pass; a tile pass at all
+            int first = 0, count = 0;                             // its problems
+            int32_t kl_wide = 0, max_T = 0;
+            int64_t max_k = 0, max_tiles = 0, fix_blocks = 0, work = 0;
+            std::vector<std::pair<int64_t, BatchItem>> staged, pipe, kl;      // (cost, item), prob counted from `first`
+            size_t o_staged = 0, o_pipe = 0, o_kl = 0;
+        };
+        Kind kinds[2];
+        std::vector<int> item;                  // the item of each problem
+        std::vector<int> pos(n_items);          // the problem of each item
+        for (int g = 0; g < 2; ++g) {
+            Kind &K = kinds[g];
+            K.mma = g == 0;
+            K.tile_kl = (f_mask & DD_F_KL) && !K.mma;
+            K.tile = K.tile_kl || (f_mask & DD_F_TV);
+            K.first = (int)item.size();
+            for (int i = 0; i < n_items; ++i)
+                if ((mma[i] != 0) == K.mma) {
+                    pos[i] = (int)item.size();
+                    item.push_back(i);
+                    K.max_T = std::max(K.max_T, T_per[i]);
+                    K.max_k = std::max(K.max_k, ms[i]->k_pad);
+                    K.work += ms[i]->n_v * ms[i]->k_pad * (int64_t)T_per[i];
+                    if (f_mask & DD_F_KL) K.fix_blocks += fix_row_blocks(ms[i]->n_v);
+                }
+            K.count = (int)item.size() - K.first;
+        }
         std::vector<BatchProblem> probs(n_items);
         int64_t so = 0;
-        for (int i = 0; i < n_items; ++i) {
-            BatchProblem &q = probs[i];
+        uint8_t *kb = reinterpret_cast<uint8_t *>(ctx->scratch[S_KLMMA]);
+        for (int j = 0; j < n_items; ++j) {
+            BatchProblem &q = probs[j];
+            const int i = item[j];
             const DevMesh &m = *ms[i];
             const int64_t blk = (int64_t)T_per[i] * m.k_pad;
             q.P = m.P;
@@ -1219,36 +1263,21 @@ dd_status dd_query_batch(dd_ctx *ctx, int32_t n_items, const int32_t *mesh_ids, 
             float *base = dfields + foff[i];
             q.out_kl = (f_mask & DD_F_KL) ? base : nullptr;
             q.out_tv = (f_mask & DD_F_TV) ? base + ((f_mask & DD_F_KL) ? (int64_t)T_per[i] * m.n_v : 0) : nullptr;
-        }
-        // KL from the tensor cores when every map qualifies (and there is room), as in dd_distance
-        bool mma = (f_mask & DD_F_KL) != 0;
-        int32_t max_T = 0;
-        size_t kb_bytes = 0;
-        for (int i = 0; i < n_items && mma; ++i) {
-            std::string err;
-            mma = kl_mma_wanted(*ms[i]);
-            if (mma && (st = prepare_kl_mma(*ms[i], ctx->stream, &mma, err)) != DD_OK) return set_err(ctx, st, err);
-            kb_bytes += kl_mma_target_bytes(ms[i]->k_pad, T_per[i], kl_mma_batch_tile(T_per[i]));
-            max_T = std::max(max_T, T_per[i]);
-        }
-        if (mma && ensure_scratch(ctx, S_KLMMA, kb_bytes) != DD_OK) {
-            cudaGetLastError();
-            ctx->err.clear();
-            mma = false;
-        }
-        if (mma) {
-            uint8_t *kb = reinterpret_cast<uint8_t *>(ctx->scratch[S_KLMMA]);
-            for (int i = 0; i < n_items; ++i) {
-                BatchProblem &q = probs[i];
-                q.KA = ms[i]->kl_a;
-                q.kex = ms[i]->kl_ex;
+            if (mma[i]) {
+                q.KA = m.kl_a;
+                q.kex = m.kl_ex;
                 q.KB = kb;
-                q.knch = kl_mma_chunks(ms[i]->k_pad);
+                q.knch = kl_mma_chunks(m.k_pad);
                 q.ktile = kl_mma_batch_tile(T_per[i]);
-                kb += kl_mma_target_bytes(ms[i]->k_pad, T_per[i], q.ktile);
+                kb += kl_mma_target_bytes(m.k_pad, T_per[i], q.ktile);
             }
         }
-        const bool tile_kl = (f_mask & DD_F_KL) && !mma;      // KL in the tile pass
+        std::vector<int32_t> tprob(nT), tloc(nT);
+        for (int i = 0; i < n_items; ++i)
+            for (int a = 0; a < T_per[i]; ++a) {
+                tprob[toff[i] + a] = pos[i];
+                tloc[toff[i] + a] = a;
+            }
         const size_t o_tprob = 0, o_tloc = align256(nT * sizeof(int32_t));
         const size_t o_probs = o_tloc + align256(nT * sizeof(int32_t));
         const size_t o_doms = o_probs + align256(n_items * sizeof(BatchProblem));
@@ -1267,147 +1296,141 @@ dd_status dd_query_batch(dd_ctx *ctx, int32_t n_items, const int32_t *mesh_ids, 
                            reinterpret_cast<const int32_t *>(dmeta + o_tloc),
                            reinterpret_cast<const int32_t *>(ctx->scratch[S_TARGETS]), nT, max_k, ctx->stream);
         CK(cudaGetLastError(), "batch staging launch");
-        if (tile_kl || (f_mask & DD_F_TV))
-            for (int i = 0; i < n_items; ++i)
-                probs[i].variant = tile_variant_for(probs[i].P, probs[i].n_v, probs[i].k_pad, probs[i].sP, probs[i].sL,
-                                                probs[i].sE, probs[i].T, tile_kl ? probs[i].out_kl : nullptr,
-                                                probs[i].out_tv, ctx->stream);
         // items: every output tile, larger row extents first for balance
-        std::vector<std::pair<int64_t, BatchItem>> order;
-        for (int i = 0; i < n_items; ++i) {
-            const int tr = tile_rows(probs[i].variant), tt = tile_targets(probs[i].variant);
-            const int64_t cost = ms[i]->k_pad * tr * (int64_t)tt;
-            for (int64_t xt = 0; xt * tr < ms[i]->n_v; ++xt)
-                for (int at = 0; at * tt < T_per[i]; ++at) order.push_back({cost, BatchItem{i, (int32_t)xt, at, 0}});
-        }
-        std::stable_sort(order.begin(), order.end(),
-                         [](const std::pair<int64_t, BatchItem> &x, const std::pair<int64_t, BatchItem> &y) {
-                             return x.first > y.first;
-                         });
-        // the pipelined launch: every mesh's tiled copy of P (built once per
-        // mesh; without room for it the batch stays staged), every problem's
-        // targets in the tiled layout, items of 128 rows x 64 targets
-        bool pipe_ok = tile_kl || (f_mask & DD_F_TV);      // (a tile pass is needed)
-        int64_t tstage_bytes = 0, max_tiles = 0;
-        for (int i = 0; i < n_items && pipe_ok; ++i) {
-            std::string err;
-            if (prepare_tiled(*ms[i], tile_kl, ctx->stream, err) != DD_OK) pipe_ok = false;
-            tstage_bytes += (int64_t)tiled_target_bytes(ms[i]->k_pad, T_per[i]);
-            max_tiles = std::max<int64_t>(max_tiles, (T_per[i] + 63) / 64 * (tiled_k32(ms[i]->k_pad) / 32));
-        }
-        if (pipe_ok && ensure_scratch(ctx, S_TSTAGE, (size_t)tstage_bytes) != DD_OK) {
-            cudaGetLastError();
-            pipe_ok = false;
-        }
         auto costliest_first = [](std::vector<std::pair<int64_t, BatchItem>> &v) {
             std::stable_sort(v.begin(), v.end(),
                              [](const std::pair<int64_t, BatchItem> &x, const std::pair<int64_t, BatchItem> &y) {
                                  return x.first > y.first;
                              });
         };
-        std::vector<std::pair<int64_t, BatchItem>> order_pipe;
-        if (pipe_ok) {
-            float *ts = reinterpret_cast<float *>(ctx->scratch[S_TSTAGE]);
-            for (int i = 0; i < n_items; ++i) {
-                BatchProblem &q = probs[i];
-                const DevMesh &m = *ms[i];
-                const int64_t half = (int64_t)tiled_target_bytes(m.k_pad, T_per[i]) / (2 * sizeof(float));
+        for (Kind &K : kinds) {
+            for (int j = 0; j < K.count && K.tile; ++j) {
+                BatchProblem &q = probs[K.first + j];
+                q.variant = tile_variant_for(q.P, q.n_v, q.k_pad, q.sP, q.sL, q.sE, q.T,
+                                             K.tile_kl ? q.out_kl : nullptr, q.out_tv, ctx->stream);
+                const int tr = tile_rows(q.variant), tt = tile_targets(q.variant);
+                const int64_t cost = q.k_pad * tr * (int64_t)tt;
+                for (int64_t xt = 0; xt * tr < q.n_v; ++xt)
+                    for (int at = 0; at * tt < q.T; ++at) K.staged.push_back({cost, BatchItem{j, (int32_t)xt, at, 0}});
+            }
+            costliest_first(K.staged);
+        }
+        // the pipelined launch: every mesh's tiled copy of P (built once per
+        // mesh; without room for it the batch stays staged), every problem's
+        // targets in the tiled layout, items of 128 rows x 64 targets
+        bool pipe_ok = true;
+        int64_t tstage_bytes = 0;
+        for (Kind &K : kinds)
+            for (int j = 0; j < K.count && K.tile && pipe_ok; ++j) {
+                DevMesh &m = *ms[item[K.first + j]];
+                const int32_t T = probs[K.first + j].T;
+                std::string err;
+                if (prepare_tiled(m, K.tile_kl, ctx->stream, err) != DD_OK) pipe_ok = false;
+                tstage_bytes += (int64_t)tiled_target_bytes(m.k_pad, T);
+                K.max_tiles = std::max<int64_t>(K.max_tiles, (T + 63) / 64 * (tiled_k32(m.k_pad) / 32));
+            }
+        if (pipe_ok && tstage_bytes && ensure_scratch(ctx, S_TSTAGE, (size_t)tstage_bytes) != DD_OK) {
+            cudaGetLastError();
+            pipe_ok = false;
+        }
+        float *ts = reinterpret_cast<float *>(ctx->scratch[S_TSTAGE]);
+        for (Kind &K : kinds) {
+            for (int j = 0; j < K.count && K.tile && pipe_ok; ++j) {
+                BatchProblem &q = probs[K.first + j];
+                const DevMesh &m = *ms[item[K.first + j]];
+                const int64_t half = (int64_t)tiled_target_bytes(m.k_pad, q.T) / (2 * sizeof(float));
                 q.PT = m.pt_p;
                 q.LT = m.pt_l;
                 q.kt = m.pt_kt;
                 q.TQ = ts;
                 q.TL = ts + half;
                 ts += 2 * half;
-                if (!tile_kl) continue;      // TV alone: order_tv
-                for (int64_t xt = 0; xt * 128 < m.n_v; ++xt)
-                    for (int at = 0; at * 64 < T_per[i]; ++at)
-                        order_pipe.push_back({m.pt_kt, BatchItem{i, (int32_t)xt, at, 0}});
-            }
-            costliest_first(order_pipe);
-        }
-        // the tensor-core KL's items, those of 128 targets first
-        std::vector<std::pair<int64_t, BatchItem>> order_kl;
-        int32_t kl_wide = 0;
-        for (int tile = 128; mma && tile >= 64; tile -= 64) {
-            std::vector<std::pair<int64_t, BatchItem>> part;
-            for (int i = 0; i < n_items; ++i) {
-                if (probs[i].ktile != tile) continue;
-                for (int64_t xt = 0; xt * 128 < ms[i]->n_v; ++xt)
-                    for (int at = 0; at * tile < T_per[i]; ++at)
-                        part.push_back({probs[i].knch, BatchItem{i, (int32_t)xt, at, 0}});
-            }
-            costliest_first(part);
-            order_kl.insert(order_kl.end(), part.begin(), part.end());
-            if (tile == 128) kl_wide = (int32_t)order_kl.size();
-        }
-        // the pipelined TV pass alone: a problem's last target tile of at most 32 or
-        // 16 targets in items of that many and more rows (twelve uneven maps of 28 to
-        // 246 targets: 13 % of padded sums instead of 25 %, the tile pass 861 -> 855 us)
-        std::vector<std::pair<int64_t, BatchItem>> order_tv;
-        if (pipe_ok && !tile_kl) {
-            for (int i = 0; i < n_items; ++i) {
-                const int nat = (T_per[i] + 63) / 64, rem = T_per[i] - 64 * (nat - 1);
-                const int last = rem <= 16 ? 2 : rem <= 32 ? 1 : 0;
+                // the pipelined TV pass alone: a problem's last target tile of at most 32 or
+                // 16 targets in items of that many and more rows (twelve uneven maps of 28 to
+                // 246 targets: 13 % of padded sums instead of 25 %, the tile pass 861 -> 855 us)
+                const int nat = (q.T + 63) / 64, rem = q.T - 64 * (nat - 1);
+                const int last = K.tile_kl ? 0 : rem <= 16 ? 2 : rem <= 32 ? 1 : 0;
                 for (int at = 0; at < nat; ++at) {
                     const int shape = at == nat - 1 ? last : 0;
-                    for (int64_t xt = 0; xt * (128 << shape) < ms[i]->n_v; ++xt)
-                        order_tv.push_back({tiled_k32(ms[i]->k_pad), BatchItem{i, (int32_t)xt, at, shape}});
+                    for (int64_t xt = 0; xt * (128 << shape) < q.n_v; ++xt)
+                        K.pipe.push_back({m.pt_kt, BatchItem{j, (int32_t)xt, at, shape}});
                 }
             }
-            costliest_first(order_tv);
+            costliest_first(K.pipe);
+            // the tensor-core KL's items, those of 128 targets first
+            for (int tile = 128; K.mma && tile >= 64; tile -= 64) {
+                std::vector<std::pair<int64_t, BatchItem>> part;
+                for (int j = 0; j < K.count; ++j) {
+                    const BatchProblem &q = probs[K.first + j];
+                    if (q.ktile != tile) continue;
+                    for (int64_t xt = 0; xt * 128 < q.n_v; ++xt)
+                        for (int at = 0; at * tile < q.T; ++at)
+                            part.push_back({q.knch, BatchItem{j, (int32_t)xt, at, 0}});
+                }
+                costliest_first(part);
+                K.kl.insert(K.kl.end(), part.begin(), part.end());
+                if (tile == 128) K.kl_wide = (int32_t)K.kl.size();
+            }
         }
-        const size_t o_items_pipe = o_items + align256(order.size() * sizeof(BatchItem));
-        const size_t o_items_tv = o_items_pipe + align256(order_pipe.size() * sizeof(BatchItem));
-        const size_t o_items_kl = o_items_tv + align256(order_tv.size() * sizeof(BatchItem));
-        meta.resize(o_items_kl + order_kl.size() * sizeof(BatchItem));
+        size_t meta_bytes = o_items;
+        auto place = [&](const std::vector<std::pair<int64_t, BatchItem>> &v) {
+            const size_t o = meta_bytes;
+            meta_bytes += align256(v.size() * sizeof(BatchItem));
+            return o;
+        };
+        for (Kind &K : kinds) {
+            K.o_staged = place(K.staged);
+            K.o_pipe = place(K.pipe);
+            K.o_kl = place(K.kl);
+        }
+        meta.resize(meta_bytes);
         std::memcpy(meta.data() + o_probs, probs.data(), n_items * sizeof(BatchProblem));
         // trace domains; gradients per item in consecutive blocks [T_i][n_t_i]
         {
             int64_t go = 0;
-            for (int i = 0; i < n_items; ++i) {
-                fill_batch_trace_dom(meta.data() + o_doms + i * dom_bytes, *ms[i],
-                                     (trace_f == DD_F_TV && probs[i].out_tv) ? probs[i].out_tv : probs[i].out_kl,
-                                     T_per[i], grads ? grads + go : nullptr);
-                go += (int64_t)trace_scratch_bytes(*ms[i], T_per[i], false);
+            for (int j = 0; j < n_items; ++j) {
+                const DevMesh &m = *ms[item[j]];
+                fill_batch_trace_dom(meta.data() + o_doms + j * dom_bytes, m,
+                                     (trace_f == DD_F_TV && probs[j].out_tv) ? probs[j].out_tv : probs[j].out_kl,
+                                     probs[j].T, grads ? grads + go : nullptr);
+                go += (int64_t)trace_scratch_bytes(m, probs[j].T, false);
             }
         }
-        for (size_t j = 0; j < order.size(); ++j)
-            std::memcpy(meta.data() + o_items + j * sizeof(BatchItem), &order[j].second, sizeof(BatchItem));
-        for (size_t j = 0; j < order_pipe.size(); ++j)
-            std::memcpy(meta.data() + o_items_pipe + j * sizeof(BatchItem), &order_pipe[j].second, sizeof(BatchItem));
-        for (size_t j = 0; j < order_tv.size(); ++j)
-            std::memcpy(meta.data() + o_items_tv + j * sizeof(BatchItem), &order_tv[j].second, sizeof(BatchItem));
-        for (size_t j = 0; j < order_kl.size(); ++j)
-            std::memcpy(meta.data() + o_items_kl + j * sizeof(BatchItem), &order_kl[j].second, sizeof(BatchItem));
+        auto write = [&](size_t o, const std::vector<std::pair<int64_t, BatchItem>> &v) {
+            for (size_t j = 0; j < v.size(); ++j)
+                std::memcpy(meta.data() + o + j * sizeof(BatchItem), &v[j].second, sizeof(BatchItem));
+        };
+        for (const Kind &K : kinds) {
+            write(K.o_staged, K.staged);
+            write(K.o_pipe, K.pipe);
+            write(K.o_kl, K.kl);
+        }
         if ((st = upload(ctx, S_META, meta.data(), meta.size())) != DD_OK) return st;
         dmeta = reinterpret_cast<uint8_t *>(ctx->scratch[S_META]);
-        int64_t fix_blocks = 0, work = 0;
-        for (int i = 0; i < n_items; ++i) {
-            if (probs[i].out_kl) fix_blocks += fix_row_blocks(probs[i].n_v);
-            work += ms[i]->n_v * ms[i]->k_pad * (int64_t)T_per[i];
-        }
-        const BatchProblem *dprobs = reinterpret_cast<const BatchProblem *>(dmeta + o_probs);
         int32_t *dcounter = reinterpret_cast<int32_t *>(dmeta + o_counter);
-        const BatchItem *ditems_pipe = reinterpret_cast<const BatchItem *>(dmeta + o_items_pipe);
-        const BatchKlMma kl{reinterpret_cast<const BatchItem *>(dmeta + o_items_kl), kl_wide, (int32_t)order_kl.size(),
-                            max_T, max_k, ctx->d_err, (f_mask & DD_F_TV) != 0};
-        const BatchKlMma *klp = mma ? &kl : nullptr;
-        auto staged = [&]() {
-            launch_batch_fields(dprobs, (int32_t)n_items, reinterpret_cast<const BatchItem *>(dmeta + o_items),
-                                (int32_t)order.size(), dcounter, ctx->stream, fix_blocks, klp);
-        };
-        auto pipelined = [&]() {
-            const bool narrow = !order_tv.empty();
-            launch_batch_fields_pipe(dprobs, (int32_t)n_items,
-                                     narrow ? reinterpret_cast<const BatchItem *>(dmeta + o_items_tv) : ditems_pipe,
-                                     (int32_t)(narrow ? order_tv.size() : order_pipe.size()), dcounter,
-                                     ctx->d_err, ctx->stream, fix_blocks, max_tiles, (f_mask & DD_F_KL) != 0,
-                                     (f_mask & DD_F_TV) != 0, klp);
-        };
-        if (pipe_ok && batch_launch_choice(n_items, work, f_mask | (mma ? kBatchTensorKl : 0), staged, pipelined, ctx->stream) == 1)
-            pipelined();
-        else
-            staged();
+        for (const Kind &K : kinds) {
+            if (K.count == 0) continue;
+            const BatchProblem *dprobs = reinterpret_cast<const BatchProblem *>(dmeta + o_probs) + K.first;
+            auto items = [&](size_t o) { return reinterpret_cast<const BatchItem *>(dmeta + o); };
+            const BatchKlMma kl{items(K.o_kl), K.kl_wide, (int32_t)K.kl.size(), K.max_T, K.max_k, ctx->d_err,
+                                (f_mask & DD_F_TV) != 0};
+            const BatchKlMma *klp = K.mma ? &kl : nullptr;
+            auto staged = [&]() {
+                launch_batch_fields(dprobs, K.count, items(K.o_staged), (int32_t)K.staged.size(), dcounter, ctx->stream,
+                                    K.fix_blocks, klp);
+            };
+            auto pipelined = [&]() {
+                launch_batch_fields_pipe(dprobs, K.count, items(K.o_pipe), (int32_t)K.pipe.size(), dcounter, ctx->d_err,
+                                         ctx->stream, K.fix_blocks, K.max_tiles, (f_mask & DD_F_KL) != 0,
+                                         (f_mask & DD_F_TV) != 0, klp);
+            };
+            if (K.tile && pipe_ok &&
+                batch_launch_choice(K.count, K.work, f_mask | (K.mma ? kBatchTensorKl : 0), staged, pipelined,
+                                    ctx->stream) == 1)
+                pipelined();
+            else
+                staged();
+        }
         CK(cudaGetLastError(), "batch field launch");
         bool host = false;
         if (sf == 0) {

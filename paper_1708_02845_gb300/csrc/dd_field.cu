@@ -1680,7 +1680,7 @@ void launch_batch_fix(const BatchProblem *d_probs, int32_t n_probs, int64_t fix_
 
 void launch_batch_fields(const BatchProblem *d_probs, int32_t n_probs, const BatchItem *d_items, int32_t n_items,
                          int32_t *d_counter, cudaStream_t s, int64_t fix_blocks, const BatchKlMma *kl_mma) {
-    if (n_items <= 0) return;
+    if (n_items <= 0 && !kl_mma) return;
     const size_t smem = (size_t)(2 * kTileB + kTileB + 4) * (256 + 16) * sizeof(float);
     auto tile = [&](auto kern) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1704,7 +1704,7 @@ void launch_batch_fields(const BatchProblem *d_probs, int32_t n_probs, const Bat
 void launch_batch_fields_pipe(const BatchProblem *d_probs, int32_t n_probs, const BatchItem *d_items,
                               int32_t n_items, int32_t *d_counter, int *err, cudaStream_t s, int64_t fix_blocks,
                               int64_t max_tiles, bool f_kl, bool f_tv, const BatchKlMma *kl_mma) {
-    if (n_items <= 0) return;
+    if (n_items <= 0 && !kl_mma) return;
     if (kl_mma) f_kl = false;        // in the tile pass
     if (f_kl || f_tv) {
         {
