@@ -266,9 +266,9 @@ dd_status fields_into(dd_ctx *ctx, DevMesh &m, const int32_t *d_targets, int32_t
         if ((st = ensure_scratch(ctx, S_STAGE, sparse_stage_bytes(m.k_pad, T))) != DD_OK) return st;
         float4 *stage = reinterpret_cast<float4 *>(ctx->scratch[S_STAGE]);
         launch_stage_targets(m.P, m.n_v, m.k_pad, d_targets, T, stage, ctx->stream);
-        // (per-kernel timing is by stream: with it on, everything stays on the caller's)
+        // (per-kernel timing is by stream: with it on for the caller's, everything stays there)
         SideStream side{};
-        const bool fork = klt && (kl || tv) && g_kt_on.load(std::memory_order_relaxed) == 0;
+        const bool fork = klt && (kl || tv) && !kernel_timing_on(ctx->stream);
         if (fork) {
             if ((st = ensure_side(ctx)) != DD_OK) return st;
             side = SideStream{ctx->side, ctx->side_ev[3], ctx->side_ev[4]};
@@ -385,6 +385,12 @@ void kt_fold(KTimer &t) {
 }  // namespace
 
 int64_t memory_releases() { return g_releases.load(std::memory_order_relaxed); }
+
+bool kernel_timing_on(cudaStream_t s) {
+    if (!g_kt_on.load(std::memory_order_relaxed)) return false;
+    std::lock_guard<std::mutex> lock(g_kt_mutex);
+    return g_kt.find(s) != g_kt.end();
+}
 
 KMark::KMark(const char *n, cudaStream_t s) {
     if (!g_kt_on.load(std::memory_order_relaxed)) return;

@@ -339,6 +339,7 @@ struct dd_ctx {
 // stream, a KMark around a launch on that stream records a CUDA event before
 // and after it; totals per kernel name are folded in when read.  Without
 // timing enabled a KMark costs one relaxed atomic load.
+bool kernel_timing_on(cudaStream_t s);      // for launches on s
 struct KMark {
     KMark(const char *name, cudaStream_t s);
     ~KMark();
