@@ -268,11 +268,12 @@ dd_status fields_into(dd_ctx *ctx, DevMesh &m, const int32_t *d_targets, int32_t
         launch_stage_targets(m.P, m.n_v, m.k_pad, d_targets, T, stage, ctx->stream);
         // (per-kernel timing is by stream: with it on for the caller's, everything stays there)
         SideStream side{};
-        const bool fork = klt && (kl || tv) && !kernel_timing_on(ctx->stream);
-        if (fork) {
-            if ((st = ensure_side(ctx)) != DD_OK) return st;
-            side = SideStream{ctx->side, ctx->side_ev[3], ctx->side_ev[4]};
+        bool fork = klt && (kl || tv) && !kernel_timing_on(ctx->stream);
+        if (fork && ensure_side(ctx) != DD_OK) {      // without a second stream all of it runs on the caller's
+            ctx->err.clear();
+            fork = false;
         }
+        if (fork) side = SideStream{ctx->side, ctx->side_ev[3], ctx->side_ev[4]};
         launch_sparse_fields(m, d_targets, stage, T, kl, tv, klt, prec == DD_PREC_SPARSE_MERGED, ctx->d_err,
                              ctx->stream, fork ? &side : nullptr);
         CK(cudaGetLastError(), "sparse field kernel launch");
