@@ -297,8 +297,9 @@ __device__ __forceinline__ void stream_rows(const float *__restrict__ P, int64_t
 }
 
 // floats per staged row of two_pass_pair_kernel: k_pad rounded up to whole groups
-// of 32 lanes x one float4
-constexpr int kMaxGroups = 104;      // 200 KB of staged rows of one target
+// of 32 lanes x one float4; eight rows (four a target) in at most 200 KB
+constexpr int64_t kPairPitch = 6400;
+constexpr int kPairGroups = kPairPitch / 128;
 __host__ __device__ constexpr int64_t two_pass_pair_pitch(int64_t k_pad) { return (k_pad + 127) / 128 * 128; }
 
 // floats per staged row of two_pass_kernel: k_pad rounded up to whole
@@ -496,17 +497,16 @@ __global__ void __launch_bounds__(512, 1) two_pass_pair_kernel(const float *__re
     constexpr int TT = 2, U = 4;             // targets; float4 per lane and buffer
     extern __shared__ __align__(16) float fsm[];
     __shared__ float tab[2 * kLogTab];
-    __shared__ unsigned char tz[kMaxGroups];      // a target's group of entries (32 float4) holds a 0
+    __shared__ unsigned char tz[kPairGroups];      // a target's group of entries (32 float4) holds a 0
     // the staged rows zero-padded to whole groups of 32 float4 (two_pass_pair_pitch):
     // every lane of a group reads its target entries without a test
     const int64_t kp = two_pass_pair_pitch(k_pad);
-    const int a = 0;
-    for (int i = threadIdx.x; i < kMaxGroups; i += blockDim.x) tz[i] = 0;
+    for (int i = threadIdx.x; i < kPairGroups; i += blockDim.x) tz[i] = 0;
     __syncthreads();
     for (int i = 0; i < TT; ++i)
         for (int64_t b = threadIdx.x; b < kp; b += blockDim.x) {
             const bool in = b < k_pad;
-            const int64_t o = (int64_t)(a + i) * k_pad + b;
+            const int64_t o = i * k_pad + b;
             float *t = fsm + 4 * i * kp + b;
             const float p = in ? sP[o] : 0.0f;
             t[0] = p;
@@ -561,7 +561,7 @@ __global__ void __launch_bounds__(512, 1) two_pass_pair_kernel(const float *__re
         if (FAM == kAlpha) {
             bool z = false;
 #pragma unroll
-            for (int u = 0; u < U; ++u) z |= has_zero(v[u]) || tz[min((c0 >> 5) + u, kMaxGroups - 1)];
+            for (int u = 0; u < U; ++u) z |= has_zero(v[u]) || tz[min((c0 >> 5) + u, kPairGroups - 1)];
             plain = !__any_sync(0xffffffffu, z) && plain;
         }
         if (plain) {
@@ -602,7 +602,7 @@ __global__ void __launch_bounds__(512, 1) two_pass_pair_kernel(const float *__re
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
             }
-            if (lane == 0) out[(int64_t)(a + i) * n_v + x] = sum;
+            if (lane == 0) out[i * n_v + x] = sum;
             sums[i] = zero2;
         }
     };
@@ -664,8 +664,9 @@ dd_status launch_fdiv(const float *P, int64_t n_v, int64_t k_pad, const float4 *
         // two passes (hardware mantissa logs, then the table form near the target)
         const float *sF = sE + (int64_t)T * k_pad;
         // two targets of a P of 256 MB or more: both in one pass
-        const size_t smem_pair = 8 * (size_t)two_pass_pair_pitch(k_pad) * sizeof(float);
-        if (T == 2 && n_v * k_pad * (int64_t)sizeof(float) >= (int64_t)256 << 20 && smem_pair <= 200 * 1024) {
+        const int64_t pitch = two_pass_pair_pitch(k_pad);
+        const size_t smem_pair = 8 * (size_t)pitch * sizeof(float);
+        if (T == 2 && n_v * k_pad * (int64_t)sizeof(float) >= (int64_t)256 << 20 && pitch <= kPairPitch) {
             auto kern = family == DD_DIV_ALPHA ? two_pass_pair_kernel<kAlpha> : two_pass_pair_kernel<kKlRev>;
             cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_pair);
             const int64_t blocks = std::min<int64_t>(sms, (n_v + 15) / 16);
