@@ -189,8 +189,9 @@ dd_status dd_check_mesh(const double *xy, int64_t n_v, const int32_t *tri, int64
 
 /* Validate (as dd_check_mesh) and copy a mesh to the device; builds the
  * triangle adjacency, the vertex-to-triangle and vertex-neighbour lists and
- * the cotangent Laplacian (Section IV).  Arguments as in dd_check_mesh, all
- * host memory.  *mesh_id receives the handle.  Errors: DD_EINVAL, DD_ENOMEM,
+ * the cotangent Laplacian (Section IV), and the walk's ready-made crossings
+ * (192 bytes a triangle on the device, besides 64 for its record).  Arguments
+ * as in dd_check_mesh, all host memory.  *mesh_id receives the handle.  Errors: DD_EINVAL, DD_ENOMEM,
  * DD_ECUDA. */
 dd_status dd_load_mesh(dd_ctx *ctx, const double *xy, int64_t n_v, const int32_t *tri, int64_t n_t,
                        const int32_t *loop_idx, const int64_t *loop_off, int32_t n_loops,

@@ -1388,6 +1388,13 @@ constexpr int kPipeShape = 3;      // the pipelined tile on the tiled layout (si
 // A last target tile of at most 32 or 16 targets goes to a launch of its own
 // with that many and more rows a CTA, where that takes less: 333 targets are
 // five tiles and 13 targets, not six tiles (300 x 300 cells: 4.44 -> 4.02 ms).
+//
+// The weights: a tile's time for its share of sums, the 128 x 64 tile's 100.
+// Measured on 18,241 to 76,609 rows of 640 and 1,216 columns: 64 x 64 96 to 102,
+// 32 x 64 97 to 109 (the upper end with one target tile, the lower with ten),
+// 256 x 32 98 to 104, 128 x 32 103 to 111, 512 x 16 108 to 119, 128 x 16 120 to
+// 136 (179 where it leaves an SM one tile).  What decides is the rounding of the
+// share, factors of two and more; the weights only order tiles of equal shares.
 void launch_pipe(const TiledArgs &ta, int64_t n_v, int32_t T, float *out_kl, float *out_tv, int *err,
                  cudaStream_t s) {
     const int nat = (T + kTiledRows - 1) / kTiledRows;
