@@ -40,7 +40,9 @@
 // where what the slices leave does not average out: below 8e-8, against 1.6e-7
 // (4.4e-7).  The pairs below kMmaExactBelow are recomputed in the exact form as
 // there.  The extra columns cost 0.3 % of a call with a chunk more (grid450,
-// 1,024 targets: 54.95 -> 55.13 ms) and up to 1 % of small ones.
+// 1,024 targets: 54.95 -> 55.13 ms) and up to 1 % of small ones.  Slicing P, once
+// a map, takes a quarter longer with the chunks' sums (201 x 201 cells: 131 -> 165
+// us, 82 % of the issue slots).
 //
 // Kernel: persistent, one CTA per SM walks 128-row x N-target output tiles.
 // The operands lie in global memory chunk by chunk in the shared-memory image
@@ -55,7 +57,7 @@
 // (45.3 ms) and a recompute of fewer pairs (1.6 against 4.1 ms) in place of
 // the 94.5 ms KL+TV tile pass: a call 98.9 -> 55.1 ms.  grid140, 64 targets:
 // 34 us (N = 64; the slices' 131 MB from memory bound it), a call 321 -> 181
-// us.  KL alone, 201 x 201 cells, 7 targets: a call 228 -> 104 us.
+// us.  KL alone, 201 x 201 cells, 7 targets: a call 228 -> 106 us.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -423,10 +425,13 @@ __device__ __forceinline__ int row_grid(float x, float y) {
     return min(max((int)(mx >> 23), 40), 200) - 7;
 }
 
+constexpr float kMagic = 12582912.0f;       // 1.5 * 2^23
+constexpr int kMagicBits = 0x4B400000;
+
 // The slices of P's rows and e_x, one warp per row (rows past n_v: zeros), two
 // columns a lane.  Rows that the exactness argument does not cover (an entry
 // that is negative, infinite or NaN, or a sum above 1.01) raise *bad.
-__global__ void __launch_bounds__(256) kl_rows_kernel(const float *__restrict__ P, int64_t n_v, int64_t n_pad,
+__global__ void __launch_bounds__(256, 8) kl_rows_kernel(const float *__restrict__ P, int64_t n_v, int64_t n_pad,
                                                       int64_t k_pad, uint8_t *__restrict__ A,
                                                       float2 *__restrict__ ex, int *__restrict__ bad) {
     __shared__ Log2Tab tab;
@@ -446,11 +451,15 @@ __global__ void __launch_bounds__(256) kl_rows_kernel(const float *__restrict__ 
             *reinterpret_cast<__nv_bfloat162 *>(img + s * BM * ROW_B) =
                 __nv_bfloat162(__float2bfloat16_rn(rx), __float2bfloat16_rn(ry));
         };
-        float2 last = make_float2(0.f, 0.f);      // the entries of a last chunk that is not whole
+        // (k_pad is a multiple of 4; the next chunk's entries are read ahead of this one's sums)
+        auto entries = [&](int c) {
+            const int b = c * BK + 2 * lane;
+            return x < n_v && b < k_pad ? *reinterpret_cast<const float2 *>(P + x * k_pad + b) : make_float2(0.f, 0.f);
+        };
+        float2 ahead = entries(0);
         for (int c = 0; c < nb; ++c) {
-            const int64_t b = (int64_t)c * BK + 2 * lane;
-            float2 p = make_float2(0.f, 0.f);
-            if (x < n_v && b < k_pad) p = *reinterpret_cast<const float2 *>(P + x * k_pad + b);   // k_pad is a multiple of 4
+            float2 p = ahead;
+            if (c + 1 < nb) ahead = entries(c + 1);
             wrong |= !(p.x >= 0.f && p.y >= 0.f && p.x <= 2.f && p.y <= 2.f);
             sum += p.x + p.y;
 #pragma unroll
@@ -463,14 +472,16 @@ __global__ void __launch_bounds__(256) kl_rows_kernel(const float *__restrict__ 
                     pair_add(es, ec, a);
                 }
             }
-            last = p;
             const int g = row_grid(p.x, p.y);
             float q = __int_as_float(g << 23), iq = __int_as_float((254 - g) << 23);
-            float n[NSA];
+            int n[NSA];
 #pragma unroll
             for (int s = 0; s < NSA; ++s) {
-                const float nx = rintf(p.x * iq), ny = rintf(p.y * iq), rx = nx * q, ry = ny * q;
-                n[s] = q * (float)__reduce_add_sync(0xffffffffu, (int)(nx + ny));    // below 2^14 of the grid
+                // to the nearest multiple by adding 1.5 * 2^23, whose last bits then hold it (rintf
+                // and conversions to int run at a quarter of the rate)
+                const float tx = __fmaf_rn(p.x, iq, kMagic), ty = __fmaf_rn(p.y, iq, kMagic);
+                const float rx = (tx - kMagic) * q, ry = (ty - kMagic) * q;
+                n[s] = __float_as_int(tx) + __float_as_int(ty) - 2 * kMagicBits;
                 if (c < whole) store(s, rx, ry);
                 p.x -= rx;
                 p.y -= ry;
@@ -478,7 +489,16 @@ __global__ void __launch_bounds__(256) kl_rows_kernel(const float *__restrict__ 
                 iq *= 0x1p9f;
             }
             if (c < whole) img += A_BYTES;
-            if (lane == 0) rs[c] = make_float2(n[0] + n[1], n[2] + n[3]);      // both exact
+            // the slices' sums, up to 2^14 of their grids: two to a word, 2^-9 of a grid apart
+            const int n01 = __reduce_add_sync(0xffffffffu, n[0] * 65536 + n[1]),
+                      n23 = __reduce_add_sync(0xffffffffu, n[2] * 65536 + n[3]);
+            if (lane == 0) {
+                auto both = [](int v, int g) {      // exact
+                    const int low = (int)(short)(v & 0xffff);
+                    return __int_as_float(g << 23) * ((float)((v - low) >> 16) + 0x1p-9f * (float)low);
+                };
+                rs[c] = make_float2(both(n01, g), both(n23, g - 18));
+            }
         }
         __syncwarp();
         // the rest: entries of P behind the whole chunks, then the sums
@@ -487,7 +507,7 @@ __global__ void __launch_bounds__(256) kl_rows_kernel(const float *__restrict__ 
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
                 const int64_t b = (int64_t)c * BK + 2 * lane + i, j = b - k_pad;
-                h[i] = j < 0 ? (i ? last.y : last.x) : 0.0f;
+                h[i] = x < n_v && j < 0 ? P[x * k_pad + b] : 0.0f;
                 l[i] = 0.0f;
                 if (j >= 0 && j < nb) two_sum(rs[j].x, rs[j].y, h[i], l[i]);
             }
