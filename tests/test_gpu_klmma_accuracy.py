@@ -53,3 +53,32 @@ def test_error_against_64_bits(N, T):
         assert np.sqrt((rel * rel).mean()) <= 8e-8
     finally:
         dd.dd_destroy(ctx)
+
+
+@pytest.mark.parametrize("k", [4300, 4352])       # 68 chunks: their sums take two more, one shared with P's columns or none
+@pytest.mark.parametrize("T", [3, 70])
+def test_more_chunks_than_one_holds_sums_of(k, T):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from synthetic.meshes import disk_rings
+    dd, ctx = ctx_and_lib()
+    try:
+        mid = load(dd, ctx, disk_rings(1, k))         # one interior vertex
+        n = k + 1
+        rng = np.random.default_rng(k)
+        P = np.exp(rng.uniform(0.3, 0.6, n)[:, None] * rng.standard_normal((n, k)))
+        P[0] = 1.0
+        P /= P.sum(1, keepdims=True)
+        dd.dd_set_poisson_kernel(ctx, mid, P)
+        P = P.astype(np.float32).astype(np.float64)
+        out = torch.full((1, T, n), float("nan"), dtype=torch.float32, device="cuda")
+        dd.dd_distance(ctx, mid, np.zeros(T, np.int32), dd.DD_F_KL, dd.DD_PREC_FP32, out)
+        dd.dd_sync(ctx)
+        got = out[0].cpu().numpy().astype(np.float64)
+        L = np.log(P)
+        ref = (P * L).sum(1) - P @ L[0]
+        assert np.array_equal(got, np.broadcast_to(got[0], got.shape)) and got[0, 0] == 0.0
+        rel = (got[0] / np.where(ref > 0, ref, 1.0) - 1.0)[(ref > 0.07) & (ref < 0.25)]
+        assert len(rel) > 1000 and np.sqrt((rel * rel).mean()) <= 8e-8
+    finally:
+        dd.dd_destroy(ctx)
