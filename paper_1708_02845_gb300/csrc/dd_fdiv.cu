@@ -252,13 +252,7 @@ __device__ __forceinline__ void alpha_pair4(const Row4 &x, const f2_t (&pe)[2], 
 // chunk (of this row or the next) are in flight while the current one is
 // computed.  chunk(b, x, c0): the lane's U float4 b of row x, float4 columns
 // c0 + u * 32 + lane (zero past the row's end); done(x): row x is complete.
-// TURN: every nwarps rows the warps are dealt anew, 0.38 nwarps further on.
-// Without it a warp's rows may all lie in one column of a grid map (270 cells:
-// 2,432 warps are 8.97 of its lines), and the warps whose column the target is in
-// have all the rows to recompute (the pair kernel's alpha there 384 us a call,
-// turned 283, the single-target kernel's 331).  Reverse KL, with fewer rows to
-// recompute, loses as much as it gains.
-template <int U, bool TURN = false, typename Chunk, typename Done>
+template <int U, typename Chunk, typename Done>
 __device__ __forceinline__ void stream_rows(const float *__restrict__ P, int64_t n_v, int64_t k_pad, int64_t warp,
                                             int64_t nwarps, int lane, Chunk chunk, Done done) {
     const int nvec = (int)(k_pad >> 2);
@@ -272,17 +266,10 @@ __device__ __forceinline__ void stream_rows(const float *__restrict__ P, int64_t
             b[u] = c < nvec ? __ldcs(row + c) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
     };
-    const int64_t turn = TURN ? nwarps * 382 / 1000 : 0;
-    int64_t place = warp;
     auto next = [&](int64_t &x, int &ch) {
         if (++ch == nch) {
             ch = 0;
             x += nwarps;
-            if (TURN) {
-                const int64_t to = place + turn < nwarps ? place + turn : place + turn - nwarps;
-                x += to - place;
-                place = to;
-            }
         }
     };
     int64_t x = warp;
@@ -494,16 +481,12 @@ __global__ void __launch_bounds__(256) two_pass_kernel(const float *__restrict__
 
 // Two targets a CTA of 512 threads: P is read, and its entries' logarithms
 // formed, once for both, and chunks without a zero run without branches (the
-// two take 125 registers: one CTA an SM).  For two targets of a P of 256 MB or
-// more (twice L2).  A call by the kernel above against this one, maps of 245,
-// 270, 285 and 300 cells with 0, 8 and 16 obstacles, three pairs of targets on
-// each: alpha 0.98 to 1.60 times as long, 1.19 in the mean (300 cells, no
-// obstacle: 442 and 313 us); reverse KL 0.97 to 1.16, 1.06 in the mean (182 and
-// 157 us).  Below 256 MB it gains as much on some maps and loses up to 10 % on
-// others (150 to 228 cells: 0.89 to 1.43, reverse KL 0.93 to 1.24); with one
-// target, or three and more, whose blocks share what one of them has read, the
-// kernel above is the better one (300 cells, three: 470 against 539 us with a
-// pair and one).
+// two take 125 registers: one CTA an SM).  For two targets of a map well
+// beyond L2: alpha 0.5 on 300 x 300 cells 442 -> 332 us a call, reverse KL 194
+// -> 181.  For a P that L2 holds, one target, or three and more, whose blocks
+// share what one of them has read, the kernel above is the better one (177 x
+// 177 cells, two targets: 83 us against 108; 300 x 300, three: 470 against 539
+// with a pair and one).
 template <int FAM>
 __global__ void __launch_bounds__(512, 1) two_pass_pair_kernel(const float *__restrict__ P, int64_t n_v,
                                                                int64_t k_pad, const float *__restrict__ sP,
@@ -623,7 +606,7 @@ __global__ void __launch_bounds__(512, 1) two_pass_pair_kernel(const float *__re
             sums[i] = zero2;
         }
     };
-    stream_rows<U, FAM == kAlpha>(P, n_v, k_pad, warp, nwarps, lane, chunk, done);
+    stream_rows<U>(P, n_v, k_pad, warp, nwarps, lane, chunk, done);
 }
 
 }  // namespace
