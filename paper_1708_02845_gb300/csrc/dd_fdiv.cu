@@ -481,12 +481,19 @@ __global__ void __launch_bounds__(256) two_pass_kernel(const float *__restrict__
 
 // Two targets a CTA of 512 threads: P is read, and its entries' logarithms
 // formed, once for both, and chunks without a zero run without branches (the
-// two take 125 registers: one CTA an SM).  For two targets of a map well
-// beyond L2: alpha 0.5 on 300 x 300 cells 442 -> 332 us a call, reverse KL 194
-// -> 181.  For a P that L2 holds, one target, or three and more, whose blocks
-// share what one of them has read, the kernel above is the better one (177 x
-// 177 cells, two targets: 83 us against 108; 300 x 300, three: 470 against 539
-// with a pair and one).
+// two take 125 registers: one CTA an SM).  For two targets of a P of 256 MB or
+// more (twice L2).  A call by the kernel above against this one, maps of 245,
+// 270, 285 and 300 cells with 0, 8 and 16 obstacles, four pairs of targets on
+// each: alpha 0.86 to 1.43 times as long, 1.18 in the mean (300 cells, no
+// obstacle: 443 and 330 us), two of 48 below 0.97 (270 cells, whose lines the
+// warps' stride nearly divides by nine: the warps at the target's column have
+// most of the rows to recompute, 331 and 385 us; other strides move that to
+// other targets); reverse KL 0.97 to 1.18, 1.07 in the mean (182 and 153 us).
+// Between 150 and 228 cells, most of whose P L2 holds: alpha 0.87 to 1.45, 1.16
+// in the mean, reverse KL 0.94 to 1.24, 1.03 in the mean, seven of 144 below
+// 0.97; smaller maps stay with the kernel above.  With one target, or three and
+// more, whose blocks share what one of them has read, the kernel above is the
+// better one (300 cells, three: 470 against 539 us with a pair and one).
 template <int FAM>
 __global__ void __launch_bounds__(512, 1) two_pass_pair_kernel(const float *__restrict__ P, int64_t n_v,
                                                                int64_t k_pad, const float *__restrict__ sP,
