@@ -489,9 +489,9 @@ __global__ void __launch_bounds__(256) two_pass_kernel(const float *__restrict__
 // warps' stride nearly divides by nine: the warps at the target's column have
 // most of the rows to recompute, 331 and 385 us; other strides move that to
 // other targets); reverse KL 0.97 to 1.18, 1.07 in the mean (182 and 153 us).
-// Between 150 and 228 cells, most of whose P L2 holds: alpha 0.87 to 1.45, 1.16
-// in the mean, reverse KL 0.94 to 1.24, 1.03 in the mean, seven of 144 below
-// 0.97; smaller maps stay with the kernel above.  With one target, or three and
+// Between 150 and 228 cells (P of 65 to 250 MB): alpha 0.87 to 1.45, 1.16 in the
+// mean, reverse KL 0.94 to 1.24, 1.03 in the mean, seven of 144 below 0.97:
+// these stay with the kernel above.  With one target, or three and
 // more, whose blocks share what one of them has read, the kernel above is the
 // better one (300 cells, three: 470 against 539 us with a pair and one).
 template <int FAM>
